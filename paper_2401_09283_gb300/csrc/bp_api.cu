@@ -86,7 +86,7 @@ constexpr int ZB = bpk::ZB_VJP;
 // Stage the per-view inputs and run the FP64 composition into ctx->geom.
 int prepare_views(bp_ctx* ctx, const bp_proj_desc* pd, const double* P, const double* motion,
                   const double* view_weight, int weight, const VolInfo& vi, cudaStream_t s,
-                  const double** dP, const double** dmotion) {
+                  const double** dP, const double** dmotion, const int** wide) {
   const int V = pd->nviews;
   const void* q = nullptr;
   CK(stage_in(ctx->s_P, P, sizeof(double) * 12 * V, s, &q), "copy P");
@@ -98,8 +98,18 @@ int prepare_views(bp_ctx* ctx, const bp_proj_desc* pd, const double* P, const do
   CK(stage_in(ctx->s_scale, pd->view_scale, sizeof(float) * V, s, &q), "copy view_scale");
   const float* dsc = (const float*)q;
   CK(ensure(ctx->geom, sizeof(ViewGeom) * (size_t)V), "alloc view table");
+  // large problems choose the kernel variant per view on the device (two
+  // launches, one of which returns at once: ~3 us, so not for small ones)
+  *wide = nullptr;
+  bpk::FitInfo fit{pd->dtype, nullptr};
+  if ((long long)vi.nx * vi.ny * vi.nz * V >= (1LL << 28)) {
+    CK(ensure(ctx->wide, sizeof(int) * (size_t)V), "alloc view flags");
+    fit.wide = (int*)ctx->wide.p;
+    *wide = fit.wide;
+  }
   CK(TL(K_COMPOSE, 1, bpk::launch_compose(*dP, *dmotion, dvw, dsc, V, weight == BP_WEIGHT_FDK,
-                                          pd->sid, vi, (ViewGeom*)ctx->geom.p, nullptr, s)),
+                                          pd->sid, vi, (ViewGeom*)ctx->geom.p, nullptr, s,
+                                          fit.wide ? &fit : nullptr)),
      "compose");
   return BP_OK;
 }
@@ -133,7 +143,7 @@ void bp_ctx_destroy(bp_ctx* ctx) {
   if (!ctx) return;
   DeviceGuard g(ctx->device);
   cudaDeviceSynchronize();
-  Buf* bufs[] = {&ctx->geom,   &ctx->grad,   &ctx->partials,   &ctx->shblk,      &ctx->fdk_tab,
+  Buf* bufs[] = {&ctx->geom,   &ctx->wide,   &ctx->grad,   &ctx->partials,   &ctx->shblk,      &ctx->fdk_tab,
                  &ctx->s_proj,
                  &ctx->s_P,    &ctx->s_motion, &ctx->s_vw,     &ctx->s_scale,    &ctx->s_vol,
                  &ctx->s_dvol, &ctx->s_out_motion, &ctx->s_out_P, &ctx->s_out_proj,
@@ -150,7 +160,7 @@ const char* bp_last_error(const bp_ctx* ctx) { return ctx ? ctx->err.c_str() : "
 
 long long bp_ctx_workspace_bytes(const bp_ctx* ctx) {
   if (!ctx) return 0;
-  const Buf* bufs[] = {&ctx->geom,   &ctx->grad,   &ctx->partials,   &ctx->shblk,      &ctx->fdk_tab,
+  const Buf* bufs[] = {&ctx->geom,   &ctx->wide,   &ctx->grad,   &ctx->partials,   &ctx->shblk,      &ctx->fdk_tab,
                        &ctx->s_proj,
                        &ctx->s_P,    &ctx->s_motion, &ctx->s_vw,     &ctx->s_scale,    &ctx->s_vol,
                        &ctx->s_dvol, &ctx->s_out_motion, &ctx->s_out_P, &ctx->s_out_proj,
@@ -270,11 +280,12 @@ int bp_forward(bp_ctx* ctx, const void* proj, const bp_proj_desc* pdesc, const d
     const void* dproj;
     CK(stage_in(ctx->s_proj, proj, proj_bytes(pdesc), s, &dproj), "copy proj");
     const double *dP, *dm;
-    st = prepare_views(ctx, pdesc, P, motion, view_weight, weight, vi, s, &dP, &dm);
+    const int* wide;
+    st = prepare_views(ctx, pdesc, P, motion, view_weight, weight, vi, s, &dP, &dm, &wide);
     if (st) return st;
-    CK(TL(K_FORWARD, 1, bpk::launch_forward(dproj, pdesc->dtype, make_projinfo(pdesc),
+    CK(TL(K_FORWARD, wide ? 2 : 1, bpk::launch_forward(dproj, pdesc->dtype, make_projinfo(pdesc),
                                           (const ViewGeom*)ctx->geom.p, vi,
-                                          weight == BP_WEIGHT_FDK, (float*)dvol, s)),
+                                          weight == BP_WEIGHT_FDK, (float*)dvol, wide, s)),
        "forward kernel");
   }
   if (host_vol) {
@@ -316,7 +327,8 @@ int bp_vjp(bp_ctx* ctx, const float* dL_dvol, const void* proj, const bp_proj_de
   const void* dproj = nullptr;
   if (want_geo) CK(stage_in(ctx->s_proj, proj, proj_bytes(pdesc), s, &dproj), "copy proj");
   const double *dP, *dm;
-  st = prepare_views(ctx, pdesc, P, motion, view_weight, weight, vi, s, &dP, &dm);
+  const int* wide;
+  st = prepare_views(ctx, pdesc, P, motion, view_weight, weight, vi, s, &dP, &dm, &wide);
   if (st) return st;
   void *om = nullptr, *oP = nullptr, *oD = nullptr;
   bool hm = false, hP = false, hD = false;
@@ -345,12 +357,12 @@ int bp_vjp(bp_ctx* ctx, const float* dL_dvol, const void* proj, const bp_proj_de
       if (blocks)
         CK(ensure(ctx->blkimg, sizeof(float) * (size_t)bpk::block_image_floats(pi)),
            "alloc block image");
-      CK(TL(fuse ? K_VJP_FUSED : K_VJP_MOTION, blocks ? 2 : 1,
+      CK(TL(fuse ? K_VJP_FUSED : K_VJP_MOTION, (wide ? 2 : 1) + (blocks ? 1 : 0),
             bpk::launch_vjp_motion(ddvol, dproj, pdesc->dtype, pi, grad,
                                    (const ViewGeom*)ctx->geom.p, vi, weight == BP_WEIGHT_FDK,
                                    deriv == BP_DERIV_BILINEAR_EXACT, (float*)ctx->partials.p,
                                    fuse ? (float*)oD : nullptr,
-                                   blocks ? (float*)ctx->blkimg.p : nullptr, s)),
+                                   blocks ? (float*)ctx->blkimg.p : nullptr, wide, s)),
          "vjp kernel");
     }
     CK(TL(K_REDUCE, 1, bpk::launch_reduce_chain((const float*)ctx->partials.p, nvox > 0 ? ntiles : 0,

@@ -78,22 +78,75 @@ __device__ static void compose_view(const double* __restrict__ P, const double* 
   geom[j] = g;
 }
 
+// Whether most of a view's tiles are wider than the staging buffer (cols x rows
+// pixels): the footprint of a tile half-way to the far end of the volume (the
+// largest w over its corners), from the derivatives of (u/w, v/w) at the
+// centre.  Pc = P' (index frame).
+__host__ __device__ static bool view_wide(const double* Pc, const VolInfo& vi, int cols, int rows) {
+  const double w = Pc[11];
+  if (!(w > 0.0)) return false;
+  double far = w, eu = 0.0, ev = 0.0;
+  const double c[3] = {vi.cx, vi.cy, vi.cz};
+  for (int k = 0; k < 3; ++k) {
+    const double e = TX - 1;  // a tile's extent, the same along every axis
+    far += fabs(Pc[8 + k]) * c[k];
+    eu += e * fabs(Pc[k] - Pc[3] / w * Pc[8 + k]);
+    ev += e * fabs(Pc[4 + k] - Pc[7] / w * Pc[8 + k]);
+  }
+  const double wm = 0.5 * (w + far);
+  return eu / wm > cols || ev / wm > rows;
+}
+
 // One thread per view.
 __global__ void compose_kernel(const double* __restrict__ P, const double* __restrict__ theta,
                                const double* __restrict__ vw, const float* __restrict__ vscale,
                                int V, int fdk, double sid, VolInfo vi, ViewGeom* __restrict__ geom,
-                               double* __restrict__ Phat) {
+                               double* __restrict__ Phat, int* __restrict__ wide, int cols,
+                               int rows) {
   int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= V) return;
   compose_view(P, theta, vw, vscale, fdk, sid, vi, geom, Phat, j);
+  if (wide) wide[j] = view_wide(geom[j].P, vi, cols, rows);
+}
+
+// Pixels of the staging buffer less the taps, their halo and the rounding to
+// 16-byte chunks.
+static void stage_limits(int dtype, int* cols, int* rows) {
+  stage_extent(dtype, cols, rows);
+  *cols -= 3;
+  *rows -= 3;
+}
+
+static const int kWideAll = 0;
+const int* const WIDE_ALL = &kWideAll;
+
+bool all_views_wide(const double* P, int V, int dtype, const VolInfo& vi) {
+  int cols, rows;
+  stage_limits(dtype, &cols, &rows);
+  for (int j = 0; j < V; ++j) {
+    double Pc[12];
+    for (int r = 0; r < 3; ++r) {
+      const double* p = P + 12 * j + 4 * r;
+      Pc[4 * r + 0] = p[0] * vi.A[0];
+      Pc[4 * r + 1] = p[1] * vi.A[5];
+      Pc[4 * r + 2] = p[2] * vi.A[10];
+      Pc[4 * r + 3] = p[0] * vi.A[3] + p[1] * vi.A[7] + p[2] * vi.A[11] + p[3];
+    }
+    if (!view_wide(Pc, vi, cols, rows)) return false;
+  }
+  return true;
 }
 
 cudaError_t launch_compose(const double* P, const double* theta, const double* view_weight,
                            const float* view_scale, int V, int fdk, double sid,
-                           const VolInfo& vi, ViewGeom* geom, double* Phat, cudaStream_t s) {
+                           const VolInfo& vi, ViewGeom* geom, double* Phat, cudaStream_t s,
+                           const FitInfo* fit) {
   if (V <= 0) return cudaSuccess;
+  int cols = 0, rows = 0;
+  if (fit) stage_limits(fit->dtype, &cols, &rows);
   compose_kernel<<<(V + 127) / 128, 128, 0, s>>>(P, theta, view_weight, view_scale, V, fdk, sid,
-                                                  vi, geom, Phat);
+                                                  vi, geom, Phat, fit ? fit->wide : nullptr, cols,
+                                                  rows);
   return cudaGetLastError();
 }
 
@@ -653,7 +706,8 @@ cudaError_t launch_batch_iteration(const BatchTable& tab, unsigned* counter, int
       e = cudaStreamWaitEvent(br->streams[m], br->fork, 0);
       if (e == cudaSuccess)
         e = launch_vjp_motion(J.dvol, J.proj, dtype, J.pi, J.grad, J.geom, J.vi, fdk, exact,
-                              J.partials, nullptr, nullptr, br->streams[m]);
+                              J.partials, nullptr, nullptr, J.unstaged ? WIDE_ALL : nullptr,
+                              br->streams[m]);
       if (e == cudaSuccess) e = cudaEventRecord(br->joins[m], br->streams[m]);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(s, br->joins[m], 0);
     }

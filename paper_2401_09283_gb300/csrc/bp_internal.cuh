@@ -14,6 +14,7 @@
 //                positions keep ~1e-6 px precision up to 1240-px detectors.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
@@ -41,27 +42,30 @@ struct ViewGeom {
   double scale;   // per-view dequantisation scale (1 for float32 data)
 };
 
-// Per (tile, view), in shared memory.
-struct TileView {
-  float U0, V0, W0;   // anchored homogeneous coordinates at the tile centre
-  float ru[3];        // d(u_rel)/d(dq)
-  float rv[3];
-  float rw[3];
-  int au, av;         // anchor pixel
-  float wgt;          // wgt * scale (FP32): weight of a stored sample
-  float wgtd;         // wgt alone: weight of a dequantised sample (data VJP)
-  int mode;           // MODE_*
-  int fu0, fv0;       // detector footprint of the tile (first pixel), clipped
-  int fw, fh;         // footprint size in pixels (0 when unbounded)
-  int csafe;          // every tap pixel and its central-difference neighbours
-                      // (one more pixel each side) lie inside the detector
-  // Staged footprint in shared memory (staged != 0): detector rows
-  // [sv0, sv0 + sh) and 16-byte chunks [sx0, sx0 + scpr * CH) at a fixed row
-  // pitch, zero where they lie off the detector.  soff turns the
-  // magic-number floor bits (bx, by) of a sample into its element index
-  // by * pitch + bx + soff (mod 2^32); srpp rows are copied per warp pass and
-  // smag = ceil(2^16 / scpr) divides a lane index by scpr.
-  int sx0, sv0, sh, scpr, srpp, smag, soff, staged;
+// Per (tile, view), in shared memory.  The first four quads are what the
+// sample loops read, one 16-byte load each.
+struct alignas(16) TileView {
+  float U0, V0, W0;     // anchored homogeneous coordinates at the tile centre
+  float wgt;            // wgt * scale (FP32): weight of a stored sample
+  float ru0, rv0, rw0;  // d(u_rel, v_rel, w)/dx
+  float ic;             // staged index constant (staged_index), exact
+  float ru1, rv1, rw1;  // .../dy
+  int mode;             // MODE_*
+  float ru2, rv2, rw2;  // .../dz
+  float wgtd;           // wgt alone: weight of a dequantised sample (data VJP)
+  int au, av;           // anchor pixel
+  // Staged footprint in shared memory (staged != 0): detector pixels from
+  // (sx0, sv0), sh rows at a fixed row pitch, zero where they lie off the
+  // detector.
+  int sx0, sv0, sh;
+  int staged;
+  int soff;             // by * pitch + bx + soff (mod 2^32) is the element index
+                        // of a sample with magic-number floor bits (bx, by)
+  // conversion of 16-bit footprints: scpr 16-byte chunks per row, srpp rows
+  // per warp pass, smag = ceil(2^16 / scpr) divides a lane index by scpr
+  int scpr, srpp, smag;
+  int csafe;            // every tap pixel and its central-difference neighbours
+                        // (one more pixel each side) lie inside the detector
 };
 
 enum { MODE_SKIP = 0, MODE_INTERIOR = 1, MODE_EDGE = 2 };
@@ -79,15 +83,40 @@ struct ProjInfo {
   long long rs, vs;   // element strides
 };
 
+// Views whose tiles project larger than the staging buffer everywhere in the
+// volume ("wide": more than ~4 px per voxel) read global memory, and do so
+// faster from a kernel variant that leaves the L1 cache its full size
+// (a job of 10 iterations on 128^3 x 360 views, 4.8 px per voxel: 61.6 ms, 76.2 ms
+// from the staged variant's fallback).  `wide` of launch_forward and launch_vjp_motion:
+// NULL, take the staged variant; WIDE_ALL, take the other one; else one flag
+// per view on the device (launch_compose, fit): both are launched and each
+// item runs in the one that suits its first view.
+struct FitInfo {
+  int dtype;
+  int* wide;  // [V]
+};
+extern const int* const WIDE_ALL;
 // ------------------------------------------------------------ launchers
 // All launchers are asynchronous on `stream` and return cudaGetLastError().
 
 cudaError_t launch_compose(const double* P, const double* theta, const double* view_weight,
                            const float* view_scale, int V, int fdk, double sid,
-                           const VolInfo& vi, ViewGeom* geom, double* Phat, cudaStream_t s);
+                           const VolInfo& vi, ViewGeom* geom, double* Phat, cudaStream_t s,
+                           const FitInfo* fit = nullptr);
+
+// The same test on the host for the nominal matrices: every view is wide.
+bool all_views_wide(const double* P, int V, int dtype, const VolInfo& vi);
+
+
+// The tensor map of a projection stack that the staging copies read; needs
+// 16-byte aligned data and strides (and a width of whole 16-byte chunks).
+// Pixels (columns, rows) of a staging buffer.
+void stage_extent(int dtype, int* cols, int* rows);
+cudaError_t make_stage_map(const void* proj, int dtype, const ProjInfo& pi, CUtensorMap* map);
 
 cudaError_t launch_forward(const void* proj, int dtype, const ProjInfo& pi, const ViewGeom* geom,
-                           const VolInfo& vi, int fdk, float* vol, cudaStream_t s);
+                           const VolInfo& vi, int fdk, float* vol, const int* wide,
+                           cudaStream_t s);
 // Set the forward / motion-VJP kernels' shared-memory attributes on the
 // current device (done by the first launch anyway; call before capturing a
 // graph).
@@ -106,7 +135,7 @@ cudaError_t launch_grad_images(const void* proj, int dtype, const ProjInfo& pi, 
 cudaError_t launch_vjp_motion(const float* dvol, const void* proj, int dtype, const ProjInfo& pi,
                               const float2* grad, const ViewGeom* geom, const VolInfo& vi,
                               int fdk, int exact, float* partials, float* dproj, float* blk,
-                              cudaStream_t s);
+                              const int* wide, cudaStream_t s);
 long long block_image_floats(const ProjInfo& pi);
 bool vjp_uses_blocks(const void* proj, int dtype, const ProjInfo& pi, int exact);
 
@@ -178,6 +207,7 @@ cudaError_t launch_fdk_filter(const float* raw, int V, int nv, int nu, int ext, 
 constexpr int BATCH_MAX_JOBS = 32;
 
 struct BatchJob {
+  CUtensorMap map;         // of proj, for the staging copies
   const void* proj;        // [V][nv][nu] compact, the batch's dtype
   const float2* grad;      // CENTRAL gradient images (NULL with BILINEAR_EXACT)
   const double* P;         // [V][12]
@@ -197,6 +227,7 @@ struct BatchJob {
   double lr_t, lr_r, beta1, beta2, eps, decay;
   float tv_eps;
   int V, ntiles_f, ntiles_v, nblk, max_iters, gauge;
+  int unstaged;            // every view is wide
 };
 
 struct BatchTable {

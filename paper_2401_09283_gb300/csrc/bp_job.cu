@@ -37,6 +37,7 @@ struct bp_job {
   cudaStream_t cap = nullptr;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
+  bool unstaged = false;        // every view is wide: the kernels that read global memory
   bool cancelled = false;
   int queued = 0;               // iterations queued so far (motion_step or batches)
   bp_batch* batch = nullptr;    // the batch this job is a member of, if any
@@ -136,7 +137,8 @@ cudaError_t record_iteration(bp_job* j, cudaStream_t s) {
   e = bpk::launch_compose(j->P, j->theta, j->vw, j->scale, V, fdk, j->pd.sid, j->vi, j->geom,
                           nullptr, s);
   if (e != cudaSuccess) return e;
-  e = bpk::launch_forward(j->proj, j->pd.dtype, j->pi, j->geom, j->vi, fdk, j->vol, s);
+  e = bpk::launch_forward(j->proj, j->pd.dtype, j->pi, j->geom, j->vi, fdk, j->vol,
+                          j->unstaged ? bpk::WIDE_ALL : nullptr, s);
   if (e != cudaSuccess) return e;
   if (j->opt.loss == BP_LOSS_TV)
     e = bpk::launch_tv(j->vol, j->vd.nx, j->vd.ny, j->vd.nz, (float)j->opt.tv_eps, j->blk, j->nblk,
@@ -146,7 +148,8 @@ cudaError_t record_iteration(bp_job* j, cudaStream_t s) {
                                    j->hist, j->iter, j->max_iters, j->dvol, s);
   if (e != cudaSuccess) return e;
   e = bpk::launch_vjp_motion(j->dvol, j->proj, j->pd.dtype, j->pi, j->grad, j->geom, j->vi, fdk,
-                             j->deriv == BP_DERIV_BILINEAR_EXACT, j->partials, nullptr, nullptr, s);
+                             j->deriv == BP_DERIV_BILINEAR_EXACT, j->partials, nullptr, nullptr,
+                             j->unstaged ? bpk::WIDE_ALL : nullptr, s);
   if (e != cudaSuccess) return e;
   e = bpk::launch_reduce_chain(j->partials, j->ntiles, j->vi, j->P, j->theta, V, nullptr, j->gth,
                                s);
@@ -341,12 +344,16 @@ int bp_job_create(bp_ctx* ctx, const void* proj, const bp_proj_desc* pdesc, cons
   if (e == cudaSuccess)
     e = bpk::prepare_vjp(pdesc->dtype, weight == BP_WEIGHT_FDK, deriv == BP_DERIV_BILINEAR_EXACT);
   if (e == cudaSuccess) e = cudaEventRecord(j->done, os);
+  std::vector<double> Ph((size_t)V * 12);  // the matrices decide the kernel variant
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(Ph.data(), j->P, 96 * (size_t)V, cudaMemcpyDeviceToHost, os);
   if (e == cudaSuccess) e = cudaStreamSynchronize(os);
   if (e != cudaSuccess) {
     release(j);
     delete j;
     return cuda_fail(ctx, e, "bp_job_create");
   }
+  j->unstaged = bpk::all_views_wide(Ph.data(), V, pdesc->dtype, j->vi);
   ctx->job_bytes += j->bytes;
   *out = j;
   return BP_OK;
@@ -485,7 +492,7 @@ bool same_config(const bp_job* a, const bp_job* b) {
 }
 
 // Fill one table from the members (host side).
-void fill_table(bp_batch* b, bpk::BatchTable& T) {
+cudaError_t fill_table(bp_batch* b, bpk::BatchTable& T) {
   const int n = (int)b->members.size();
   T.njobs = n;
   T.off_view[0] = T.off_fwd[0] = T.off_loss[0] = 0;
@@ -510,6 +517,8 @@ void fill_table(bp_batch* b, bpk::BatchTable& T) {
     J.hist = j->hist;
     J.iter = j->iter;
     J.pi = j->pi;
+    const cudaError_t e = bpk::make_stage_map(j->proj, j->pd.dtype, j->pi, &J.map);
+    if (e != cudaSuccess) return e;
     J.vi = j->vi;
     J.vif = j->vi;
     J.vif.zb = zbf;
@@ -528,10 +537,12 @@ void fill_table(bp_batch* b, bpk::BatchTable& T) {
     J.nblk = j->nblk;
     J.max_iters = j->max_iters;
     J.gauge = j->opt.gauge;
+    J.unstaged = j->unstaged;
     T.off_view[k + 1] = T.off_view[k] + J.V;
     T.off_fwd[k + 1] = T.off_fwd[k] + J.ntiles_f;
     T.off_loss[k + 1] = T.off_loss[k] + J.nblk;
   }
+  return cudaSuccess;
 }
 
 }  // namespace
@@ -653,8 +664,8 @@ int bp_batch_step(bp_batch* b, int n_iters, void* stream) {
       b->graph = nullptr;
       b->exec = nullptr;
     }
-    fill_table(b, b->table);
-    e = bpk::prepare_batch(j0->pd.dtype, fdk, exact);
+    e = fill_table(b, b->table);
+    if (e == cudaSuccess) e = bpk::prepare_batch(j0->pd.dtype, fdk, exact);
     if (e == cudaSuccess) e = bpk::prepare_vjp(j0->pd.dtype, fdk, exact);
     if (e == cudaSuccess && !b->br_fork)
       e = cudaEventCreateWithFlags(&b->br_fork, cudaEventDisableTiming);

@@ -3,57 +3,59 @@
 //
 // Work decomposition: a CTA of 256 threads owns a 16 x 16 x ZB box of voxels
 // (one z-column of ZB voxels per thread, warps of 8 x 4 columns) and loops
-// over all views.  For each batch of 32 views one thread per view computes,
-// in FP64, the anchored per-tile view record (TileView): the integer pixel
-// nearest the projection of the tile centre, the anchored rows and the
-// classification of the whole box as entirely off the detector (SKIP),
-// entirely inside it (INTERIOR: no bounds checks) or crossing an edge (EDGE:
-// clamped coordinates and checked taps).  The inner loops are plain FP32:
-// three FMAs for (u, v, w), one MUFU reciprocal, floor via a round-down add
-// of 1.5*2^23, bilinear interpolation with FP32 lerps (hardware texture
-// filtering is not used: its weights are 8-bit fixed point).
+// over views.  For each batch of 32 views eight threads per view compute, in
+// FP64 where it matters, the anchored per-tile view record (TileView): the
+// integer pixel nearest the projection of the tile centre, the anchored rows and
+// the classification of the whole box as entirely off the detector (SKIP),
+// entirely inside it (INTERIOR) or crossing an edge (EDGE).  Each view's detector
+// footprint comes to shared memory by TMA, views ahead, through a pipe of slots
+// that the warps pass at their own pace.  The inner loops are plain FP32: three
+// FMAs for (u, v, w), one MUFU reciprocal, floor via a round-down add of
+// 1.5*2^23, bilinear interpolation with FP32 lerps (hardware texture filtering is
+// not used: its weights are 8-bit fixed point).
+//
+// What bounds them (ncu, c2): the motion VJP's central-safe loop, the L1 data
+// pipe (12 taps per voxel-view at 1.4 wavefronts each, 80 % of its peak); the
+// forward, that pipe (63 %), the FMA pipe (54 %) and issue (58 %) together.
 #include "bp_internal.cuh"
+#include "bp_tma.cuh"
 
 namespace bpk {
 
 // CTAs per SM the register budget is sized for (256 threads each).
-#ifndef BP_FWD_MINB
-#define BP_FWD_MINB 4
-#endif
-#ifndef BP_VJP_MINB
-#define BP_VJP_MINB 3
-#endif
-constexpr int FWD_MINB = BP_FWD_MINB;
-constexpr int VJP_MINB = BP_VJP_MINB;
+constexpr int FWD_MINB = 4;
+constexpr int VJP_MINB = 3;
+// Staging slots (three at three CTAs per SM in the forward, three or four at
+// two in the VJP: slower, 3.69 against 3.58 and 10.9 against 9.9 ms on c2).
+constexpr int FWD_NS = 2;
+constexpr int VJP_NS = 2;
 
 constexpr float MAGIC = 12582912.0f;   // 1.5 * 2^23
 constexpr int MAGIC_BITS = 0x4B400000;
+// 1.5 * 2^21: one unit is 4 in the bit pattern, so INDEX_MAGIC + i has the
+// bits INDEX_BITS + 4 i, a byte offset, for integers |i| < 2^19.
+constexpr float INDEX_MAGIC = 3145728.0f;
+constexpr unsigned INDEX_BITS = 0x4A400000u;
 
-// Footprint staging buffers: fixed row pitch (so tap offsets are
-// immediates), rows of 21 16-byte chunks, 64 rows.  (A pitch of 80 floats,
-// which a simulation of the c2 tap positions gave 3 % fewer bank-conflict
-// wavefronts, measured the same: c2 step 19.448 against 19.445 ms.)
-#ifndef BP_STAGE_PITCH_BYTES
-#define BP_STAGE_PITCH_BYTES 336
-#endif
-constexpr int STAGE_PITCH_BYTES = BP_STAGE_PITCH_BYTES;
+// Footprint staging buffers: 64 rows at a fixed row pitch P (elements), so tap
+// offsets are immediates, filled by TMA in boxes of P x 8 pixels.  FP32
+// footprints are sampled in place (pitch 84; 80 measured the same).  FP16 and
+// BF16 footprints arrive raw (pitch 80; 88 bank-conflicts more, 30.8 against
+// 30.5 ms for a 384^3 x 248 VJP) and are converted once per (tile, view) into an
+// FP32 buffer of the same pitch, which the sample loops read like FP32 data.
 constexpr int STAGE_ROWS = 64;
-constexpr int STAGE_BYTES = STAGE_PITCH_BYTES * STAGE_ROWS;
+constexpr int BOX_ROWS = 8;
 template <typename T>
 struct StageGeom {
-  static constexpr int CH = 16 / (int)sizeof(T);                // elements per chunk
-  static constexpr int P = STAGE_PITCH_BYTES / (int)sizeof(T);  // row pitch in elements
+  static constexpr int CH = 16 / (int)sizeof(T);               // elements per 16 bytes
+  static constexpr int P = sizeof(T) == 4 ? 84 : 80;           // row pitch in elements
+  static constexpr int BOX_BYTES = P * BOX_ROWS * (int)sizeof(T);
+  static constexpr int BYTES = P * STAGE_ROWS * (int)sizeof(T);  // one footprint buffer
 };
-// FP16/BF16 data staged with conversion: raw rows of 16-byte chunks (8
-// pixels) at a pitch of CONV_P elements are converted into an FP32 buffer of
-// the same pitch (in floats), which the sample loops read like FP32 data.
-constexpr int CONV_P = 88;
-struct ConvGeom {
-  static constexpr int CH = 8;
-  static constexpr int P = CONV_P;
-};
-constexpr int CONV_F_BYTES = CONV_P * STAGE_ROWS * 4;  // FP32 buffer
-constexpr int CONV_R_BYTES = CONV_P * STAGE_ROWS * 2;  // raw buffer
+constexpr int CONV_F_BYTES = StageGeom<__half>::P * STAGE_ROWS * 4;  // converted footprint
+static_assert(StageGeom<float>::BOX_BYTES % 128 == 0 && StageGeom<__half>::BOX_BYTES % 128 == 0 &&
+                  CONV_F_BYTES % 128 == 0,
+              "TMA boxes land on 128-byte boundaries");
 
 template <typename T>
 __device__ __forceinline__ float ldv(const T* p);
@@ -189,11 +191,12 @@ struct TileIdx {
   int tx, ty, tz, lx, ly;
   float dx, dy;
   double qc[3];
-  float half[3];
+  float hx, hy, zlo, zhi;  // extent of the CTA's box about the tile centre
 };
 
-template <int ZB>
-__device__ __forceinline__ TileIdx tile_index(const VolInfo& vi, int tile) {
+// zs: the CTA's slices of the tile, [zs * ZS, zs * ZS + ZS).
+template <int ZB, int ZS = ZB>
+__device__ __forceinline__ TileIdx tile_index(const VolInfo& vi, int tile, int zs = 0) {
   TileIdx ti;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   ti.lx = (warp & 1) * 8 + (lane & 7);
@@ -206,9 +209,10 @@ __device__ __forceinline__ TileIdx tile_index(const VolInfo& vi, int tile) {
   ti.qc[0] = ti.tx * TX + 0.5 * (TX - 1) - vi.cx;
   ti.qc[1] = ti.ty * TY + 0.5 * (TY - 1) - vi.cy;
   ti.qc[2] = ti.tz * ZB + 0.5 * (ZB - 1) - vi.cz;
-  ti.half[0] = 0.5f * (TX - 1);
-  ti.half[1] = 0.5f * (TY - 1);
-  ti.half[2] = 0.5f * (ZB - 1);
+  ti.hx = 0.5f * (TX - 1);
+  ti.hy = 0.5f * (TY - 1);
+  ti.zlo = zs * ZS - 0.5f * (ZB - 1);
+  ti.zhi = ti.zlo + (ZS - 1);
   return ti;
 }
 
@@ -225,18 +229,13 @@ __device__ __forceinline__ TileIdx tile_index(const VolInfo& vi, int tile) {
 //   SKIP      every sample is 0 (projection at or beyond -1 / n),
 //   INTERIOR  every tap (floor and floor+1) lies on the detector,
 //   EDGE      otherwise (clamped coordinates, checked taps).
-// The footprint is the clipped pixel rectangle that the box's taps can
-// touch (unbounded, fw = 0, when some corner has w <= 0).
-//
 // With STAGE, bounded boxes also get a staging plan: the rectangle of
 // detector pixels that any tap (plus `halo` pixels each side) can read,
 // NOT clipped to the detector (off-detector pixels are staged as zeros, so
 // the sample loop needs neither checks nor clamps), if it fits the buffer.
-// With `need_csafe` only central-safe boxes are staged.
-template <typename T, bool STAGE, class G = StageGeom<T>>
+template <typename T, bool STAGE>
 __device__ void setup_batch(TileView* tvs, const ViewGeom* __restrict__ geom, int j0, int nb,
-                            const TileIdx& ti, int nu, int nv, bool with_scale, int halo = 0,
-                            bool need_csafe = false) {
+                            const TileIdx& ti, int nu, int nv, bool with_scale, int halo = 0) {
   const int b = threadIdx.x >> 3, c = threadIdx.x & 7;
   const ViewGeom& g = geom[j0 + min(b, nb - 1)];
   const double* M = g.P;
@@ -256,24 +255,26 @@ __device__ void setup_batch(TileView* tvs, const ViewGeom* __restrict__ geom, in
   t.V0 = (float)fma(-(double)av, wc, vc);
   t.W0 = (float)wc;
   const float fau = (float)au, fav = (float)av;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const float m2 = (float)M[8 + k];
-    t.ru[k] = fmaf(-fau, m2, (float)M[k]);
-    t.rv[k] = fmaf(-fav, m2, (float)M[4 + k]);
-    t.rw[k] = m2;
-  }
+  t.rw0 = (float)M[8];
+  t.rw1 = (float)M[9];
+  t.rw2 = (float)M[10];
+  t.ru0 = fmaf(-fau, t.rw0, (float)M[0]);
+  t.ru1 = fmaf(-fau, t.rw1, (float)M[1]);
+  t.ru2 = fmaf(-fau, t.rw2, (float)M[2]);
+  t.rv0 = fmaf(-fav, t.rw0, (float)M[4]);
+  t.rv1 = fmaf(-fav, t.rw1, (float)M[5]);
+  t.rv2 = fmaf(-fav, t.rw2, (float)M[6]);
   t.au = au;
   t.av = av;
   t.wgt = (float)(with_scale ? g.wgt * g.scale : g.wgt);
   t.wgtd = (float)g.wgt;
   // this lane's corner
-  const float d0 = (c & 1) ? ti.half[0] : -ti.half[0];
-  const float d1 = (c & 2) ? ti.half[1] : -ti.half[1];
-  const float d2 = (c & 4) ? ti.half[2] : -ti.half[2];
-  const float w = fmaf(t.rw[2], d2, fmaf(t.rw[1], d1, fmaf(t.rw[0], d0, t.W0)));
-  const float u = fmaf(t.ru[2], d2, fmaf(t.ru[1], d1, fmaf(t.ru[0], d0, t.U0)));
-  const float v = fmaf(t.rv[2], d2, fmaf(t.rv[1], d1, fmaf(t.rv[0], d0, t.V0)));
+  const float d0 = (c & 1) ? ti.hx : -ti.hx;
+  const float d1 = (c & 2) ? ti.hy : -ti.hy;
+  const float d2 = (c & 4) ? ti.zhi : ti.zlo;
+  const float w = fmaf(t.rw2, d2, fmaf(t.rw1, d1, fmaf(t.rw0, d0, t.W0)));
+  const float u = fmaf(t.ru2, d2, fmaf(t.ru1, d1, fmaf(t.ru0, d0, t.U0)));
+  const float v = fmaf(t.rv2, d2, fmaf(t.rv1, d1, fmaf(t.rv0, d0, t.V0)));
   const bool pos = w > 0.0f;
   int npos = pos ? 1 : 0;
   float xmin = INFINITY, xmax = -INFINITY, ymin = INFINITY, ymax = -INFINITY;
@@ -293,9 +294,8 @@ __device__ void setup_batch(TileView* tvs, const ViewGeom* __restrict__ geom, in
   const float m = 0.01f;
   // detector [0, n-1] in the anchored frame
   const float ulo = -fau, uhi = (float)(nu - 1) - fau, vlo = -fav, vhi = (float)(nv - 1) - fav;
-  t.fu0 = t.fv0 = t.fw = t.fh = 0;
-  t.csafe = 0;
-  t.sx0 = t.sv0 = t.sh = t.scpr = t.srpp = t.smag = t.soff = t.staged = 0;
+  t.ic = 0.0f;
+  t.sx0 = t.sv0 = t.sh = t.scpr = t.srpp = t.smag = t.soff = t.staged = t.csafe = 0;
   if (npos == 0) {
     t.mode = MODE_SKIP;
   } else if (npos < 8) {
@@ -309,21 +309,13 @@ __device__ void setup_batch(TileView* tvs, const ViewGeom* __restrict__ geom, in
                  : MODE_EDGE;
     // central differences at the tap pixels use interior neighbours only:
     // taps in [1, n-2], i.e. floor in [1, n-3]
-    t.csafe = xmin >= ulo + 1.0f + m && xmax <= uhi - 1.0f - m && ymin >= vlo + 1.0f + m &&
-              ymax <= vhi - 1.0f - m;
-    const int fl_u0 = (int)floorf(xmin - m) + au, fl_u1 = (int)floorf(xmax + m) + 1 + au;
-    const int fl_v0 = (int)floorf(ymin - m) + av, fl_v1 = (int)floorf(ymax + m) + 1 + av;
-    const int u0 = max(fl_u0, 0), u1 = min(fl_u1, nu - 1);
-    const int v0 = max(fl_v0, 0), v1 = min(fl_v1, nv - 1);
-    if (u1 >= u0 && v1 >= v0) {
-      t.fu0 = u0;
-      t.fv0 = v0;
-      t.fw = u1 - u0 + 1;
-      t.fh = v1 - v0 + 1;
-    }
-    if (STAGE && t.mode != MODE_SKIP && (!need_csafe || t.csafe)) {
-      constexpr int CH = G::CH, P = G::P;
-      const int x0 = (fl_u0 - halo) & ~(CH - 1);  // floor to a chunk boundary
+    t.csafe = xmin >= ulo + 1.0f + m && xmax <= uhi - 1.0f - m &&
+              ymin >= vlo + 1.0f + m && ymax <= vhi - 1.0f - m;
+    if (STAGE) {
+      constexpr int CH = StageGeom<T>::CH, P = StageGeom<T>::P;
+      const int fl_u0 = (int)floorf(xmin - m) + au, fl_u1 = (int)floorf(xmax + m) + 1 + au;
+      const int fl_v0 = (int)floorf(ymin - m) + av, fl_v1 = (int)floorf(ymax + m) + 1 + av;
+      const int x0 = (fl_u0 - halo) & ~(CH - 1);  // floor to a 16-byte boundary
       const int y0 = fl_v0 - halo;
       const int cpr = (fl_u1 + halo - x0) / CH + 1;
       const int h = fl_v1 + halo - y0 + 1;
@@ -337,6 +329,7 @@ __device__ void setup_batch(TileView* tvs, const ViewGeom* __restrict__ geom, in
         t.smag = (65536 + cpr - 1) / cpr;
         t.soff = (int)((unsigned)(av - y0) * (unsigned)P - (unsigned)MAGIC_BITS * (unsigned)P +
                        (unsigned)(au - x0) - (unsigned)MAGIC_BITS);
+        t.ic = INDEX_MAGIC + (float)((av - y0) * P + (au - x0));
       }
     }
   }
@@ -423,56 +416,89 @@ __device__ __forceinline__ f2 bilerp2(f2 tu, f2 tv, f2 d00, f2 d10, f2 d01, f2 d
 // footprint from the set-up).  Voxels project ~2.6 px apart on the larger
 // detectors, so a warp's 32 taps of one load are scattered over 4-6 L1
 // lines; from shared memory the same taps are a single wavefront (bar bank
-// conflicts).  The footprint is therefore copied to shared memory with
-// cp.async in 16-byte chunks, one view ahead: the copy of view j+1 overlaps
-// the arithmetic of view j.  Footprints that do not fit the buffer, or are
-// unbounded, read global memory instead.
+// conflicts).  The footprint is therefore copied to shared memory by TMA, in
+// boxes of P x 8 pixels (pixels off the detector arrive as zeros), two views
+// ahead: one warp issues at most eight copies per view, where a cp.async copy
+// by all threads cost ~50 of the ~540 instructions of a (thread, view) and two
+// CTA barriers.  Footprints that do not fit the buffer, or are unbounded,
+// read global memory instead.
 
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-__device__ __forceinline__ void cp_async_wait1() {
-  asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-}
+// NS staging slots, used by consecutive views in turn.  full[s] completes once
+// per view (when its footprint has arrived, at once if it has none); done[s]
+// counts the warps that have finished the view, and the warp that finishes
+// last refills the slot, so no warp waits for another one to free a slot.
+// Every warp waits on full[s] for every view, staged or not: it may then be at
+// most one phase behind, which the parity tells apart.
+template <int NS>
+struct StagePipe {
+  unsigned long long full[NS];
+  unsigned done[NS];
+};
 
-// All threads: copy the staged rectangle of record t (rows per warp pass,
-// one chunk per lane, no divisions).  A chunk lies wholly on or off the
-// detector (chunk starts are multiples of CH and nu is), so off-detector
-// chunks and rows are written as zeros.
-template <typename T, int P = StageGeom<T>::P>
-__device__ __forceinline__ void stage_issue(T* buf, const T* img, long long rs, int nu, int nv,
-                                            const TileView& t) {
-  constexpr int CH = StageGeom<T>::CH;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int lr = (lane * t.smag) >> 16, lc = lane - lr * t.scpr;
-  if (lr >= t.srpp) return;
-  const int cu = t.sx0 + lc * CH;
-  const bool uin = cu >= 0 && cu < nu;
-  for (int r = warp * t.srpp + lr; r < t.sh; r += (NT / 32) * t.srpp) {
-#ifdef BP_BOUNDS_CHECK
-    if (!(r < STAGE_ROWS && lc * CH + CH <= P)) {
-      bc_fail(BC_STAGE_DST, r, lc);
-      break;
-    }
-#endif
-    T* dst = buf + r * P + lc * CH;
-    const int row = t.sv0 + r;
-    if (uin && (unsigned)row < (unsigned)nv)
-      cp_async16(dst, img + (long long)row * rs + cu);
-    else
-      *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
+template <int NS>
+__device__ __forceinline__ void pipe_init(StagePipe<NS>& p) {  // ends with a CTA barrier
+  if (threadIdx.x < NS) {
+    mbar_init(&p.full[threadIdx.x], 1);
+    p.done[threadIdx.x] = 0u;
+    mbar_init_fence();
   }
+  __syncthreads();
+}
+
+// A warp's place in the pipe: the slot of its current view and the parity of
+// that slot's phase.
+template <int NS>
+struct PipePos {
+  unsigned slot = 0, parity = 0;
+  __device__ __forceinline__ void next() {
+    if (++slot == NS) {
+      slot = 0;
+      parity ^= 1u;
+    }
+  }
+};
+
+// One whole warp: request the footprint of record t (view v) into buf.
+template <typename T>
+__device__ __forceinline__ void stage_issue(unsigned char* buf, const CUtensorMap* map,
+                                            const TileView& t, int v, unsigned long long* bar) {
+  constexpr int BOX = StageGeom<T>::BOX_BYTES;
+  const int lane = threadIdx.x & 31;
+  int nb = t.staged ? (t.sh + BOX_ROWS - 1) / BOX_ROWS : 0;
+#ifdef BP_BOUNDS_CHECK
+  if (nb > STAGE_ROWS / BOX_ROWS || (t.sx0 & (StageGeom<T>::CH - 1))) {
+    if (lane == 0) bc_fail(BC_STAGE_DST, t.sh, t.sx0);
+    nb = 0;
+  }
+#endif
+  if (lane == 0) {
+    if (nb) mbar_arrive_expect(bar, (unsigned)(nb * BOX));
+    else mbar_arrive(bar);
+  }
+  __syncwarp();
+  if (lane < nb) tma_load_3d(buf + lane * BOX, map, t.sx0, t.sv0 + lane * BOX_ROWS, v, bar);
+}
+
+// Whether the calling warp is the last of the CTA's warps to finish with a
+// slot.  Acquire-release: the last warp sees what every other warp wrote
+// before, and its refill comes after all their reads.
+__device__ __forceinline__ bool last_warp(unsigned* done) {
+  __syncwarp();
+  unsigned old = 0;
+  if ((threadIdx.x & 31) == 0)
+    asm volatile("atom.acq_rel.cta.shared::cta.inc.u32 %0, [%1], %2;"
+                 : "=r"(old)
+                 : "r"(smem_addr(done)), "r"(NT / 32 - 1)
+                 : "memory");
+  return __shfl_sync(0xffffffffu, old, 0) == NT / 32 - 1;
 }
 
 // All threads: convert the raw FP16/BF16 rectangle of record t (staged by
-// stage_issue<T, CONV_P>) into FP32 at the same pitch, chunk by chunk with the
-// copy's thread mapping.
+// stage_issue<T>) into FP32 at the same pitch, in 16-byte chunks, rows per warp
+// pass (no divisions).
 template <typename T>
 __device__ __forceinline__ void convert_stage(float* F, const T* R, const TileView& t) {
+  constexpr int CONV_P = StageGeom<T>::P;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int lr = (lane * t.smag) >> 16, lc = lane - lr * t.scpr;
   if (lr >= t.srpp) return;
@@ -497,61 +523,88 @@ __device__ __forceinline__ void convert_stage(float* F, const T* R, const TileVi
   }
 }
 
-__device__ __forceinline__ void cp_async_wait0() {
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+// Sampling of the staged FP32 footprint.  buf is its shared-memory address, P
+// the row pitch, H the stencil's reach beyond the bilinear taps (1 for the
+// CENTRAL 4x4-minus-corners stencil, 0 otherwise; the staging plan covers it).
+
+template <int OFF>  // OFF in floats
+__device__ __forceinline__ float lds(unsigned a) {
+  float r;
+  asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(r) : "r"(a), "n"(OFF * 4));
+  return r;
+}
+template <int OFF>
+__device__ __forceinline__ f2 lds2(unsigned a, unsigned b) {
+  const float lo = lds<OFF>(a), hi = lds<OFF>(b);
+  return pk2(lo, hi);
 }
 
-template <typename T>
-__device__ __forceinline__ float tof(T x);
-template <>
-__device__ __forceinline__ float tof<float>(float x) {
-  return x;
-}
-template <>
-__device__ __forceinline__ float tof<__half>(__half x) {
-  return __half2float(x);
-}
-template <>
-__device__ __forceinline__ float tof<__nv_bfloat16>(__nv_bfloat16 x) {
-  return __bfloat162float(x);
-}
-
-// A sample's position in the staged buffer: (bx, by) are the bit patterns
-// of x + MAGIC and y + MAGIC rounded down, i.e. MAGIC_BITS + floor.
-// H is the stencil's reach beyond the bilinear taps (1 for the CENTRAL
-// 4x4-minus-corners stencil, 0 otherwise); the staging plan covers it.
-template <int P, int H = 0, typename T>
-__device__ __forceinline__ const T* staged_tap(const T* buf, const TileView& t, int bx, int by) {
 #ifdef BP_BOUNDS_CHECK
-  constexpr int CHK = (P == CONV_P) ? 8 : 16 / (int)sizeof(T);  // elements per staged chunk
-  const int ru = bx - MAGIC_BITS + t.au - t.sx0, rv = by - MAGIC_BITS + t.av - t.sv0;
-  if (!(t.staged && ru - H >= 0 && ru + 1 + H < t.scpr * CHK && rv - H >= 0 &&
-        rv + 1 + H < t.sh)) {
-    bc_fail(BC_STAGED_TAP, ru, rv);
+// Column and row of the floor pixel in the staged rectangle; true if bad.
+template <typename T, int H>
+__device__ __forceinline__ bool bc_staged(const TileView& t, int fx, int fy) {
+  const int ru = fx + t.au - t.sx0, rv = fy + t.av - t.sv0;
+  if (t.staged && ru - H >= 0 && ru + 1 + H < t.scpr * StageGeom<T>::CH && rv - H >= 0 &&
+      rv + 1 + H < t.sh)
+    return false;
+  bc_fail(BC_STAGED_TAP, ru, rv);
+  return true;
+}
+#endif
+
+// Address of one sample's floor pixel: (bx, by) are the bit patterns of
+// x + MAGIC and y + MAGIC rounded down, i.e. MAGIC_BITS + floor.
+template <typename T, int H>
+__device__ __forceinline__ unsigned staged_tap(unsigned buf, const TileView& t, int bx, int by) {
+  constexpr int P = StageGeom<T>::P;
+#ifdef BP_BOUNDS_CHECK
+  if (bc_staged<T, H>(t, bx - MAGIC_BITS, by - MAGIC_BITS)) {
     bx = MAGIC_BITS + t.sx0 + H - t.au;
     by = MAGIC_BITS + t.sv0 + H - t.av;
   }
 #endif
   const unsigned o = (unsigned)by * (unsigned)P + (unsigned)bx + (unsigned)t.soff;
-  return buf + (int)o;
+  return buf + 4u * o;
 }
 
-
+// Addresses of a pair of samples' floor pixels from their floors (fx, fy), as
+// floats: fy * P + (fx + ic) is exact and its bit pattern is INDEX_BITS plus
+// the byte offset, so a pair costs two packed instructions where integer
+// arithmetic on the floor bits took four to six (7.4 integer instructions per
+// voxel-view in the forward before, 40 % of its issue slots with the moves).
+template <typename T, int H>
+__device__ __forceinline__ void staged_pair(unsigned buf, const TileView& t, f2 ic, f2 fx, f2 fy,
+                                            unsigned& al, unsigned& ah) {
+  constexpr float P = (float)StageGeom<T>::P;
+  const f2 o = fma2(fy, pk2(P, P), add2(fx, ic));
+  float lo, hi;
+  up2(o, lo, hi);
+#ifdef BP_BOUNDS_CHECK
+  float xl, xh, yl, yh;
+  up2(fx, xl, xh);
+  up2(fy, yl, yh);
+  const float safe = INDEX_MAGIC + (float)(H * StageGeom<T>::P + H);
+  if (bc_staged<T, H>(t, (int)xl, (int)yl)) lo = safe;
+  if (bc_staged<T, H>(t, (int)xh, (int)yh)) hi = safe;
+#endif
+  al = __float_as_uint(lo) + (buf - INDEX_BITS);
+  ah = __float_as_uint(hi) + (buf - INDEX_BITS);
+}
 
 // ------------------------------------------------------------------ forward
 
 // One view from global memory (footprint not staged).
 template <int ZB, typename T, bool FDK, bool EDGE>
 __device__ __forceinline__ void forward_view(const T* img, long long rs, int nu, int nv,
-                                             const TileView& t, float dx, float dy,
+                                             const TileView& t, float dx, float dy, float zlo,
                                              float (&acc)[ZB]) {
-  float u0 = fmaf(dy, t.ru[1], fmaf(dx, t.ru[0], t.U0));
-  float v0 = fmaf(dy, t.rv[1], fmaf(dx, t.rv[0], t.V0));
-  float w0 = fmaf(dy, t.rw[1], fmaf(dx, t.rw[0], t.W0));
+  float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
+  float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
+  float w0 = fmaf(dy, t.rw1, fmaf(dx, t.rw0, t.W0));
 #pragma unroll
   for (int k = 0; k < ZB; ++k) {
-    const float dz = k - 0.5f * (ZB - 1);
-    Sample s = locate<EDGE>(fmaf(dz, t.ru[2], u0), fmaf(dz, t.rv[2], v0), fmaf(dz, t.rw[2], w0),
+    const float dz = zlo + k;
+    Sample s = locate<EDGE>(fmaf(dz, t.ru2, u0), fmaf(dz, t.rv2, v0), fmaf(dz, t.rw2, w0),
                             t, nu, nv);
     if (EDGE && !s.ok) continue;
     float d00, d10, d01, d11;
@@ -565,177 +618,162 @@ __device__ __forceinline__ void forward_view(const T* img, long long rs, int nu,
 // One view from its staged, zero-padded footprint (no checks, no clamps, tap
 // offsets are compile-time constants), with packed pairs of voxels (k, k+1):
 // every step of the scalar loop above, in the same order, on f32x2 pairs.
-// E is the staged element type, P the staged row pitch.
-template <int ZB, typename T, bool FDK, int P = StageGeom<T>::P>
-__device__ __forceinline__ void forward_view_staged2(const T* buf, const TileView& t, float dx,
-                                                     float dy, f2 (&acc)[ZB / 2]) {
-  const float u0 = fmaf(dy, t.ru[1], fmaf(dx, t.ru[0], t.U0));
-  const float v0 = fmaf(dy, t.rv[1], fmaf(dx, t.rv[0], t.V0));
-  const float w0 = fmaf(dy, t.rw[1], fmaf(dx, t.rw[0], t.W0));
+// buf is the FP32 footprint's shared-memory address, T the stored type.
+template <int ZS, typename T, bool FDK>
+__device__ __forceinline__ void forward_view_staged2(unsigned buf, const TileView& t, float dx,
+                                                     float dy, float zlo, f2 (&acc)[ZS / 2]) {
+  constexpr int P = StageGeom<T>::P;
+  const float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
+  const float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
+  const float w0 = fmaf(dy, t.rw1, fmaf(dx, t.rw0, t.W0));
   const f2 U0 = pk2(u0, u0), V0 = pk2(v0, v0), W0 = pk2(w0, w0);
-  const f2 RU = pk2(t.ru[2], t.ru[2]), RV = pk2(t.rv[2], t.rv[2]), RW = pk2(t.rw[2], t.rw[2]);
+  const f2 RU = pk2(t.ru2, t.ru2), RV = pk2(t.rv2, t.rv2), RW = pk2(t.rw2, t.rw2);
   const f2 M2 = pk2(MAGIC, MAGIC), TWO = pk2(2.0f, 2.0f), WG = pk2(t.wgt, t.wgt);
-  f2 dz = pk2(-0.5f * (ZB - 1), 1.0f - 0.5f * (ZB - 1));  // exact: halves of small integers
+  const f2 IC = pk2(t.ic, t.ic);
+  f2 dz = pk2(zlo, zlo + 1.0f);  // exact: halves of small integers
 #pragma unroll
-  for (int p = 0; p < ZB / 2; ++p) {
+  for (int p = 0; p < ZS / 2; ++p) {
     if (p) dz = add2(dz, TWO);
     const f2 u = fma2(dz, RU, U0), v = fma2(dz, RV, V0), w = fma2(dz, RW, W0);
     float wl, wh;
     up2(w, wl, wh);
     const f2 r = pk2(rcp_approx(wl), rcp_approx(wh));
     const f2 x = mul2(u, r), y = mul2(v, r);
-    const f2 rx = add2_rd(x, M2), ry = add2_rd(y, M2);
-    const f2 tu = sub2(x, sub2(rx, M2)), tv = sub2(y, sub2(ry, M2));
-    float bxl, bxh, byl, byh;
-    up2(rx, bxl, bxh);
-    up2(ry, byl, byh);
-    const T* ql = staged_tap<P>(buf, t, __float_as_int(bxl), __float_as_int(byl));
-    const T* qh = staged_tap<P>(buf, t, __float_as_int(bxh), __float_as_int(byh));
-    const f2 d00 = pk2(tof(ql[0]), tof(qh[0])), d10 = pk2(tof(ql[1]), tof(qh[1]));
-    const f2 d01 = pk2(tof(ql[P]), tof(qh[P])), d11 = pk2(tof(ql[P + 1]), tof(qh[P + 1]));
+    const f2 fx = sub2(add2_rd(x, M2), M2), fy = sub2(add2_rd(y, M2), M2);
+    const f2 tu = sub2(x, fx), tv = sub2(y, fy);
+    unsigned ql, qh;
+    staged_pair<T, 0>(buf, t, IC, fx, fy, ql, qh);
+    const f2 d00 = lds2<0>(ql, qh), d10 = lds2<1>(ql, qh);
+    const f2 d01 = lds2<P>(ql, qh), d11 = lds2<P + 1>(ql, qh);
     const f2 val = bilerp2(tu, tv, d00, d10, d01, d11);
     acc[p] = fma2(val, FDK ? mul2(r, mul2(r, WG)) : WG, acc[p]);
   }
 }
 
-// Views are processed in order; the records of batch k+1 are built at the
-// start of batch k (two record slots), so the footprint of view j+1 is
-// known, and its copy issued, while view j is computed.  With two staging
-// buffers a second barrier per view guards their reuse; with three it is
-// not needed (the copy into buffer (j+1) mod 3 cannot overlap a read of it:
-// view j-2 was finished by every thread before the barrier of view j-1),
-// but the third buffer costs occupancy: two buffers at 4 CTAs/SM measured
-// faster on GB300 than three at 3 CTAs/SM.
-#ifndef BP_FWD_NBUF
-#define BP_FWD_NBUF 2
-#endif
-constexpr int FWD_NBUF = BP_FWD_NBUF;
-
-//
-// FP16/BF16 data (CONV) is staged through a raw buffer and converted once per
-// (tile, view) into an FP32 buffer, so the sample loop is the FP32 one
-// (no conversion per tap): wait for the raw copy of view j, barrier, convert,
-// barrier, issue the raw copy of view j+1, compute view j.
+// FP16/BF16 data (CONV) is converted once per (tile, view) from the raw slot
+// into one FP32 buffer that all warps share, so that path has CTA barriers:
+// wait for view v, barrier (every warp is done with the FP32 buffer), convert,
+// barrier, refill the raw slot, compute.
 template <typename T>
 __host__ __device__ constexpr bool conv_staging() {
   return !std::is_same<T, float>::value;
 }
-template <typename T>
-__host__ __device__ constexpr int fwd_smem_bytes() {
-  return conv_staging<T>() ? CONV_F_BYTES + CONV_R_BYTES : FWD_NBUF * STAGE_BYTES;
+template <typename T, int NS>
+__host__ __device__ constexpr int stage_smem_bytes() {
+  return (conv_staging<T>() ? CONV_F_BYTES : 0) + NS * StageGeom<T>::BYTES;
 }
 
-// One tile of the forward: every view, in order, accumulated per voxel.
-// All threads of the CTA call it; tvs and dyn_smem are the CTA's shared
-// memory (the kernel's static record slots and dynamic staging buffers).
-template <int ZB, typename T, bool FDK, bool STAGE>
-__device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const ProjInfo& pi,
-                                             const ViewGeom* __restrict__ geom, const VolInfo& vi,
-                                             float* __restrict__ vol, int tile,
-                                             TileView (*tvs)[VB], unsigned char* dyn_smem) {
+// One tile of the forward (its slices [zs ZS, zs ZS + ZS)): every view, in
+// order, accumulated per voxel.  All threads of the CTA call it; tvs, pipe and
+// dyn_smem are the CTA's shared memory.  seq counts the views the CTA has X.  The records of batch k+1 are built at the start of batch
+// k (two record slots), so the footprints of the next views are known.
+// A copy that never arrives (the bounded wait gives up) shows as NaN voxels.
+template <int ZB, int ZS, int NS, typename T, bool FDK, bool STAGE>
+__device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const CUtensorMap* map,
+                                             const ProjInfo& pi, const ViewGeom* __restrict__ geom,
+                                             const VolInfo& vi, float* __restrict__ vol, int tile,
+                                             int zs, TileView (*tvs)[VB],
+                                             StagePipe<NS>& pipe, unsigned char* dyn_smem,
+                                             PipePos<NS>& pos) {
   constexpr bool CONV = STAGE && conv_staging<T>();
-  using G = typename std::conditional<CONV, ConvGeom, StageGeom<T>>::type;
-  T* bufs = reinterpret_cast<T*>(dyn_smem);  // plain: FWD_NBUF buffers of T
-  float* F = reinterpret_cast<float*>(dyn_smem);  // CONV: FP32 buffer, then the raw one
-  T* R = reinterpret_cast<T*>(dyn_smem + CONV_F_BYTES);
-  constexpr int CAP = STAGE_BYTES / (int)sizeof(T);
-  static_assert(ZB % 2 == 0, "voxel pairs");
-  const TileIdx ti = tile_index<ZB>(vi, tile);
-  f2 acc[ZB / 2];
+  constexpr int SLOT = StageGeom<T>::BYTES;
+  unsigned char* slots = dyn_smem + (CONV ? CONV_F_BYTES : 0);
+  static_assert(ZS % 2 == 0 && ZB % ZS == 0, "voxel pairs");
+  const TileIdx ti = tile_index<ZB, ZS>(vi, tile, zs);
+  const int warp = threadIdx.x >> 5;
+  f2 acc[ZS / 2];
 #pragma unroll
-  for (int k = 0; k < ZB / 2; ++k) acc[k] = pk2(0.0f, 0.0f);
+  for (int k = 0; k < ZS / 2; ++k) acc[k] = pk2(0.0f, 0.0f);
+  bool bad = false;
   const int V = pi.nviews;
   const int nbatch = (V + VB - 1) / VB;
-  setup_batch<T, STAGE, G>(tvs[0], geom, 0, min(VB, V), ti, pi.nu, pi.nv, true);
+  setup_batch<T, STAGE>(tvs[0], geom, 0, min(VB, V), ti, pi.nu, pi.nv, true);
   if (nbatch > 1)
-    setup_batch<T, STAGE, G>(tvs[1], geom, VB, min(VB, V - VB), ti, pi.nu, pi.nv, true);
+    setup_batch<T, STAGE>(tvs[1], geom, VB, min(VB, V - VB), ti, pi.nu, pi.nv, true);
   __syncthreads();
-  if (STAGE && V > 0 && tvs[0][0].staged) {
-    if constexpr (CONV)
-      stage_issue<T, CONV_P>(R, proj, pi.rs, pi.nu, pi.nv, tvs[0][0]);
-    else
-      stage_issue(bufs, proj, pi.rs, pi.nu, pi.nv, tvs[0][0]);
+  if (STAGE && warp < NS && warp < V) {
+    const unsigned s = (pos.slot + warp) % NS;
+    stage_issue<T>(slots + s * SLOT, map, tvs[0][warp], warp, &pipe.full[s]);
   }
-  cp_async_commit();
-  int cur = 0;  // buffer of view v
   for (int v = 0; v < V; ++v) {
     const int k = v / VB, b = v - k * VB;
     if (b == 0 && k >= 1 && k + 1 < nbatch) {
-      setup_batch<T, STAGE, G>(tvs[(k + 1) & 1], geom, (k + 1) * VB, min(VB, V - (k + 1) * VB),
-                               ti, pi.nu, pi.nv, true);
+      __syncthreads();  // every warp is done with batch k-1
+      setup_batch<T, STAGE>(tvs[(k + 1) & 1], geom, (k + 1) * VB, min(VB, V - (k + 1) * VB), ti,
+                            pi.nu, pi.nv, true);
       __syncthreads();
     }
-    const TileView t = tvs[k & 1][b];
-    const int nxt = cur == FWD_NBUF - 1 ? 0 : cur + 1;
-    const int kn = (v + 1) / VB;
-    const TileView* tn = v + 1 < V ? &tvs[kn & 1][v + 1 - kn * VB] : nullptr;
+    // without the pipe, a barrier per view keeps the warps' footprints together
+    // in the L1 cache
+    if (!STAGE) __syncthreads();
+    const TileView& t = tvs[k & 1][b];
+    const unsigned slot = pos.slot;
+    unsigned char* buf = slots + slot * SLOT;
+    if (STAGE && !bad) bad = !mbar_wait(&pipe.full[slot], pos.parity);
+    pos.next();
+    const int vn = v + NS;
+    const TileView& tn = tvs[(vn / VB) & 1][vn % VB];
     if constexpr (CONV) {
-      cp_async_wait0();
-      __syncthreads();  // raw view v complete; every thread is done with F
-      if (t.staged) convert_stage<T>(F, R, t);
-      __syncthreads();  // F holds view v; R is free
-      if (tn && tn->staged)
-        stage_issue<T, CONV_P>(R, proj + (long long)(v + 1) * pi.vs, pi.rs, pi.nu, pi.nv, *tn);
-      cp_async_commit();
-    } else {
-      if (STAGE && tn && tn->staged)
-        stage_issue(bufs + nxt * CAP, proj + (long long)(v + 1) * pi.vs, pi.rs, pi.nu, pi.nv, *tn);
-      cp_async_commit();
-      cp_async_wait1();
-      __syncthreads();
+      __syncthreads();  // every warp has seen this phase and is done with F
+      if (t.staged) {
+        convert_stage<T>(reinterpret_cast<float*>(dyn_smem), reinterpret_cast<const T*>(buf), t);
+        __syncthreads();  // F holds view v; the raw slot is free
+      }
+      if (warp == (v & 7) && vn < V && !bad) stage_issue<T>(buf, map, tn, vn, &pipe.full[slot]);
     }
     if (t.mode != MODE_SKIP) {
       if (STAGE && t.staged) {
-        if constexpr (CONV)
-          forward_view_staged2<ZB, float, FDK, CONV_P>(F, t, ti.dx, ti.dy, acc);
-        else
-          forward_view_staged2<ZB, T, FDK>(bufs + cur * CAP, t, ti.dx, ti.dy, acc);
+        forward_view_staged2<ZS, T, FDK>(smem_addr(CONV ? dyn_smem : buf), t, ti.dx, ti.dy, ti.zlo,
+                                         acc);
       } else {
         const T* img = proj + (long long)v * pi.vs;
-        float a[ZB];
+        float a[ZS];
 #pragma unroll
-        for (int k = 0; k < ZB / 2; ++k) up2(acc[k], a[2 * k], a[2 * k + 1]);
+        for (int k2 = 0; k2 < ZS / 2; ++k2) up2(acc[k2], a[2 * k2], a[2 * k2 + 1]);
         if (t.mode == MODE_INTERIOR)
-          forward_view<ZB, T, FDK, false>(img, pi.rs, pi.nu, pi.nv, t, ti.dx, ti.dy, a);
+          forward_view<ZS, T, FDK, false>(img, pi.rs, pi.nu, pi.nv, t, ti.dx, ti.dy, ti.zlo, a);
         else
-          forward_view<ZB, T, FDK, true>(img, pi.rs, pi.nu, pi.nv, t, ti.dx, ti.dy, a);
+          forward_view<ZS, T, FDK, true>(img, pi.rs, pi.nu, pi.nv, t, ti.dx, ti.dy, ti.zlo, a);
 #pragma unroll
-        for (int k = 0; k < ZB / 2; ++k) acc[k] = pk2(a[2 * k], a[2 * k + 1]);
+        for (int k2 = 0; k2 < ZS / 2; ++k2) acc[k2] = pk2(a[2 * k2], a[2 * k2 + 1]);
       }
     }
-    if (!CONV && FWD_NBUF == 2) __syncthreads();
-    cur = nxt;
+    if constexpr (STAGE && !CONV) {
+      if (last_warp(&pipe.done[slot]) && vn < V && !bad)
+        stage_issue<T>(buf, map, tn, vn, &pipe.full[slot]);
+    }
   }
   const int i = ti.tx * TX + ti.lx, j = ti.ty * TY + ti.ly;
   if (i < vi.nx && j < vi.ny) {
 #pragma unroll
-    for (int k = 0; k < ZB / 2; ++k) {
+    for (int k = 0; k < ZS / 2; ++k) {
       float lo, hi;
       up2(acc[k], lo, hi);
-      const int z = ti.tz * ZB + 2 * k;
+      if (STAGE && bad) lo = hi = __int_as_float(0x7fc00000);
+      const int z = ti.tz * ZB + zs * ZS + 2 * k;
       if (z < vi.nz) vol[((long long)z * vi.ny + j) * vi.nx + i] = lo;
       if (z + 1 < vi.nz) vol[((long long)(z + 1) * vi.ny + j) * vi.nx + i] = hi;
     }
   }
 }
 
-template <int ZB, typename T, bool FDK, bool STAGE>
-__global__ void __launch_bounds__(NT, FWD_MINB)
-    forward_kernel(const T* __restrict__ proj, ProjInfo pi, const ViewGeom* __restrict__ geom,
-                   VolInfo vi, float* __restrict__ vol) {
+template <int ZB, int ZS, int NS, typename T, bool FDK, bool STAGE>
+__global__ void __launch_bounds__(NT, NS > FWD_NS ? 2 : FWD_MINB)
+    forward_kernel(const T* __restrict__ proj, const __grid_constant__ CUtensorMap map, ProjInfo pi,
+                   const ViewGeom* __restrict__ geom, VolInfo vi, float* __restrict__ vol,
+                   const int* __restrict__ wide) {
+  if (wide && (wide[0] != 0) == STAGE) return;  // the other variant's launch
   __shared__ TileView tvs[2][VB];
-  extern __shared__ __align__(16) unsigned char dyn_smem[];
-  forward_tile<ZB, T, FDK, STAGE>(proj, pi, geom, vi, vol, blockIdx.x, tvs, dyn_smem);
+  __shared__ StagePipe<NS> pipe;
+  extern __shared__ __align__(128) unsigned char dyn_smem[];
+  if (STAGE) pipe_init(pipe);
+  PipePos<NS> pos;
+  forward_tile<ZB, ZS, NS, T, FDK, STAGE>(proj, &map, pi, geom, vi, vol, blockIdx.x / (ZB / ZS),
+                                      blockIdx.x % (ZB / ZS), tvs, pipe, dyn_smem, pos);
 }
 
-// z-extent of the forward's tiles (its own tiling; the VJP's is ZB_VJP)
-#ifndef BP_ZB_FWD
-#define BP_ZB_FWD 16
-#endif
-#ifndef BP_FWD_STAGE
-#define BP_FWD_STAGE 1
-#endif
-constexpr int ZB_FWD = BP_ZB_FWD;
+// z-extent of the forward's tiles
+constexpr int ZB_FWD = 16;
 
 // Staging needs 16-byte aligned rows and whole 16-byte chunks per row.
 template <typename T>
@@ -759,46 +797,123 @@ static cudaError_t smem_attr_once(int bytes) {
   return e;
 }
 
-template <typename T, bool FDK>
-static cudaError_t forward_dispatch(const void* proj, const ProjInfo& pi, const ViewGeom* geom,
-                                    const VolInfo& vi, float* vol, cudaStream_t s) {
-  const int ntiles = vi.tiles_x * vi.tiles_y * vi.tiles_z;
-  const int smem = fwd_smem_bytes<T>();
-  if (BP_FWD_STAGE && stageable<T>(proj, pi)) {
-    cudaError_t e = smem_attr_once<forward_kernel<ZB_FWD, T, FDK, true>>(smem);
+// The tensor map that the staging copies read: dimensions (nu, nv, views), box
+// P x BOX_ROWS x 1.  (cuTensorMapEncodeTiled is a driver call without a stream;
+// it only fills in the descriptor.)
+cudaError_t make_stage_map(const void* proj, int dtype, const ProjInfo& pi, CUtensorMap* map) {
+  using Fn = decltype(&cuTensorMapEncodeTiled);
+  static const Fn encode = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault,
+                                         &r) != cudaSuccess ||
+        r != cudaDriverEntryPointSuccess)
+      f = nullptr;
+    return reinterpret_cast<Fn>(f);
+  }();
+  if (!encode) return cudaErrorNotSupported;
+  const cuuint64_t es = dtype == 0 ? 4 : 2;
+  const cuuint64_t dims[3] = {(cuuint64_t)pi.nu, (cuuint64_t)pi.nv, (cuuint64_t)pi.nviews};
+  const cuuint64_t strides[2] = {(cuuint64_t)pi.rs * es, (cuuint64_t)pi.vs * es};
+  const cuuint32_t box[3] = {
+      (cuuint32_t)(dtype == 0 ? StageGeom<float>::P : StageGeom<__half>::P), BOX_ROWS, 1};
+  const cuuint32_t ones[3] = {1, 1, 1};
+  const CUtensorMapDataType dt = dtype == 0   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+                                 : dtype == 1 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
+                                              : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+  const CUresult rc =
+      encode(map, dt, 3, const_cast<void*>(proj), dims, strides, box, ones,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return rc == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+void stage_extent(int dtype, int* cols, int* rows) {
+  *cols = dtype == 0 ? StageGeom<float>::P : StageGeom<__half>::P;
+  *rows = STAGE_ROWS;
+}
+
+template <typename T>
+constexpr int dtype_id() {
+  return std::is_same<T, float>::value ? 0 : std::is_same<T, __half>::value ? 1 : 2;
+}
+
+template <int ZS, int NS, typename T, bool FDK>
+static cudaError_t forward_launch(const void* proj, const ProjInfo& pi, const ViewGeom* geom,
+                                  const VolInfo& vi, float* vol, const int* wide, cudaStream_t s) {
+  const int nblocks = vi.tiles_x * vi.tiles_y * vi.tiles_z * (ZB_FWD / ZS);
+  CUtensorMap map{};
+  const bool stage = stageable<T>(proj, pi) && wide != WIDE_ALL &&
+                     make_stage_map(proj, dtype_id<T>(), pi, &map) == cudaSuccess;
+  const int* sel = stage ? wide : nullptr;
+  if (stage) {
+    const int smem = stage_smem_bytes<T, NS>();
+    cudaError_t e = smem_attr_once<forward_kernel<ZB_FWD, ZS, NS, T, FDK, true>>(smem);
     if (e != cudaSuccess) return e;
-    forward_kernel<ZB_FWD, T, FDK, true><<<ntiles, NT, smem, s>>>((const T*)proj, pi, geom, vi, vol);
-  } else {
-    forward_kernel<ZB_FWD, T, FDK, false><<<ntiles, NT, 0, s>>>((const T*)proj, pi, geom, vi, vol);
+    forward_kernel<ZB_FWD, ZS, NS, T, FDK, true>
+        <<<nblocks, NT, smem, s>>>((const T*)proj, map, pi, geom, vi, vol, sel);
+    e = cudaGetLastError();
+    if (e != cudaSuccess || !sel) return e;
   }
+  forward_kernel<ZB_FWD, ZS, FWD_NS, T, FDK, false>
+      <<<nblocks, NT, 0, s>>>((const T*)proj, map, pi, geom, vi, vol, sel);
   return cudaGetLastError();
 }
 
+// Slices of a tile per CTA and staging slots, by the number of 16^3 tiles: with
+// too few tiles to fill the SMs, half tiles, and with few enough for one CTA per
+// SM, four slots (a view's arithmetic there is shorter than a copy's latency).
+// Measured, ms, 16 slices and 2 slots / 8 and 2 / 8 and 4: 64 tiles x 60 views
+// 0.095 / 0.071 / 0.067, 216 x 248 0.452 / 0.383 / 0.510, 512 x 248 0.748 /
+// 0.794 / 1.044; quarter tiles were slower throughout.
+constexpr int FWD_FEW_TILES = 76, FWD_SOME_TILES = 304;
+constexpr int FWD_NS_FEW = 4;
+
+template <typename T, bool FDK>
+static cudaError_t forward_dispatch(const void* proj, const ProjInfo& pi, const ViewGeom* geom,
+                                    const VolInfo& vi, float* vol, const int* wide,
+                                    cudaStream_t s) {
+  const int n = vi.tiles_x * vi.tiles_y * vi.tiles_z;
+  if (n <= FWD_FEW_TILES)
+    return forward_launch<8, FWD_NS_FEW, T, FDK>(proj, pi, geom, vi, vol, wide, s);
+  if (n <= FWD_SOME_TILES)
+    return forward_launch<8, FWD_NS, T, FDK>(proj, pi, geom, vi, vol, wide, s);
+  return forward_launch<16, FWD_NS, T, FDK>(proj, pi, geom, vi, vol, wide, s);
+}
+
+template <typename T, bool FDK>
+static cudaError_t prepare_forward_t() {
+  constexpr int smem = stage_smem_bytes<T, FWD_NS>();
+  cudaError_t e = smem_attr_once<forward_kernel<ZB_FWD, 16, FWD_NS, T, FDK, true>>(smem);
+  if (e == cudaSuccess) e = smem_attr_once<forward_kernel<ZB_FWD, 8, FWD_NS, T, FDK, true>>(smem);
+  if (e == cudaSuccess)
+    e = smem_attr_once<forward_kernel<ZB_FWD, 8, FWD_NS_FEW, T, FDK, true>>(
+        stage_smem_bytes<T, FWD_NS_FEW>());
+  return e;
+}
+
 cudaError_t prepare_forward(int dtype, int fdk) {
-  if (dtype == 0)
-    return fdk ? smem_attr_once<forward_kernel<ZB_FWD, float, true, true>>(fwd_smem_bytes<float>())
-               : smem_attr_once<forward_kernel<ZB_FWD, float, false, true>>(fwd_smem_bytes<float>());
+  if (dtype == 0) return fdk ? prepare_forward_t<float, true>() : prepare_forward_t<float, false>();
   if (dtype == 1)
-    return fdk ? smem_attr_once<forward_kernel<ZB_FWD, __half, true, true>>(fwd_smem_bytes<__half>())
-               : smem_attr_once<forward_kernel<ZB_FWD, __half, false, true>>(fwd_smem_bytes<__half>());
-  constexpr int sb = fwd_smem_bytes<__nv_bfloat16>();
-  return fdk ? smem_attr_once<forward_kernel<ZB_FWD, __nv_bfloat16, true, true>>(sb)
-             : smem_attr_once<forward_kernel<ZB_FWD, __nv_bfloat16, false, true>>(sb);
+    return fdk ? prepare_forward_t<__half, true>() : prepare_forward_t<__half, false>();
+  return fdk ? prepare_forward_t<__nv_bfloat16, true>()
+             : prepare_forward_t<__nv_bfloat16, false>();
 }
 
 cudaError_t launch_forward(const void* proj, int dtype, const ProjInfo& pi, const ViewGeom* geom,
-                           const VolInfo& vi_in, int fdk, float* vol, cudaStream_t s) {
+                           const VolInfo& vi_in, int fdk, float* vol, const int* wide,
+                           cudaStream_t s) {
   VolInfo vi = vi_in;  // the forward tiles z by ZB_FWD
   vi.zb = ZB_FWD;
   vi.tiles_z = (vi.nz + ZB_FWD - 1) / ZB_FWD;
   if (dtype == 0)
-    return fdk ? forward_dispatch<float, true>(proj, pi, geom, vi, vol, s)
-               : forward_dispatch<float, false>(proj, pi, geom, vi, vol, s);
+    return fdk ? forward_dispatch<float, true>(proj, pi, geom, vi, vol, wide, s)
+               : forward_dispatch<float, false>(proj, pi, geom, vi, vol, wide, s);
   if (dtype == 1)
-    return fdk ? forward_dispatch<__half, true>(proj, pi, geom, vi, vol, s)
-               : forward_dispatch<__half, false>(proj, pi, geom, vi, vol, s);
-  return fdk ? forward_dispatch<__nv_bfloat16, true>(proj, pi, geom, vi, vol, s)
-             : forward_dispatch<__nv_bfloat16, false>(proj, pi, geom, vi, vol, s);
+    return fdk ? forward_dispatch<__half, true>(proj, pi, geom, vi, vol, wide, s)
+               : forward_dispatch<__half, false>(proj, pi, geom, vi, vol, wide, s);
+  return fdk ? forward_dispatch<__nv_bfloat16, true>(proj, pi, geom, vi, vol, wide, s)
+             : forward_dispatch<__nv_bfloat16, false>(proj, pi, geom, vi, vol, wide, s);
 }
 
 // ------------------------------------------------------- gradient images
@@ -991,11 +1106,8 @@ __device__ __forceinline__ int scatter_slot(int lane) {
 //
 // Sources of the samples (SRC):
 //   SRC_GLOBAL  gradient images (CENTRAL) or raw taps (EXACT) from global memory;
-//   SRC_SMEM    the tile footprint staged in shared memory -- raw taps for
-//               EXACT, and for CENTRAL the 4x4-minus-corners neighbourhood
-//               whose central differences equal the gradient images there
-//               (only for "central-safe" tiles, whose differences never use
-//               the one-sided edge rule).
+//   SRC_SMEM    the tile footprint staged in shared memory (EXACT; staged
+//               CENTRAL tiles run vjp_view_central2 below).
 enum { SRC_GLOBAL = 0, SRC_SMEM = 1 };
 
 //
@@ -1003,31 +1115,31 @@ enum { SRC_GLOBAL = 0, SRC_SMEM = 1 };
 // the coordinates are never clamped (EDGE then only guards the scatter of
 // the fused data VJP).
 template <int ZB, typename T, bool FDK, bool EXACT, bool EDGE, bool PROJ, int SRC,
-          typename E = T, int P = StageGeom<T>::P>
-__device__ __forceinline__ void vjp_view(const T* img, const float2* gimg, const E* buf,
+          int P = StageGeom<T>::P>
+__device__ __forceinline__ void vjp_view(const T* img, const float2* gimg, unsigned buf,
                                          float* pout, float* qout, long long rs, int nu, int nv,
                                          const TileView& t, float dx, float dy,
                                          const float (&delta)[ZB], float (&S)[3], float (&Z)[3]) {
   constexpr bool CLAMP = EDGE && SRC == SRC_GLOBAL;
   
-  float u0 = fmaf(dy, t.ru[1], fmaf(dx, t.ru[0], t.U0));
-  float v0 = fmaf(dy, t.rv[1], fmaf(dx, t.rv[0], t.V0));
-  float w0 = fmaf(dy, t.rw[1], fmaf(dx, t.rw[0], t.W0));
+  float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
+  float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
+  float w0 = fmaf(dy, t.rw1, fmaf(dx, t.rw0, t.W0));
 #pragma unroll
   for (int k = 0; k < ZB; ++k) {
     const float dz = k - 0.5f * (ZB - 1);
-    Sample s = locate<CLAMP>(fmaf(dz, t.ru[2], u0), fmaf(dz, t.rv[2], v0), fmaf(dz, t.rw[2], w0),
+    Sample s = locate<CLAMP>(fmaf(dz, t.ru2, u0), fmaf(dz, t.rv2, v0), fmaf(dz, t.rw2, w0),
                              t, nu, nv);
     if (CLAMP && !s.ok) continue;
-    float gu, gv, val = 0.0f, gscale = 1.0f;
+    float gu, gv, val = 0.0f;
     if (EXACT) {
       float d00, d10, d01, d11;
       if (SRC == SRC_SMEM) {
-        const E* q = staged_tap<P>(buf, t, s.bx, s.by);
-        d00 = tof(q[0]);
-        d10 = tof(q[1]);
-        d01 = tof(q[P]);
-        d11 = tof(q[P + 1]);
+        const unsigned q = staged_tap<T, 0>(buf, t, s.bx, s.by);
+        d00 = lds<0>(q);
+        d10 = lds<1>(q);
+        d01 = lds<P>(q);
+        d11 = lds<P + 1>(q);
       } else {
         taps<EDGE>(img, rs, nu, nv, s, d00, d10, d01, d11);
       }
@@ -1036,19 +1148,6 @@ __device__ __forceinline__ void vjp_view(const T* img, const float2* gimg, const
       const float c = d01 - d00, d = d11 - d10;
       gv = fmaf(s.tu, d - c, c);
       if (FDK) val = bilerp(s.tu, s.tv, d00, d10, d01, d11);
-    } else if (SRC == SRC_SMEM) {
-      // central-safe interior tile: 12 staged taps around (iu, iv)
-      constexpr int p = P;
-      const E* q = staged_tap<P, 1>(buf, t, s.bx, s.by);
-      const float a0 = tof(q[-p]), a1 = tof(q[-p + 1]);
-      const float b0 = tof(q[-1]), b1 = tof(q[0]), b2 = tof(q[1]), b3 = tof(q[2]);
-      const float c0 = tof(q[p - 1]), c1 = tof(q[p]), c2 = tof(q[p + 1]), c3 = tof(q[p + 2]);
-      const float e0 = tof(q[2 * p]), e1 = tof(q[2 * p + 1]);
-      // twice the central-difference gradient images at the four tap pixels
-      gu = bilerp(s.tu, s.tv, b2 - b0, b3 - b1, c2 - c0, c3 - c1);
-      gv = bilerp(s.tu, s.tv, c1 - a0, c2 - a1, e0 - b1, e1 - b2);
-      gscale = 0.5f;
-      if (FDK) val = bilerp(s.tu, s.tv, b1, b2, c1, c2);
     } else {
       float2 g00, g10, g01, g11;
       const float2 z2 = make_float2(0.0f, 0.0f);
@@ -1079,8 +1178,7 @@ __device__ __forceinline__ void vjp_view(const T* img, const float2* gimg, const
     }
     float sd = delta[k] * (FDK ? s.rwi * (s.rwi * t.wgt) : t.wgt);
     const float sr = sd * s.rwi;
-    const float sg = sr * gscale;
-    const float a0 = gu * sg, a1 = gv * sg;
+    const float a0 = gu * sr, a1 = gv * sr;
     float a2 = -fmaf(a0, s.x, a1 * s.y);
     if (FDK) a2 = fmaf(-2.0f * sr, val, a2);
     S[0] += a0;
@@ -1095,22 +1193,322 @@ __device__ __forceinline__ void vjp_view(const T* img, const float2* gimg, const
   }
 }
 
+// The tile's dL/dvol in shared memory, element k of thread tid's column.  The
+// fused data VJP's line pass needs [z][y][x] (row pitch TX + 1); otherwise the
+// columns are stored as [k / 2][thread] pairs, one conflict-free 8-byte load
+// per pair of voxels.
+template <bool PROJ>
+__device__ __forceinline__ int delta_base(int lx, int ly) {
+  return PROJ ? ly * (TX + 1) + lx : 2 * (int)threadIdx.x;
+}
+template <bool PROJ>
+__device__ __forceinline__ int delta_off(int k) {
+  return PROJ ? k * (TY * (TX + 1)) : (k >> 1) * (2 * NT) + (k & 1);
+}
+
+// The sums of one thread's column over a view (see vjp_view).
+struct Sums6 {
+  float S[3], Z[3];
+};
+
+// One view from global memory of a tile that crosses the detector's edge (or
+// whose footprint is not staged): the arithmetic of vjp_view, in the same
+// order.  A loop over pairs of voxels, not one unrolled body: such a body was
+// ~30 KB of code, and the warps, which drift apart, streamed it through the
+// instruction cache.  A pair that is off the detector for the whole warp is
+// left out (its gradients are 0; a non-finite upstream value keeps its pair,
+// 0 * inf must stay NaN).  delta(k) gives the upstream gradient of voxel k.
+template <int ZB, typename T, bool FDK, bool EXACT, bool PROJ>
+__device__ __forceinline__ Sums6 vjp_view_edge(const T* img, const float2* gimg, float* pout,
+                                            long long rs, int nu, int nv, const TileView& t,
+                                            float dx, float dy, const float* delta) {
+  float S[3] = {0.0f, 0.0f, 0.0f}, Z[3] = {0.0f, 0.0f, 0.0f};
+  const float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
+  const float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
+  const float w0 = fmaf(dy, t.rw1, fmaf(dx, t.rw0, t.W0));
+#pragma unroll 1
+  for (int k0 = 0; k0 < ZB; k0 += 2) {
+    constexpr int G = 2;
+    Sample s[G];
+    float d[G], gu[G], gv[G], val[G];
+    bool live = false;
+#pragma unroll
+    for (int q = 0; q < G; ++q) {
+      const float dz = (k0 + q) - 0.5f * (ZB - 1);
+      s[q] = locate<true>(fmaf(dz, t.ru2, u0), fmaf(dz, t.rv2, v0), fmaf(dz, t.rw2, w0), t, nu, nv);
+      d[q] = delta[delta_off<PROJ>(k0 + q)];
+      val[q] = 0.0f;
+      live |= (s[q].ok && (unsigned)(s[q].iu + 1) <= (unsigned)nu &&
+               (unsigned)(s[q].iv + 1) <= (unsigned)nv) ||
+              !(fabsf(d[q]) <= 3.402823466e38f);
+    }
+    if (!__any_sync(0xffffffffu, live)) continue;
+#pragma unroll
+    for (int q = 0; q < G; ++q) {
+      float d00, d10, d01, d11;
+      if (EXACT || FDK) taps<true>(img, rs, nu, nv, s[q], d00, d10, d01, d11);
+      if (EXACT) {
+        const float a = d10 - d00, b = d11 - d01;
+        gu[q] = fmaf(s[q].tv, b - a, a);
+        const float c = d01 - d00, e = d11 - d10;
+        gv[q] = fmaf(s[q].tu, e - c, c);
+      } else {
+        const float2 z2 = make_float2(0.0f, 0.0f);
+        const bool uu0 = (unsigned)s[q].iu < (unsigned)nu;
+        const bool uu1 = (unsigned)(s[q].iu + 1) < (unsigned)nu;
+        const bool vv0 = (unsigned)s[q].iv < (unsigned)nv;
+        const bool vv1 = (unsigned)(s[q].iv + 1) < (unsigned)nv;
+        const float2* p = gimg + (long long)s[q].iv * nu + s[q].iu;
+        const float2 g00 = (uu0 && vv0 && s[q].ok) ? __ldg(p) : z2;
+        const float2 g10 = (uu1 && vv0 && s[q].ok) ? __ldg(p + 1) : z2;
+        const float2 g01 = (uu0 && vv1 && s[q].ok) ? __ldg(p + nu) : z2;
+        const float2 g11 = (uu1 && vv1 && s[q].ok) ? __ldg(p + nu + 1) : z2;
+        gu[q] = bilerp(s[q].tu, s[q].tv, g00.x, g10.x, g01.x, g11.x);
+        gv[q] = bilerp(s[q].tu, s[q].tv, g00.y, g10.y, g01.y, g11.y);
+      }
+      if (FDK) val[q] = bilerp(s[q].tu, s[q].tv, d00, d10, d01, d11);
+    }
+#pragma unroll
+    for (int q = 0; q < G; ++q) {
+      if (!s[q].ok) continue;
+      const float dz = (k0 + q) - 0.5f * (ZB - 1);
+      const float sd = d[q] * (FDK ? s[q].rwi * (s[q].rwi * t.wgt) : t.wgt);
+      const float sr = sd * s[q].rwi;
+      const float a0 = gu[q] * sr, a1 = gv[q] * sr;
+      float a2 = -fmaf(a0, s[q].x, a1 * s[q].y);
+      if (FDK) a2 = fmaf(-2.0f * sr, val[q], a2);
+      S[0] += a0;
+      S[1] += a1;
+      S[2] += a2;
+      Z[0] = fmaf(a0, dz, Z[0]);
+      Z[1] = fmaf(a1, dz, Z[1]);
+      Z[2] = fmaf(a2, dz, Z[2]);
+      if (PROJ && d[q] != 0.0f)
+        scatter_sample<true>(pout, nullptr, nu, nv, s[q],
+                             d[q] * (FDK ? s[q].rwi * (s[q].rwi * t.wgtd) : t.wgtd));
+    }
+  }
+  return Sums6{{S[0], S[1], S[2]}, {Z[0], Z[1], Z[2]}};
+}
+
+// Twice the difference of one tap pixel along an axis from its neighbours l, r
+// (c is the pixel itself): r - l inside, twice the one-sided difference on the
+// first and last pixel, 0 off the detector -- the gradient images' values, bit
+// for bit (times 2).  f is the pixel's coordinate, [lo, hi] the detector's, as
+// floats that hold integers.
+struct EdgeRule {
+  bool first, last, off;
+  __device__ __forceinline__ EdgeRule(float f, float lo, float hi)
+      : first(f == lo), last(f == hi), off(f < lo || f > hi) {}
+  __device__ __forceinline__ float operator()(float l, float c, float r) const {
+    const float d = (last ? c : r) - (first ? c : l);
+    return off ? 0.0f : (first || last) ? d + d : d;
+  }
+};
+
+// Range of dz with a + b dz >= 0, intersected into [lo, hi].
+__device__ __forceinline__ void clip_range(float a, float b, float& lo, float& hi) {
+  const float q = __fdividef(-a, b);
+  if (b > 0.0f) lo = fmaxf(lo, q);
+  else if (b < 0.0f) hi = fminf(hi, q);
+  else if (a < 0.0f) hi = -INFINITY;
+}
+
+// Range of dz in which a column's samples lie in [x0, x1] x [y0, y1] (anchored
+// pixels; w > 0): u/w >= x0 is linear in dz, u - x0 w >= 0.
+__device__ __forceinline__ void column_range(const TileView& t, float u0, float v0, float w0,
+                                             float x0, float x1, float y0, float y1, float& lo,
+                                             float& hi) {
+  lo = -INFINITY;
+  hi = INFINITY;
+  clip_range(fmaf(-x0, w0, u0), fmaf(-x0, t.rw2, t.ru2), lo, hi);
+  clip_range(fmaf(x1, w0, -u0), fmaf(x1, t.rw2, -t.ru2), lo, hi);
+  clip_range(fmaf(-y0, w0, v0), fmaf(-y0, t.rw2, t.rv2), lo, hi);
+  clip_range(fmaf(y1, w0, -v0), fmaf(y1, t.rw2, -t.rv2), lo, hi);
+}
+
+// One view of a staged CENTRAL tile that crosses the detector's edge: the
+// packed arithmetic of vjp_view_central2 on the zero-padded footprint, the sums
+// taken sample by sample as vjp_view_edge takes them.  Per column the slices
+// that touch the detector and those that are central-safe are intervals (a
+// linear inequality per detector side), so a warp visits only the pairs some
+// lane needs, and pairs that are safe for every lane run without any test; in
+// the others each sample is classified, the edge rules of the gradient images
+// are applied to the differences where needed, and only samples that touch the
+// detector are added.  The intervals are taken 0.01 px wide (on) and narrow
+// (safe), far beyond their rounding error.  Reading the gradient images from
+// global memory here instead (eight scattered loads per sample) took 2.5 times
+// as long per (tile, view) as a central-safe one.
+template <int ZB, typename T, bool FDK, bool PROJ>
+__device__ __forceinline__ Sums6 vjp_view_edge2(unsigned buf, float* pout, float* qout, int nu, int nv,
+                                             const TileView& t, float dx, float dy,
+                                             const float* delta, bool finite) {
+  float S[3] = {0.0f, 0.0f, 0.0f}, Z[3] = {0.0f, 0.0f, 0.0f};
+  constexpr int P = StageGeom<T>::P;
+  const float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
+  const float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
+  const float w0 = fmaf(dy, t.rw1, fmaf(dx, t.rw0, t.W0));
+  const f2 M2 = pk2(MAGIC, MAGIC), HALF = pk2(0.5f, 0.5f), IC = pk2(t.ic, t.ic);
+  const f2 WG = pk2(t.wgt, t.wgt), WGD = pk2(t.wgtd, t.wgtd);
+  // detector pixels [xl, xr] x [yl, yr] in the anchored frame
+  const float xl = -(float)t.au, xr = (float)(nu - 1 - t.au);
+  const float yl = -(float)t.av, yr = (float)(nv - 1 - t.av);
+  constexpr float M = 0.01f, HZ = 0.5f * (ZB - 1);
+  float lo, hi;
+  column_range(t, u0, v0, w0, xl - 1.0f - M, xr + 1.0f + M, yl - 1.0f - M, yr + 1.0f + M, lo, hi);
+  int k0 = 0, k1 = ZB;  // slices that touch the detector in some lane
+  if (finite) {
+    const bool some = lo <= hi;
+    k0 = __reduce_min_sync(0xffffffffu,
+                           some ? (int)ceilf(fminf(fmaxf(lo + HZ, 0.0f), (float)ZB)) : ZB);
+    k1 = __reduce_max_sync(0xffffffffu,
+                           some ? (int)floorf(fminf(fmaxf(hi + HZ, -1.0f), ZB - 1.0f)) + 1 : 0);
+  }
+  column_range(t, u0, v0, w0, xl + 1.0f + M, xr - 1.0f - M, yl + 1.0f + M, yr - 1.0f - M, lo, hi);
+  // slices [s0, s1) are central-safe in every lane
+  const bool some = finite && lo <= hi;
+  const int s0 = __reduce_max_sync(
+      0xffffffffu, some ? (int)ceilf(fminf(fmaxf(lo + HZ, 0.0f), (float)ZB)) : ZB);
+  const int s1 = __reduce_min_sync(
+      0xffffffffu, some ? (int)floorf(fminf(fmaxf(hi + HZ, -1.0f), ZB - 1.0f)) + 1 : 0);
+#pragma unroll 1
+  for (int k = k0 & ~1; k < k1; k += 2) {
+    const bool safe = k >= s0 && k + 2 <= s1;
+    const float dz0 = k - HZ;
+    const f2 dz = pk2(dz0, dz0 + 1.0f);
+    const f2 u = fma2(dz, pk2(t.ru2, t.ru2), pk2(u0, u0));
+    const f2 v = fma2(dz, pk2(t.rv2, t.rv2), pk2(v0, v0));
+    const f2 w = fma2(dz, pk2(t.rw2, t.rw2), pk2(w0, w0));
+    float wl, wh;
+    up2(w, wl, wh);
+    const f2 r = pk2(rcp_approx(wl), rcp_approx(wh));
+    const f2 x = mul2(u, r), y = mul2(v, r);
+    const f2 fx = sub2(add2_rd(x, M2), M2), fy = sub2(add2_rd(y, M2), M2);
+    float d[2], xs[2], ys[2], fxs[2], fys[2];
+    up2(x, xs[0], xs[1]);
+    up2(y, ys[0], ys[1]);
+    up2(fx, fxs[0], fxs[1]);
+    up2(fy, fys[0], fys[1]);
+    bool use[2] = {true, true};
+    unsigned flags = safe ? 1u : 0u;  // 1: a sample to add, 2 / 4: one at the border along u / v
+#pragma unroll
+    for (int q = 0; q < 2; ++q) d[q] = delta[delta_off<PROJ>(k + q)];
+    if (!safe) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      use[q] = (fxs[q] >= xl - 1.0f && fxs[q] <= xr && fys[q] >= yl - 1.0f && fys[q] <= yr) ||
+               !(fabsf(d[q]) <= 3.402823466e38f);
+      if (use[q])  // a central-safe sample has its floor pixel in [1, n-3]
+        flags |= 1u | (fxs[q] >= xl + 1.0f && fxs[q] <= xr - 2.0f ? 0u : 2u) |
+                 (fys[q] >= yl + 1.0f && fys[q] <= yr - 2.0f ? 0u : 4u);
+    }
+    flags = __reduce_or_sync(0xffffffffu, flags);
+    if (!flags) continue;
+    }
+    const f2 tu = sub2(x, fx), tv = sub2(y, fy);
+    unsigned ql, qh;
+    staged_pair<T, 1>(buf, t, IC, fx, fy, ql, qh);
+    const f2 a0 = lds2<-P>(ql, qh), a1 = lds2<-P + 1>(ql, qh);
+    const f2 b0 = lds2<-1>(ql, qh), b1 = lds2<0>(ql, qh), b2 = lds2<1>(ql, qh),
+             b3 = lds2<2>(ql, qh);
+    const f2 c0 = lds2<P - 1>(ql, qh), c1 = lds2<P>(ql, qh), c2 = lds2<P + 1>(ql, qh),
+             c3 = lds2<P + 2>(ql, qh);
+    const f2 e0 = lds2<2 * P>(ql, qh), e1 = lds2<2 * P + 1>(ql, qh);
+    // twice the gradient images' values at the four tap pixels
+    f2 gu00, gu10, gu01, gu11, gv00, gv10, gv01, gv11;
+#define BP_RULE(rule, g, l, c, r_)                                        \
+  {                                                                       \
+    float l0, l1, m0, m1, n0, n1;                                         \
+    up2(l, l0, l1);                                                       \
+    up2(c, m0, m1);                                                       \
+    up2(r_, n0, n1);                                                      \
+    g = pk2(rule##0(l0, m0, n0), rule##1(l1, m1, n1));                    \
+  }
+    if (flags & 2u) {
+      const EdgeRule p0(fxs[0], xl, xr), p1(fxs[1], xl, xr);
+      BP_RULE(p, gu00, b0, b1, b2)
+      BP_RULE(p, gu01, c0, c1, c2)
+      const EdgeRule q0(fxs[0] + 1.0f, xl, xr), q1(fxs[1] + 1.0f, xl, xr);
+      BP_RULE(q, gu10, b1, b2, b3)
+      BP_RULE(q, gu11, c1, c2, c3)
+    } else {
+      gu00 = sub2(b2, b0);
+      gu10 = sub2(b3, b1);
+      gu01 = sub2(c2, c0);
+      gu11 = sub2(c3, c1);
+    }
+    if (flags & 4u) {
+      const EdgeRule p0(fys[0], yl, yr), p1(fys[1], yl, yr);
+      BP_RULE(p, gv00, a0, b1, c1)
+      BP_RULE(p, gv10, a1, b2, c2)
+      const EdgeRule q0(fys[0] + 1.0f, yl, yr), q1(fys[1] + 1.0f, yl, yr);
+      BP_RULE(q, gv01, b1, c1, e0)
+      BP_RULE(q, gv11, b2, c2, e1)
+    } else {
+      gv00 = sub2(c1, a0);
+      gv10 = sub2(c2, a1);
+      gv01 = sub2(e0, b1);
+      gv11 = sub2(e1, b2);
+    }
+#undef BP_RULE
+    const f2 D = pk2(d[0], d[1]);
+    const f2 sr = mul2(mul2(D, FDK ? mul2(r, mul2(r, WG)) : WG), r);
+    float gu[2], gv[2], val[2], srs[2], sgs[2];
+    up2(bilerp2(tu, tv, gu00, gu10, gu01, gu11), gu[0], gu[1]);
+    up2(bilerp2(tu, tv, gv00, gv10, gv01, gv11), gv[0], gv[1]);
+    if (FDK) up2(bilerp2(tu, tv, b1, b2, c1, c2), val[0], val[1]);
+    up2(sr, srs[0], srs[1]);
+    up2(mul2(sr, HALF), sgs[0], sgs[1]);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      if (!use[q]) continue;
+      const float a0s = gu[q] * sgs[q], a1s = gv[q] * sgs[q];
+      float a2s = -fmaf(a0s, xs[q], a1s * ys[q]);
+      if (FDK) a2s = fmaf(-2.0f * srs[q], val[q], a2s);
+      S[0] += a0s;
+      S[1] += a1s;
+      S[2] += a2s;
+      Z[0] = fmaf(a0s, dz0 + q, Z[0]);
+      Z[1] = fmaf(a1s, dz0 + q, Z[1]);
+      Z[2] = fmaf(a2s, dz0 + q, Z[2]);
+    }
+    if (PROJ) {
+      float tus[2], tvs_[2], sp[2];
+      up2(tu, tus[0], tus[1]);
+      up2(tv, tvs_[0], tvs_[1]);
+      up2(mul2(D, FDK ? mul2(r, mul2(r, WGD)) : WGD), sp[0], sp[1]);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        if (!use[q] || d[q] == 0.0f) continue;
+        Sample s;
+        s.tu = tus[q];
+        s.tv = tvs_[q];
+        s.iu = (int)fxs[q] + t.au;
+        s.iv = (int)fys[q] + t.av;
+        scatter_sample<true>(pout, qout, nu, nv, s, sp[q]);
+      }
+    }
+  }
+  return Sums6{{S[0], S[1], S[2]}, {Z[0], Z[1], Z[2]}};
+}
+
 // The CENTRAL sample loop from a staged central-safe footprint with packed
 // pairs of voxels (k, k+1): the steps of vjp_view in the same order on
 // f32x2 pairs, with the w-component kept negated (na2 = -a2) so that no
 // negation instruction is needed.  Even and odd voxels are summed in the two
 // halves of the pair accumulators and added at the end.
-template <int ZB, typename T, bool FDK, bool EDGE, bool PROJ, int P = StageGeom<T>::P>
-__device__ __forceinline__ void vjp_view_central2(const T* buf, float* pout, float* qout, int nu,
+template <int ZB, typename T, bool FDK, bool PROJ, bool LINES>
+__device__ __forceinline__ void vjp_view_central2(unsigned buf, float* pout, float* qout, int nu,
                                                   int nv, const TileView& t, float dx, float dy,
-                                                  const float (&delta)[ZB], float (&S)[3],
+                                                  const float* dcol, float (&S)[3],
                                                   float (&Z)[3]) {
-  
-  const float u0 = fmaf(dy, t.ru[1], fmaf(dx, t.ru[0], t.U0));
-  const float v0 = fmaf(dy, t.rv[1], fmaf(dx, t.rv[0], t.V0));
-  const float w0 = fmaf(dy, t.rw[1], fmaf(dx, t.rw[0], t.W0));
+  constexpr int P = StageGeom<T>::P;
+  const f2 IC = pk2(t.ic, t.ic);
+  const float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
+  const float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
+  const float w0 = fmaf(dy, t.rw1, fmaf(dx, t.rw0, t.W0));
   const f2 U0 = pk2(u0, u0), V0 = pk2(v0, v0), W0 = pk2(w0, w0);
-  const f2 RU = pk2(t.ru[2], t.ru[2]), RV = pk2(t.rv[2], t.rv[2]), RW = pk2(t.rw[2], t.rw[2]);
+  const f2 RU = pk2(t.ru2, t.ru2), RV = pk2(t.rv2, t.rv2), RW = pk2(t.rw2, t.rw2);
   const f2 M2 = pk2(MAGIC, MAGIC), TWO = pk2(2.0f, 2.0f), HALF = pk2(0.5f, 0.5f);
   const f2 WG = pk2(t.wgt, t.wgt);
   const f2 WGD = pk2(t.wgtd, t.wgtd);
@@ -1132,22 +1530,23 @@ __device__ __forceinline__ void vjp_view_central2(const T* buf, float* pout, flo
     const f2 r = pk2(rcp_approx(wl), rcp_approx(wh));
     const f2 x = mul2(u, r), y = mul2(v, r);
     const f2 rx = add2_rd(x, M2), ry = add2_rd(y, M2);
-    const f2 tu = sub2(x, sub2(rx, M2)), tv = sub2(y, sub2(ry, M2));
-    float bxl, bxh, byl, byh;
-    up2(rx, bxl, bxh);
-    up2(ry, byl, byh);
-    const T* ql = staged_tap<P, 1>(buf, t, __float_as_int(bxl), __float_as_int(byl));
-    const T* qh = staged_tap<P, 1>(buf, t, __float_as_int(bxh), __float_as_int(byh));
-#define BP_TAP2(o) pk2(tof(ql[o]), tof(qh[o]))
-    const f2 a0 = BP_TAP2(-P), a1 = BP_TAP2(-P + 1);
-    const f2 b0 = BP_TAP2(-1), b1 = BP_TAP2(0), b2 = BP_TAP2(1), b3 = BP_TAP2(2);
-    const f2 c0 = BP_TAP2(P - 1), c1 = BP_TAP2(P), c2 = BP_TAP2(P + 1), c3 = BP_TAP2(P + 2);
-    const f2 e0 = BP_TAP2(2 * P), e1 = BP_TAP2(2 * P + 1);
-#undef BP_TAP2
+    const f2 fx = sub2(rx, M2), fy = sub2(ry, M2);
+    const f2 tu = sub2(x, fx), tv = sub2(y, fy);
+    unsigned ql, qh;
+    staged_pair<T, 1>(buf, t, IC, fx, fy, ql, qh);
+    const f2 a0 = lds2<-P>(ql, qh), a1 = lds2<-P + 1>(ql, qh);
+    const f2 b0 = lds2<-1>(ql, qh), b1 = lds2<0>(ql, qh), b2 = lds2<1>(ql, qh),
+             b3 = lds2<2>(ql, qh);
+    const f2 c0 = lds2<P - 1>(ql, qh), c1 = lds2<P>(ql, qh), c2 = lds2<P + 1>(ql, qh),
+             c3 = lds2<P + 2>(ql, qh);
+    const f2 e0 = lds2<2 * P>(ql, qh), e1 = lds2<2 * P + 1>(ql, qh);
     // twice the central-difference gradient images at the four tap pixels
     const f2 gu = bilerp2(tu, tv, sub2(b2, b0), sub2(b3, b1), sub2(c2, c0), sub2(c3, c1));
     const f2 gv = bilerp2(tu, tv, sub2(c1, a0), sub2(c2, a1), sub2(e0, b1), sub2(e1, b2));
-    const f2 D = pk2(delta[2 * p], delta[2 * p + 1]);
+    // (from shared memory: the column's 16 registers would spill others; fused VJP
+    // of c2 15.85 -> 15.32 ms, motion VJP 10.5 -> 10.0 ms when it was measured)
+    const f2 D = LINES ? pk2(dcol[delta_off<true>(2 * p)], dcol[delta_off<true>(2 * p + 1)])
+                       : *reinterpret_cast<const f2*>(dcol + delta_off<false>(2 * p));
     const f2 sd = mul2(D, FDK ? mul2(r, mul2(r, WG)) : WG);
     const f2 sr = mul2(sd, r);
     const f2 sg = mul2(sr, HALF);
@@ -1167,6 +1566,9 @@ __device__ __forceinline__ void vjp_view_central2(const T* buf, float* pout, flo
       const f2 SD = mul2(D, FDK ? mul2(r, mul2(r, WGD)) : WGD);
       const f2 Q1 = mul2(SD, tv), Q0 = sub2(SD, Q1);
       const f2 W11 = mul2(Q1, tu), W01 = sub2(Q1, W11), W10 = mul2(Q0, tu), W00 = sub2(Q0, W10);
+      float bxl, bxh, byl, byh;
+      up2(rx, bxl, bxh);
+      up2(ry, byl, byh);
       float w[4][2];
       up2(W00, w[0][0], w[0][1]);
       up2(W10, w[1][0], w[1][1]);
@@ -1230,16 +1632,16 @@ __device__ __forceinline__ void proj_lines(float* __restrict__ pout, float* __re
                                            const float* __restrict__ dsm) {
   static_assert(ZB == TX && TY == TX, "lines run along a 16-voxel tile edge");
   const int a = threadIdx.x & (TX - 1), b = threadIdx.x / TX;
-  const bool alongx = fabsf(t.ru[0]) <= fabsf(t.ru[1]);
+  const bool alongx = fabsf(t.ru0) <= fabsf(t.ru1);
   const float fa = a - 0.5f * (TX - 1), fb = b - 0.5f * (ZB - 1);
   // x-lines: voxels (k, a, b); y-lines: (a, k, b)
-  const float ou = alongx ? t.ru[1] : t.ru[0], ov = alongx ? t.rv[1] : t.rv[0];
-  const float ow = alongx ? t.rw[1] : t.rw[0];
-  float su = alongx ? t.ru[0] : t.ru[1], sv = alongx ? t.rv[0] : t.rv[1];
-  float sw = alongx ? t.rw[0] : t.rw[1];
-  const float u0 = fmaf(fb, t.ru[2], fmaf(fa, ou, t.U0));
-  const float v0 = fmaf(fb, t.rv[2], fmaf(fa, ov, t.V0));
-  const float w0 = fmaf(fb, t.rw[2], fmaf(fa, ow, t.W0));
+  const float ou = alongx ? t.ru1 : t.ru0, ov = alongx ? t.rv1 : t.rv0;
+  const float ow = alongx ? t.rw1 : t.rw0;
+  float su = alongx ? t.ru0 : t.ru1, sv = alongx ? t.rv0 : t.rv1;
+  float sw = alongx ? t.rw0 : t.rw1;
+  const float u0 = fmaf(fb, t.ru2, fmaf(fa, ou, t.U0));
+  const float v0 = fmaf(fb, t.rv2, fmaf(fa, ov, t.V0));
+  const float w0 = fmaf(fb, t.rw2, fmaf(fa, ow, t.W0));
   // walk in the direction of increasing u: step kk visits voxel k = 15 - kk
   // when the axis runs against u (the negated steps give the same positions)
   const bool rev = su < 0.0f;
@@ -1328,46 +1730,64 @@ __device__ __forceinline__ void proj_lines(float* __restrict__ pout, float* __re
 // Staged CENTRAL (central-safe) tiles run the packed motion loop and, when
 // the data VJP is fused, the line pass above; the other tiles scatter the
 // data VJP per sample.
-template <int ZB, typename T, bool FDK, bool EXACT, bool PROJ, typename E, int P>
-__device__ __forceinline__ void vjp_tile_view(const T* img, const float2* gimg, const E* buf,
+template <int ZB, typename T, bool FDK, bool EXACT, bool PROJ, bool STAGE>
+__device__ __forceinline__ void vjp_tile_view(const T* img, const float2* gimg, unsigned buf,
                                               bool staged, float* pout, float* qout,
                                               const ProjInfo& pi, const TileView& t,
                                               const TileIdx& ti,
-                                              const float (&delta)[ZB], const float* dsm,
-                                              float (*redv)[12]) {
+                                              const float (&delta)[ZB], const float* dcol,
+                                              bool finite, const float* dsm, float (*redv)[12]) {
   float S[3] = {0.0f, 0.0f, 0.0f}, Z[3] = {0.0f, 0.0f, 0.0f};
-  if (staged && !EXACT) {
-    // CENTRAL footprints are staged only for central-safe, hence interior,
-    // tiles.  With the fused data VJP: the line pass where samples along
+  if (staged && !EXACT && t.csafe) {
+    // With the fused data VJP: the line pass where samples along
     // the ray-parallel axis move by at most BP_VJP_LINE_DU px per voxel
     // (there it merges most: about 4 (du + 1/16) atomics per sample), else
     // four atomics per sample from the packed loop, with fewer instructions
     if (PROJ && BP_VJP_LINES &&
-        fminf(fabsf(t.ru[0]), fabsf(t.ru[1])) <= BP_VJP_LINE_DU * t.W0) {
-      vjp_view_central2<ZB, E, FDK, false, false, P>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy,
-                                                     delta, S, Z);
+        fminf(fabsf(t.ru0), fabsf(t.ru1)) <= BP_VJP_LINE_DU * t.W0) {
+      vjp_view_central2<ZB, T, FDK, false, PROJ>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy,
+                                                 dcol, S, Z);
       proj_lines<ZB, FDK>(pout, qout, pi.nu, pi.nv, t, dsm);
     } else {
-      vjp_view_central2<ZB, E, FDK, false, PROJ, P>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy,
-                                                    delta, S, Z);
+      vjp_view_central2<ZB, T, FDK, PROJ, PROJ>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy,
+                                                dcol, S, Z);
     }
-  } else if (staged) {
+  } else if (!EXACT && staged) {
+    const Sums6 q =
+        vjp_view_edge2<ZB, T, FDK, PROJ>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy, dcol,
+                                         finite);
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      S[r] = q.S[r];
+      Z[r] = q.Z[r];
+    }
+  } else if (EXACT && staged) {
     // (the per-sample paths keep scalar scatters in the fused kernel: block
     // reductions of their in-range samples measured 1 % slower there,
     // 15.12 against 14.94 ms on c2, while the data VJP alone gains 10 %)
     if (t.mode == MODE_INTERIOR || !PROJ)
-      vjp_view<ZB, T, FDK, EXACT, false, PROJ, SRC_SMEM, E, P>(
-          img, gimg, buf, pout, nullptr, pi.rs, pi.nu, pi.nv, t, ti.dx, ti.dy, delta, S, Z);
+      vjp_view<ZB, T, FDK, EXACT, false, PROJ, SRC_SMEM>(img, gimg, buf, pout, nullptr, pi.rs,
+                                                         pi.nu, pi.nv, t, ti.dx, ti.dy, delta, S,
+                                                         Z);
     else
-      vjp_view<ZB, T, FDK, EXACT, true, PROJ, SRC_SMEM, E, P>(
-          img, gimg, buf, pout, nullptr, pi.rs, pi.nu, pi.nv, t, ti.dx, ti.dy, delta, S, Z);
+      vjp_view<ZB, T, FDK, EXACT, true, PROJ, SRC_SMEM>(img, gimg, buf, pout, nullptr, pi.rs, pi.nu,
+                                                        pi.nv, t, ti.dx, ti.dy, delta, S, Z);
   } else {
-    if (t.mode == MODE_INTERIOR)
-      vjp_view<ZB, T, FDK, EXACT, false, PROJ, SRC_GLOBAL, E, P>(
-          img, gimg, buf, pout, nullptr, pi.rs, pi.nu, pi.nv, t, ti.dx, ti.dy, delta, S, Z);
-    else
-      vjp_view<ZB, T, FDK, EXACT, true, PROJ, SRC_GLOBAL, E, P>(
-          img, gimg, buf, pout, nullptr, pi.rs, pi.nu, pi.nv, t, ti.dx, ti.dy, delta, S, Z);
+    // (where footprints can be staged, interior tiles come here only beside
+    // the detector's edge: they take the checked path, one code path less)
+    if (!STAGE && t.mode == MODE_INTERIOR)
+      vjp_view<ZB, T, FDK, EXACT, false, PROJ, SRC_GLOBAL>(img, gimg, buf, pout, nullptr, pi.rs,
+                                                           pi.nu, pi.nv, t, ti.dx, ti.dy, delta, S,
+                                                           Z);
+    else {
+      const Sums6 q = vjp_view_edge<ZB, T, FDK, EXACT, PROJ>(img, gimg, pout, pi.rs, pi.nu, pi.nv, t,
+                                                             ti.dx, ti.dy, dcol);
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        S[r] = q.S[r];
+        Z[r] = q.Z[r];
+      }
+    }
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float v[16];
@@ -1385,16 +1805,16 @@ __device__ __forceinline__ void vjp_tile_view(const T* img, const float2* gimg, 
 }
 
 // Write the record of one (tile, view): fixed-order sum of the 8 warps'
-// values, plus the anchors (threads 0..PSLOTS-1).
+// values, plus the anchors (16 consecutive threads, slot = 0 .. PSLOTS-1).
 __device__ __forceinline__ void vjp_write_record(const TileView& t, const float (*redv)[12],
-                                                 bool any, int j, int tile, int ntiles,
+                                                 bool bad, int slot, int j, int tile, int ntiles,
                                                  float* __restrict__ partials) {
-  const int slot = threadIdx.x;
   if (slot >= PSLOTS) return;
   float val = 0.0f;
   if (slot < 12) {
-    if (any && t.mode != MODE_SKIP)
+    if (t.mode != MODE_SKIP)
       for (int w = 0; w < NT / 32; ++w) val += redv[w][slot];
+    if (bad) val = __int_as_float(0x7fc00000);
   } else if (slot == 12) {
     val = (float)t.au;
   } else if (slot == 13) {
@@ -1406,45 +1826,45 @@ __device__ __forceinline__ void vjp_write_record(const TileView& t, const float 
 // Motion VJP (optionally fused with the data VJP).  Grid: (view chunk, tile),
 // tiles fastest, so the CTAs resident at any time share a few views whose
 // data and dL/dproj rows stay in L2.  Per tile the views of the chunk are
-// processed in order with the footprint of view j+1 copied to shared memory
-// while view j is computed (STAGE), like the forward.
+// processed in order through the staging pipe (STAGE), like the forward.  The
+// warp that finishes a view last also sums the 8 warps' values and writes the
+// view's record, before it refills the slot (so the next writers of the
+// slot's red[] come after it).
 //
-// FP16/BF16 data (CONV) is staged through a raw buffer and converted once per
-// (tile, view) into an FP32 buffer: convert view j, barrier, issue the raw
-// copy of view j+1, compute view j, wait for the copy, barrier.
 // With the fused data VJP the tile's dL/dvol is also kept in shared memory
 // ([z][y][x], row pitch TX + 1) for the line pass.
 constexpr int DSM_BYTES = ZB_VJP * TY * (TX + 1) * 4;
-template <typename T, bool PROJ = false>
+template <typename T, int NS>
 __host__ __device__ constexpr int vjp_smem_bytes() {
-  return (conv_staging<T>() ? CONV_F_BYTES + CONV_R_BYTES : 2 * STAGE_BYTES) +
-         (PROJ ? DSM_BYTES : 0);
+  return stage_smem_bytes<T, NS>() + DSM_BYTES;
 }
 
 // One work item of the VJP: views [item / ntiles * vchunk, + vchunk) of tile
 // item % ntiles.  All threads of the CTA call it with the CTA's shared memory.
-template <int ZB, typename T, bool FDK, bool EXACT, bool PROJ, bool STAGE>
+template <int ZB, int NS, typename T, bool FDK, bool EXACT, bool PROJ, bool STAGE>
 __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T* __restrict__ proj,
-                                         const ProjInfo& pi, const float2* __restrict__ grad,
+                                         const CUtensorMap* map, const ProjInfo& pi,
+                                         const float2* __restrict__ grad,
                                          const ViewGeom* __restrict__ geom, const VolInfo& vi,
                                          float* __restrict__ partials, float* __restrict__ dproj,
-                                         float* __restrict__ dblk, int vchunk, int item, TileView (*tvs)[VB],
-                                         float (*red)[NT / 32][12], unsigned char* dyn_smem) {
+                                         float* __restrict__ dblk, int vchunk, int item,
+                                         TileView (*tvs)[VB], float (*red)[NT / 32][12],
+                                         StagePipe<NS>& pipe,
+                                         unsigned char* dyn_smem) {
   constexpr bool CONV = STAGE && conv_staging<T>();
-  using G = typename std::conditional<CONV, ConvGeom, StageGeom<T>>::type;
-  T* bufs = reinterpret_cast<T*>(dyn_smem);  // plain: two buffers of T
-  float* F = reinterpret_cast<float*>(dyn_smem);  // CONV: FP32 buffer, then the raw one
-  T* R = reinterpret_cast<T*>(dyn_smem + CONV_F_BYTES);
-  float* dsm = reinterpret_cast<float*>(dyn_smem + vjp_smem_bytes<T, false>());
-  constexpr int CAP = STAGE_BYTES / (int)sizeof(T);
+  constexpr int SLOT = StageGeom<T>::BYTES;
+  unsigned char* slots = dyn_smem + (CONV ? CONV_F_BYTES : 0);
+  float* dsm =
+      reinterpret_cast<float*>(dyn_smem + (STAGE ? stage_smem_bytes<T, NS>() : 0));
   constexpr int HALO = EXACT ? 0 : 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int ntiles = vi.tiles_x * vi.tiles_y * vi.tiles_z;
   const int tile = item % ntiles;
   const int vbeg = (item / ntiles) * vchunk, vend = min(pi.nviews, vbeg + vchunk);
   const TileIdx ti = tile_index<ZB>(vi, tile);
   const int i = ti.tx * TX + ti.lx, j = ti.ty * TY + ti.ly;
   float delta[ZB];
-  bool nz = false;
+  bool nz = false, finite = true;
 #pragma unroll
   for (int k = 0; k < ZB; ++k) {
     const int z = ti.tz * ZB + k;
@@ -1452,162 +1872,194 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
                    ? __ldg(dvol + ((long long)z * vi.ny + j) * vi.nx + i)
                    : 0.0f;
     nz |= delta[k] != 0.0f;
+    finite = finite && fabsf(delta[k]) <= 3.402823466e38f;
   }
-  if (PROJ && STAGE && !EXACT && BP_VJP_LINES) {
+  finite = __all_sync(0xffffffffu, finite);
+  float* dcol = dsm + delta_base<PROJ>(ti.lx, ti.ly);  // this thread's column
 #pragma unroll
-    for (int k = 0; k < ZB; ++k) dsm[(k * TY + ti.ly) * (TX + 1) + ti.lx] = delta[k];
-  }
-  const bool any = __syncthreads_or(nz);
+  for (int k = 0; k < ZB; ++k) dcol[delta_off<PROJ>(k)] = delta[k];
   const int nvw = vend - vbeg, nbatch = (nvw + VB - 1) / VB;
-  setup_batch<T, STAGE, G>(tvs[0], geom, vbeg, min(VB, nvw), ti, pi.nu, pi.nv, true, HALO, !EXACT);
+  if (!__syncthreads_or(nz)) {  // no upstream gradient in this tile: zero records
+    for (int e = threadIdx.x; e < nvw * PSLOTS; e += NT)
+      partials[((long long)(vbeg + e / PSLOTS) * ntiles + tile) * PSLOTS + e % PSLOTS] = 0.0f;
+    return;
+  }
+  setup_batch<T, STAGE>(tvs[0], geom, vbeg, min(VB, nvw), ti, pi.nu, pi.nv, true, HALO);
   if (nbatch > 1)
-    setup_batch<T, STAGE, G>(tvs[1], geom, vbeg + VB, min(VB, nvw - VB), ti, pi.nu, pi.nv, true,
-                             HALO, !EXACT);
+    setup_batch<T, STAGE>(tvs[1], geom, vbeg + VB, min(VB, nvw - VB), ti, pi.nu, pi.nv, true,
+                          HALO);
   __syncthreads();
-  if (STAGE && any && tvs[0][0].staged) {
-    if constexpr (CONV)
-      stage_issue<T, CONV_P>(R, proj + (long long)vbeg * pi.vs, pi.rs, pi.nu, pi.nv, tvs[0][0]);
-    else
-      stage_issue(bufs, proj + (long long)vbeg * pi.vs, pi.rs, pi.nu, pi.nv, tvs[0][0]);
-  }
-  cp_async_commit();
-  if constexpr (CONV) {
-    cp_async_wait0();
-    __syncthreads();
-  }
+  if (STAGE && warp < NS && warp < nvw)
+    stage_issue<T>(slots + warp * SLOT, map, tvs[0][warp], vbeg + warp, &pipe.full[warp]);
+  bool bad = false;
+  PipePos<NS> pos;
   for (int v = vbeg; v < vend; ++v) {
     const int idx = v - vbeg, k = idx / VB, b = idx - k * VB;
     if (b == 0 && k >= 1) {
-      // batch k-1 is complete: write its last record, then reuse its slot
-      vjp_write_record(tvs[(k - 1) & 1][VB - 1], red[(idx - 1) & 1], any, v - 1, tile, ntiles,
-                       partials);
-      __syncthreads();
+      __syncthreads();  // every warp is done with batch k-1, its records are written
+      if (CONV && warp == 0)  // (the barrier path writes them one view late)
+        vjp_write_record(tvs[(k - 1) & 1][VB - 1], red[(idx - 1) % NS], bad, lane, v - 1, tile,
+                         ntiles, partials);
+      if (CONV) __syncthreads();
       if (k + 1 < nbatch)
-        setup_batch<T, STAGE, G>(tvs[(k + 1) & 1], geom, vbeg + (k + 1) * VB,
-                                 min(VB, nvw - (k + 1) * VB), ti, pi.nu, pi.nv, true, HALO,
-                                 !EXACT);
+        setup_batch<T, STAGE>(tvs[(k + 1) & 1], geom, vbeg + (k + 1) * VB,
+                              min(VB, nvw - (k + 1) * VB), ti, pi.nu, pi.nv, true, HALO);
       __syncthreads();
     }
-    const TileView t = tvs[k & 1][b];
-    const int kn = (idx + 1) / VB;
-    const TileView* tn = v + 1 < vend ? &tvs[kn & 1][idx + 1 - kn * VB] : nullptr;
+    const TileView& t = tvs[k & 1][b];
+    const unsigned slot = pos.slot;
+    unsigned char* buf = slots + slot * SLOT;
+    if (STAGE && !bad) bad = !mbar_wait(&pipe.full[slot], pos.parity);
+    pos.next();
+    const int in = idx + NS;
+    const TileView& tn = tvs[(in / VB) & 1][in % VB];
     if constexpr (CONV) {
-      if (any && t.staged) convert_stage<T>(F, R, t);
-      __syncthreads();  // F holds view v; R is free
-      if (any && tn && tn->staged)
-        stage_issue<T, CONV_P>(R, proj + (long long)(v + 1) * pi.vs, pi.rs, pi.nu, pi.nv, *tn);
-      cp_async_commit();
-    } else {
-      if (STAGE && any && tn && tn->staged)
-        stage_issue(bufs + ((idx + 1) & 1) * CAP, proj + (long long)(v + 1) * pi.vs, pi.rs, pi.nu,
-                    pi.nv, *tn);
-      cp_async_commit();
-      cp_async_wait1();
-      __syncthreads();
+      __syncthreads();  // every warp has seen this phase and is done with F and view v-1
+      if (b > 0 && warp == ((v + 4) & 7))
+        vjp_write_record(tvs[k & 1][b - 1], red[(idx - 1) % NS], bad, lane, v - 1, tile, ntiles,
+                         partials);
+      if (t.staged) {
+        convert_stage<T>(reinterpret_cast<float*>(dyn_smem), reinterpret_cast<const T*>(buf), t);
+        __syncthreads();  // F holds view v; the raw slot is free
+      }
+      if (warp == (v & 7) && in < nvw && !bad)
+        stage_issue<T>(buf, map, tn, vbeg + in, &pipe.full[slot]);
     }
-    // the record of view v-1 (its sums are complete since the last barrier;
-    // red[(idx - 1) & 1] is next written by view v+1, after another barrier)
-    if (idx > 0 && b > 0)
-      vjp_write_record(tvs[k & 1][b - 1], red[(idx - 1) & 1], any, v - 1, tile, ntiles, partials);
-    if (any && t.mode != MODE_SKIP) {
+    if (t.mode != MODE_SKIP) {
       const T* img = proj + (long long)v * pi.vs;
       const float2* gimg = EXACT ? nullptr : grad + (long long)v * pi.nv * pi.nu;
       float* pout = PROJ ? dproj + (long long)v * pi.nv * pi.nu : nullptr;
       float* qout =
           PROJ && dblk ? dblk + (long long)v * 4 * pi.nv * pi.nu : nullptr;
-      if constexpr (CONV)
-        vjp_tile_view<ZB, T, FDK, EXACT, PROJ, float, CONV_P>(img, gimg, F, t.staged, pout, qout,
-                                                              pi, t, ti, delta, dsm, red[idx & 1]);
-      else
-        vjp_tile_view<ZB, T, FDK, EXACT, PROJ, T, StageGeom<T>::P>(
-            img, gimg, bufs + (idx & 1) * CAP, STAGE && t.staged, pout, qout, pi, t, ti, delta,
-            dsm, red[idx & 1]);
+      vjp_tile_view<ZB, T, FDK, EXACT, PROJ, STAGE>(img, gimg, smem_addr(CONV ? dyn_smem : buf),
+                                             STAGE && t.staged, pout, qout, pi, t, ti, delta, dcol, finite,
+                                                    dsm, red[slot]);
     }
-    if constexpr (CONV) cp_async_wait0();  // the raw copy of view v+1
-    __syncthreads();  // F and the staging buffers are free; red[idx & 1] complete
+    if constexpr (!CONV) {
+      if (!STAGE) __syncthreads();  // no pipe to keep the warps within two views
+      if (last_warp(&pipe.done[slot])) {
+        vjp_write_record(t, red[slot], bad, lane, v, tile, ntiles, partials);
+        __syncwarp();
+        if (STAGE && in < nvw && !bad) stage_issue<T>(buf, map, tn, vbeg + in, &pipe.full[slot]);
+      }
+    }
   }
-  if (nvw > 0) {
+  if (CONV) {
+    __syncthreads();
     const int il = nvw - 1, kl = il / VB;
-    vjp_write_record(tvs[kl & 1][il - kl * VB], red[il & 1], any, vend - 1, tile, ntiles,
-                     partials);
+    if (warp == 0)
+      vjp_write_record(tvs[kl & 1][il - kl * VB], red[il % NS], bad, lane, vend - 1, tile, ntiles,
+                       partials);
   }
 }
 
-template <int ZB, typename T, bool FDK, bool EXACT, bool PROJ, bool STAGE>
-__global__ void __launch_bounds__(NT, VJP_MINB)
-    vjp_motion_kernel(const float* __restrict__ dvol, const T* __restrict__ proj, ProjInfo pi,
+template <int ZB, int NS, typename T, bool FDK, bool EXACT, bool PROJ, bool STAGE>
+__global__ void __launch_bounds__(NT, NS > VJP_NS ? 2 : VJP_MINB)
+    vjp_motion_kernel(const float* __restrict__ dvol, const T* __restrict__ proj,
+                      const __grid_constant__ CUtensorMap map, ProjInfo pi,
                       const float2* __restrict__ grad, const ViewGeom* __restrict__ geom,
                       VolInfo vi, float* __restrict__ partials, float* __restrict__ dproj,
-                      float* __restrict__ dblk, int vchunk) {
+                      float* __restrict__ dblk, int vchunk, const int* __restrict__ wide) {
+  // the other variant's launch takes this item
+  if (wide && (wide[blockIdx.x / (vi.tiles_x * vi.tiles_y * vi.tiles_z) * vchunk] != 0) == STAGE)
+    return;
   __shared__ TileView tvs[2][VB];
-  __shared__ float red[2][NT / 32][12];
-  extern __shared__ __align__(16) unsigned char dyn_smem[];
-  vjp_item<ZB, T, FDK, EXACT, PROJ, STAGE>(dvol, proj, pi, grad, geom, vi, partials, dproj, dblk,
-                                           vchunk, blockIdx.x, tvs, red, dyn_smem);
+  __shared__ float red[NS][NT / 32][12];
+  __shared__ StagePipe<NS> pipe;
+  extern __shared__ __align__(128) unsigned char dyn_smem[];
+  pipe_init(pipe);
+  vjp_item<ZB, NS, T, FDK, EXACT, PROJ, STAGE>(dvol, proj, &map, pi, grad, geom, vi, partials, dproj,
+                                           dblk, vchunk, blockIdx.x, tvs, red, pipe, dyn_smem);
 }
 
 #ifndef BP_VJP_CHUNK_MIB
 #define BP_VJP_CHUNK_MIB 128
 #endif
-// Views per chunk of the view-chunked VJP grids: the bytes that one chunk's
-// views touch (projections, gradient images, dL/dproj rows) are kept near
-// BP_VJP_CHUNK_MIB, at most 32 views.  Measured on c2 (fused VJP, before
-// the block image): 16 MiB 23.1 ms, 32 MiB 20.3 ms, 64 MiB 18.1 ms, 128 MiB
-// 17.4 ms.
-static int view_chunk(const ProjInfo& pi, long long bytes_per_px) {
+// Views per chunk of the view-chunked VJP grids.  Large problems: the bytes that
+// one chunk's views touch (projections, gradient images, dL/dproj rows) are kept
+// near BP_VJP_CHUNK_MIB, at most 32 views (c2, fused VJP before the block image:
+// 16 MiB 23.1 ms, 32 MiB 20.3 ms, 64 MiB 18.1 ms, 128 MiB 17.4 ms).  Small ones:
+// one wave of CTAs (a CTA's views are a serial chain) up to ten views each, then
+// at least three waves, so that the last one is not a large part (motion VJP
+// with 32 / 16 / 8 / 4 views per chunk, in a step of 60 views: 96^3 voxels 467 /
+// 438 / 430 / 440 us, 32^3 268 / 231 / 212 / 204 us).
+constexpr int VJP_WAVE = 152 * VJP_MINB;
+// Items up to which the VJP runs two CTAs per SM with four staging slots.
+constexpr int VJP_FEW = 304, VJP_NS_FEW = 4;
+static int view_chunk(const ProjInfo& pi, long long bytes_per_px, int ntiles) {
   const long long per_view = (long long)pi.nu * pi.nv * bytes_per_px;
   long long c = ((long long)BP_VJP_CHUNK_MIB << 20) / (per_view > 0 ? per_view : 1);
-  if (c < 1) c = 1;
   if (c > VB) c = VB;
-  return (int)c;
+  const long long n = (long long)ntiles * pi.nviews;
+  const long long f = n <= 10LL * VJP_WAVE ? (n + VJP_WAVE - 1) / VJP_WAVE
+                                           : (n / (3 * VJP_WAVE) > 8 ? n / (3 * VJP_WAVE) : 8);
+  if (c > f) c = f;
+  return c < 1 ? 1 : (int)c;
 }
 
-template <typename T, bool FDK, bool EXACT, bool PROJ, bool STAGE>
-static cudaError_t vjp_launch(const float* dvol, const void* proj, const ProjInfo& pi,
+template <int NS, typename T, bool FDK, bool EXACT, bool PROJ, bool STAGE>
+static cudaError_t vjp_launch(const float* dvol, const void* proj, const CUtensorMap& map,
+                              const ProjInfo& pi,
                               const float2* grad, const ViewGeom* geom, const VolInfo& vi,
                               float* partials, float* dproj, float* blk, int vc,
-                              unsigned nblocks, cudaStream_t s) {
-  const int smem = STAGE ? vjp_smem_bytes<T, PROJ && !EXACT && BP_VJP_LINES>() : 0;
+                              unsigned nblocks, const int* wide, cudaStream_t s) {
+  const int smem = STAGE ? vjp_smem_bytes<T, NS>() : DSM_BYTES;
   if (STAGE) {
-    cudaError_t e = smem_attr_once<vjp_motion_kernel<ZB_VJP, T, FDK, EXACT, PROJ, STAGE>>(smem);
+    const cudaError_t e =
+        smem_attr_once<vjp_motion_kernel<ZB_VJP, NS, T, FDK, EXACT, PROJ, STAGE>>(smem);
     if (e != cudaSuccess) return e;
   }
-  vjp_motion_kernel<ZB_VJP, T, FDK, EXACT, PROJ, STAGE><<<nblocks, NT, smem, s>>>(
-      dvol, (const T*)proj, pi, grad, geom, vi, partials, dproj, blk, vc);
+  vjp_motion_kernel<ZB_VJP, NS, T, FDK, EXACT, PROJ, STAGE><<<nblocks, NT, smem, s>>>(
+      dvol, (const T*)proj, map, pi, grad, geom, vi, partials, dproj, blk, vc, wide);
   return cudaGetLastError();
+}
+
+template <typename T, bool FDK, bool EXACT, bool PROJ>
+static cudaError_t vjp_variants(const float* dvol, const void* proj, const ProjInfo& pi,
+                                const float2* grad, const ViewGeom* geom, const VolInfo& vi,
+                                float* partials, float* dproj, float* blk, int vc,
+                                unsigned nblocks, const int* wide, cudaStream_t s) {
+  CUtensorMap map{};
+  const bool stage = stageable<T>(proj, pi) && wide != WIDE_ALL &&
+                     make_stage_map(proj, dtype_id<T>(), pi, &map) == cudaSuccess;
+  const int* sel = stage ? wide : nullptr;
+  if (stage) {
+    const cudaError_t e =
+        nblocks <= (unsigned)VJP_FEW
+            ? vjp_launch<VJP_NS_FEW, T, FDK, EXACT, PROJ, true>(
+                  dvol, proj, map, pi, grad, geom, vi, partials, dproj, blk, vc, nblocks, sel, s)
+            : vjp_launch<VJP_NS, T, FDK, EXACT, PROJ, true>(
+                  dvol, proj, map, pi, grad, geom, vi, partials, dproj, blk, vc, nblocks, sel, s);
+    if (e != cudaSuccess || !sel) return e;
+  }
+  return vjp_launch<VJP_NS, T, FDK, EXACT, PROJ, false>(dvol, proj, map, pi, grad, geom, vi, partials,
+                                                        dproj, nullptr, vc, nblocks, sel, s);
 }
 
 template <typename T, bool FDK, bool EXACT>
 static cudaError_t vjp_dispatch(const float* dvol, const void* proj, const ProjInfo& pi,
                                 const float2* grad, const ViewGeom* geom, const VolInfo& vi,
-                                float* partials, float* dproj, float* blk, cudaStream_t s) {
+                                float* partials, float* dproj, float* blk, const int* wide,
+                                cudaStream_t s) {
   const int ntiles = vi.tiles_x * vi.tiles_y * vi.tiles_z;
-  const bool stage = stageable<T>(proj, pi);
   // block images only where the staged CENTRAL paths scatter
-  const bool useb = dproj && blk && stage && !EXACT && BP_VJP_BLOCKS;
+  const bool useb = dproj && blk && stageable<T>(proj, pi) && !EXACT && BP_VJP_BLOCKS;
   // the block image is left out of the chunk's byte count: measured on c2,
   // counting its 16 bytes per pixel (smaller chunks) made the fused VJP 2.8 %
   // slower (15.37 against 14.94 ms), counting 8 bytes 1.7 %
   const long long bpp = (long long)sizeof(T) + (EXACT ? 0 : 8) + (dproj ? 4 : 0);
-  const int vc = view_chunk(pi, bpp);
+  const int vc = view_chunk(pi, bpp, ntiles);
   const unsigned nblocks = (unsigned)((long long)ntiles * ((pi.nviews + vc - 1) / vc));
-  if (dproj) {
-    cudaError_t e = cudaSuccess;
-    if (useb) e = cudaMemsetAsync(blk, 0, sizeof(float) * (size_t)block_image_floats(pi), s);
-    if (e == cudaSuccess)
-      e = stage ? vjp_launch<T, FDK, EXACT, true, true>(dvol, proj, pi, grad, geom, vi, partials,
-                                                        dproj, useb ? blk : nullptr, vc, nblocks,
-                                                        s)
-                : vjp_launch<T, FDK, EXACT, true, false>(dvol, proj, pi, grad, geom, vi,
-                                                         partials, dproj, nullptr, vc, nblocks, s);
-    if (e == cudaSuccess && useb) e = launch_block_combine(blk, pi, dproj, s);
-    return e;
-  }
-  return stage ? vjp_launch<T, FDK, EXACT, false, true>(dvol, proj, pi, grad, geom, vi, partials,
-                                                        nullptr, nullptr, vc, nblocks, s)
-               : vjp_launch<T, FDK, EXACT, false, false>(dvol, proj, pi, grad, geom, vi,
-                                                         partials, nullptr, nullptr, vc, nblocks,
-                                                         s);
+  if (!dproj)
+    return vjp_variants<T, FDK, EXACT, false>(dvol, proj, pi, grad, geom, vi, partials, nullptr,
+                                              nullptr, vc, nblocks, wide, s);
+  cudaError_t e = cudaSuccess;
+  if (useb) e = cudaMemsetAsync(blk, 0, sizeof(float) * (size_t)block_image_floats(pi), s);
+  if (e == cudaSuccess)
+    e = vjp_variants<T, FDK, EXACT, true>(dvol, proj, pi, grad, geom, vi, partials, dproj,
+                                          useb ? blk : nullptr, vc, nblocks, wide, s);
+  if (e == cudaSuccess && useb) e = launch_block_combine(blk, pi, dproj, s);
+  return e;
 }
 
 bool vjp_uses_blocks(const void* proj, int dtype, const ProjInfo& pi, int exact) {
@@ -1619,52 +2071,57 @@ bool vjp_uses_blocks(const void* proj, int dtype, const ProjInfo& pi, int exact)
 
 // Set the VJP kernels' shared-memory attributes on the current device
 // (call before capturing a graph).
-cudaError_t prepare_vjp(int dtype, int fdk, int exact) {
-  cudaError_t e = cudaSuccess;
-#define BP_PREP(T)                                                                                 \
-  do {                                                                                             \
-    const int smem = vjp_smem_bytes<T>();                                                          \
-    if (fdk && exact) e = smem_attr_once<vjp_motion_kernel<ZB_VJP, T, true, true, false, true>>(smem); \
-    if (fdk && !exact) e = smem_attr_once<vjp_motion_kernel<ZB_VJP, T, true, false, false, true>>(smem); \
-    if (!fdk && exact) e = smem_attr_once<vjp_motion_kernel<ZB_VJP, T, false, true, false, true>>(smem); \
-    if (!fdk && !exact) e = smem_attr_once<vjp_motion_kernel<ZB_VJP, T, false, false, false, true>>(smem); \
-  } while (0)
-  if (dtype == 0) BP_PREP(float);
-  else if (dtype == 1) BP_PREP(__half);
-  else BP_PREP(__nv_bfloat16);
-#undef BP_PREP
+template <typename T, bool FDK, bool EXACT>
+static cudaError_t prepare_vjp_t() {
+  cudaError_t e = smem_attr_once<vjp_motion_kernel<ZB_VJP, VJP_NS, T, FDK, EXACT, false, true>>(
+      vjp_smem_bytes<T, VJP_NS>());
+  if (e == cudaSuccess)
+    e = smem_attr_once<vjp_motion_kernel<ZB_VJP, VJP_NS_FEW, T, FDK, EXACT, false, true>>(
+        vjp_smem_bytes<T, VJP_NS_FEW>());
   return e;
+}
+
+template <typename T>
+static cudaError_t prepare_vjp_d(int fdk, int exact) {
+  if (fdk) return exact ? prepare_vjp_t<T, true, true>() : prepare_vjp_t<T, true, false>();
+  return exact ? prepare_vjp_t<T, false, true>() : prepare_vjp_t<T, false, false>();
+}
+
+cudaError_t prepare_vjp(int dtype, int fdk, int exact) {
+  if (dtype == 0) return prepare_vjp_d<float>(fdk, exact);
+  if (dtype == 1) return prepare_vjp_d<__half>(fdk, exact);
+  return prepare_vjp_d<__nv_bfloat16>(fdk, exact);
 }
 
 template <typename T>
 static cudaError_t vjp_dispatch_t(int fdk, int exact, const float* dvol, const void* proj,
                                   const ProjInfo& pi, const float2* grad, const ViewGeom* geom,
                                   const VolInfo& vi, float* partials, float* dproj,
-                                  float* blk, cudaStream_t s) {
+                                  float* blk, const int* wide, cudaStream_t s) {
   if (fdk)
     return exact ? vjp_dispatch<T, true, true>(dvol, proj, pi, grad, geom, vi, partials, dproj,
-                                               blk, s)
+                                               blk, wide, s)
                  : vjp_dispatch<T, true, false>(dvol, proj, pi, grad, geom, vi, partials, dproj,
-                                                blk, s);
+                                                blk, wide, s);
   return exact ? vjp_dispatch<T, false, true>(dvol, proj, pi, grad, geom, vi, partials, dproj,
-                                              blk, s)
+                                              blk, wide, s)
                : vjp_dispatch<T, false, false>(dvol, proj, pi, grad, geom, vi, partials, dproj,
-                                               blk, s);
+                                               blk, wide, s);
 }
 
 cudaError_t launch_vjp_motion(const float* dvol, const void* proj, int dtype, const ProjInfo& pi,
                               const float2* grad, const ViewGeom* geom, const VolInfo& vi,
                               int fdk, int exact, float* partials, float* dproj, float* blk,
-                              cudaStream_t s) {
+                              const int* wide, cudaStream_t s) {
   if (vi.zb != ZB_VJP) return cudaErrorInvalidValue;
   if (dtype == 0)
     return vjp_dispatch_t<float>(fdk, exact, dvol, proj, pi, grad, geom, vi, partials, dproj, blk,
-                                 s);
+                                 wide, s);
   if (dtype == 1)
     return vjp_dispatch_t<__half>(fdk, exact, dvol, proj, pi, grad, geom, vi, partials, dproj,
-                                  blk, s);
+                                  blk, wide, s);
   return vjp_dispatch_t<__nv_bfloat16>(fdk, exact, dvol, proj, pi, grad, geom, vi, partials,
-                                       dproj, blk, s);
+                                       dproj, blk, wide, s);
 }
 
 // ------------------------------------------------- VJP w.r.t. the data
@@ -1681,14 +2138,14 @@ template <int ZB, bool FDK, bool EDGE>
 __device__ __forceinline__ void proj_view(float* out, float* bout, int nu, int nv,
                                           const TileView& t, float dx, float dy,
                                           const float (&delta)[ZB]) {
-  const float u0 = fmaf(dy, t.ru[1], fmaf(dx, t.ru[0], t.U0));
-  const float v0 = fmaf(dy, t.rv[1], fmaf(dx, t.rv[0], t.V0));
-  const float w0 = fmaf(dy, t.rw[1], fmaf(dx, t.rw[0], t.W0));
+  const float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
+  const float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
+  const float w0 = fmaf(dy, t.rw1, fmaf(dx, t.rw0, t.W0));
 #pragma unroll
   for (int k = 0; k < ZB; ++k) {
     if (delta[k] == 0.0f) continue;
     const float dz = k - 0.5f * (ZB - 1);
-    Sample s = locate<EDGE>(fmaf(dz, t.ru[2], u0), fmaf(dz, t.rv[2], v0), fmaf(dz, t.rw[2], w0),
+    Sample s = locate<EDGE>(fmaf(dz, t.ru2, u0), fmaf(dz, t.rv2, v0), fmaf(dz, t.rw2, w0),
                             t, nu, nv);
     if (EDGE && !s.ok) continue;
     const float sd = delta[k] * (FDK ? s.rwi * (s.rwi * t.wgtd) : t.wgtd);
@@ -1740,7 +2197,7 @@ cudaError_t launch_vjp_proj(const float* dvol, const ProjInfo& pi, const ViewGeo
   if (vi.zb != ZB_VJP) return cudaErrorInvalidValue;
   if (!BP_VJP_BLOCKS) blk = nullptr;
   const int ntiles = vi.tiles_x * vi.tiles_y * vi.tiles_z;
-  const int vc = view_chunk(pi, blk ? 20 : 4);
+  const int vc = view_chunk(pi, blk ? 20 : 4, ntiles);
   const unsigned nblocks = (unsigned)((long long)ntiles * ((pi.nviews + vc - 1) / vc));
   if (blk) {
     cudaError_t e = cudaMemsetAsync(blk, 0, sizeof(float) * (size_t)block_image_floats(pi), s);
@@ -1775,8 +2232,11 @@ template <int ZB, typename T, bool FDK>
 __global__ void __launch_bounds__(NT, FWD_MINB)
     batch_forward_kernel(const __grid_constant__ BatchTable t, unsigned* __restrict__ counter) {
   __shared__ TileView tvs[2][VB];
+  __shared__ StagePipe<FWD_NS> pipe;
   __shared__ int item;
-  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  extern __shared__ __align__(128) unsigned char dyn_smem[];
+  pipe_init(pipe);
+  PipePos<FWD_NS> pos;
   const int n = t.njobs, total = t.off_fwd[n];
   for (;;) {
     __syncthreads();  // every thread is done with the previous tile
@@ -1786,8 +2246,8 @@ __global__ void __launch_bounds__(NT, FWD_MINB)
     if (w >= total) break;
     const int j = batch_find(t.off_fwd, n, w);
     const BatchJob& J = t.job[j];
-    forward_tile<ZB, T, FDK, true>((const T*)J.proj, J.pi, J.geom, J.vif, J.vol, w - t.off_fwd[j],
-                                   tvs, dyn_smem);
+    forward_tile<ZB, ZB, FWD_NS, T, FDK, true>((const T*)J.proj, &J.map, J.pi, J.geom, J.vif, J.vol,
+                                       w - t.off_fwd[j], 0, tvs, pipe, dyn_smem, pos);
   }
 }
 
@@ -1796,7 +2256,7 @@ int forward_zb() { return ZB_FWD; }
 template <typename T, bool FDK>
 static cudaError_t batch_forward_t(const BatchTable& tab, unsigned* counter, int sms,
                                    cudaStream_t s) {
-  const int smem = fwd_smem_bytes<T>();
+  const int smem = stage_smem_bytes<T, FWD_NS>();
   cudaError_t e = smem_attr_once<batch_forward_kernel<ZB_FWD, T, FDK>>(smem);
   if (e != cudaSuccess) return e;
   batch_forward_kernel<ZB_FWD, T, FDK><<<sms * FWD_MINB, NT, smem, s>>>(tab, counter);
@@ -1819,15 +2279,15 @@ cudaError_t launch_batch_forward(const BatchTable& tab, unsigned* counter, int d
 cudaError_t prepare_batch(int dtype, int fdk, int exact) {
   (void)exact;
   if (dtype == 0)
-    return fdk ? smem_attr_once<batch_forward_kernel<ZB_FWD, float, true>>(fwd_smem_bytes<float>())
-               : smem_attr_once<batch_forward_kernel<ZB_FWD, float, false>>(fwd_smem_bytes<float>());
+    return fdk ? smem_attr_once<batch_forward_kernel<ZB_FWD, float, true>>(stage_smem_bytes<float, FWD_NS>())
+               : smem_attr_once<batch_forward_kernel<ZB_FWD, float, false>>(stage_smem_bytes<float, FWD_NS>());
   if (dtype == 1)
-    return fdk ? smem_attr_once<batch_forward_kernel<ZB_FWD, __half, true>>(fwd_smem_bytes<__half>())
-               : smem_attr_once<batch_forward_kernel<ZB_FWD, __half, false>>(fwd_smem_bytes<__half>());
+    return fdk ? smem_attr_once<batch_forward_kernel<ZB_FWD, __half, true>>(stage_smem_bytes<__half, FWD_NS>())
+               : smem_attr_once<batch_forward_kernel<ZB_FWD, __half, false>>(stage_smem_bytes<__half, FWD_NS>());
   return fdk ? smem_attr_once<batch_forward_kernel<ZB_FWD, __nv_bfloat16, true>>(
-                   fwd_smem_bytes<__nv_bfloat16>())
+                   stage_smem_bytes<__nv_bfloat16, FWD_NS>())
              : smem_attr_once<batch_forward_kernel<ZB_FWD, __nv_bfloat16, false>>(
-                   fwd_smem_bytes<__nv_bfloat16>());
+                   stage_smem_bytes<__nv_bfloat16, FWD_NS>());
 }
 
 }  // namespace bpk
