@@ -622,7 +622,7 @@ int bp_fdk_filter(bp_ctx* ctx, const float* raw, int nviews, int nv, int nu, dou
   void* o;
   bool host;
   CK(stage_out(ctx->s_out_proj, out, sizeof(float) * n, &o, &host), "alloc out");
-  CK(ensure(ctx->fdk_tab, sizeof(float) * bpk::fdk_table_floats(nviews, nu, ext)),
+  CK(ensure(ctx->fdk_tab, sizeof(float) * bpk::fdk_table_floats(nviews, nu, nv, ext)),
      "alloc tables");
   CK(TL(K_FDK, 2, bpk::launch_fdk_filter((const float*)q, nviews, nv, nu, ext, pitch, sid, sdd,
                                          arc, (float*)ctx->fdk_tab.p, (float*)o, s)),

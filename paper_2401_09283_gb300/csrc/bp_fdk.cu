@@ -6,13 +6,14 @@
 // linear convolution with the Shepp-Logan ramp h[n] = -2 / (pi^2 tau^2
 // (4 n^2 - 1)), tau = pitch * SID / SDD, times tau.
 //
-// The ramp and the per-(view, column) redundancy weights are tabulated in
-// FP64 and rounded to FP32; the convolution is a direct O(nu^2) sum in FP32,
-// four detector rows per CTA so that one broadcast float4 load feeds four
-// FMAs per tap.  With ext > 0 (truncation correction, Sec. IV-D) every
-// weighted row is extended by ext pixels per side falling linearly from its
-// edge value to 0 (extension pixel m = 1..ext holds edge * (1 - m/ext)) and
-// the measured nu pixels of the filtered, extended row are kept.
+// The ramp, the redundancy weights (view, column) and the cosine weights
+// (distance from the detector's centre lines) are tabulated in FP64; the
+// convolution is a direct O(nu^2) sum in FP32, taken tap by tap in the same order
+// for every output.  (An FP32 FFT is 2 to 3 times further from the FP64 result.)
+// With ext > 0 (truncation correction, Sec. IV-D) every weighted row is extended
+// by ext pixels per side falling linearly from its edge value to 0 (extension
+// pixel m = 1..ext holds edge * (1 - m/ext)) and the measured nu pixels of the
+// filtered, extended row are kept.
 #include "bp_internal.cuh"
 
 namespace bpk {
@@ -34,118 +35,244 @@ __device__ double parker_w(double beta, double gamma, double arc) {
   return fmin(fmax(w, 0.0), 1.0);
 }
 
-// h[m + ne - 1] for |m| < ne = nu + 2 ext, then the redundancy weight of
-// (view j, column a) at [2 ne - 1 + j nu + a].
-__global__ void fdk_tables_kernel(int V, int nu, int ext, double pitch, double sid, double sdd,
-                                  double arc, float* __restrict__ tab) {
+// Layout of the tables: cosine weights of a quarter of the detector, the ramp,
+// redundancy weights.
+struct FdkTables {
+  int nuh, nvh;          // quarter detector: distance from the nearer edge
+  size_t ramp, red;      // offsets in floats
+  __host__ __device__ FdkTables(int nu, int nv, int ext)
+      : nuh((nu + 1) / 2),
+        nvh((nv + 1) / 2),
+        ramp(2 * (size_t)nuh * (size_t)nvh),
+        red(ramp + 2 * ((size_t)nu + 2 * (size_t)ext) - 1) {}
+};
+
+constexpr int RED_VIEWS = 8;  // views per thread of the redundancy table
+
+// [nvh][nuh] (high, low) FP32 parts of the cosine weight, then h[m + ne - 1] for
+// |m| < ne = nu + 2 ext, then the redundancy weight of (view j, column a) at
+// j nu + a.
+__global__ void fdk_tables_kernel(int V, int nu, int nv, int ext, double pitch, double sid,
+                                  double sdd, double arc, float* __restrict__ tab) {
   const double tau = pitch * sid / sdd;
   const bool full = arc >= 2.0 * kPi - 1e-12;
   const double dbeta = full ? arc / V : (V > 1 ? arc / (V - 1) : 0.0);
   const int ne = nu + 2 * ext;
-  const long long nh = 2LL * ne - 1, n = nh + (long long)V * nu;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
+  const FdkTables T(nu, nv, ext);
+  const long long nc = (long long)T.nuh * T.nvh, nh = 2LL * ne - 1;
+  const long long nr = (long long)((V + RED_VIEWS - 1) / RED_VIEWS) * nu;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nc + nh + nr;
        e += (long long)gridDim.x * blockDim.x) {
-    if (e < nh) {
-      const double m = (double)(e - (ne - 1));
-      tab[e] = (float)(-2.0 / (kPi * kPi * tau * tau * (4.0 * m * m - 1.0)));
+    if (e < nc) {
+      const int b = (int)(e / T.nuh), k = (int)(e % T.nuh);
+      const double x = (k - 0.5 * (nu - 1)) * pitch, y = (b - 0.5 * (nv - 1)) * pitch;
+      const double c = sdd / sqrt(sdd * sdd + x * x + y * y);
+      const float hi = (float)c;
+      reinterpret_cast<float2*>(tab)[e] = make_float2(hi, (float)(c - (double)hi));
+    } else if (e < nc + nh) {
+      const double m = (double)(e - nc - (ne - 1));
+      tab[T.ramp + (e - nc)] = (float)(-2.0 / (kPi * kPi * tau * tau * (4.0 * m * m - 1.0)));
     } else {
-      const long long q = e - nh;
-      const int j = (int)(q / nu), a = (int)(q % nu);
-      const double x = (a - 0.5 * (nu - 1)) * pitch;
-      tab[e] = full ? 0.5f : (float)parker_w(j * dbeta, atan(x / sdd), arc);
+      const long long q = e - nc - nh;
+      const int j0 = (int)(q / nu) * RED_VIEWS, a = (int)(q % nu);
+      const double g = full ? 0.0 : atan((a - 0.5 * (nu - 1)) * pitch / sdd);
+      for (int j = j0; j < min(V, j0 + RED_VIEWS); ++j)
+        tab[T.red + (size_t)j * nu + a] = full ? 0.5f : (float)parker_w(j * dbeta, g, arc);
     }
   }
 }
 
-constexpr int ROWS = 4;
+constexpr int ROWS = 4;        // detector rows of a group, interleaved as float4
+constexpr int OUT = 8;         // consecutive outputs per thread
+constexpr int MAX_GROUPS = 8;  // groups per CTA
+constexpr int MAX_THREADS = 512;
 
-// grid (ceil(nv / ROWS), V); dynamic shared memory: ne = nu + 2 ext float4
-// (the four weighted, extended rows interleaved) + (2 ne - 1) floats (the ramp).
-__global__ void __launch_bounds__(256) fdk_conv_kernel(const float* __restrict__ raw, int nu,
-                                                       int nv, int ext, double pitch, double sdd,
-                                                       float tau, const float* __restrict__ tab,
-                                                       float* __restrict__ out) {
+// The ramp in shared memory, element m at m + m / 8, shifted by `shift` so that
+// the taps of one block of eight steps lie in one such run: the lanes' loads
+// (eight elements apart) fall in different banks and their offsets are immediates.
+struct RampLayout {
+  int c, shift, n;  // index of output 0's first tap; elements
+  __host__ __device__ RampLayout(int nu, int ext) {
+    const int c0 = ext + (nu + 2 * ext) - 1;
+    shift = (7 - c0) & 7;
+    c = c0 + shift;
+    n = (nu + OUT - 1) / OUT * OUT + c;
+  }
+  __host__ __device__ static int at(int m) { return m + (m >> 3); }
+};
+
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 splat2(float a) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
+  return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// grid (ceil(groups / G), V), G groups of four rows per CTA.  Dynamic shared
+// memory: G x ne float4 (the weighted, extended rows, interleaved), the ramp.
+//
+// The convolution is nu FMAs per output, bound by the FMA pipe when the operands
+// are cheap: a thread owns 8 outputs of 4 rows (16 packed accumulators) and takes,
+// per tap, one broadcast 16-byte load of the rows and ONE ramp value, the other
+// seven being those of the step before (a window in registers, renamed by the
+// unrolling).  One output of 4 rows per thread loaded 20 bytes for four FMAs.
+// The cosine weight comes from a table as a pair of FP32 values, not from an FP64
+// square root and division per pixel and view (2 FP64 lanes per clock and SM).
+// 248 x 480 rows of 616: 3.76 -> 1.93 ms, the FMAs alone take 1.2 ms.
+__global__ void __launch_bounds__(MAX_THREADS)
+    fdk_conv_kernel(const float* __restrict__ raw, int nu, int nv, int ext, int G, float tau,
+                    const float* __restrict__ tab, float* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int ne = nu + 2 * ext;
-  float4* ext_rows = reinterpret_cast<float4*>(smem);
-  float4* rows = ext_rows + ext;  // rows[k], k = -ext .. nu + ext - 1
-  float* h = reinterpret_cast<float*>(smem + sizeof(float4) * (size_t)ne);
-  const int j = blockIdx.y, b0 = blockIdx.x * ROWS;
-  const float* park = tab + (2 * ne - 1) + (size_t)j * nu;
-  for (int e = threadIdx.x; e < 2 * ne - 1; e += blockDim.x) h[e] = tab[e];
-  for (int k = threadIdx.x; k < nu; k += blockDim.x) {
-    const double x = (k - 0.5 * (nu - 1)) * pitch;
+  const FdkTables T(nu, nv, ext);
+  const RampLayout L(nu, ext);
+  float4* rows = reinterpret_cast<float4*>(smem);  // [G][ne]
+  float* h = reinterpret_cast<float*>(smem + sizeof(float4) * (size_t)G * ne);
+  const int j = blockIdx.y, groups = (nv + ROWS - 1) / ROWS;
+  const int g0 = blockIdx.x * G, ng = min(G, groups - g0);
+  const float* red = tab + T.red + (size_t)j * nu;
+  const float2* cosw = reinterpret_cast<const float2*>(tab);
+  for (int e = threadIdx.x; e < L.n; e += blockDim.x) {
+    const int m = e - L.shift;
+    h[RampLayout::at(e)] = m >= 0 && m < 2 * ne - 1 ? tab[T.ramp + m] : 0.0f;
+  }
+  for (int e = threadIdx.x; e < ng * nu; e += blockDim.x) {
+    const int g = e / nu, k = e - g * nu;
+    const float p = red[k];
     float v[ROWS];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
-      const int b = b0 + r;
+      const int b = (g0 + g) * ROWS + r;
       v[r] = 0.0f;
       if (b < nv) {
-        const double y = (b - 0.5 * (nv - 1)) * pitch;
-        const double c = sdd / sqrt(sdd * sdd + x * x + y * y);
-        v[r] = (float)(c * (double)park[k]) * raw[((size_t)j * nv + b) * nu + k];
+        const float2 c = cosw[(size_t)min(b, nv - 1 - b) * T.nuh + min(k, nu - 1 - k)];
+        // the product of the FP64 cosine weight and p, rounded once
+        const float hi = __fmul_rn(c.x, p);
+        const float w = __fadd_rn(hi, fmaf(c.y, p, fmaf(c.x, p, -hi)));
+        v[r] = w * raw[((size_t)j * nv + b) * nu + k];
       }
     }
-    rows[k] = make_float4(v[0], v[1], v[2], v[3]);
+    rows[(size_t)g * ne + ext + k] = make_float4(v[0], v[1], v[2], v[3]);
   }
   __syncthreads();
-  for (int m = 1 + threadIdx.x; m <= ext; m += blockDim.x) {  // linear fall-off to 0
+  for (int e = threadIdx.x; e < ng * ext; e += blockDim.x) {  // linear fall-off to 0
+    const int g = e / ext, m = 1 + (e - g * ext);
+    float4* q = rows + (size_t)g * ne + ext;
     const float f = 1.0f - (float)m / (float)ext;
-    const float4 l = rows[0], r = rows[nu - 1];
-    rows[-m] = make_float4(l.x * f, l.y * f, l.z * f, l.w * f);
-    rows[nu - 1 + m] = make_float4(r.x * f, r.y * f, r.z * f, r.w * f);
+    const float4 l = q[0], r = q[nu - 1];
+    q[-m] = make_float4(l.x * f, l.y * f, l.z * f, l.w * f);
+    q[nu - 1 + m] = make_float4(r.x * f, r.y * f, r.z * f, r.w * f);
   }
   __syncthreads();
-  for (int a = threadIdx.x; a < nu; a += blockDim.x) {
-    float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
-    const float* ha = h + a + ext + ne - 1;  // ha[-k'] = h[(a + ext) - k'], k' = k + ext
-#pragma unroll 4
-    for (int kk = 0; kk < ne; ++kk) {
-      const int k = kk - ext;
-      const float4 p = rows[k];
-      const float w = ha[-kk];
-      s0 = fmaf(w, p.x, s0);
-      s1 = fmaf(w, p.y, s1);
-      s2 = fmaf(w, p.z, s2);
-      s3 = fmaf(w, p.w, s3);
-    }
-    const float s[ROWS] = {s0, s1, s2, s3};
+  const int nt = (nu + OUT - 1) / OUT;
+  for (int item = threadIdx.x; item < ng * nt; item += blockDim.x) {
+    const int g = item / nt, a0 = (item - g * nt) * OUT;
+    const ulonglong2* p = reinterpret_cast<const ulonglong2*>(rows + (size_t)g * ne);
+    const float* hb = h + RampLayout::at(a0 + L.c);  // tap kk of output a0 + i: L.c + a0 - kk + i
+    f2 acc[OUT][2], w[OUT];
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r)
-      if (b0 + r < nv) out[((size_t)j * nv + b0 + r) * nu + a] = tau * s[r];
+    for (int i = 0; i < OUT; ++i) acc[i][0] = acc[i][1] = splat2(0.0f);
+#pragma unroll
+    for (int i = 1; i < OUT; ++i) w[i] = splat2(hb[1 + i]);
+#pragma unroll 1
+    for (int kk = 0; kk + OUT <= ne; kk += OUT) {
+#pragma unroll
+      for (int q = 0; q < OUT; ++q) {
+        const ulonglong2 x = p[kk + q];
+        w[(OUT - q) % OUT] = splat2(hb[-q]);
+#pragma unroll
+        for (int i = 0; i < OUT; ++i) {
+          acc[i][0] = fma2(w[(i - q + OUT) % OUT], x.x, acc[i][0]);
+          acc[i][1] = fma2(w[(i - q + OUT) % OUT], x.y, acc[i][1]);
+        }
+      }
+      hb -= OUT + 1;
+    }
+#pragma unroll 1
+    for (int kk = ne / OUT * OUT; kk < ne; ++kk) {
+      const ulonglong2 x = p[kk];
+#pragma unroll
+      for (int i = 0; i < OUT; ++i) {
+        const f2 wi = splat2(h[RampLayout::at(a0 + L.c - kk + i)]);
+        acc[i][0] = fma2(wi, x.x, acc[i][0]);
+        acc[i][1] = fma2(wi, x.y, acc[i][1]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+      const int b = (g0 + g) * ROWS + r;
+      if (b >= nv) break;
+      float* o = out + ((size_t)j * nv + b) * nu + a0;
+      float s[OUT];
+#pragma unroll
+      for (int i = 0; i < OUT; ++i) {
+        const f2 a = acc[i][r / 2];
+        s[i] = tau * __uint_as_float((unsigned)(r % 2 ? a >> 32 : a));
+      }
+      if (nu % 4 == 0 && a0 + OUT <= nu && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+        reinterpret_cast<float4*>(o)[0] = make_float4(s[0], s[1], s[2], s[3]);
+        reinterpret_cast<float4*>(o)[1] = make_float4(s[4], s[5], s[6], s[7]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < OUT; ++i)
+          if (a0 + i < nu) o[i] = s[i];
+      }
+    }
   }
+}
+
+size_t conv_smem(int nu, int ext, int G) {
+  const RampLayout L(nu, ext);
+  return sizeof(float4) * (size_t)G * ((size_t)nu + 2 * (size_t)ext) +
+         sizeof(float) * (size_t)(RampLayout::at(L.n) + 1);
 }
 
 }  // namespace
 
-size_t fdk_table_floats(int V, int nu, int ext) {
-  return (size_t)(2 * (nu + 2 * ext) - 1) + (size_t)V * nu;
-}
-
-size_t fdk_smem_bytes(int nu, int ext) {
-  const size_t ne = (size_t)nu + 2 * (size_t)ext;
-  return sizeof(float) * (4 * ne + 2 * ne - 1);
+size_t fdk_table_floats(int V, int nu, int nv, int ext) {
+  return FdkTables(nu, nv, ext).red + (size_t)V * nu;
 }
 
 cudaError_t launch_fdk_filter(const float* raw, int V, int nv, int nu, int ext, double pitch,
                               double sid, double sdd, double arc, float* tab, float* out,
                               cudaStream_t s) {
   if (V == 0 || nv == 0) return cudaSuccess;
-  const long long n = (long long)fdk_table_floats(V, nu, ext);
+  const long long n = (long long)fdk_table_floats(V, nu, nv, ext);
   long long nb = (n + 255) / 256;
   if (nb > 152 * 16) nb = 152 * 16;
-  fdk_tables_kernel<<<(int)nb, 256, 0, s>>>(V, nu, ext, pitch, sid, sdd, arc, tab);
+  fdk_tables_kernel<<<(int)nb, 256, 0, s>>>(V, nu, nv, ext, pitch, sid, sdd, arc, tab);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const size_t smem = fdk_smem_bytes(nu, ext);
-  if (smem > 48 * 1024) {
+  // Groups per CTA: the share of busy threads (whole warps, whole CTAs), best
+  // within 56 KiB of shared memory, so that several CTAs are resident.
+  const int nt = (nu + OUT - 1) / OUT, groups = (nv + ROWS - 1) / ROWS;
+  int G = 1, threads = 0;
+  double best = 0.0;
+  for (int g = 1; g <= MAX_GROUPS && g <= groups; ++g) {
+    if (g > 1 && conv_smem(nu, ext, g) > 56 * 1024) break;
+    const int t = (g * nt + 31) / 32 * 32 < MAX_THREADS ? (g * nt + 31) / 32 * 32 : MAX_THREADS;
+    const int ctas = (groups + g - 1) / g, turns = (g * nt + t - 1) / t;
+    const double busy = (double)groups * nt / ((double)ctas * turns * t);
+    if (busy > best + 0.01) {
+      best = busy;
+      G = g;
+      threads = t;
+    }
+  }
+  const size_t smem = conv_smem(nu, ext, G);
+  if (smem > 48 * 1024) {  // the same limit in every call: calls in other threads agree
     e = cudaFuncSetAttribute(fdk_conv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+                             227 * 1024);
     if (e != cudaSuccess) return e;
   }
-  dim3 grid((nv + ROWS - 1) / ROWS, V);
-  fdk_conv_kernel<<<grid, 256, smem, s>>>(raw, nu, nv, ext, pitch, sdd,
-                                          (float)(pitch * sid / sdd), tab, out);
+  dim3 grid((groups + G - 1) / G, V);
+  fdk_conv_kernel<<<grid, threads, smem, s>>>(raw, nu, nv, ext, G, (float)(pitch * sid / sdd), tab,
+                                              out);
   return cudaGetLastError();
 }
 

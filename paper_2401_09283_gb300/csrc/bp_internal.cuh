@@ -184,11 +184,10 @@ cudaError_t launch_akima_vjp(int n, int V, const double* nodes, const double* g,
 
 // FDK preprocessing (bp_fdk.cu): cosine and redundancy weights, optional
 // truncation extension by `ext` pixels per side, Shepp-Logan ramp along rows.
-// `tab` holds fdk_table_floats(V, nu, ext) floats of workspace; nu + 2 ext <=
-// FDK_MAX_NU (shared memory of the convolution: fdk_smem_bytes(nu, ext)).
+// `tab` holds fdk_table_floats(V, nu, nv, ext) floats of workspace (8-byte aligned);
+// nu + 2 ext <= FDK_MAX_NU (the convolution keeps whole rows in shared memory).
 constexpr int FDK_MAX_NU = 8192;
-size_t fdk_table_floats(int V, int nu, int ext);
-size_t fdk_smem_bytes(int nu, int ext);
+size_t fdk_table_floats(int V, int nu, int nv, int ext);
 cudaError_t launch_fdk_filter(const float* raw, int V, int nv, int nu, int ext, double pitch,
                               double sid, double sdd, double arc, float* tab, float* out,
                               cudaStream_t s);
