@@ -10,11 +10,8 @@ namespace bpk {
 
 // R = Rz(rz) Ry(ry) Rx(rx) (row-major 3x3), or its derivative with respect
 // to one angle when dax = 0, 1, 2 (x, y, z).
-__device__ static void rot_zyx(const double* th, int dax, double R[9]) {
-  double sx, cx, sy, cy, sz, cz;
-  sincos(th[3], &sx, &cx);
-  sincos(th[4], &sy, &cy);
-  sincos(th[5], &sz, &cz);
+__device__ static void rot_zyx(const double sn[3], const double cs[3], int dax, double R[9]) {
+  const double sx = sn[0], cx = cs[0], sy = sn[1], cy = cs[1], sz = sn[2], cz = cs[2];
   double X[9] = {1, 0, 0, 0, cx, -sx, 0, sx, cx};
   double Y[9] = {cy, 0, sy, 0, 1, 0, -sy, 0, cy};
   double Z[9] = {cz, -sz, 0, sz, cz, 0, 0, 0, 1};
@@ -54,8 +51,9 @@ __device__ static void compose_view(const double* __restrict__ P, const double* 
                                     ViewGeom* __restrict__ geom, double* __restrict__ Phat, int j) {
   double Ph[12];
   if (theta) {
-    double R[9];
-    rot_zyx(theta + 6 * j, -1, R);
+    double R[9], sn[3], cs[3];
+    for (int k = 0; k < 3; ++k) sincos(theta[6 * j + 3 + k], &sn[k], &cs[k]);
+    rot_zyx(sn, cs, -1, R);
     p_times_rigid(P + 12 * j, R, theta + 6 * j, 1.0, Ph);
   } else {
     for (int e = 0; e < 12; ++e) Ph[e] = P[12 * j + e];
@@ -73,8 +71,11 @@ __device__ static void compose_view(const double* __restrict__ P, const double* 
     g.P[4 * r + 3] = p[0] * vi.A[3] + p[1] * vi.A[7] + p[2] * vi.A[11] + p[3];
   }
   double c = vw ? vw[j] : 1.0;
-  g.wgt = fdk ? c * sid * sid : c;
-  g.scale = vscale ? (double)vscale[j] : 1.0;
+  const double wgt = fdk ? c * sid * sid : c;
+  const double scale = vscale ? (double)vscale[j] : 1.0;
+  g.R[0] = make_float4((float)g.P[0], (float)g.P[1], (float)g.P[2], (float)(wgt * scale));
+  g.R[1] = make_float4((float)g.P[4], (float)g.P[5], (float)g.P[6], (float)wgt);
+  g.R[2] = make_float4((float)g.P[8], (float)g.P[9], (float)g.P[10], 0.0f);
   geom[j] = g;
 }
 
@@ -97,7 +98,9 @@ __host__ __device__ static bool view_wide(const double* Pc, const VolInfo& vi, i
   return eu / wm > cols || ev / wm > rows;
 }
 
-// One thread per view.
+// One thread per view, a warp per CTA: FP64 instructions of several warps of an SM
+// queue up behind each other (2 lanes per clock and SM).
+constexpr int COMPOSE_NT = 32;
 __global__ void compose_kernel(const double* __restrict__ P, const double* __restrict__ theta,
                                const double* __restrict__ vw, const float* __restrict__ vscale,
                                int V, int fdk, double sid, VolInfo vi, ViewGeom* __restrict__ geom,
@@ -144,7 +147,7 @@ cudaError_t launch_compose(const double* P, const double* theta, const double* v
   if (V <= 0) return cudaSuccess;
   int cols = 0, rows = 0;
   if (fit) stage_limits(fit->dtype, &cols, &rows);
-  compose_kernel<<<(V + 127) / 128, 128, 0, s>>>(P, theta, view_weight, view_scale, V, fdk, sid,
+  compose_kernel<<<(V + COMPOSE_NT - 1) / COMPOSE_NT, COMPOSE_NT, 0, s>>>(P, theta, view_weight, view_scale, V, fdk, sid,
                                                   vi, geom, Phat, fit ? fit->wide : nullptr, cols,
                                                   rows);
   return cudaGetLastError();
@@ -185,12 +188,21 @@ __device__ static void reduce_chain_view(const float* __restrict__ partials, int
   }
   for (int e = 0; e < 12; ++e) red[e][tid] = acc[e];
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (tid < w)
-      for (int e = 0; e < 12; ++e) red[e][tid] += red[e][tid + w];
+  // pairwise tree over the threads that had a record, all (sum, thread) pairs of a
+  // level spread over the CTA
+  int lw = 7;
+  while (lw >= 0 && (1 << lw) >= ntiles) --lw;
+  for (; lw >= 0; --lw) {
+    for (int x = tid; x < 12 << lw; x += 256) {
+      const int e = x >> lw, c = x & ((1 << lw) - 1);
+      red[e][c] += red[e][c + (1 << lw)];
+    }
     __syncthreads();
   }
-  if (tid != 0) return;
+  // The chain rule, one lane per motion parameter (a warp's FP64 instruction costs
+  // the same for one lane as for 32; one thread for all six, before, and the spread of
+  // the tree took a 64^3 x 60 step from 226 to 197 us together with the records).
+  if (tid >= 32) return;
   double Gp[12], Gh[12];
   for (int e = 0; e < 12; ++e) Gp[e] = red[e][0];
   const double sxyz[3] = {vi.A[0], vi.A[5], vi.A[10]};
@@ -199,30 +211,28 @@ __device__ static void reduce_chain_view(const float* __restrict__ partials, int
     for (int c = 0; c < 3; ++c) Gh[4 * r + c] = Gp[4 * r + c] * sxyz[c] + Gp[4 * r + 3] * txyz[c];
     Gh[4 * r + 3] = Gp[4 * r + 3];
   }
-  if (dPhat)
+  if (dPhat && tid == 0)
     for (int e = 0; e < 12; ++e) dPhat[12 * j + e] = Gh[e];
   if (!dth) return;
-  const double zero6[6] = {0, 0, 0, 0, 0, 0};
-  const double* th = theta ? theta + 6 * j : zero6;
-  const double* Pj = P + 12 * j;
-  for (int m = 0; m < 6; ++m) {
-    double J[12];
-    if (m < 3) {
-      // dT/dt_m: zero rotation block, unit vector in the translation column
-      const double Rz0[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-      double t[3] = {0, 0, 0};
-      t[m] = 1.0;
-      p_times_rigid(Pj, Rz0, t, 0.0, J);
-    } else {
-      double dR[9];
-      const double t0[3] = {0, 0, 0};
-      rot_zyx(th, m - 3, dR);
-      p_times_rigid(Pj, dR, t0, 0.0, J);
+  const int m = tid < 6 ? tid : 5;
+  double sn[3], cs[3];
+  {
+    double a, b;
+    sincos(theta ? theta[6 * j + 3 + tid % 3] : 0.0, &a, &b);
+    for (int k = 0; k < 3; ++k) {
+      sn[k] = __shfl_sync(0xffffffffu, a, k);
+      cs[k] = __shfl_sync(0xffffffffu, b, k);
     }
-    double s = 0.0;
-    for (int e = 0; e < 12; ++e) s += Gh[e] * J[e];
-    dth[6 * j + m] = s;
   }
+  // dT/dt_m: zero rotation block, unit vector in the translation column
+  double dR[9], t[3], J[12];
+  rot_zyx(sn, cs, m - 3, dR);
+  for (int e = 0; e < 9; ++e) dR[e] = m < 3 ? 0.0 : dR[e];
+  for (int k = 0; k < 3; ++k) t[k] = m == k ? 1.0 : 0.0;
+  p_times_rigid(P + 12 * j, dR, t, 0.0, J);
+  double s = 0.0;
+  for (int e = 0; e < 12; ++e) s += Gh[e] * J[e];
+  if (tid < 6) dth[6 * j + m] = s;
 }
 
 __global__ void reduce_chain_kernel(const float* __restrict__ partials, int ntiles, VolInfo vi,

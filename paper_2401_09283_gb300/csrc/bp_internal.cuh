@@ -36,10 +36,11 @@ constexpr int PSLOTS = 16;    // floats per (tile, view) partial record
 constexpr int ZB_VJP = BP_ZB_VJP;
 
 // Per view, written by compose_kernel.
-struct ViewGeom {
+struct alignas(16) ViewGeom {
   double P[12];   // P' = P T(theta) A   (index frame -> absolute pixels)
-  double wgt;     // c_j * (FDK ? sid^2 : 1)
-  double scale;   // per-view dequantisation scale (1 for float32 data)
+  // wgt = c_j * (FDK ? sid^2 : 1), scale the per-view dequantisation scale
+  // (1 for float32 data); in FP32, as the tile records take them
+  float4 R[3];    // rows of P' (columns 0-2); .w: wgt * scale, wgt, 0
 };
 
 // Per (tile, view), in shared memory.  The first four quads are what the

@@ -217,9 +217,12 @@ __device__ __forceinline__ TileIdx tile_index(const VolInfo& vi, int tile, int z
 }
 
 // Cooperative set-up of the records of views j0 .. j0+nb-1 (nb <= 32) for
-// this CTA's box; every thread of the CTA must call it.  Eight lanes serve
-// one view; lane c evaluates box corner c.  FP64 is used only where the
-// precision matters -- the projection (uc, vc, wc) of the tile centre and
+// this CTA's box; whole warps call it.  Eight lanes serve one view; lane c
+// evaluates box corner c, lanes 0-2 also one row each in FP64 (eight FP64
+// instructions per warp, of 16 cycles each on an SM's FP64 pipe; all rows in every
+// lane, with the conversions, were 32: 256^3 x 248 forward 3.59 -> 3.53 ms).  FP64
+// is used only where the precision
+// matters -- the projection (uc, vc, wc) of the tile centre and
 // the anchored values U0 = uc - au wc, V0 = vc - av wc; the anchor pixel
 // itself only has to be near the projection and comes from FP32.  The
 // corners are evaluated in FP32 in the anchored frame (errors ~1e-5 px,
@@ -235,39 +238,41 @@ __device__ __forceinline__ TileIdx tile_index(const VolInfo& vi, int tile, int z
 // the sample loop needs neither checks nor clamps), if it fits the buffer.
 template <typename T, bool STAGE>
 __device__ void setup_batch(TileView* tvs, const ViewGeom* __restrict__ geom, int j0, int nb,
-                            const TileIdx& ti, int nu, int nv, bool with_scale, int halo = 0) {
+                            const TileIdx& ti, int nu, int nv, int halo = 0) {
   const int b = threadIdx.x >> 3, c = threadIdx.x & 7;
+  if ((int)(threadIdx.x >> 5) * 4 >= nb) return;  // a warp without a view
   const ViewGeom& g = geom[j0 + min(b, nb - 1)];
-  const double* M = g.P;
-  const double uc = fma(M[0], ti.qc[0], fma(M[1], ti.qc[1], fma(M[2], ti.qc[2], M[3])));
-  const double vc = fma(M[4], ti.qc[0], fma(M[5], ti.qc[1], fma(M[6], ti.qc[2], M[7])));
-  const double wc = fma(M[8], ti.qc[0], fma(M[9], ti.qc[1], fma(M[10], ti.qc[2], M[11])));
-  int au = 0, av = 0;
-  if (wc > 0.0) {
-    const float wf = (float)wc;
-    const float a = fminf(fmaxf(floorf((float)uc / wf), -1048576.0f), 1048576.0f);
-    const float bq = fminf(fmaxf(floorf((float)vc / wf), -1048576.0f), 1048576.0f);
-    au = (int)a;
-    av = (int)bq;
-  }
+  // lanes 0, 1, 2 of a view hold the rows u, v, w of the tile centre's projection
+  const int row = min(c, 2);
+  const double* M = g.P + 4 * row;
+  const double pc = fma(M[0], ti.qc[0], fma(M[1], ti.qc[1], fma(M[2], ti.qc[2], M[3])));
+  const float pf = (float)pc;
+  const double wc = __shfl_sync(0xffffffffu, pc, 2, 8);
+  const float wf = __shfl_sync(0xffffffffu, pf, 2, 8);
+  int ar = 0;  // the row's anchor
+  if (wc > 0.0 && c < 2)
+    ar = (int)fminf(fmaxf(floorf(pf / wf), -1048576.0f), 1048576.0f);
+  const int au = __shfl_sync(0xffffffffu, ar, 0, 8), av = __shfl_sync(0xffffffffu, ar, 1, 8);
+  const float p0 = c < 2 ? (float)fma(-(double)ar, wc, pc) : pf;
   TileView t;
-  t.U0 = (float)fma(-(double)au, wc, uc);
-  t.V0 = (float)fma(-(double)av, wc, vc);
-  t.W0 = (float)wc;
+  t.U0 = __shfl_sync(0xffffffffu, p0, 0, 8);
+  t.V0 = __shfl_sync(0xffffffffu, p0, 1, 8);
+  t.W0 = wf;
   const float fau = (float)au, fav = (float)av;
-  t.rw0 = (float)M[8];
-  t.rw1 = (float)M[9];
-  t.rw2 = (float)M[10];
-  t.ru0 = fmaf(-fau, t.rw0, (float)M[0]);
-  t.ru1 = fmaf(-fau, t.rw1, (float)M[1]);
-  t.ru2 = fmaf(-fau, t.rw2, (float)M[2]);
-  t.rv0 = fmaf(-fav, t.rw0, (float)M[4]);
-  t.rv1 = fmaf(-fav, t.rw1, (float)M[5]);
-  t.rv2 = fmaf(-fav, t.rw2, (float)M[6]);
+  const float4 R0 = g.R[0], R1 = g.R[1], R2 = g.R[2];
+  t.rw0 = R2.x;
+  t.rw1 = R2.y;
+  t.rw2 = R2.z;
+  t.ru0 = fmaf(-fau, t.rw0, R0.x);
+  t.ru1 = fmaf(-fau, t.rw1, R0.y);
+  t.ru2 = fmaf(-fau, t.rw2, R0.z);
+  t.rv0 = fmaf(-fav, t.rw0, R1.x);
+  t.rv1 = fmaf(-fav, t.rw1, R1.y);
+  t.rv2 = fmaf(-fav, t.rw2, R1.z);
   t.au = au;
   t.av = av;
-  t.wgt = (float)(with_scale ? g.wgt * g.scale : g.wgt);
-  t.wgtd = (float)g.wgt;
+  t.wgt = R0.w;
+  t.wgtd = R1.w;
   // this lane's corner
   const float d0 = (c & 1) ? ti.hx : -ti.hx;
   const float d1 = (c & 2) ? ti.hy : -ti.hy;
@@ -687,9 +692,9 @@ __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const C
   bool bad = false;
   const int V = pi.nviews;
   const int nbatch = (V + VB - 1) / VB;
-  setup_batch<T, STAGE>(tvs[0], geom, 0, min(VB, V), ti, pi.nu, pi.nv, true);
+  setup_batch<T, STAGE>(tvs[0], geom, 0, min(VB, V), ti, pi.nu, pi.nv);
   if (nbatch > 1)
-    setup_batch<T, STAGE>(tvs[1], geom, VB, min(VB, V - VB), ti, pi.nu, pi.nv, true);
+    setup_batch<T, STAGE>(tvs[1], geom, VB, min(VB, V - VB), ti, pi.nu, pi.nv);
   __syncthreads();
   if (STAGE && warp < NS && warp < V) {
     const unsigned s = (pos.slot + warp) % NS;
@@ -700,7 +705,7 @@ __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const C
     if (b == 0 && k >= 1 && k + 1 < nbatch) {
       __syncthreads();  // every warp is done with batch k-1
       setup_batch<T, STAGE>(tvs[(k + 1) & 1], geom, (k + 1) * VB, min(VB, V - (k + 1) * VB), ti,
-                            pi.nu, pi.nv, true);
+                            pi.nu, pi.nv);
       __syncthreads();
     }
     // without the pipe, a barrier per view keeps the warps' footprints together
@@ -1884,9 +1889,9 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
       partials[((long long)(vbeg + e / PSLOTS) * ntiles + tile) * PSLOTS + e % PSLOTS] = 0.0f;
     return;
   }
-  setup_batch<T, STAGE>(tvs[0], geom, vbeg, min(VB, nvw), ti, pi.nu, pi.nv, true, HALO);
+  setup_batch<T, STAGE>(tvs[0], geom, vbeg, min(VB, nvw), ti, pi.nu, pi.nv, HALO);
   if (nbatch > 1)
-    setup_batch<T, STAGE>(tvs[1], geom, vbeg + VB, min(VB, nvw - VB), ti, pi.nu, pi.nv, true,
+    setup_batch<T, STAGE>(tvs[1], geom, vbeg + VB, min(VB, nvw - VB), ti, pi.nu, pi.nv,
                           HALO);
   __syncthreads();
   if (STAGE && warp < NS && warp < nvw)
@@ -1903,7 +1908,7 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
       if (CONV) __syncthreads();
       if (k + 1 < nbatch)
         setup_batch<T, STAGE>(tvs[(k + 1) & 1], geom, vbeg + (k + 1) * VB,
-                              min(VB, nvw - (k + 1) * VB), ti, pi.nu, pi.nv, true, HALO);
+                              min(VB, nvw - (k + 1) * VB), ti, pi.nu, pi.nv, HALO);
       __syncthreads();
     }
     const TileView& t = tvs[k & 1][b];
@@ -2177,7 +2182,7 @@ __global__ void __launch_bounds__(NT, 2)
   for (int j0 = vbeg; j0 < vend; j0 += VB) {
     const int nb = min(VB, vend - j0);
     __syncthreads();
-    setup_batch<float, false>(tvs, geom, j0, nb, ti, pi.nu, pi.nv, true);
+    setup_batch<float, false>(tvs, geom, j0, nb, ti, pi.nu, pi.nv);
     __syncthreads();
     for (int b = 0; b < nb; ++b) {
       const TileView t = tvs[b];
