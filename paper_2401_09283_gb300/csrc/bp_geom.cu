@@ -115,17 +115,35 @@ __global__ void compose_kernel(const double* __restrict__ P, const double* __res
 // Pixels of the staging buffer less the taps, their halo and the rounding to
 // 16-byte chunks.
 static void stage_limits(int dtype, int* cols, int* rows) {
-  stage_extent(dtype, cols, rows);
+  stage_extent(dtype, false, cols, rows);
   *cols -= 3;
   *rows -= 3;
 }
 
-static const int kWideAll = 0;
-const int* const WIDE_ALL = &kWideAll;
+static const int kWide[2] = {};
+const int* const WIDE_ALL = kWide;
+const int* const WIDE_HALF = kWide + 1;
 
-bool all_views_wide(const double* P, int V, int dtype, const VolInfo& vi) {
+// Whether the half tiles at the volume's centre fit the half-tile buffers in this
+// view, with room for the spread of a tile's magnification over the rows.
+static bool half_tiles_fit(const double* Pc, const VolInfo& vi, int dtype) {
+  const double w = Pc[11];
+  if (!(w > 0.0)) return false;
+  int cols, rows;
+  stage_extent(dtype, true, &cols, &rows);
+  double eu = 0.0, ev = 0.0;
+  for (int k = 0; k < 3; ++k) {
+    const double e = k < 2 ? TX - 1 : TX / 2 - 1;
+    eu += e * fabs(Pc[k] - Pc[3] / w * Pc[8 + k]) / w;
+    ev += e * fabs(Pc[4 + k] - Pc[7] / w * Pc[8 + k]) / w;
+  }
+  return eu <= cols - (dtype == 0 ? 7 : 11) && ev <= rows - 16;
+}
+
+const int* scan_variant(const double* P, int V, int dtype, const VolInfo& vi) {
   int cols, rows;
   stage_limits(dtype, &cols, &rows);
+  bool half = true;
   for (int j = 0; j < V; ++j) {
     double Pc[12];
     for (int r = 0; r < 3; ++r) {
@@ -135,9 +153,10 @@ bool all_views_wide(const double* P, int V, int dtype, const VolInfo& vi) {
       Pc[4 * r + 2] = p[2] * vi.A[10];
       Pc[4 * r + 3] = p[0] * vi.A[3] + p[1] * vi.A[7] + p[2] * vi.A[11] + p[3];
     }
-    if (!view_wide(Pc, vi, cols, rows)) return false;
+    if (!view_wide(Pc, vi, cols, rows)) return nullptr;
+    half = half && half_tiles_fit(Pc, vi, dtype);
   }
-  return true;
+  return half ? WIDE_HALF : WIDE_ALL;
 }
 
 cudaError_t launch_compose(const double* P, const double* theta, const double* view_weight,
@@ -716,8 +735,7 @@ cudaError_t launch_batch_iteration(const BatchTable& tab, unsigned* counter, int
       e = cudaStreamWaitEvent(br->streams[m], br->fork, 0);
       if (e == cudaSuccess)
         e = launch_vjp_motion(J.dvol, J.proj, dtype, J.pi, J.grad, J.geom, J.vi, fdk, exact,
-                              J.partials, nullptr, nullptr, J.unstaged ? WIDE_ALL : nullptr,
-                              br->streams[m]);
+                              J.partials, nullptr, nullptr, J.wide, br->streams[m]);
       if (e == cudaSuccess) e = cudaEventRecord(br->joins[m], br->streams[m]);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(s, br->joins[m], 0);
     }

@@ -86,17 +86,18 @@ struct ProjInfo {
 
 // Views whose tiles project larger than the staging buffer everywhere in the
 // volume ("wide": more than ~4 px per voxel) read global memory, and do so
-// faster from a kernel variant that leaves the L1 cache its full size
-// (a job of 10 iterations on 128^3 x 360 views, 4.8 px per voxel: 61.6 ms, 76.2 ms
-// from the staged variant's fallback).  `wide` of launch_forward and launch_vjp_motion:
-// NULL, take the staged variant; WIDE_ALL, take the other one; else one flag
-// per view on the device (launch_compose, fit): both are launched and each
-// item runs in the one that suits its first view.
+// faster from a kernel variant that leaves the L1 cache its full size, unless
+// most half tiles fit the wider half-tile buffers.  `wide` of launch_forward and
+// launch_vjp_motion: NULL, take the staged variant; WIDE_ALL, take the one that
+// reads global memory; WIDE_HALF, stage half tiles (the same job: 59.9 -> 50.6 ms);
+// else one flag per view on the device (launch_compose, fit): the first two are launched and each item runs in
+// the one that suits its first view.
 struct FitInfo {
   int dtype;
   int* wide;  // [V]
 };
 extern const int* const WIDE_ALL;
+extern const int* const WIDE_HALF;
 // ------------------------------------------------------------ launchers
 // All launchers are asynchronous on `stream` and return cudaGetLastError().
 
@@ -105,15 +106,18 @@ cudaError_t launch_compose(const double* P, const double* theta, const double* v
                            const VolInfo& vi, ViewGeom* geom, double* Phat, cudaStream_t s,
                            const FitInfo* fit = nullptr);
 
-// The same test on the host for the nominal matrices: every view is wide.
-bool all_views_wide(const double* P, int V, int dtype, const VolInfo& vi);
+// The choice for a whole scan from its nominal matrices, on the host: WIDE_ALL or
+// WIDE_HALF where every view is wide, else NULL.
+const int* scan_variant(const double* P, int V, int dtype, const VolInfo& vi);
 
 
 // The tensor map of a projection stack that the staging copies read; needs
 // 16-byte aligned data and strides (and a width of whole 16-byte chunks).
+// half: the boxes of the half-tile buffers.
+cudaError_t make_stage_map(const void* proj, int dtype, const ProjInfo& pi, CUtensorMap* map,
+                           bool half);
 // Pixels (columns, rows) of a staging buffer.
-void stage_extent(int dtype, int* cols, int* rows);
-cudaError_t make_stage_map(const void* proj, int dtype, const ProjInfo& pi, CUtensorMap* map);
+void stage_extent(int dtype, bool half, int* cols, int* rows);
 
 cudaError_t launch_forward(const void* proj, int dtype, const ProjInfo& pi, const ViewGeom* geom,
                            const VolInfo& vi, int fdk, float* vol, const int* wide,
@@ -227,7 +231,7 @@ struct BatchJob {
   double lr_t, lr_r, beta1, beta2, eps, decay;
   float tv_eps;
   int V, ntiles_f, ntiles_v, nblk, max_iters, gauge;
-  int unstaged;            // every view is wide
+  const int* wide;         // scan_variant of the scan (host value)
 };
 
 struct BatchTable {

@@ -37,7 +37,7 @@ struct bp_job {
   cudaStream_t cap = nullptr;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
-  bool unstaged = false;        // every view is wide: the kernels that read global memory
+  const int* wide = nullptr;    // the kernel variant of the scan (scan_variant)
   bool cancelled = false;
   int queued = 0;               // iterations queued so far (motion_step or batches)
   bp_batch* batch = nullptr;    // the batch this job is a member of, if any
@@ -138,7 +138,7 @@ cudaError_t record_iteration(bp_job* j, cudaStream_t s) {
                           nullptr, s);
   if (e != cudaSuccess) return e;
   e = bpk::launch_forward(j->proj, j->pd.dtype, j->pi, j->geom, j->vi, fdk, j->vol,
-                          j->unstaged ? bpk::WIDE_ALL : nullptr, s);
+                          j->wide, s);
   if (e != cudaSuccess) return e;
   if (j->opt.loss == BP_LOSS_TV)
     e = bpk::launch_tv(j->vol, j->vd.nx, j->vd.ny, j->vd.nz, (float)j->opt.tv_eps, j->blk, j->nblk,
@@ -149,7 +149,7 @@ cudaError_t record_iteration(bp_job* j, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   e = bpk::launch_vjp_motion(j->dvol, j->proj, j->pd.dtype, j->pi, j->grad, j->geom, j->vi, fdk,
                              j->deriv == BP_DERIV_BILINEAR_EXACT, j->partials, nullptr, nullptr,
-                             j->unstaged ? bpk::WIDE_ALL : nullptr, s);
+                             j->wide, s);
   if (e != cudaSuccess) return e;
   e = bpk::launch_reduce_chain(j->partials, j->ntiles, j->vi, j->P, j->theta, V, nullptr, j->gth,
                                s);
@@ -353,7 +353,7 @@ int bp_job_create(bp_ctx* ctx, const void* proj, const bp_proj_desc* pdesc, cons
     delete j;
     return cuda_fail(ctx, e, "bp_job_create");
   }
-  j->unstaged = bpk::all_views_wide(Ph.data(), V, pdesc->dtype, j->vi);
+  j->wide = bpk::scan_variant(Ph.data(), V, pdesc->dtype, j->vi);
   ctx->job_bytes += j->bytes;
   *out = j;
   return BP_OK;
@@ -517,7 +517,7 @@ cudaError_t fill_table(bp_batch* b, bpk::BatchTable& T) {
     J.hist = j->hist;
     J.iter = j->iter;
     J.pi = j->pi;
-    const cudaError_t e = bpk::make_stage_map(j->proj, j->pd.dtype, j->pi, &J.map);
+    const cudaError_t e = bpk::make_stage_map(j->proj, j->pd.dtype, j->pi, &J.map, false);
     if (e != cudaSuccess) return e;
     J.vi = j->vi;
     J.vif = j->vi;
@@ -537,7 +537,7 @@ cudaError_t fill_table(bp_batch* b, bpk::BatchTable& T) {
     J.nblk = j->nblk;
     J.max_iters = j->max_iters;
     J.gauge = j->opt.gauge;
-    J.unstaged = j->unstaged;
+    J.wide = j->wide;
     T.off_view[k + 1] = T.off_view[k] + J.V;
     T.off_fwd[k + 1] = T.off_fwd[k] + J.ntiles_f;
     T.off_loss[k + 1] = T.off_loss[k] + J.nblk;

@@ -43,19 +43,51 @@ constexpr unsigned INDEX_BITS = 0x4A400000u;
 // BF16 footprints arrive raw (pitch 80; 88 bank-conflicts more, 30.8 against
 // 30.5 ms for a 384^3 x 248 VJP) and are converted once per (tile, view) into an
 // FP32 buffer of the same pitch, which the sample loops read like FP32 data.
-constexpr int STAGE_ROWS = 64;
 constexpr int BOX_ROWS = 8;
-template <typename T>
+template <typename G>
 struct StageGeom {
-  static constexpr int CH = 16 / (int)sizeof(T);               // elements per 16 bytes
-  static constexpr int P = sizeof(T) == 4 ? 84 : 80;           // row pitch in elements
-  static constexpr int BOX_BYTES = P * BOX_ROWS * (int)sizeof(T);
-  static constexpr int BYTES = P * STAGE_ROWS * (int)sizeof(T);  // one footprint buffer
+  static constexpr bool CONV = sizeof(G) != 4;                 // converted to FP32
+  static constexpr int CH = 16 / (int)sizeof(G);               // elements per 16 bytes
+  static constexpr int P = CONV ? 80 : 84;                     // row pitch in elements
+  static constexpr int ROWS = 64;
+  static constexpr int BOX_BYTES = P * BOX_ROWS * (int)sizeof(G);
+  static constexpr int BYTES = P * ROWS * (int)sizeof(G);      // one footprint buffer
+  static constexpr int F_BYTES = CONV ? P * ROWS * 4 : 0;      // converted footprint
 };
-constexpr int CONV_F_BYTES = StageGeom<__half>::P * STAGE_ROWS * 4;  // converted footprint
-static_assert(StageGeom<float>::BOX_BYTES % 128 == 0 && StageGeom<__half>::BOX_BYTES % 128 == 0 &&
-                  CONV_F_BYTES % 128 == 0,
+// Buffers of half tiles (16 x 16 x 8 voxels), for scans of 4 to 5 pixels per voxel,
+// whose whole tiles project wider and higher than the buffers above.  116 floats:
+// 93 % of the half tiles of a 128^3 volume at 4.8 px per voxel fit (108 wide 80 %,
+// 48 rows 77 %), four CTAs per SM, and as few bank conflicts as 84 (124 has more).
+template <typename T>
+struct Half {};
+template <typename T>
+struct StageGeom<Half<T>> {
+  static constexpr bool CONV = sizeof(T) != 4;
+  static constexpr int CH = 16 / (int)sizeof(T);
+  static constexpr int P = CONV ? 120 : 116;
+  static constexpr int ROWS = 56;
+  static constexpr int BOX_BYTES = P * BOX_ROWS * (int)sizeof(T);
+  static constexpr int BYTES = P * ROWS * (int)sizeof(T);
+  static constexpr int F_BYTES = CONV ? P * ROWS * 4 : 0;
+};
+template <typename G>
+constexpr bool aligned_boxes() {  // TMA boxes land on 128-byte boundaries
+  return StageGeom<G>::BOX_BYTES % 128 == 0 && StageGeom<G>::F_BYTES % 128 == 0;
+}
+static_assert(aligned_boxes<float>() && aligned_boxes<__half>() && aligned_boxes<Half<float>>() &&
+                  aligned_boxes<Half<__half>>(),
               "TMA boxes land on 128-byte boundaries");
+
+// How a kernel variant gets its footprints: from global memory, staged whole tiles,
+// staged half tiles.
+enum { STAGE_NONE = 0, STAGE_TILE = 1, STAGE_HALF = 2 };
+template <typename T, int STAGE>
+using Geo = std::conditional_t<STAGE == STAGE_HALF, Half<T>, T>;
+// Records per batch of views (half tiles: two records per view in the VJP).
+template <int STAGE>
+__host__ __device__ constexpr int batch_records() {
+  return STAGE == STAGE_HALF ? VB / 2 : VB;
+}
 
 template <typename T>
 __device__ __forceinline__ float ldv(const T* p);
@@ -236,12 +268,17 @@ __device__ __forceinline__ TileIdx tile_index(const VolInfo& vi, int tile, int z
 // detector pixels that any tap (plus `halo` pixels each side) can read,
 // NOT clipped to the detector (off-detector pixels are staged as zeros, so
 // the sample loop needs neither checks nor clamps), if it fits the buffer.
-template <typename T, bool STAGE>
+// With HALVES = 2 record b is the lower (even b) or upper half, in z, of the box in
+// view j0 + b / 2 (whole views: j0 is of a lower half).
+template <typename G, bool STAGE, int HALVES = 1>
 __device__ void setup_batch(TileView* tvs, const ViewGeom* __restrict__ geom, int j0, int nb,
                             const TileIdx& ti, int nu, int nv, int halo = 0) {
   const int b = threadIdx.x >> 3, c = threadIdx.x & 7;
   if ((int)(threadIdx.x >> 5) * 4 >= nb) return;  // a warp without a view
-  const ViewGeom& g = geom[j0 + min(b, nb - 1)];
+  const ViewGeom& g = geom[j0 + min(b, nb - 1) / HALVES];
+  const float zmid = 0.5f * (ti.zlo + ti.zhi);
+  const float zlo = HALVES == 2 && (b & 1) ? zmid + 0.5f : ti.zlo;
+  const float zhi = HALVES == 2 && !(b & 1) ? zmid - 0.5f : ti.zhi;
   // lanes 0, 1, 2 of a view hold the rows u, v, w of the tile centre's projection
   const int row = min(c, 2);
   const double* M = g.P + 4 * row;
@@ -276,7 +313,7 @@ __device__ void setup_batch(TileView* tvs, const ViewGeom* __restrict__ geom, in
   // this lane's corner
   const float d0 = (c & 1) ? ti.hx : -ti.hx;
   const float d1 = (c & 2) ? ti.hy : -ti.hy;
-  const float d2 = (c & 4) ? ti.zhi : ti.zlo;
+  const float d2 = (c & 4) ? zhi : zlo;
   const float w = fmaf(t.rw2, d2, fmaf(t.rw1, d1, fmaf(t.rw0, d0, t.W0)));
   const float u = fmaf(t.ru2, d2, fmaf(t.ru1, d1, fmaf(t.ru0, d0, t.U0)));
   const float v = fmaf(t.rv2, d2, fmaf(t.rv1, d1, fmaf(t.rv0, d0, t.V0)));
@@ -317,14 +354,14 @@ __device__ void setup_batch(TileView* tvs, const ViewGeom* __restrict__ geom, in
     t.csafe = xmin >= ulo + 1.0f + m && xmax <= uhi - 1.0f - m &&
               ymin >= vlo + 1.0f + m && ymax <= vhi - 1.0f - m;
     if (STAGE) {
-      constexpr int CH = StageGeom<T>::CH, P = StageGeom<T>::P;
+      constexpr int CH = StageGeom<G>::CH, P = StageGeom<G>::P;
       const int fl_u0 = (int)floorf(xmin - m) + au, fl_u1 = (int)floorf(xmax + m) + 1 + au;
       const int fl_v0 = (int)floorf(ymin - m) + av, fl_v1 = (int)floorf(ymax + m) + 1 + av;
       const int x0 = (fl_u0 - halo) & ~(CH - 1);  // floor to a 16-byte boundary
       const int y0 = fl_v0 - halo;
       const int cpr = (fl_u1 + halo - x0) / CH + 1;
       const int h = fl_v1 + halo - y0 + 1;
-      if (cpr * CH <= P && h <= STAGE_ROWS) {
+      if (cpr * CH <= P && h <= StageGeom<G>::ROWS) {
         t.staged = 1;
         t.sx0 = x0;
         t.sv0 = y0;
@@ -464,14 +501,14 @@ struct PipePos {
 };
 
 // One whole warp: request the footprint of record t (view v) into buf.
-template <typename T>
+template <typename G>
 __device__ __forceinline__ void stage_issue(unsigned char* buf, const CUtensorMap* map,
                                             const TileView& t, int v, unsigned long long* bar) {
-  constexpr int BOX = StageGeom<T>::BOX_BYTES;
+  constexpr int BOX = StageGeom<G>::BOX_BYTES;
   const int lane = threadIdx.x & 31;
   int nb = t.staged ? (t.sh + BOX_ROWS - 1) / BOX_ROWS : 0;
 #ifdef BP_BOUNDS_CHECK
-  if (nb > STAGE_ROWS / BOX_ROWS || (t.sx0 & (StageGeom<T>::CH - 1))) {
+  if (nb > StageGeom<G>::ROWS / BOX_ROWS || (t.sx0 & (StageGeom<G>::CH - 1))) {
     if (lane == 0) bc_fail(BC_STAGE_DST, t.sh, t.sx0);
     nb = 0;
   }
@@ -501,9 +538,9 @@ __device__ __forceinline__ bool last_warp(unsigned* done) {
 // All threads: convert the raw FP16/BF16 rectangle of record t (staged by
 // stage_issue<T>) into FP32 at the same pitch, in 16-byte chunks, rows per warp
 // pass (no divisions).
-template <typename T>
+template <typename T, typename G>
 __device__ __forceinline__ void convert_stage(float* F, const T* R, const TileView& t) {
-  constexpr int CONV_P = StageGeom<T>::P;
+  constexpr int CONV_P = StageGeom<G>::P;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int lr = (lane * t.smag) >> 16, lc = lane - lr * t.scpr;
   if (lr >= t.srpp) return;
@@ -546,10 +583,10 @@ __device__ __forceinline__ f2 lds2(unsigned a, unsigned b) {
 
 #ifdef BP_BOUNDS_CHECK
 // Column and row of the floor pixel in the staged rectangle; true if bad.
-template <typename T, int H>
+template <typename G, int H>
 __device__ __forceinline__ bool bc_staged(const TileView& t, int fx, int fy) {
   const int ru = fx + t.au - t.sx0, rv = fy + t.av - t.sv0;
-  if (t.staged && ru - H >= 0 && ru + 1 + H < t.scpr * StageGeom<T>::CH && rv - H >= 0 &&
+  if (t.staged && ru - H >= 0 && ru + 1 + H < t.scpr * StageGeom<G>::CH && rv - H >= 0 &&
       rv + 1 + H < t.sh)
     return false;
   bc_fail(BC_STAGED_TAP, ru, rv);
@@ -559,11 +596,11 @@ __device__ __forceinline__ bool bc_staged(const TileView& t, int fx, int fy) {
 
 // Address of one sample's floor pixel: (bx, by) are the bit patterns of
 // x + MAGIC and y + MAGIC rounded down, i.e. MAGIC_BITS + floor.
-template <typename T, int H>
+template <typename G, int H>
 __device__ __forceinline__ unsigned staged_tap(unsigned buf, const TileView& t, int bx, int by) {
-  constexpr int P = StageGeom<T>::P;
+  constexpr int P = StageGeom<G>::P;
 #ifdef BP_BOUNDS_CHECK
-  if (bc_staged<T, H>(t, bx - MAGIC_BITS, by - MAGIC_BITS)) {
+  if (bc_staged<G, H>(t, bx - MAGIC_BITS, by - MAGIC_BITS)) {
     bx = MAGIC_BITS + t.sx0 + H - t.au;
     by = MAGIC_BITS + t.sv0 + H - t.av;
   }
@@ -577,10 +614,10 @@ __device__ __forceinline__ unsigned staged_tap(unsigned buf, const TileView& t, 
 // the byte offset, so a pair costs two packed instructions where integer
 // arithmetic on the floor bits took four to six (7.4 integer instructions per
 // voxel-view in the forward before, 40 % of its issue slots with the moves).
-template <typename T, int H>
+template <typename G, int H>
 __device__ __forceinline__ void staged_pair(unsigned buf, const TileView& t, f2 ic, f2 fx, f2 fy,
                                             unsigned& al, unsigned& ah) {
-  constexpr float P = (float)StageGeom<T>::P;
+  constexpr float P = (float)StageGeom<G>::P;
   const f2 o = fma2(fy, pk2(P, P), add2(fx, ic));
   float lo, hi;
   up2(o, lo, hi);
@@ -588,9 +625,9 @@ __device__ __forceinline__ void staged_pair(unsigned buf, const TileView& t, f2 
   float xl, xh, yl, yh;
   up2(fx, xl, xh);
   up2(fy, yl, yh);
-  const float safe = INDEX_MAGIC + (float)(H * StageGeom<T>::P + H);
-  if (bc_staged<T, H>(t, (int)xl, (int)yl)) lo = safe;
-  if (bc_staged<T, H>(t, (int)xh, (int)yh)) hi = safe;
+  const float safe = INDEX_MAGIC + (float)(H * StageGeom<G>::P + H);
+  if (bc_staged<G, H>(t, (int)xl, (int)yl)) lo = safe;
+  if (bc_staged<G, H>(t, (int)xh, (int)yh)) hi = safe;
 #endif
   al = __float_as_uint(lo) + (buf - INDEX_BITS);
   ah = __float_as_uint(hi) + (buf - INDEX_BITS);
@@ -623,11 +660,11 @@ __device__ __forceinline__ void forward_view(const T* img, long long rs, int nu,
 // One view from its staged, zero-padded footprint (no checks, no clamps, tap
 // offsets are compile-time constants), with packed pairs of voxels (k, k+1):
 // every step of the scalar loop above, in the same order, on f32x2 pairs.
-// buf is the FP32 footprint's shared-memory address, T the stored type.
-template <int ZS, typename T, bool FDK>
+// buf is the FP32 footprint's shared-memory address, G the buffers' geometry.
+template <int ZS, typename G, bool FDK>
 __device__ __forceinline__ void forward_view_staged2(unsigned buf, const TileView& t, float dx,
                                                      float dy, float zlo, f2 (&acc)[ZS / 2]) {
-  constexpr int P = StageGeom<T>::P;
+  constexpr int P = StageGeom<G>::P;
   const float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
   const float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
   const float w0 = fmaf(dy, t.rw1, fmaf(dx, t.rw0, t.W0));
@@ -647,7 +684,7 @@ __device__ __forceinline__ void forward_view_staged2(unsigned buf, const TileVie
     const f2 fx = sub2(add2_rd(x, M2), M2), fy = sub2(add2_rd(y, M2), M2);
     const f2 tu = sub2(x, fx), tv = sub2(y, fy);
     unsigned ql, qh;
-    staged_pair<T, 0>(buf, t, IC, fx, fy, ql, qh);
+    staged_pair<G, 0>(buf, t, IC, fx, fy, ql, qh);
     const f2 d00 = lds2<0>(ql, qh), d10 = lds2<1>(ql, qh);
     const f2 d01 = lds2<P>(ql, qh), d11 = lds2<P + 1>(ql, qh);
     const f2 val = bilerp2(tu, tv, d00, d10, d01, d11);
@@ -659,13 +696,9 @@ __device__ __forceinline__ void forward_view_staged2(unsigned buf, const TileVie
 // into one FP32 buffer that all warps share, so that path has CTA barriers:
 // wait for view v, barrier (every warp is done with the FP32 buffer), convert,
 // barrier, refill the raw slot, compute.
-template <typename T>
-__host__ __device__ constexpr bool conv_staging() {
-  return !std::is_same<T, float>::value;
-}
-template <typename T, int NS>
+template <typename G, int NS>
 __host__ __device__ constexpr int stage_smem_bytes() {
-  return (conv_staging<T>() ? CONV_F_BYTES : 0) + NS * StageGeom<T>::BYTES;
+  return StageGeom<G>::F_BYTES + NS * StageGeom<G>::BYTES;
 }
 
 // One tile of the forward (its slices [zs ZS, zs ZS + ZS)): every view, in
@@ -673,16 +706,17 @@ __host__ __device__ constexpr int stage_smem_bytes() {
 // dyn_smem are the CTA's shared memory.  seq counts the views the CTA has X.  The records of batch k+1 are built at the start of batch
 // k (two record slots), so the footprints of the next views are known.
 // A copy that never arrives (the bounded wait gives up) shows as NaN voxels.
-template <int ZB, int ZS, int NS, typename T, bool FDK, bool STAGE>
+template <int ZB, int ZS, int NS, typename T, bool FDK, int STAGE>
 __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const CUtensorMap* map,
                                              const ProjInfo& pi, const ViewGeom* __restrict__ geom,
                                              const VolInfo& vi, float* __restrict__ vol, int tile,
-                                             int zs, TileView (*tvs)[VB],
+                                             int zs, TileView (*tvs)[batch_records<STAGE>()],
                                              StagePipe<NS>& pipe, unsigned char* dyn_smem,
                                              PipePos<NS>& pos) {
-  constexpr bool CONV = STAGE && conv_staging<T>();
-  constexpr int SLOT = StageGeom<T>::BYTES;
-  unsigned char* slots = dyn_smem + (CONV ? CONV_F_BYTES : 0);
+  using G = Geo<T, STAGE>;
+  constexpr bool CONV = STAGE && StageGeom<G>::CONV;
+  constexpr int SLOT = StageGeom<G>::BYTES, NB = batch_records<STAGE>();
+  unsigned char* slots = dyn_smem + StageGeom<G>::F_BYTES;
   static_assert(ZS % 2 == 0 && ZB % ZS == 0, "voxel pairs");
   const TileIdx ti = tile_index<ZB, ZS>(vi, tile, zs);
   const int warp = threadIdx.x >> 5;
@@ -691,20 +725,20 @@ __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const C
   for (int k = 0; k < ZS / 2; ++k) acc[k] = pk2(0.0f, 0.0f);
   bool bad = false;
   const int V = pi.nviews;
-  const int nbatch = (V + VB - 1) / VB;
-  setup_batch<T, STAGE>(tvs[0], geom, 0, min(VB, V), ti, pi.nu, pi.nv);
+  const int nbatch = (V + NB - 1) / NB;
+  setup_batch<G, STAGE != STAGE_NONE>(tvs[0], geom, 0, min(NB, V), ti, pi.nu, pi.nv);
   if (nbatch > 1)
-    setup_batch<T, STAGE>(tvs[1], geom, VB, min(VB, V - VB), ti, pi.nu, pi.nv);
+    setup_batch<G, STAGE != STAGE_NONE>(tvs[1], geom, NB, min(NB, V - NB), ti, pi.nu, pi.nv);
   __syncthreads();
   if (STAGE && warp < NS && warp < V) {
     const unsigned s = (pos.slot + warp) % NS;
-    stage_issue<T>(slots + s * SLOT, map, tvs[0][warp], warp, &pipe.full[s]);
+    stage_issue<G>(slots + s * SLOT, map, tvs[0][warp], warp, &pipe.full[s]);
   }
   for (int v = 0; v < V; ++v) {
-    const int k = v / VB, b = v - k * VB;
+    const int k = v / NB, b = v - k * NB;
     if (b == 0 && k >= 1 && k + 1 < nbatch) {
       __syncthreads();  // every warp is done with batch k-1
-      setup_batch<T, STAGE>(tvs[(k + 1) & 1], geom, (k + 1) * VB, min(VB, V - (k + 1) * VB), ti,
+      setup_batch<G, STAGE != STAGE_NONE>(tvs[(k + 1) & 1], geom, (k + 1) * NB, min(NB, V - (k + 1) * NB), ti,
                             pi.nu, pi.nv);
       __syncthreads();
     }
@@ -717,18 +751,18 @@ __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const C
     if (STAGE && !bad) bad = !mbar_wait(&pipe.full[slot], pos.parity);
     pos.next();
     const int vn = v + NS;
-    const TileView& tn = tvs[(vn / VB) & 1][vn % VB];
+    const TileView& tn = tvs[(vn / NB) & 1][vn % NB];
     if constexpr (CONV) {
       __syncthreads();  // every warp has seen this phase and is done with F
       if (t.staged) {
-        convert_stage<T>(reinterpret_cast<float*>(dyn_smem), reinterpret_cast<const T*>(buf), t);
+        convert_stage<T, G>(reinterpret_cast<float*>(dyn_smem), reinterpret_cast<const T*>(buf), t);
         __syncthreads();  // F holds view v; the raw slot is free
       }
-      if (warp == (v & 7) && vn < V && !bad) stage_issue<T>(buf, map, tn, vn, &pipe.full[slot]);
+      if (warp == (v & 7) && vn < V && !bad) stage_issue<G>(buf, map, tn, vn, &pipe.full[slot]);
     }
     if (t.mode != MODE_SKIP) {
       if (STAGE && t.staged) {
-        forward_view_staged2<ZS, T, FDK>(smem_addr(CONV ? dyn_smem : buf), t, ti.dx, ti.dy, ti.zlo,
+        forward_view_staged2<ZS, G, FDK>(smem_addr(CONV ? dyn_smem : buf), t, ti.dx, ti.dy, ti.zlo,
                                          acc);
       } else {
         const T* img = proj + (long long)v * pi.vs;
@@ -745,7 +779,7 @@ __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const C
     }
     if constexpr (STAGE && !CONV) {
       if (last_warp(&pipe.done[slot]) && vn < V && !bad)
-        stage_issue<T>(buf, map, tn, vn, &pipe.full[slot]);
+        stage_issue<G>(buf, map, tn, vn, &pipe.full[slot]);
     }
   }
   const int i = ti.tx * TX + ti.lx, j = ti.ty * TY + ti.ly;
@@ -762,13 +796,13 @@ __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const C
   }
 }
 
-template <int ZB, int ZS, int NS, typename T, bool FDK, bool STAGE>
+template <int ZB, int ZS, int NS, typename T, bool FDK, int STAGE>
 __global__ void __launch_bounds__(NT, NS > FWD_NS ? 2 : FWD_MINB)
     forward_kernel(const T* __restrict__ proj, const __grid_constant__ CUtensorMap map, ProjInfo pi,
                    const ViewGeom* __restrict__ geom, VolInfo vi, float* __restrict__ vol,
                    const int* __restrict__ wide) {
-  if (wide && (wide[0] != 0) == STAGE) return;  // the other variant's launch
-  __shared__ TileView tvs[2][VB];
+  if (wide && (wide[0] != 0) == (STAGE != STAGE_NONE)) return;  // the other variant's launch
+  __shared__ TileView tvs[2][batch_records<STAGE>()];
   __shared__ StagePipe<NS> pipe;
   extern __shared__ __align__(128) unsigned char dyn_smem[];
   if (STAGE) pipe_init(pipe);
@@ -802,10 +836,21 @@ static cudaError_t smem_attr_once(int bytes) {
   return e;
 }
 
+void stage_extent(int dtype, bool half, int* cols, int* rows) {
+  if (half) {
+    *cols = dtype == 0 ? StageGeom<Half<float>>::P : StageGeom<Half<__half>>::P;
+    *rows = StageGeom<Half<float>>::ROWS;
+  } else {
+    *cols = dtype == 0 ? StageGeom<float>::P : StageGeom<__half>::P;
+    *rows = StageGeom<float>::ROWS;
+  }
+}
+
 // The tensor map that the staging copies read: dimensions (nu, nv, views), box
 // P x BOX_ROWS x 1.  (cuTensorMapEncodeTiled is a driver call without a stream;
 // it only fills in the descriptor.)
-cudaError_t make_stage_map(const void* proj, int dtype, const ProjInfo& pi, CUtensorMap* map) {
+cudaError_t make_stage_map(const void* proj, int dtype, const ProjInfo& pi, CUtensorMap* map,
+                           bool half) {
   using Fn = decltype(&cuTensorMapEncodeTiled);
   static const Fn encode = [] {
     void* f = nullptr;
@@ -820,8 +865,9 @@ cudaError_t make_stage_map(const void* proj, int dtype, const ProjInfo& pi, CUte
   const cuuint64_t es = dtype == 0 ? 4 : 2;
   const cuuint64_t dims[3] = {(cuuint64_t)pi.nu, (cuuint64_t)pi.nv, (cuuint64_t)pi.nviews};
   const cuuint64_t strides[2] = {(cuuint64_t)pi.rs * es, (cuuint64_t)pi.vs * es};
-  const cuuint32_t box[3] = {
-      (cuuint32_t)(dtype == 0 ? StageGeom<float>::P : StageGeom<__half>::P), BOX_ROWS, 1};
+  int cols, rows;
+  stage_extent(dtype, half, &cols, &rows);
+  const cuuint32_t box[3] = {(cuuint32_t)cols, BOX_ROWS, 1};
   const cuuint32_t ones[3] = {1, 1, 1};
   const CUtensorMapDataType dt = dtype == 0   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                  : dtype == 1 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
@@ -833,10 +879,6 @@ cudaError_t make_stage_map(const void* proj, int dtype, const ProjInfo& pi, CUte
   return rc == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-void stage_extent(int dtype, int* cols, int* rows) {
-  *cols = dtype == 0 ? StageGeom<float>::P : StageGeom<__half>::P;
-  *rows = STAGE_ROWS;
-}
 
 template <typename T>
 constexpr int dtype_id() {
@@ -848,19 +890,29 @@ static cudaError_t forward_launch(const void* proj, const ProjInfo& pi, const Vi
                                   const VolInfo& vi, float* vol, const int* wide, cudaStream_t s) {
   const int nblocks = vi.tiles_x * vi.tiles_y * vi.tiles_z * (ZB_FWD / ZS);
   CUtensorMap map{};
-  const bool stage = stageable<T>(proj, pi) && wide != WIDE_ALL &&
-                     make_stage_map(proj, dtype_id<T>(), pi, &map) == cudaSuccess;
+  if (wide == WIDE_HALF && stageable<T>(proj, pi) &&
+      make_stage_map(proj, dtype_id<T>(), pi, &map, true) == cudaSuccess) {
+    const int smem = stage_smem_bytes<Half<T>, FWD_NS>();
+    cudaError_t e = smem_attr_once<forward_kernel<ZB_FWD, 8, FWD_NS, T, FDK, STAGE_HALF>>(smem);
+    if (e != cudaSuccess) return e;
+    forward_kernel<ZB_FWD, 8, FWD_NS, T, FDK, STAGE_HALF>
+        <<<vi.tiles_x * vi.tiles_y * vi.tiles_z * (ZB_FWD / 8), NT, smem, s>>>(
+            (const T*)proj, map, pi, geom, vi, vol, nullptr);
+    return cudaGetLastError();
+  }
+  const bool stage = stageable<T>(proj, pi) && wide != WIDE_ALL && wide != WIDE_HALF &&
+                     make_stage_map(proj, dtype_id<T>(), pi, &map, false) == cudaSuccess;
   const int* sel = stage ? wide : nullptr;
   if (stage) {
     const int smem = stage_smem_bytes<T, NS>();
-    cudaError_t e = smem_attr_once<forward_kernel<ZB_FWD, ZS, NS, T, FDK, true>>(smem);
+    cudaError_t e = smem_attr_once<forward_kernel<ZB_FWD, ZS, NS, T, FDK, STAGE_TILE>>(smem);
     if (e != cudaSuccess) return e;
-    forward_kernel<ZB_FWD, ZS, NS, T, FDK, true>
+    forward_kernel<ZB_FWD, ZS, NS, T, FDK, STAGE_TILE>
         <<<nblocks, NT, smem, s>>>((const T*)proj, map, pi, geom, vi, vol, sel);
     e = cudaGetLastError();
     if (e != cudaSuccess || !sel) return e;
   }
-  forward_kernel<ZB_FWD, ZS, FWD_NS, T, FDK, false>
+  forward_kernel<ZB_FWD, ZS, FWD_NS, T, FDK, STAGE_NONE>
       <<<nblocks, NT, 0, s>>>((const T*)proj, map, pi, geom, vi, vol, sel);
   return cudaGetLastError();
 }
@@ -889,11 +941,14 @@ static cudaError_t forward_dispatch(const void* proj, const ProjInfo& pi, const 
 template <typename T, bool FDK>
 static cudaError_t prepare_forward_t() {
   constexpr int smem = stage_smem_bytes<T, FWD_NS>();
-  cudaError_t e = smem_attr_once<forward_kernel<ZB_FWD, 16, FWD_NS, T, FDK, true>>(smem);
-  if (e == cudaSuccess) e = smem_attr_once<forward_kernel<ZB_FWD, 8, FWD_NS, T, FDK, true>>(smem);
+  cudaError_t e = smem_attr_once<forward_kernel<ZB_FWD, 16, FWD_NS, T, FDK, STAGE_TILE>>(smem);
+  if (e == cudaSuccess) e = smem_attr_once<forward_kernel<ZB_FWD, 8, FWD_NS, T, FDK, STAGE_TILE>>(smem);
   if (e == cudaSuccess)
-    e = smem_attr_once<forward_kernel<ZB_FWD, 8, FWD_NS_FEW, T, FDK, true>>(
+    e = smem_attr_once<forward_kernel<ZB_FWD, 8, FWD_NS_FEW, T, FDK, STAGE_TILE>>(
         stage_smem_bytes<T, FWD_NS_FEW>());
+  if (e == cudaSuccess)
+    e = smem_attr_once<forward_kernel<ZB_FWD, 8, FWD_NS, T, FDK, STAGE_HALF>>(
+        stage_smem_bytes<Half<T>, FWD_NS>());
   return e;
 }
 
@@ -1223,23 +1278,23 @@ struct Sums6 {
 // instruction cache.  A pair that is off the detector for the whole warp is
 // left out (its gradients are 0; a non-finite upstream value keeps its pair,
 // 0 * inf must stay NaN).  delta(k) gives the upstream gradient of voxel k.
-template <int ZB, typename T, bool FDK, bool EXACT, bool PROJ>
+template <int ZS, typename T, bool FDK, bool EXACT, bool PROJ>
 __device__ __forceinline__ Sums6 vjp_view_edge(const T* img, const float2* gimg, float* pout,
                                             long long rs, int nu, int nv, const TileView& t,
-                                            float dx, float dy, const float* delta) {
+                                            float dx, float dy, const float* delta, float zlo) {
   float S[3] = {0.0f, 0.0f, 0.0f}, Z[3] = {0.0f, 0.0f, 0.0f};
   const float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
   const float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
   const float w0 = fmaf(dy, t.rw1, fmaf(dx, t.rw0, t.W0));
 #pragma unroll 1
-  for (int k0 = 0; k0 < ZB; k0 += 2) {
+  for (int k0 = 0; k0 < ZS; k0 += 2) {
     constexpr int G = 2;
     Sample s[G];
     float d[G], gu[G], gv[G], val[G];
     bool live = false;
 #pragma unroll
     for (int q = 0; q < G; ++q) {
-      const float dz = (k0 + q) - 0.5f * (ZB - 1);
+      const float dz = (k0 + q) + zlo;
       s[q] = locate<true>(fmaf(dz, t.ru2, u0), fmaf(dz, t.rv2, v0), fmaf(dz, t.rw2, w0), t, nu, nv);
       d[q] = delta[delta_off<PROJ>(k0 + q)];
       val[q] = 0.0f;
@@ -1276,7 +1331,7 @@ __device__ __forceinline__ Sums6 vjp_view_edge(const T* img, const float2* gimg,
 #pragma unroll
     for (int q = 0; q < G; ++q) {
       if (!s[q].ok) continue;
-      const float dz = (k0 + q) - 0.5f * (ZB - 1);
+      const float dz = (k0 + q) + zlo;
       const float sd = d[q] * (FDK ? s[q].rwi * (s[q].rwi * t.wgt) : t.wgt);
       const float sr = sd * s[q].rwi;
       const float a0 = gu[q] * sr, a1 = gv[q] * sr;
@@ -1344,12 +1399,12 @@ __device__ __forceinline__ void column_range(const TileView& t, float u0, float 
 // (safe), far beyond their rounding error.  Reading the gradient images from
 // global memory here instead (eight scattered loads per sample) took 2.5 times
 // as long per (tile, view) as a central-safe one.
-template <int ZB, typename T, bool FDK, bool PROJ>
+template <int ZS, typename G, bool FDK, bool PROJ>
 __device__ __forceinline__ Sums6 vjp_view_edge2(unsigned buf, float* pout, float* qout, int nu, int nv,
                                              const TileView& t, float dx, float dy,
-                                             const float* delta, bool finite) {
+                                             const float* delta, float zlo, bool finite) {
   float S[3] = {0.0f, 0.0f, 0.0f}, Z[3] = {0.0f, 0.0f, 0.0f};
-  constexpr int P = StageGeom<T>::P;
+  constexpr int P = StageGeom<G>::P;
   const float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
   const float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
   const float w0 = fmaf(dy, t.rw1, fmaf(dx, t.rw0, t.W0));
@@ -1358,24 +1413,25 @@ __device__ __forceinline__ Sums6 vjp_view_edge2(unsigned buf, float* pout, float
   // detector pixels [xl, xr] x [yl, yr] in the anchored frame
   const float xl = -(float)t.au, xr = (float)(nu - 1 - t.au);
   const float yl = -(float)t.av, yr = (float)(nv - 1 - t.av);
-  constexpr float M = 0.01f, HZ = 0.5f * (ZB - 1);
+  constexpr float M = 0.01f;
+  const float HZ = -zlo;
   float lo, hi;
   column_range(t, u0, v0, w0, xl - 1.0f - M, xr + 1.0f + M, yl - 1.0f - M, yr + 1.0f + M, lo, hi);
-  int k0 = 0, k1 = ZB;  // slices that touch the detector in some lane
+  int k0 = 0, k1 = ZS;  // slices that touch the detector in some lane
   if (finite) {
     const bool some = lo <= hi;
     k0 = __reduce_min_sync(0xffffffffu,
-                           some ? (int)ceilf(fminf(fmaxf(lo + HZ, 0.0f), (float)ZB)) : ZB);
+                           some ? (int)ceilf(fminf(fmaxf(lo + HZ, 0.0f), (float)ZS)) : ZS);
     k1 = __reduce_max_sync(0xffffffffu,
-                           some ? (int)floorf(fminf(fmaxf(hi + HZ, -1.0f), ZB - 1.0f)) + 1 : 0);
+                           some ? (int)floorf(fminf(fmaxf(hi + HZ, -1.0f), ZS - 1.0f)) + 1 : 0);
   }
   column_range(t, u0, v0, w0, xl + 1.0f + M, xr - 1.0f - M, yl + 1.0f + M, yr - 1.0f - M, lo, hi);
   // slices [s0, s1) are central-safe in every lane
   const bool some = finite && lo <= hi;
   const int s0 = __reduce_max_sync(
-      0xffffffffu, some ? (int)ceilf(fminf(fmaxf(lo + HZ, 0.0f), (float)ZB)) : ZB);
+      0xffffffffu, some ? (int)ceilf(fminf(fmaxf(lo + HZ, 0.0f), (float)ZS)) : ZS);
   const int s1 = __reduce_min_sync(
-      0xffffffffu, some ? (int)floorf(fminf(fmaxf(hi + HZ, -1.0f), ZB - 1.0f)) + 1 : 0);
+      0xffffffffu, some ? (int)floorf(fminf(fmaxf(hi + HZ, -1.0f), ZS - 1.0f)) + 1 : 0);
 #pragma unroll 1
   for (int k = k0 & ~1; k < k1; k += 2) {
     const bool safe = k >= s0 && k + 2 <= s1;
@@ -1412,7 +1468,7 @@ __device__ __forceinline__ Sums6 vjp_view_edge2(unsigned buf, float* pout, float
     }
     const f2 tu = sub2(x, fx), tv = sub2(y, fy);
     unsigned ql, qh;
-    staged_pair<T, 1>(buf, t, IC, fx, fy, ql, qh);
+    staged_pair<G, 1>(buf, t, IC, fx, fy, ql, qh);
     const f2 a0 = lds2<-P>(ql, qh), a1 = lds2<-P + 1>(ql, qh);
     const f2 b0 = lds2<-1>(ql, qh), b1 = lds2<0>(ql, qh), b2 = lds2<1>(ql, qh),
              b3 = lds2<2>(ql, qh);
@@ -1501,13 +1557,14 @@ __device__ __forceinline__ Sums6 vjp_view_edge2(unsigned buf, float* pout, float
 // pairs of voxels (k, k+1): the steps of vjp_view in the same order on
 // f32x2 pairs, with the w-component kept negated (na2 = -a2) so that no
 // negation instruction is needed.  Even and odd voxels are summed in the two
-// halves of the pair accumulators and added at the end.
-template <int ZB, typename T, bool FDK, bool PROJ, bool LINES>
+// halves of the pair accumulators and added at the end.  ZS slices from dz = zlo on,
+// dcol their upstream gradients.
+template <int ZS, typename G, bool FDK, bool PROJ, bool LINES>
 __device__ __forceinline__ void vjp_view_central2(unsigned buf, float* pout, float* qout, int nu,
                                                   int nv, const TileView& t, float dx, float dy,
-                                                  const float* dcol, float (&S)[3],
-                                                  float (&Z)[3]) {
-  constexpr int P = StageGeom<T>::P;
+                                                  const float* dcol, float zlo,
+                                                  float (&S)[3], float (&Z)[3]) {
+  constexpr int P = StageGeom<G>::P;
   const f2 IC = pk2(t.ic, t.ic);
   const float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
   const float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
@@ -1520,11 +1577,11 @@ __device__ __forceinline__ void vjp_view_central2(unsigned buf, float* pout, flo
   // pixel index offset of the floor bits: (av - MAGIC_BITS) nu + au - MAGIC_BITS
   const unsigned pofs = (unsigned)(t.av - MAGIC_BITS) * (unsigned)nu + (unsigned)(t.au - MAGIC_BITS);
   const f2 zero = pk2(0.0f, 0.0f);
-  f2 dz = pk2(-0.5f * (ZB - 1), 1.0f - 0.5f * (ZB - 1));
-  f2 ndz = pk2(0.5f * (ZB - 1), 0.5f * (ZB - 1) - 1.0f);
+  f2 dz = pk2(zlo, zlo + 1.0f);
+  f2 ndz = pk2(-zlo, -zlo - 1.0f);
   f2 S0 = zero, S1 = zero, S2 = zero, Z0 = zero, Z1 = zero, Z2 = zero;
 #pragma unroll
-  for (int p = 0; p < ZB / 2; ++p) {
+  for (int p = 0; p < ZS / 2; ++p) {
     if (p) {
       dz = add2(dz, TWO);
       ndz = sub2(ndz, TWO);
@@ -1538,7 +1595,7 @@ __device__ __forceinline__ void vjp_view_central2(unsigned buf, float* pout, flo
     const f2 fx = sub2(rx, M2), fy = sub2(ry, M2);
     const f2 tu = sub2(x, fx), tv = sub2(y, fy);
     unsigned ql, qh;
-    staged_pair<T, 1>(buf, t, IC, fx, fy, ql, qh);
+    staged_pair<G, 1>(buf, t, IC, fx, fy, ql, qh);
     const f2 a0 = lds2<-P>(ql, qh), a1 = lds2<-P + 1>(ql, qh);
     const f2 b0 = lds2<-1>(ql, qh), b1 = lds2<0>(ql, qh), b2 = lds2<1>(ql, qh),
              b3 = lds2<2>(ql, qh);
@@ -1730,71 +1787,80 @@ __device__ __forceinline__ void proj_lines(float* __restrict__ pout, float* __re
   atomicAdd(q + nu + 1, b1);
 }
 
-// One view of one tile: the sample loop (from the staged footprint when it
-// was staged), then the warp reduce-scatter of the 12 sums into redv[warp].
-// Staged CENTRAL (central-safe) tiles run the packed motion loop and, when
-// the data VJP is fused, the line pass above; the other tiles scatter the
-// data VJP per sample.
-template <int ZB, typename T, bool FDK, bool EXACT, bool PROJ, bool STAGE>
+// One view of one tile, or of one half of it: the sample loop (from the staged
+// footprint when it was staged), added to the thread's sums.  Staged CENTRAL
+// (central-safe) tiles run the packed motion loop and, when the data VJP is fused,
+// the line pass above; the other tiles scatter the data VJP per sample.  ZS slices
+// from dz = zlo on, dcol their upstream gradients.
+template <int ZB, int ZS, typename T, bool FDK, bool EXACT, bool PROJ, int STAGE>
 __device__ __forceinline__ void vjp_tile_view(const T* img, const float2* gimg, unsigned buf,
                                               bool staged, float* pout, float* qout,
                                               const ProjInfo& pi, const TileView& t,
-                                              const TileIdx& ti,
+                                              const TileIdx& ti, float zlo,
                                               const float (&delta)[ZB], const float* dcol,
-                                              bool finite, const float* dsm, float (*redv)[12]) {
-  float S[3] = {0.0f, 0.0f, 0.0f}, Z[3] = {0.0f, 0.0f, 0.0f};
-  if (staged && !EXACT && t.csafe) {
+                                              bool finite, const float* dsm, float (&S)[3],
+                                              float (&Z)[3]) {
+  using G = Geo<T, STAGE>;
+  static_assert(ZS == ZB || (!EXACT && !PROJ), "half tiles: CENTRAL motion VJP only");
+  auto take = [&](const Sums6& q) {
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      S[r] = ZS == ZB ? q.S[r] : S[r] + q.S[r];
+      Z[r] = ZS == ZB ? q.Z[r] : Z[r] + q.Z[r];
+    }
+  };
+  if (!EXACT && staged && t.csafe) {
     // With the fused data VJP: the line pass where samples along
     // the ray-parallel axis move by at most BP_VJP_LINE_DU px per voxel
     // (there it merges most: about 4 (du + 1/16) atomics per sample), else
     // four atomics per sample from the packed loop, with fewer instructions
-    if (PROJ && BP_VJP_LINES &&
-        fminf(fabsf(t.ru0), fabsf(t.ru1)) <= BP_VJP_LINE_DU * t.W0) {
-      vjp_view_central2<ZB, T, FDK, false, PROJ>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy,
-                                                 dcol, S, Z);
-      proj_lines<ZB, FDK>(pout, qout, pi.nu, pi.nv, t, dsm);
-    } else {
-      vjp_view_central2<ZB, T, FDK, PROJ, PROJ>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy,
-                                                dcol, S, Z);
+    if constexpr (PROJ) {
+      if (BP_VJP_LINES && fminf(fabsf(t.ru0), fabsf(t.ru1)) <= BP_VJP_LINE_DU * t.W0) {
+        vjp_view_central2<ZB, G, FDK, false, PROJ>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy,
+                                                   dcol, zlo, S, Z);
+        proj_lines<ZB, FDK>(pout, qout, pi.nu, pi.nv, t, dsm);
+        return;
+      }
     }
+    vjp_view_central2<ZS, G, FDK, PROJ, PROJ>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy, dcol,
+                                              zlo, S, Z);
   } else if (!EXACT && staged) {
-    const Sums6 q =
-        vjp_view_edge2<ZB, T, FDK, PROJ>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy, dcol,
-                                         finite);
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      S[r] = q.S[r];
-      Z[r] = q.Z[r];
-    }
+    take(vjp_view_edge2<ZS, G, FDK, PROJ>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy, dcol, zlo,
+                                          finite));
   } else if (EXACT && staged) {
     // (the per-sample paths keep scalar scatters in the fused kernel: block
     // reductions of their in-range samples measured 1 % slower there,
     // 15.12 against 14.94 ms on c2, while the data VJP alone gains 10 %)
-    if (t.mode == MODE_INTERIOR || !PROJ)
-      vjp_view<ZB, T, FDK, EXACT, false, PROJ, SRC_SMEM>(img, gimg, buf, pout, nullptr, pi.rs,
-                                                         pi.nu, pi.nv, t, ti.dx, ti.dy, delta, S,
-                                                         Z);
-    else
-      vjp_view<ZB, T, FDK, EXACT, true, PROJ, SRC_SMEM>(img, gimg, buf, pout, nullptr, pi.rs, pi.nu,
-                                                        pi.nv, t, ti.dx, ti.dy, delta, S, Z);
+    if constexpr (EXACT) {
+      if (t.mode == MODE_INTERIOR || !PROJ)
+        vjp_view<ZB, T, FDK, EXACT, false, PROJ, SRC_SMEM>(img, gimg, buf, pout, nullptr, pi.rs,
+                                                           pi.nu, pi.nv, t, ti.dx, ti.dy, delta, S,
+                                                           Z);
+      else
+        vjp_view<ZB, T, FDK, EXACT, true, PROJ, SRC_SMEM>(img, gimg, buf, pout, nullptr, pi.rs,
+                                                          pi.nu, pi.nv, t, ti.dx, ti.dy, delta, S,
+                                                          Z);
+    }
   } else {
     // (where footprints can be staged, interior tiles come here only beside
     // the detector's edge: they take the checked path, one code path less)
-    if (!STAGE && t.mode == MODE_INTERIOR)
-      vjp_view<ZB, T, FDK, EXACT, false, PROJ, SRC_GLOBAL>(img, gimg, buf, pout, nullptr, pi.rs,
-                                                           pi.nu, pi.nv, t, ti.dx, ti.dy, delta, S,
-                                                           Z);
-    else {
-      const Sums6 q = vjp_view_edge<ZB, T, FDK, EXACT, PROJ>(img, gimg, pout, pi.rs, pi.nu, pi.nv, t,
-                                                             ti.dx, ti.dy, dcol);
-#pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        S[r] = q.S[r];
-        Z[r] = q.Z[r];
+    if constexpr (STAGE == STAGE_NONE) {
+      if (t.mode == MODE_INTERIOR) {
+        vjp_view<ZB, T, FDK, EXACT, false, PROJ, SRC_GLOBAL>(img, gimg, buf, pout, nullptr, pi.rs,
+                                                             pi.nu, pi.nv, t, ti.dx, ti.dy, delta,
+                                                             S, Z);
+        return;
       }
     }
+    take(vjp_view_edge<ZS, T, FDK, EXACT, PROJ>(img, gimg, pout, pi.rs, pi.nu, pi.nv, t, ti.dx,
+                                                ti.dy, dcol, zlo));
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+}
+
+// The warp's reduce-scatter of the 12 sums of one (tile, view) into redv.
+__device__ __forceinline__ void vjp_reduce(const TileIdx& ti, const float (&S)[3],
+                                           const float (&Z)[3], float (&redv)[12]) {
+  const int lane = threadIdx.x & 31;
   float v[16];
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
@@ -1806,18 +1872,20 @@ __device__ __forceinline__ void vjp_tile_view(const T* img, const float2* gimg, 
   v[12] = v[13] = v[14] = v[15] = 0.0f;
   const float tot = warp_reduce_scatter16(v, lane);
   const int slot = scatter_slot(lane);
-  if (!(lane & 1) && slot < 12) redv[warp][slot] = tot;
+  if (!(lane & 1) && slot < 12) redv[slot] = tot;
 }
 
 // Write the record of one (tile, view): fixed-order sum of the 8 warps'
-// values, plus the anchors (16 consecutive threads, slot = 0 .. PSLOTS-1).
-__device__ __forceinline__ void vjp_write_record(const TileView& t, const float (*redv)[12],
-                                                 bool bad, int slot, int j, int tile, int ntiles,
+// values (0 when the tile is off the detector: not live), plus the anchors (16
+// consecutive threads, slot = 0 .. PSLOTS-1).
+__device__ __forceinline__ void vjp_write_record(const TileView& t, bool live,
+                                                 const float (*redv)[12], bool bad, int slot, int j,
+                                                 int tile, int ntiles,
                                                  float* __restrict__ partials) {
   if (slot >= PSLOTS) return;
   float val = 0.0f;
   if (slot < 12) {
-    if (t.mode != MODE_SKIP)
+    if (live)
       for (int w = 0; w < NT / 32; ++w) val += redv[w][slot];
     if (bad) val = __int_as_float(0x7fc00000);
   } else if (slot == 12) {
@@ -1839,28 +1907,34 @@ __device__ __forceinline__ void vjp_write_record(const TileView& t, const float 
 // With the fused data VJP the tile's dL/dvol is also kept in shared memory
 // ([z][y][x], row pitch TX + 1) for the line pass.
 constexpr int DSM_BYTES = ZB_VJP * TY * (TX + 1) * 4;
-template <typename T, int NS>
+constexpr int COL_BYTES = ZB_VJP * NT * 4;  // without the line pass
+template <typename G, int NS, bool PROJ>
 __host__ __device__ constexpr int vjp_smem_bytes() {
-  return stage_smem_bytes<T, NS>() + DSM_BYTES;
+  return stage_smem_bytes<G, NS>() + (PROJ ? DSM_BYTES : COL_BYTES);
 }
 
 // One work item of the VJP: views [item / ntiles * vchunk, + vchunk) of tile
 // item % ntiles.  All threads of the CTA call it with the CTA's shared memory.
-template <int ZB, int NS, typename T, bool FDK, bool EXACT, bool PROJ, bool STAGE>
+template <int ZB, int NS, typename T, bool FDK, bool EXACT, bool PROJ, int STAGE>
 __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T* __restrict__ proj,
                                          const CUtensorMap* map, const ProjInfo& pi,
                                          const float2* __restrict__ grad,
                                          const ViewGeom* __restrict__ geom, const VolInfo& vi,
                                          float* __restrict__ partials, float* __restrict__ dproj,
                                          float* __restrict__ dblk, int vchunk, int item,
-                                         TileView (*tvs)[VB], float (*red)[NT / 32][12],
+                                         TileView (*tvs)[batch_records<STAGE>()],
+                                         float (*red)[NT / 32][12],
                                          StagePipe<NS>& pipe,
                                          unsigned char* dyn_smem) {
-  constexpr bool CONV = STAGE && conv_staging<T>();
-  constexpr int SLOT = StageGeom<T>::BYTES;
-  unsigned char* slots = dyn_smem + (CONV ? CONV_F_BYTES : 0);
+  using G = Geo<T, STAGE>;
+  constexpr bool CONV = STAGE && StageGeom<G>::CONV;
+  constexpr int SLOT = StageGeom<G>::BYTES, NB = batch_records<STAGE>();
+  // steps per view; step idx is half idx % HALVES of view vbeg + idx / HALVES
+  constexpr int HALVES = STAGE == STAGE_HALF ? 2 : 1, ZS = ZB / HALVES;
+  static_assert(NB % HALVES == 0 && ZS % 2 == 0, "whole views per batch, whole pairs per half");
+  unsigned char* slots = dyn_smem + StageGeom<G>::F_BYTES;
   float* dsm =
-      reinterpret_cast<float*>(dyn_smem + (STAGE ? stage_smem_bytes<T, NS>() : 0));
+      reinterpret_cast<float*>(dyn_smem + (STAGE ? stage_smem_bytes<G, NS>() : 0));
   constexpr int HALO = EXACT ? 0 : 1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int ntiles = vi.tiles_x * vi.tiles_y * vi.tiles_z;
@@ -1883,32 +1957,39 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
   float* dcol = dsm + delta_base<PROJ>(ti.lx, ti.ly);  // this thread's column
 #pragma unroll
   for (int k = 0; k < ZB; ++k) dcol[delta_off<PROJ>(k)] = delta[k];
-  const int nvw = vend - vbeg, nbatch = (nvw + VB - 1) / VB;
+  const int nvw = vend - vbeg, nst = nvw * HALVES, nbatch = (nst + NB - 1) / NB;
   if (!__syncthreads_or(nz)) {  // no upstream gradient in this tile: zero records
     for (int e = threadIdx.x; e < nvw * PSLOTS; e += NT)
       partials[((long long)(vbeg + e / PSLOTS) * ntiles + tile) * PSLOTS + e % PSLOTS] = 0.0f;
     return;
   }
-  setup_batch<T, STAGE>(tvs[0], geom, vbeg, min(VB, nvw), ti, pi.nu, pi.nv, HALO);
-  if (nbatch > 1)
-    setup_batch<T, STAGE>(tvs[1], geom, vbeg + VB, min(VB, nvw - VB), ti, pi.nu, pi.nv,
-                          HALO);
+  auto setup = [&](int k) {  // the records of batch k
+    setup_batch<G, STAGE != STAGE_NONE, HALVES>(tvs[k & 1], geom, vbeg + k * (NB / HALVES),
+                                                min(NB, nst - k * NB), ti, pi.nu, pi.nv, HALO);
+  };
+  // the record of step x's view (x is the view's last step)
+  auto record = [&](int x, bool bad) {
+    const TileView* q = tvs[(x / NB) & 1] + x % NB;
+    bool live = q->mode != MODE_SKIP;
+    if (HALVES == 2) live = live || q[-1].mode != MODE_SKIP;
+    vjp_write_record(*q, live, red[x % NS], bad, lane, vbeg + x / HALVES, tile, ntiles, partials);
+  };
+  setup(0);
+  if (nbatch > 1) setup(1);
   __syncthreads();
-  if (STAGE && warp < NS && warp < nvw)
-    stage_issue<T>(slots + warp * SLOT, map, tvs[0][warp], vbeg + warp, &pipe.full[warp]);
+  if (STAGE && warp < NS && warp < nst)
+    stage_issue<G>(slots + warp * SLOT, map, tvs[0][warp], vbeg + warp / HALVES, &pipe.full[warp]);
   bool bad = false;
   PipePos<NS> pos;
-  for (int v = vbeg; v < vend; ++v) {
-    const int idx = v - vbeg, k = idx / VB, b = idx - k * VB;
+  float S[3], Z[3];
+  for (int idx = 0; idx < nst; ++idx) {
+    const int v = vbeg + idx / HALVES, half = idx % HALVES, k = idx / NB, b = idx - k * NB;
     if (b == 0 && k >= 1) {
       __syncthreads();  // every warp is done with batch k-1, its records are written
-      if (CONV && warp == 0)  // (the barrier path writes them one view late)
-        vjp_write_record(tvs[(k - 1) & 1][VB - 1], red[(idx - 1) % NS], bad, lane, v - 1, tile,
-                         ntiles, partials);
+      if (CONV && warp == 0)  // (the barrier path writes them one step late)
+        record(idx - 1, bad);
       if (CONV) __syncthreads();
-      if (k + 1 < nbatch)
-        setup_batch<T, STAGE>(tvs[(k + 1) & 1], geom, vbeg + (k + 1) * VB,
-                              min(VB, nvw - (k + 1) * VB), ti, pi.nu, pi.nv, HALO);
+      if (k + 1 < nbatch) setup(k + 1);
       __syncthreads();
     }
     const TileView& t = tvs[k & 1][b];
@@ -1917,18 +1998,20 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
     if (STAGE && !bad) bad = !mbar_wait(&pipe.full[slot], pos.parity);
     pos.next();
     const int in = idx + NS;
-    const TileView& tn = tvs[(in / VB) & 1][in % VB];
+    const TileView& tn = tvs[(in / NB) & 1][in % NB];
     if constexpr (CONV) {
-      __syncthreads();  // every warp has seen this phase and is done with F and view v-1
-      if (b > 0 && warp == ((v + 4) & 7))
-        vjp_write_record(tvs[k & 1][b - 1], red[(idx - 1) % NS], bad, lane, v - 1, tile, ntiles,
-                         partials);
+      __syncthreads();  // every warp has seen this phase and is done with F and step idx-1
+      if (b > 0 && half == 0 && warp == ((idx + 4) & 7)) record(idx - 1, bad);
       if (t.staged) {
-        convert_stage<T>(reinterpret_cast<float*>(dyn_smem), reinterpret_cast<const T*>(buf), t);
-        __syncthreads();  // F holds view v; the raw slot is free
+        convert_stage<T, G>(reinterpret_cast<float*>(dyn_smem), reinterpret_cast<const T*>(buf), t);
+        __syncthreads();  // F holds this step's footprint; the raw slot is free
       }
-      if (warp == (v & 7) && in < nvw && !bad)
-        stage_issue<T>(buf, map, tn, vbeg + in, &pipe.full[slot]);
+      if (warp == (idx & 7) && in < nst && !bad)
+        stage_issue<G>(buf, map, tn, vbeg + in / HALVES, &pipe.full[slot]);
+    }
+    if (half == 0) {
+#pragma unroll
+      for (int r = 0; r < 3; ++r) S[r] = Z[r] = 0.0f;
     }
     if (t.mode != MODE_SKIP) {
       const T* img = proj + (long long)v * pi.vs;
@@ -1936,29 +2019,29 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
       float* pout = PROJ ? dproj + (long long)v * pi.nv * pi.nu : nullptr;
       float* qout =
           PROJ && dblk ? dblk + (long long)v * 4 * pi.nv * pi.nu : nullptr;
-      vjp_tile_view<ZB, T, FDK, EXACT, PROJ, STAGE>(img, gimg, smem_addr(CONV ? dyn_smem : buf),
-                                             STAGE && t.staged, pout, qout, pi, t, ti, delta, dcol, finite,
-                                                    dsm, red[slot]);
+      vjp_tile_view<ZB, ZS, T, FDK, EXACT, PROJ, STAGE>(
+          img, gimg, smem_addr(CONV ? dyn_smem : buf), STAGE && t.staged, pout, qout, pi, t, ti,
+          half * ZS - 0.5f * (ZB - 1), delta, dcol + delta_off<PROJ>(half * ZS), finite, dsm, S, Z);
+      if (HALVES == 1) vjp_reduce(ti, S, Z, red[slot][warp]);
     }
+    if (HALVES == 2 && half == 1) vjp_reduce(ti, S, Z, red[slot][warp]);
     if constexpr (!CONV) {
       if (!STAGE) __syncthreads();  // no pipe to keep the warps within two views
       if (last_warp(&pipe.done[slot])) {
-        vjp_write_record(t, red[slot], bad, lane, v, tile, ntiles, partials);
+        if (half == HALVES - 1) record(idx, bad);
         __syncwarp();
-        if (STAGE && in < nvw && !bad) stage_issue<T>(buf, map, tn, vbeg + in, &pipe.full[slot]);
+        if (STAGE && in < nst && !bad)
+          stage_issue<G>(buf, map, tn, vbeg + in / HALVES, &pipe.full[slot]);
       }
     }
   }
   if (CONV) {
     __syncthreads();
-    const int il = nvw - 1, kl = il / VB;
-    if (warp == 0)
-      vjp_write_record(tvs[kl & 1][il - kl * VB], red[il % NS], bad, lane, vend - 1, tile, ntiles,
-                       partials);
+    if (warp == 0) record(nst - 1, bad);
   }
 }
 
-template <int ZB, int NS, typename T, bool FDK, bool EXACT, bool PROJ, bool STAGE>
+template <int ZB, int NS, typename T, bool FDK, bool EXACT, bool PROJ, int STAGE>
 __global__ void __launch_bounds__(NT, NS > VJP_NS ? 2 : VJP_MINB)
     vjp_motion_kernel(const float* __restrict__ dvol, const T* __restrict__ proj,
                       const __grid_constant__ CUtensorMap map, ProjInfo pi,
@@ -1966,9 +2049,10 @@ __global__ void __launch_bounds__(NT, NS > VJP_NS ? 2 : VJP_MINB)
                       VolInfo vi, float* __restrict__ partials, float* __restrict__ dproj,
                       float* __restrict__ dblk, int vchunk, const int* __restrict__ wide) {
   // the other variant's launch takes this item
-  if (wide && (wide[blockIdx.x / (vi.tiles_x * vi.tiles_y * vi.tiles_z) * vchunk] != 0) == STAGE)
+  if (wide && (wide[blockIdx.x / (vi.tiles_x * vi.tiles_y * vi.tiles_z) * vchunk] != 0) ==
+                  (STAGE != STAGE_NONE))
     return;
-  __shared__ TileView tvs[2][VB];
+  __shared__ TileView tvs[2][batch_records<STAGE>()];
   __shared__ float red[NS][NT / 32][12];
   __shared__ StagePipe<NS> pipe;
   extern __shared__ __align__(128) unsigned char dyn_smem[];
@@ -2002,13 +2086,13 @@ static int view_chunk(const ProjInfo& pi, long long bytes_per_px, int ntiles) {
   return c < 1 ? 1 : (int)c;
 }
 
-template <int NS, typename T, bool FDK, bool EXACT, bool PROJ, bool STAGE>
+template <int NS, typename T, bool FDK, bool EXACT, bool PROJ, int STAGE>
 static cudaError_t vjp_launch(const float* dvol, const void* proj, const CUtensorMap& map,
                               const ProjInfo& pi,
                               const float2* grad, const ViewGeom* geom, const VolInfo& vi,
                               float* partials, float* dproj, float* blk, int vc,
                               unsigned nblocks, const int* wide, cudaStream_t s) {
-  const int smem = STAGE ? vjp_smem_bytes<T, NS>() : DSM_BYTES;
+  const int smem = STAGE ? vjp_smem_bytes<Geo<T, STAGE>, NS, PROJ>() : PROJ ? DSM_BYTES : COL_BYTES;
   if (STAGE) {
     const cudaError_t e =
         smem_attr_once<vjp_motion_kernel<ZB_VJP, NS, T, FDK, EXACT, PROJ, STAGE>>(smem);
@@ -2025,19 +2109,25 @@ static cudaError_t vjp_variants(const float* dvol, const void* proj, const ProjI
                                 float* partials, float* dproj, float* blk, int vc,
                                 unsigned nblocks, const int* wide, cudaStream_t s) {
   CUtensorMap map{};
-  const bool stage = stageable<T>(proj, pi) && wide != WIDE_ALL &&
-                     make_stage_map(proj, dtype_id<T>(), pi, &map) == cudaSuccess;
+  if constexpr (!EXACT && !PROJ) {
+    if (wide == WIDE_HALF && stageable<T>(proj, pi) &&
+        make_stage_map(proj, dtype_id<T>(), pi, &map, true) == cudaSuccess)
+      return vjp_launch<VJP_NS, T, FDK, EXACT, PROJ, STAGE_HALF>(
+          dvol, proj, map, pi, grad, geom, vi, partials, dproj, blk, vc, nblocks, nullptr, s);
+  }
+  const bool stage = stageable<T>(proj, pi) && wide != WIDE_ALL && wide != WIDE_HALF &&
+                     make_stage_map(proj, dtype_id<T>(), pi, &map, false) == cudaSuccess;
   const int* sel = stage ? wide : nullptr;
   if (stage) {
     const cudaError_t e =
         nblocks <= (unsigned)VJP_FEW
-            ? vjp_launch<VJP_NS_FEW, T, FDK, EXACT, PROJ, true>(
+            ? vjp_launch<VJP_NS_FEW, T, FDK, EXACT, PROJ, STAGE_TILE>(
                   dvol, proj, map, pi, grad, geom, vi, partials, dproj, blk, vc, nblocks, sel, s)
-            : vjp_launch<VJP_NS, T, FDK, EXACT, PROJ, true>(
+            : vjp_launch<VJP_NS, T, FDK, EXACT, PROJ, STAGE_TILE>(
                   dvol, proj, map, pi, grad, geom, vi, partials, dproj, blk, vc, nblocks, sel, s);
     if (e != cudaSuccess || !sel) return e;
   }
-  return vjp_launch<VJP_NS, T, FDK, EXACT, PROJ, false>(dvol, proj, map, pi, grad, geom, vi, partials,
+  return vjp_launch<VJP_NS, T, FDK, EXACT, PROJ, STAGE_NONE>(dvol, proj, map, pi, grad, geom, vi, partials,
                                                         dproj, nullptr, vc, nblocks, sel, s);
 }
 
@@ -2078,11 +2168,16 @@ bool vjp_uses_blocks(const void* proj, int dtype, const ProjInfo& pi, int exact)
 // (call before capturing a graph).
 template <typename T, bool FDK, bool EXACT>
 static cudaError_t prepare_vjp_t() {
-  cudaError_t e = smem_attr_once<vjp_motion_kernel<ZB_VJP, VJP_NS, T, FDK, EXACT, false, true>>(
-      vjp_smem_bytes<T, VJP_NS>());
+  cudaError_t e = smem_attr_once<vjp_motion_kernel<ZB_VJP, VJP_NS, T, FDK, EXACT, false,
+                                                   STAGE_TILE>>(vjp_smem_bytes<T, VJP_NS, false>());
+  if constexpr (!EXACT) {
+    if (e == cudaSuccess)
+      e = smem_attr_once<vjp_motion_kernel<ZB_VJP, VJP_NS, T, FDK, EXACT, false, STAGE_HALF>>(
+          vjp_smem_bytes<Half<T>, VJP_NS, false>());
+  }
   if (e == cudaSuccess)
-    e = smem_attr_once<vjp_motion_kernel<ZB_VJP, VJP_NS_FEW, T, FDK, EXACT, false, true>>(
-        vjp_smem_bytes<T, VJP_NS_FEW>());
+    e = smem_attr_once<vjp_motion_kernel<ZB_VJP, VJP_NS_FEW, T, FDK, EXACT, false, STAGE_TILE>>(
+        vjp_smem_bytes<T, VJP_NS_FEW, false>());
   return e;
 }
 
@@ -2251,7 +2346,7 @@ __global__ void __launch_bounds__(NT, FWD_MINB)
     if (w >= total) break;
     const int j = batch_find(t.off_fwd, n, w);
     const BatchJob& J = t.job[j];
-    forward_tile<ZB, ZB, FWD_NS, T, FDK, true>((const T*)J.proj, &J.map, J.pi, J.geom, J.vif, J.vol,
+    forward_tile<ZB, ZB, FWD_NS, T, FDK, STAGE_TILE>((const T*)J.proj, &J.map, J.pi, J.geom, J.vif, J.vol,
                                        w - t.off_fwd[j], 0, tvs, pipe, dyn_smem, pos);
   }
 }
