@@ -111,9 +111,12 @@ cudaError_t launch_compose(const double* P, const double* theta, const double* v
 const int* scan_variant(const double* P, int V, int dtype, const VolInfo& vi);
 
 
-// The tensor map of a projection stack that the staging copies read; needs
-// 16-byte aligned data and strides (and a width of whole 16-byte chunks).
-// half: the boxes of the half-tile buffers.
+// Whether the staging copies can read a stack (16-byte aligned data and strides),
+// and a copy of one with a row pitch of rs elements.
+bool stage_aligned(const void* proj, int dtype, const ProjInfo& pi);
+cudaError_t launch_align_rows(const void* proj, int dtype, const ProjInfo& pi, void* dst,
+                              long long rs, cudaStream_t s);
+// The tensor map that the staging copies read.  half: boxes of the half-tile buffers.
 cudaError_t make_stage_map(const void* proj, int dtype, const ProjInfo& pi, CUtensorMap* map,
                            bool half);
 // Pixels (columns, rows) of a staging buffer.

@@ -814,12 +814,39 @@ __global__ void __launch_bounds__(NT, NS > FWD_NS ? 2 : FWD_MINB)
 // z-extent of the forward's tiles
 constexpr int ZB_FWD = 16;
 
-// Staging needs 16-byte aligned rows and whole 16-byte chunks per row.
+// Staging needs 16-byte aligned rows; their length does not matter (TMA fills
+// with zeros beyond it).
+bool stage_aligned(const void* proj, int dtype, const ProjInfo& pi) {
+  const long long es = dtype == 0 ? 4 : 2;
+  return ((reinterpret_cast<uintptr_t>(proj) & 15) == 0) && (pi.rs * es) % 16 == 0 &&
+         (pi.vs * es) % 16 == 0;
+}
 template <typename T>
 static bool stageable(const void* proj, const ProjInfo& pi) {
-  const long long es = (long long)sizeof(T), ch = 16 / es;
-  return ((reinterpret_cast<uintptr_t>(proj) & 15) == 0) && (pi.rs * es) % 16 == 0 &&
-         (pi.vs * es) % 16 == 0 && pi.nu % ch == 0;
+  return stage_aligned(proj, sizeof(T) == 4 ? 0 : 1, pi);
+}
+
+template <typename U>
+__global__ void __launch_bounds__(256)
+    align_rows_kernel(const U* __restrict__ src, ProjInfo pi, U* __restrict__ dst, long long rs) {
+  const long long row = blockIdx.x;  // one CTA per detector row
+  const long long j = row / pi.nv, b = row - j * pi.nv;
+  const U* p = src + j * pi.vs + b * pi.rs;
+  U* q = dst + row * rs;
+  for (int a = threadIdx.x; a < pi.nu; a += blockDim.x) q[a] = p[a];
+}
+
+cudaError_t launch_align_rows(const void* proj, int dtype, const ProjInfo& pi, void* dst,
+                              long long rs, cudaStream_t s) {
+  const long long rows = (long long)pi.nviews * pi.nv;
+  if (rows <= 0 || pi.nu <= 0) return cudaSuccess;
+  if (rows > 0x7fffffffLL) return cudaErrorInvalidValue;
+  if (dtype == 0)
+    align_rows_kernel<<<(unsigned)rows, 256, 0, s>>>((const unsigned*)proj, pi, (unsigned*)dst, rs);
+  else
+    align_rows_kernel<<<(unsigned)rows, 256, 0, s>>>((const unsigned short*)proj, pi,
+                                                     (unsigned short*)dst, rs);
+  return cudaGetLastError();
 }
 
 // Opt a kernel into more than 48 KiB of dynamic shared memory, once per

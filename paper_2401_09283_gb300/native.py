@@ -221,7 +221,7 @@ def proj_desc(proj, sid=0.0, view_scale=None):
 
 
 KERNELS = ("compose", "forward", "grad_images", "vjp_motion", "reduce_chain", "vjp_proj",
-           "vjp_fused", "sharpness", "optimizer", "spline", "fdk_filter")
+           "vjp_fused", "sharpness", "optimizer", "spline", "fdk_filter", "align_rows")
 
 
 def set_timing(enable=True, device=None):
