@@ -29,7 +29,8 @@ def nvcc() -> str:
 
 
 def _flags(extra=()):
-    return ARCH + ["-O3", "-lineinfo", "-std=c++17", "--split-compile=0", "-Xcompiler", "-fPIC,-O2",
+    # a fixed number of parts: with 0 it follows the machine's cores, and code with it
+    return ARCH + ["-O3", "-lineinfo", "-std=c++17", "--split-compile=16", "-Xcompiler", "-fPIC,-O2",
                    "-I", os.path.join(ROOT, "include"), "-I", CSRC] + list(extra)
 
 

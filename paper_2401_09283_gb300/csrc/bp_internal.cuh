@@ -49,7 +49,7 @@ struct alignas(16) TileView {
   float U0, V0, W0;     // anchored homogeneous coordinates at the tile centre
   float wgt;            // wgt * scale (FP32): weight of a stored sample
   float ru0, rv0, rw0;  // d(u_rel, v_rel, w)/dx
-  float ic;             // staged index constant (staged_index), exact
+  float ic;             // anchor pixel's index in the staged footprint, exact
   float ru1, rv1, rw1;  // .../dy
   int mode;             // MODE_*
   float ru2, rv2, rw2;  // .../dz

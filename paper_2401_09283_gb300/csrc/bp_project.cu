@@ -32,10 +32,10 @@ constexpr int VJP_NS = 2;
 
 constexpr float MAGIC = 12582912.0f;   // 1.5 * 2^23
 constexpr int MAGIC_BITS = 0x4B400000;
-// 1.5 * 2^21: one unit is 4 in the bit pattern, so INDEX_MAGIC + i has the
-// bits INDEX_BITS + 4 i, a byte offset, for integers |i| < 2^19.
-constexpr float INDEX_MAGIC = 3145728.0f;
-constexpr unsigned INDEX_BITS = 0x4A400000u;
+// Staged byte addresses are computed as subnormal floats: a float whose value is
+// n 2^-149 (0 <= n < 2^23) has the bit pattern n, and sums and products of such
+// values are exact.  One pixel is four bytes, 2^-147.
+#define BP_PIXEL 5.60519385729926828e-45f
 
 // Footprint staging buffers: 64 rows at a fixed row pitch P (elements), so tap
 // offsets are immediates, filled by TMA in boxes of P x 8 pixels.  FP32
@@ -271,7 +271,7 @@ __device__ __forceinline__ TileIdx tile_index(const VolInfo& vi, int tile, int z
 // With HALVES = 2 record b is the lower (even b) or upper half, in z, of the box in
 // view j0 + b / 2 (whole views: j0 is of a lower half).
 template <typename G, bool STAGE, int HALVES = 1>
-__device__ void setup_batch(TileView* tvs, const ViewGeom* __restrict__ geom, int j0, int nb,
+__device__ __forceinline__ void setup_batch(TileView* tvs, const ViewGeom* __restrict__ geom, int j0, int nb,
                             const TileIdx& ti, int nu, int nv, int halo = 0) {
   const int b = threadIdx.x >> 3, c = threadIdx.x & 7;
   if ((int)(threadIdx.x >> 5) * 4 >= nb) return;  // a warp without a view
@@ -371,11 +371,20 @@ __device__ void setup_batch(TileView* tvs, const ViewGeom* __restrict__ geom, in
         t.smag = (65536 + cpr - 1) / cpr;
         t.soff = (int)((unsigned)(av - y0) * (unsigned)P - (unsigned)MAGIC_BITS * (unsigned)P +
                        (unsigned)(au - x0) - (unsigned)MAGIC_BITS);
-        t.ic = INDEX_MAGIC + (float)((av - y0) * P + (au - x0));
+        t.ic = (float)((av - y0) * P + (au - x0));
       }
     }
   }
   tvs[b] = t;
+}
+
+// The same as a call, for the forward: inlined three times it took registers from the
+// sample loop (3.43 against 3.46 ms on 256^3 x 248).  The VJP inlines it: as a call,
+// or left to the compiler, its loop spilled (11.1 against 9.6 ms).
+template <typename G, bool STAGE>
+__device__ __noinline__ void setup_batch_call(TileView* tvs, const ViewGeom* __restrict__ geom,
+                                              int j0, int nb, const TileIdx& ti, int nu, int nv) {
+  setup_batch<G, STAGE>(tvs, geom, j0, nb, ti, nu, nv);
 }
 
 // Detector position of one voxel in the anchored frame.
@@ -609,28 +618,46 @@ __device__ __forceinline__ unsigned staged_tap(unsigned buf, const TileView& t, 
   return buf + 4u * o;
 }
 
-// Addresses of a pair of samples' floor pixels from their floors (fx, fy), as
-// floats: fy * P + (fx + ic) is exact and its bit pattern is INDEX_BITS plus
-// the byte offset, so a pair costs two packed instructions where integer
-// arithmetic on the floor bits took four to six (7.4 integer instructions per
-// voxel-view in the forward before, 40 % of its issue slots with the moves).
+// Address of the anchor pixel in the footprint at buf (it may lie outside it, even
+// before it), as the subnormal float of staged_pair.
+__device__ __forceinline__ f2 staged_anchor(unsigned buf, const TileView& t) {
+  const float a = fmaf(t.ic, BP_PIXEL, __uint_as_float(buf));
+  return pk2(a, a);
+}
+
+// Addresses of a pair of samples' floor pixels from their floors (fx, fy) as floats
+// and the anchor's: two packed FMAs whose results' bit patterns are the addresses.
+// (Index arithmetic on the floor bits took four to six integer instructions, a sum
+// around 1.5 * 2^21 still one per sample to take the magic number out and the buffer
+// in: 256^3 x 248 forward 3.52 -> 3.43 ms, motion VJP 9.60 -> 9.39, a BF16 384^3 x 248
+// VJP 30.2 -> 29.3, with the two packed operations less in the VJP's loop.)
 template <typename G, int H>
 __device__ __forceinline__ void staged_pair(unsigned buf, const TileView& t, f2 ic, f2 fx, f2 fy,
                                             unsigned& al, unsigned& ah) {
   constexpr float P = (float)StageGeom<G>::P;
-  const f2 o = fma2(fy, pk2(P, P), add2(fx, ic));
+  const f2 o = fma2(fy, pk2(P * BP_PIXEL, P * BP_PIXEL), fma2(fx, pk2(BP_PIXEL, BP_PIXEL), ic));
   float lo, hi;
   up2(o, lo, hi);
+  al = __float_as_uint(lo);
+  ah = __float_as_uint(hi);
 #ifdef BP_BOUNDS_CHECK
   float xl, xh, yl, yh;
   up2(fx, xl, xh);
   up2(fy, yl, yh);
-  const float safe = INDEX_MAGIC + (float)(H * StageGeom<G>::P + H);
-  if (bc_staged<G, H>(t, (int)xl, (int)yl)) lo = safe;
-  if (bc_staged<G, H>(t, (int)xh, (int)yh)) hi = safe;
+  const unsigned safe = buf + 4u * (unsigned)(H * StageGeom<G>::P + H);
+  if (bc_staged<G, H>(t, (int)xl, (int)yl)) al = safe;
+  if (bc_staged<G, H>(t, (int)xh, (int)yh)) ah = safe;
+  // the address must also be the one that integer arithmetic gives
+  const unsigned rl = buf + 4u * (unsigned)(((int)yl + t.av - t.sv0) * StageGeom<G>::P + (int)xl +
+                                            t.au - t.sx0);
+  const unsigned rh = buf + 4u * (unsigned)(((int)yh + t.av - t.sv0) * StageGeom<G>::P + (int)xh +
+                                            t.au - t.sx0);
+  if (al != safe && al != rl) { bc_fail(BC_STAGED_TAP, (int)al, (int)rl); al = safe; }
+  if (ah != safe && ah != rh) { bc_fail(BC_STAGED_TAP, (int)ah, (int)rh); ah = safe; }
+#else
+  (void)buf;
+  (void)t;
 #endif
-  al = __float_as_uint(lo) + (buf - INDEX_BITS);
-  ah = __float_as_uint(hi) + (buf - INDEX_BITS);
 }
 
 // ------------------------------------------------------------------ forward
@@ -671,7 +698,7 @@ __device__ __forceinline__ void forward_view_staged2(unsigned buf, const TileVie
   const f2 U0 = pk2(u0, u0), V0 = pk2(v0, v0), W0 = pk2(w0, w0);
   const f2 RU = pk2(t.ru2, t.ru2), RV = pk2(t.rv2, t.rv2), RW = pk2(t.rw2, t.rw2);
   const f2 M2 = pk2(MAGIC, MAGIC), TWO = pk2(2.0f, 2.0f), WG = pk2(t.wgt, t.wgt);
-  const f2 IC = pk2(t.ic, t.ic);
+  const f2 IC = staged_anchor(buf, t);
   f2 dz = pk2(zlo, zlo + 1.0f);  // exact: halves of small integers
 #pragma unroll
   for (int p = 0; p < ZS / 2; ++p) {
@@ -726,9 +753,9 @@ __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const C
   bool bad = false;
   const int V = pi.nviews;
   const int nbatch = (V + NB - 1) / NB;
-  setup_batch<G, STAGE != STAGE_NONE>(tvs[0], geom, 0, min(NB, V), ti, pi.nu, pi.nv);
+  setup_batch_call<G, STAGE != STAGE_NONE>(tvs[0], geom, 0, min(NB, V), ti, pi.nu, pi.nv);
   if (nbatch > 1)
-    setup_batch<G, STAGE != STAGE_NONE>(tvs[1], geom, NB, min(NB, V - NB), ti, pi.nu, pi.nv);
+    setup_batch_call<G, STAGE != STAGE_NONE>(tvs[1], geom, NB, min(NB, V - NB), ti, pi.nu, pi.nv);
   __syncthreads();
   if (STAGE && warp < NS && warp < V) {
     const unsigned s = (pos.slot + warp) % NS;
@@ -738,7 +765,7 @@ __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const C
     const int k = v / NB, b = v - k * NB;
     if (b == 0 && k >= 1 && k + 1 < nbatch) {
       __syncthreads();  // every warp is done with batch k-1
-      setup_batch<G, STAGE != STAGE_NONE>(tvs[(k + 1) & 1], geom, (k + 1) * NB, min(NB, V - (k + 1) * NB), ti,
+      setup_batch_call<G, STAGE != STAGE_NONE>(tvs[(k + 1) & 1], geom, (k + 1) * NB, min(NB, V - (k + 1) * NB), ti,
                             pi.nu, pi.nv);
       __syncthreads();
     }
@@ -1435,7 +1462,7 @@ __device__ __forceinline__ Sums6 vjp_view_edge2(unsigned buf, float* pout, float
   const float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
   const float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
   const float w0 = fmaf(dy, t.rw1, fmaf(dx, t.rw0, t.W0));
-  const f2 M2 = pk2(MAGIC, MAGIC), HALF = pk2(0.5f, 0.5f), IC = pk2(t.ic, t.ic);
+  const f2 M2 = pk2(MAGIC, MAGIC), HALF = pk2(0.5f, 0.5f), IC = staged_anchor(buf, t);
   const f2 WG = pk2(t.wgt, t.wgt), WGD = pk2(t.wgtd, t.wgtd);
   // detector pixels [xl, xr] x [yl, yr] in the anchored frame
   const float xl = -(float)t.au, xr = (float)(nu - 1 - t.au);
@@ -1592,27 +1619,23 @@ __device__ __forceinline__ void vjp_view_central2(unsigned buf, float* pout, flo
                                                   const float* dcol, float zlo,
                                                   float (&S)[3], float (&Z)[3]) {
   constexpr int P = StageGeom<G>::P;
-  const f2 IC = pk2(t.ic, t.ic);
+  const f2 IC = staged_anchor(buf, t);
   const float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
   const float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
   const float w0 = fmaf(dy, t.rw1, fmaf(dx, t.rw0, t.W0));
   const f2 U0 = pk2(u0, u0), V0 = pk2(v0, v0), W0 = pk2(w0, w0);
   const f2 RU = pk2(t.ru2, t.ru2), RV = pk2(t.rv2, t.rv2), RW = pk2(t.rw2, t.rw2);
-  const f2 M2 = pk2(MAGIC, MAGIC), TWO = pk2(2.0f, 2.0f), HALF = pk2(0.5f, 0.5f);
-  const f2 WG = pk2(t.wgt, t.wgt);
+  const f2 M2 = pk2(MAGIC, MAGIC), TWO = pk2(2.0f, 2.0f), FOUR = pk2(4.0f, 4.0f);
+  const f2 WG = pk2(0.5f * t.wgt, 0.5f * t.wgt);  // half: the differences are twice the gradients
   const f2 WGD = pk2(t.wgtd, t.wgtd);
   // pixel index offset of the floor bits: (av - MAGIC_BITS) nu + au - MAGIC_BITS
   const unsigned pofs = (unsigned)(t.av - MAGIC_BITS) * (unsigned)nu + (unsigned)(t.au - MAGIC_BITS);
   const f2 zero = pk2(0.0f, 0.0f);
   f2 dz = pk2(zlo, zlo + 1.0f);
-  f2 ndz = pk2(-zlo, -zlo - 1.0f);
   f2 S0 = zero, S1 = zero, S2 = zero, Z0 = zero, Z1 = zero, Z2 = zero;
 #pragma unroll
   for (int p = 0; p < ZS / 2; ++p) {
-    if (p) {
-      dz = add2(dz, TWO);
-      ndz = sub2(ndz, TWO);
-    }
+    if (p) dz = add2(dz, TWO);
     const f2 u = fma2(dz, RU, U0), v = fma2(dz, RV, V0), w = fma2(dz, RW, W0);
     float wl, wh;
     up2(w, wl, wh);
@@ -1637,17 +1660,16 @@ __device__ __forceinline__ void vjp_view_central2(unsigned buf, float* pout, flo
     const f2 D = LINES ? pk2(dcol[delta_off<true>(2 * p)], dcol[delta_off<true>(2 * p + 1)])
                        : *reinterpret_cast<const f2*>(dcol + delta_off<false>(2 * p));
     const f2 sd = mul2(D, FDK ? mul2(r, mul2(r, WG)) : WG);
-    const f2 sr = mul2(sd, r);
-    const f2 sg = mul2(sr, HALF);
+    const f2 sg = mul2(sd, r);
     const f2 A0 = mul2(gu, sg), A1 = mul2(gv, sg);
     f2 NA2 = fma2(A0, x, mul2(A1, y));
-    if (FDK) NA2 = fma2(add2(sr, sr), bilerp2(tu, tv, b1, b2, c1, c2), NA2);
+    if (FDK) NA2 = fma2(mul2(sg, FOUR), bilerp2(tu, tv, b1, b2, c1, c2), NA2);
     S0 = add2(S0, A0);
     S1 = add2(S1, A1);
     S2 = sub2(S2, NA2);
     Z0 = fma2(A0, dz, Z0);
     Z1 = fma2(A1, dz, Z1);
-    Z2 = fma2(NA2, ndz, Z2);
+    Z2 = fma2(NA2, dz, Z2);  // minus the sum
     if (PROJ) {
       // fused data VJP, per voxel: the same sample's bilinear weights (the
       // scalar scatter's formulas, packed), dequantised view weight, four
@@ -1692,7 +1714,7 @@ __device__ __forceinline__ void vjp_view_central2(unsigned buf, float* pout, flo
   up2(S2, lo, hi); S[2] += lo + hi;
   up2(Z0, lo, hi); Z[0] += lo + hi;
   up2(Z1, lo, hi); Z[1] += lo + hi;
-  up2(Z2, lo, hi); Z[2] += lo + hi;
+  up2(Z2, lo, hi); Z[2] -= lo + hi;
 }
 
 // Fused data VJP by lines (below) or per sample (the scalar loop).
