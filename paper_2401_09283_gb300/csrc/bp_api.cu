@@ -114,14 +114,9 @@ int prepare_views(bp_ctx* ctx, const bp_proj_desc* pd, const double* P, const do
   return BP_OK;
 }
 
-// Grow a workspace that a call can do without: false where that fails, or where it
-// would break a stream capture.
-bool ensure_optional(Buf& b, size_t bytes, cudaStream_t s) {
-  if (b.n >= bytes) return true;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone &&
-      ensure(b, bytes) == cudaSuccess)
-    return true;
+// Grow a workspace that a call can do without: false where that fails.
+bool ensure_optional(Buf& b, size_t bytes) {
+  if (ensure(b, bytes) == cudaSuccess) return true;
   cudaGetLastError();
   return false;
 }
@@ -131,7 +126,9 @@ bool ensure_optional(Buf& b, size_t bytes, cudaStream_t s) {
 // stack is copied once per call to a workspace with aligned rows, where the work is
 // worth the copy: as many voxel-views as pixels (the copy moves 4 to 8 bytes per
 // pixel, 1-2 ps; staging saves more than 1 ps per voxel-view) and 2^22 of them (~4 us,
-// the launch).  Without memory for it the call runs as before.  Measured: BF16 rows of
+// the launch).  Without memory for it the call runs as before; so does one that is
+// being captured (its graph would hold a workspace that a later, larger call
+// replaces).  Measured: BF16 rows of
 // 401 pixels, 143 x 187 x 161 voxels x 111 views, forward and both gradients 4.35 ->
 // 3.18 ms.
 int align_rows(bp_ctx* ctx, const bp_proj_desc* pd, long long nvox, cudaStream_t s,
@@ -140,8 +137,13 @@ int align_rows(bp_ctx* ctx, const bp_proj_desc* pd, long long nvox, cudaStream_t
   const long long rows = (long long)pi->nviews * pi->nv, work = nvox * pi->nviews;
   if (bpk::stage_aligned(*dproj, pd->dtype, *pi) || work < (1LL << 22) || work < rows * pi->nu)
     return BP_OK;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return BP_OK;
+  }
   const long long es = pd->dtype == BP_F32 ? 4 : 2, rs = (pi->nu * es + 15) / 16 * 16 / es;
-  if (!ensure_optional(ctx->aligned, (size_t)(rows * rs * es), s)) return BP_OK;
+  if (!ensure_optional(ctx->aligned, (size_t)(rows * rs * es))) return BP_OK;
   CK(TL(K_ALIGN, 1, bpk::launch_align_rows(*dproj, pd->dtype, *pi, ctx->aligned.p, rs, s)),
      "align rows");
   *dproj = ctx->aligned.p;
@@ -401,7 +403,7 @@ int bp_vjp(bp_ctx* ctx, const float* dL_dvol, const void* proj, const bp_proj_de
       bool blocks = fuse && bpk::vjp_uses_blocks(dproj, pdesc->dtype, pi,
                                                  deriv == BP_DERIV_BILINEAR_EXACT);
       if (blocks && copied)  // (unaligned stacks never needed its memory)
-        blocks = ensure_optional(ctx->blkimg, sizeof(float) * (size_t)bpk::block_image_floats(pi), s);
+        blocks = ensure_optional(ctx->blkimg, sizeof(float) * (size_t)bpk::block_image_floats(pi));
       else if (blocks)
         CK(ensure(ctx->blkimg, sizeof(float) * (size_t)bpk::block_image_floats(pi)),
            "alloc block image");

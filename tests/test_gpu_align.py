@@ -76,9 +76,9 @@ def test_unaligned_rows_match_oracle(dtype, nu, deriv, shape):
         assert rel_l2(gd.cpu().numpy(), oD) <= 1e-5
 
 
-def test_capture_without_a_warm_workspace_runs_unstaged():
-    # a context's first call on unaligned rows, of this size or larger, inside a capture:
-    # no allocation, the result of the plain call
+def test_captured_call_holds_no_copy():
+    # a captured call on unaligned rows neither allocates nor keeps the workspace: its
+    # graph gives the plain call's result, also after a larger call has replaced that
     views, nu, nv, shape = 64, 71, 50, (40, 41, 42)
     cfg, P, th, proj, _, origin = random_case(5, shape, views, nu, nv, 1.2, 1.0)
     p, Pd, thd = (torch.as_tensor(x, device=DEV) for x in (proj, P, th))
@@ -90,5 +90,8 @@ def test_capture_without_a_warm_workspace_runs_unstaged():
     g = torch.cuda.CUDAGraph()
     with torch.cuda.graph(g):
         vol = bp.bp_forward(p, Pd, thd, **args)
+    big = torch.zeros(views, nv * 4, nu, device=DEV)
+    bp.bp_forward(big, Pd, thd, **args)
+    del big
     g.replay()
     assert rel_l2(vol.cpu().numpy(), bp.bp_forward(p, Pd, thd, **args).cpu().numpy()) <= 1e-5
