@@ -123,8 +123,9 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
 // unrolling).  One output of 4 rows per thread loaded 20 bytes for four FMAs.
 // The cosine weight comes from a table as a pair of FP32 values, not from an FP64
 // square root and division per pixel and view (2 FP64 lanes per clock and SM).
-// 248 x 480 rows of 616: 3.76 -> 1.93 ms, the FMAs alone take 1.2 ms.
-__global__ void __launch_bounds__(MAX_THREADS)
+// 248 x 480 rows of 616: 3.76 -> 1.90 ms, the FMAs alone take 1.2 ms (1.93 at 78
+// registers and two CTAs per SM; 2.14 with 8 rows per thread and 126 registers).
+__global__ void __launch_bounds__(MAX_THREADS, 2)
     fdk_conv_kernel(const float* __restrict__ raw, int nu, int nv, int ext, int G, float tau,
                     const float* __restrict__ tab, float* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
