@@ -82,6 +82,7 @@ struct VolInfo {
 struct ProjInfo {
   int nu, nv, nviews;
   long long rs, vs;   // element strides
+  int seq;            // motion VJP: sums sample by sample, as from global memory
 };
 
 // Views whose tiles project larger than the staging buffer everywhere in the
@@ -89,7 +90,7 @@ struct ProjInfo {
 // faster from a kernel variant that leaves the L1 cache its full size, unless
 // most half tiles fit the wider half-tile buffers.  `wide` of launch_forward and
 // launch_vjp_motion: NULL, take the staged variant; WIDE_ALL, take the one that
-// reads global memory; WIDE_HALF, stage half tiles (the same job: 59.9 -> 50.6 ms);
+// reads global memory; WIDE_HALF, stage half tiles (the same job: 59.9 -> 47.0 ms);
 // else one flag per view on the device (launch_compose, fit): the first two are launched and each item runs in
 // the one that suits its first view.
 struct FitInfo {

@@ -14,9 +14,10 @@
 // 1.5*2^23, bilinear interpolation with FP32 lerps (hardware texture filtering is
 // not used: its weights are 8-bit fixed point).
 //
-// What bounds them (ncu, c2): the motion VJP's central-safe loop, the L1 data
-// pipe (12 taps per voxel-view at 1.4 wavefronts each, 80 % of its peak); the
-// forward, that pipe (63 %), the FMA pipe (54 %) and issue (58 %) together.
+// What bounds them (ncu, 256^3 x 128 views): no unit alone.  The L1 data pipe is at
+// 75 % (forward) and 74 % (motion VJP: 12 taps per voxel-view at 1.4 wavefronts),
+// issue at 62 and 59 % (21 and 51 instructions per voxel-view), the FMA pipe at 57 and
+// 50 %, with the 32 and 24 warps per SM that their registers allow.
 #include "bp_sample.cuh"
 
 namespace bpk {
@@ -337,8 +338,9 @@ struct Sums6 {
 template <int ZS, typename T, bool FDK, bool EXACT, bool PROJ>
 __device__ __forceinline__ Sums6 vjp_view_edge(const T* img, const float2* gimg, float* pout,
                                             long long rs, int nu, int nv, const TileView& t,
-                                            float dx, float dy, const float* delta, float zlo) {
-  float S[3] = {0.0f, 0.0f, 0.0f}, Z[3] = {0.0f, 0.0f, 0.0f};
+                                            float dx, float dy, const float* delta, float zlo,
+                                            const Sums6& from) {
+  float S[3] = {from.S[0], from.S[1], from.S[2]}, Z[3] = {from.Z[0], from.Z[1], from.Z[2]};
   const float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
   const float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
   const float w0 = fmaf(dy, t.rw1, fmaf(dx, t.rw0, t.W0));
@@ -458,8 +460,9 @@ __device__ __forceinline__ void column_range(const TileView& t, float u0, float 
 template <int ZS, typename G, bool FDK, bool PROJ>
 __device__ __forceinline__ Sums6 vjp_view_edge2(unsigned buf, float* pout, float* qout, int nu, int nv,
                                              const TileView& t, float dx, float dy,
-                                             const float* delta, float zlo, bool finite) {
-  float S[3] = {0.0f, 0.0f, 0.0f}, Z[3] = {0.0f, 0.0f, 0.0f};
+                                             const float* delta, float zlo, bool finite,
+                                             const Sums6& from) {
+  float S[3] = {from.S[0], from.S[1], from.S[2]}, Z[3] = {from.Z[0], from.Z[1], from.Z[2]};
   constexpr int P = StageGeom<G>::P;
   const float u0 = fmaf(dy, t.ru1, fmaf(dx, t.ru0, t.U0));
   const float v0 = fmaf(dy, t.rv1, fmaf(dx, t.rv0, t.V0));
@@ -615,7 +618,8 @@ __device__ __forceinline__ Sums6 vjp_view_edge2(unsigned buf, float* pout, float
 // negation instruction is needed.  Even and odd voxels are summed in the two
 // halves of the pair accumulators and added at the end.  ZS slices from dz = zlo on,
 // dcol their upstream gradients.
-template <int ZS, typename G, bool FDK, bool PROJ, bool LINES>
+// With SEQ the sums are taken sample by sample instead, on top of S and Z.
+template <int ZS, typename G, bool FDK, bool PROJ, bool LINES, bool SEQ = false>
 __device__ __forceinline__ void vjp_view_central2(unsigned buf, float* pout, float* qout, int nu,
                                                   int nv, const TileView& t, float dx, float dy,
                                                   const float* dcol, float zlo,
@@ -666,6 +670,23 @@ __device__ __forceinline__ void vjp_view_central2(unsigned buf, float* pout, flo
     const f2 A0 = mul2(gu, sg), A1 = mul2(gv, sg);
     f2 NA2 = fma2(A0, x, mul2(A1, y));
     if (FDK) NA2 = fma2(mul2(sg, FOUR), bilerp2(tu, tv, b1, b2, c1, c2), NA2);
+    if constexpr (SEQ) {
+      float a0[2], a1[2], n2[2], z[2];
+      up2(A0, a0[0], a0[1]);
+      up2(A1, a1[0], a1[1]);
+      up2(NA2, n2[0], n2[1]);
+      up2(dz, z[0], z[1]);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        S[0] += a0[q];
+        S[1] += a1[q];
+        S[2] -= n2[q];
+        Z[0] = fmaf(a0[q], z[q], Z[0]);
+        Z[1] = fmaf(a1[q], z[q], Z[1]);
+        Z[2] = fmaf(-n2[q], z[q], Z[2]);
+      }
+      continue;
+    }
     S0 = add2(S0, A0);
     S1 = add2(S1, A1);
     S2 = sub2(S2, NA2);
@@ -710,6 +731,7 @@ __device__ __forceinline__ void vjp_view_central2(unsigned buf, float* pout, flo
       }
     }
   }
+  if (SEQ) return;
   float lo, hi;
   up2(S0, lo, hi); S[0] += lo + hi;
   up2(S1, lo, hi); S[1] += lo + hi;
@@ -853,11 +875,14 @@ __device__ __forceinline__ void vjp_tile_view(const T* img, const float2* gimg, 
                                               float (&Z)[3]) {
   using G = Geo<T, STAGE>;
   static_assert(ZS == ZB || (!EXACT && !PROJ), "half tiles: CENTRAL motion VJP only");
+  // the lower half's sums go on in the upper half, in the order of the slices
+  const Sums6 from = ZS == ZB ? Sums6{{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}}
+                              : Sums6{{S[0], S[1], S[2]}, {Z[0], Z[1], Z[2]}};
   auto take = [&](const Sums6& q) {
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
-      S[r] = ZS == ZB ? q.S[r] : S[r] + q.S[r];
-      Z[r] = ZS == ZB ? q.Z[r] : Z[r] + q.Z[r];
+      S[r] = q.S[r];
+      Z[r] = q.Z[r];
     }
   };
   if (!EXACT && staged && t.csafe) {
@@ -873,11 +898,11 @@ __device__ __forceinline__ void vjp_tile_view(const T* img, const float2* gimg, 
         return;
       }
     }
-    vjp_view_central2<ZS, G, FDK, PROJ, PROJ>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy, dcol,
+    vjp_view_central2<ZS, G, FDK, PROJ, PROJ, ZS != ZB>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy, dcol,
                                               zlo, S, Z);
   } else if (!EXACT && staged) {
     take(vjp_view_edge2<ZS, G, FDK, PROJ>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy, dcol, zlo,
-                                          finite));
+                                          finite, from));
   } else if (EXACT && staged) {
     // (the per-sample paths keep scalar scatters in the fused kernel: block
     // reductions of their in-range samples measured 1 % slower there,
@@ -904,7 +929,7 @@ __device__ __forceinline__ void vjp_tile_view(const T* img, const float2* gimg, 
       }
     }
     take(vjp_view_edge<ZS, T, FDK, EXACT, PROJ>(img, gimg, pout, pi.rs, pi.nu, pi.nv, t, ti.dx,
-                                                ti.dy, dcol, zlo));
+                                                ti.dy, dcol, zlo, from));
   }
 }
 
@@ -1016,7 +1041,8 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
   }
   auto setup = [&](int k) {  // the records of batch k
     setup_batch<G, STAGE != STAGE_NONE, HALVES>(tvs[k & 1], geom, vbeg + k * (NB / HALVES),
-                                                min(NB, nst - k * NB), ti, pi.nu, pi.nv, HALO);
+                                                min(NB, nst - k * NB), ti, pi.nu, pi.nv, HALO,
+                                                pi.seq != 0);
   };
   // the record of step x's view (x is the view's last step)
   auto record = [&](int x, bool bad) {

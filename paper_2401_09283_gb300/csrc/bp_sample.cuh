@@ -14,7 +14,9 @@ namespace bpk {
 constexpr int FWD_MINB = 4;
 constexpr int VJP_MINB = 3;
 // Staging slots (three at three CTAs per SM in the forward, three or four at
-// two in the VJP: slower, 3.69 against 3.58 and 10.9 against 9.9 ms on c2).
+// two in the VJP: slower, 3.69 against 3.58 and 10.9 against 9.9 ms on c2; three at
+// the same occupancy, in buffers of 76 x 56 pixels and batches of 16 views: 3.49
+// against 3.45 and 9.62 against 9.46).
 constexpr int FWD_NS = 2;
 constexpr int VJP_NS = 2;
 
@@ -256,11 +258,12 @@ __device__ __forceinline__ TileIdx tile_index(const VolInfo& vi, int tile, int z
 // detector pixels that any tap (plus `halo` pixels each side) can read,
 // NOT clipped to the detector (off-detector pixels are staged as zeros, so
 // the sample loop needs neither checks nor clamps), if it fits the buffer.
+// seq: no tile counts as central-safe (its sums are then taken sample by sample).
 // With HALVES = 2 record b is the lower (even b) or upper half, in z, of the box in
 // view j0 + b / 2 (whole views: j0 is of a lower half).
 template <typename G, bool STAGE, int HALVES = 1>
 __device__ __forceinline__ void setup_batch(TileView* tvs, const ViewGeom* __restrict__ geom, int j0, int nb,
-                            const TileIdx& ti, int nu, int nv, int halo = 0) {
+                            const TileIdx& ti, int nu, int nv, int halo = 0, bool seq = false) {
   const int b = threadIdx.x >> 3, c = threadIdx.x & 7;
   if ((int)(threadIdx.x >> 5) * 4 >= nb) return;  // a warp without a view
   const ViewGeom& g = geom[j0 + min(b, nb - 1) / HALVES];
@@ -339,7 +342,7 @@ __device__ __forceinline__ void setup_batch(TileView* tvs, const ViewGeom* __res
                  : MODE_EDGE;
     // central differences at the tap pixels use interior neighbours only:
     // taps in [1, n-2], i.e. floor in [1, n-3]
-    t.csafe = xmin >= ulo + 1.0f + m && xmax <= uhi - 1.0f - m &&
+    t.csafe = !seq && xmin >= ulo + 1.0f + m && xmax <= uhi - 1.0f - m &&
               ymin >= vlo + 1.0f + m && ymax <= vhi - 1.0f - m;
     if (STAGE) {
       constexpr int CH = StageGeom<G>::CH, P = StageGeom<G>::P;
