@@ -69,8 +69,6 @@ struct alignas(16) TileView {
                         // (one more pixel each side) lie inside the detector
 };
 
-enum { MODE_SKIP = 0, MODE_INTERIOR = 1, MODE_EDGE = 2 };
-
 struct VolInfo {
   int nx, ny, nz;
   int tiles_x, tiles_y, tiles_z;

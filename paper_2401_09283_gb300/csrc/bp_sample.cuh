@@ -6,6 +6,7 @@
 #pragma once
 
 #include "bp_internal.cuh"
+#include "bp_plan.h"
 #include "bp_tma.cuh"
 
 namespace bpk {
@@ -253,7 +254,8 @@ __device__ __forceinline__ TileIdx tile_index(const VolInfo& vi, int tile, int z
 // extremes are at the corners, and the box is
 //   SKIP      every sample is 0 (projection at or beyond -1 / n),
 //   INTERIOR  every tap (floor and floor+1) lies on the detector,
-//   EDGE      otherwise (clamped coordinates, checked taps).
+//   EDGE      otherwise (clamped coordinates, checked taps)
+// (plan_box, which also guards against boxes that come near the source plane).
 // With STAGE, bounded boxes also get a staging plan: the rectangle of
 // detector pixels that any tap (plus `halo` pixels each side) can read,
 // NOT clipped to the detector (off-detector pixels are staged as zeros, so
@@ -261,7 +263,9 @@ __device__ __forceinline__ TileIdx tile_index(const VolInfo& vi, int tile, int z
 // seq: no tile counts as central-safe (its sums are then taken sample by sample).
 // With HALVES = 2 record b is the lower (even b) or upper half, in z, of the box in
 // view j0 + b / 2 (whole views: j0 is of a lower half).
-template <typename G, bool STAGE, int HALVES = 1>
+// EARLY: what the corners give goes to the record before the plan, which then needs
+// fewer registers (the forward's call; inlined in the VJP it spilled more).
+template <typename G, bool STAGE, int HALVES = 1, bool EARLY = false>
 __device__ __forceinline__ void setup_batch(TileView* tvs, const ViewGeom* __restrict__ geom, int j0, int nb,
                             const TileIdx& ti, int nu, int nv, int halo = 0, bool seq = false) {
   const int b = threadIdx.x >> 3, c = threadIdx.x & 7;
@@ -297,10 +301,6 @@ __device__ __forceinline__ void setup_batch(TileView* tvs, const ViewGeom* __res
   t.rv0 = fmaf(-fav, t.rw0, R1.x);
   t.rv1 = fmaf(-fav, t.rw1, R1.y);
   t.rv2 = fmaf(-fav, t.rw2, R1.z);
-  t.au = au;
-  t.av = av;
-  t.wgt = R0.w;
-  t.wgtd = R1.w;
   // this lane's corner
   const float d0 = (c & 1) ? ti.hx : -ti.hx;
   const float d1 = (c & 2) ? ti.hy : -ti.hy;
@@ -308,9 +308,17 @@ __device__ __forceinline__ void setup_batch(TileView* tvs, const ViewGeom* __res
   const float w = fmaf(t.rw2, d2, fmaf(t.rw1, d1, fmaf(t.rw0, d0, t.W0)));
   const float u = fmaf(t.ru2, d2, fmaf(t.ru1, d1, fmaf(t.ru0, d0, t.U0)));
   const float v = fmaf(t.rv2, d2, fmaf(t.rv1, d1, fmaf(t.rv0, d0, t.V0)));
-  const bool pos = w > 0.0f;
+  t.au = au;
+  t.av = av;
+  t.wgt = R0.w;
+  t.wgtd = R1.w;
+  t.ic = 0.0f;
+  t.mode = t.csafe = t.staged = t.sx0 = t.sv0 = t.sh = t.scpr = t.srpp = t.smag = t.soff = 0;
+  const bool mine = c == 0 && b < nb;
+  if (EARLY && mine) tvs[b] = t;
+  const bool pos = in_front(w);
   int npos = pos ? 1 : 0;
-  float xmin = INFINITY, xmax = -INFINITY, ymin = INFINITY, ymax = -INFINITY;
+  float xmin = INFINITY, xmax = -INFINITY, ymin = INFINITY, ymax = -INFINITY, wmin = w;
   if (pos) {
     xmin = xmax = u / w;
     ymin = ymax = v / w;
@@ -318,55 +326,35 @@ __device__ __forceinline__ void setup_batch(TileView* tvs, const ViewGeom* __res
 #pragma unroll
   for (int o = 1; o < 8; o <<= 1) {
     npos += __shfl_xor_sync(0xffffffffu, npos, o);
+    wmin = fminf(wmin, __shfl_xor_sync(0xffffffffu, wmin, o));
     xmin = fminf(xmin, __shfl_xor_sync(0xffffffffu, xmin, o));
     xmax = fmaxf(xmax, __shfl_xor_sync(0xffffffffu, xmax, o));
     ymin = fminf(ymin, __shfl_xor_sync(0xffffffffu, ymin, o));
     ymax = fmaxf(ymax, __shfl_xor_sync(0xffffffffu, ymax, o));
   }
-  if (c != 0 || b >= nb) return;
-  const float m = 0.01f;
-  // detector [0, n-1] in the anchored frame
-  const float ulo = -fau, uhi = (float)(nu - 1) - fau, vlo = -fav, vhi = (float)(nv - 1) - fav;
-  t.ic = 0.0f;
-  t.sx0 = t.sv0 = t.sh = t.scpr = t.srpp = t.smag = t.soff = t.staged = t.csafe = 0;
-  if (npos == 0) {
-    t.mode = MODE_SKIP;
-  } else if (npos < 8) {
-    t.mode = MODE_EDGE;
-  } else if (xmax <= ulo - 1.0f - m || xmin >= uhi + 1.0f + m || ymax <= vlo - 1.0f - m ||
-             ymin >= vhi + 1.0f + m) {
-    t.mode = MODE_SKIP;
-  } else {
-    t.mode = (xmin >= ulo + m && xmax <= uhi - m && ymin >= vlo + m && ymax <= vhi - m)
-                 ? MODE_INTERIOR
-                 : MODE_EDGE;
-    // central differences at the tap pixels use interior neighbours only:
-    // taps in [1, n-2], i.e. floor in [1, n-3]
-    t.csafe = !seq && xmin >= ulo + 1.0f + m && xmax <= uhi - 1.0f - m &&
-              ymin >= vlo + 1.0f + m && ymax <= vhi - 1.0f - m;
-    if (STAGE) {
-      constexpr int CH = StageGeom<G>::CH, P = StageGeom<G>::P;
-      const int fl_u0 = (int)floorf(xmin - m) + au, fl_u1 = (int)floorf(xmax + m) + 1 + au;
-      const int fl_v0 = (int)floorf(ymin - m) + av, fl_v1 = (int)floorf(ymax + m) + 1 + av;
-      const int x0 = (fl_u0 - halo) & ~(CH - 1);  // floor to a 16-byte boundary
-      const int y0 = fl_v0 - halo;
-      const int cpr = (fl_u1 + halo - x0) / CH + 1;
-      const int h = fl_v1 + halo - y0 + 1;
-      if (cpr * CH <= P && h <= StageGeom<G>::ROWS) {
-        t.staged = 1;
-        t.sx0 = x0;
-        t.sv0 = y0;
-        t.sh = h;
-        t.scpr = cpr;
-        t.srpp = 32 / cpr;
-        t.smag = (65536 + cpr - 1) / cpr;
-        t.soff = (int)((unsigned)(av - y0) * (unsigned)P - (unsigned)MAGIC_BITS * (unsigned)P +
-                       (unsigned)(au - x0) - (unsigned)MAGIC_BITS);
-        t.ic = (float)((av - y0) * P + (au - x0));
-      }
-    }
+  if (!mine) return;
+  constexpr int CH = StageGeom<G>::CH, P = StageGeom<G>::P;
+  // w is linear: its extremes lie symmetrically about the box's centre
+  const float wmax = 2.0f * fmaf(t.rw2, 0.5f * (zlo + zhi), t.W0) - wmin;
+  const BoxRange q = {xmin, xmax, ymin, ymax, wmin, wmax, npos};
+  const BoxPlan plan = plan_box(q, nu, nv, au, av, CH, P, STAGE ? StageGeom<G>::ROWS : 0, halo, seq);
+  const int du = au - plan.sx0, dv = av - plan.sv0;
+  TileView& o = EARLY ? tvs[b] : t;
+  o.mode = plan.mode;
+  o.csafe = plan.csafe;
+  o.staged = plan.staged;
+  if (STAGE && plan.staged) {
+    o.sx0 = plan.sx0;
+    o.sv0 = plan.sv0;
+    o.sh = plan.sh;
+    o.scpr = plan.scpr;
+    o.srpp = 32 / plan.scpr;
+    o.smag = (65536 + plan.scpr - 1) / plan.scpr;
+    o.soff = (int)((unsigned)dv * (unsigned)P - (unsigned)MAGIC_BITS * (unsigned)P + (unsigned)du -
+                   (unsigned)MAGIC_BITS);
+    o.ic = (float)(dv * P + du);
   }
-  tvs[b] = t;
+  if (!EARLY) tvs[b] = t;
 }
 
 // The same as a call, for the forward: inlined three times it took registers from the
@@ -375,7 +363,7 @@ __device__ __forceinline__ void setup_batch(TileView* tvs, const ViewGeom* __res
 template <typename G, bool STAGE>
 __device__ __noinline__ void setup_batch_call(TileView* tvs, const ViewGeom* __restrict__ geom,
                                               int j0, int nb, const TileIdx& ti, int nu, int nv) {
-  setup_batch<G, STAGE>(tvs, geom, j0, nb, ti, nu, nv);
+  setup_batch<G, STAGE, 1, STAGE>(tvs, geom, j0, nb, ti, nu, nv);
 }
 
 // Detector position of one voxel in the anchored frame.
@@ -508,7 +496,7 @@ __device__ __forceinline__ void stage_issue(unsigned char* buf, const CUtensorMa
   const int lane = threadIdx.x & 31;
   int nb = t.staged ? (t.sh + BOX_ROWS - 1) / BOX_ROWS : 0;
 #ifdef BP_BOUNDS_CHECK
-  if (nb > StageGeom<G>::ROWS / BOX_ROWS || (t.sx0 & (StageGeom<G>::CH - 1))) {
+  if ((unsigned)nb > StageGeom<G>::ROWS / BOX_ROWS || (t.sx0 & (StageGeom<G>::CH - 1))) {
     if (lane == 0) bc_fail(BC_STAGE_DST, t.sh, t.sx0);
     nb = 0;
   }
