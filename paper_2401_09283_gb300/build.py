@@ -16,8 +16,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libbp_gb300.so")
-SOURCES = ["bp_api.cu", "bp_job.cu", "bp_geom.cu", "bp_forward.cu", "bp_project.cu", "bp_noalloc.cu", "bp_spline.cu",
-           "bp_fdk.cu", "bp_probe.cu"]
+SOURCES = ["bp_api.cu", "bp_job.cu", "bp_geom.cu", "bp_forward.cu", "bp_vjp_motion.cu", "bp_vjp_fused.cu",
+           "bp_vjp_exact.cu", "bp_project.cu", "bp_noalloc.cu", "bp_spline.cu", "bp_fdk.cu", "bp_probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -26,12 +26,6 @@ def nvcc() -> str:
     if not os.path.exists(cand):
         raise RuntimeError("nvcc not found: the CUDA toolkit is required to build bp_gb300")
     return cand
-
-
-# The VJP's file compiles in a fixed number of parts: half the time, and 9.46 against
-# 9.65 ms for a 256^3 x 248 motion VJP (fewer spills).  Not "0", which follows the
-# machine's cores, and the code with them.
-FILE_FLAGS = {"bp_project.cu": ["--split-compile=2"]}
 
 
 def _flags(extra=()):
@@ -65,8 +59,7 @@ def build_library(force: bool = False, verbose: bool = False, extra=(), variant=
 
     def compile_one(src):
         obj = os.path.join(build_dir, os.path.splitext(src)[0] + ".o")
-        cmd = [cc, "-c", os.path.join(CSRC, src), "-o", obj] + _flags(
-            FILE_FLAGS.get(src, []) + list(vflags) + list(extra))
+        cmd = [cc, "-c", os.path.join(CSRC, src), "-o", obj] + _flags(list(vflags) + list(extra))
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError("nvcc failed for %s:\n%s\n%s" % (src, " ".join(cmd), r.stderr))

@@ -308,8 +308,11 @@ constexpr int BATCH_KERNELS = 6;  // launches per batched iteration besides the 
 // failure first (self test of the reporting path).  cudaErrorNotSupported in
 // release builds.
 cudaError_t bounds_status(unsigned* flags, long long* first, int op, cudaStream_t s);
-// bounds_status of bp_forward.cu (bounds_status combines both).
+// bounds_status of the other files (bounds_status combines them).
 cudaError_t bounds_status_forward(unsigned* flags, long long* first, int op, cudaStream_t s);
+cudaError_t bounds_status_vjp_motion(unsigned* flags, long long* first, int op, cudaStream_t s);
+cudaError_t bounds_status_vjp_fused(unsigned* flags, long long* first, int op, cudaStream_t s);
+cudaError_t bounds_status_vjp_exact(unsigned* flags, long long* first, int op, cudaStream_t s);
 
 // Throughput probes (bp_probe.cu): kind 0 scalar FP32 FMA lane-ops/s, 1 packed
 // f32x2 FMA lane-ops/s, 2 coalesced FP32 L2 atomic adds/s, 3 atomic adds/s in

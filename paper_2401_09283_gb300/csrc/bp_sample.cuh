@@ -1,8 +1,6 @@
-// What the forward (bp_forward.cu) and the VJP kernels (bp_project.cu) share: packed
-// arithmetic, the tile records, the staging of footprints and the taps.  They are
-// separate files so that the compiler's choices for one do not depend on the other
-// (in one file, and with nvcc's split compilation, the forward spilled: 3.44
-// against 3.30 ms on 256^3 x 248).
+// What the forward (bp_forward.cu), the motion VJP (bp_vjp.cuh) and the data VJP
+// (bp_project.cu) share: packed arithmetic, the tile records, the staging of footprints
+// and the taps.
 #pragma once
 
 #include "bp_internal.cuh"
