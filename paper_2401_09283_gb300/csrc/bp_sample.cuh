@@ -509,7 +509,8 @@ __device__ __forceinline__ void stage_issue(unsigned char* buf, const CUtensorMa
 
 // Whether the calling warp is the last of the CTA's warps to finish with a
 // slot.  Acquire-release: the last warp sees what every other warp wrote
-// before, and its refill comes after all their reads.
+// before, and its refill comes after all their reads (lane 0 acquires, the second
+// __syncwarp hands that on: a shuffle orders no memory).
 __device__ __forceinline__ bool last_warp(unsigned* done) {
   __syncwarp();
   unsigned old = 0;
@@ -518,7 +519,9 @@ __device__ __forceinline__ bool last_warp(unsigned* done) {
                  : "=r"(old)
                  : "r"(smem_addr(done)), "r"(NT / 32 - 1)
                  : "memory");
-  return __shfl_sync(0xffffffffu, old, 0) == NT / 32 - 1;
+  const bool last = __shfl_sync(0xffffffffu, old, 0) == NT / 32 - 1;
+  __syncwarp();
+  return last;
 }
 
 // All threads: convert the raw FP16/BF16 rectangle of record t (staged by
