@@ -135,7 +135,9 @@ int bp_probe(bp_ctx* ctx, int kind, double* result, void* stream);
  * the two offending coordinates; -1 when none), and redirects the access to
  * a safe position -- nothing traps and nothing outside the buffers is
  * touched.  op: 0 read, 1 read and clear, 2 record a synthetic failure first
- * (tests the reporting path without touching memory).  Synchronises the
+ * (tests the reporting path without touching memory), 3 from now on the staged
+ * footprints of view *first_failure never arrive (negative: all do), so that the
+ * bounded waits for them run out and the results are NaN.  0 to 2 synchronise the
  * device's legacy default stream.  Release builds return BP_ERR_UNSUPPORTED.
  * The paper has no counterpart (a debugging aid). */
 int bp_bounds_check(bp_ctx* ctx, int op, unsigned int* flags, long long* first_failure);

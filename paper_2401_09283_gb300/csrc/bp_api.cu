@@ -255,7 +255,7 @@ int bp_probe(bp_ctx* ctx, int kind, double* result, void* stream) {
 }
 
 int bp_bounds_check(bp_ctx* ctx, int op, unsigned int* flags, long long* first_failure) {
-  if (!ctx || !flags || !first_failure || op < 0 || op > 2) return BP_ERR_INVALID_ARG;
+  if (!ctx || !flags || !first_failure || op < 0 || op > 3) return BP_ERR_INVALID_ARG;
   ctx->err.clear();
   DeviceGuard g(ctx->device);
   const cudaError_t e = bpk::bounds_status(flags, first_failure, op, nullptr);

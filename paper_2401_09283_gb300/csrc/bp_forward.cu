@@ -70,16 +70,17 @@ __device__ __forceinline__ void forward_view_staged2(unsigned buf, const TileVie
 // barrier, refill the raw slot, compute.
 // One tile of the forward (its slices [zs ZS, zs ZS + ZS)): every view, in
 // order, accumulated per voxel.  All threads of the CTA call it; tvs, pipe and
-// dyn_smem are the CTA's shared memory.  seq counts the views the CTA has X.  The records of batch k+1 are built at the start of batch
-// k (two record slots), so the footprints of the next views are known.
-// A copy that never arrives (the bounded wait gives up) shows as NaN voxels.
+// dyn_smem are the CTA's shared memory.  The records of batch k+1 are built at the
+// start of batch k (two record slots), so the footprints of the next views are known.
+// bad: a copy has never arrived (the bounded wait gave up; the same in all warps when a
+// tile begins); the tile's voxels are then NaN.
 template <int ZB, int ZS, int NS, typename T, bool FDK, int STAGE>
 __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const CUtensorMap* map,
                                              const ProjInfo& pi, const ViewGeom* __restrict__ geom,
                                              const VolInfo& vi, float* __restrict__ vol, int tile,
                                              int zs, TileView (*tvs)[batch_records<STAGE>()],
                                              StagePipe<NS>& pipe, unsigned char* dyn_smem,
-                                             PipePos<NS>& pos) {
+                                             PipePos<NS>& pos, bool& bad) {
   using G = Geo<T, STAGE>;
   constexpr bool CONV = STAGE && StageGeom<G>::CONV;
   constexpr int SLOT = StageGeom<G>::BYTES, NB = batch_records<STAGE>();
@@ -90,14 +91,13 @@ __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const C
   f2 acc[ZS / 2];
 #pragma unroll
   for (int k = 0; k < ZS / 2; ++k) acc[k] = pk2(0.0f, 0.0f);
-  bool bad = false;
   const int V = pi.nviews;
   const int nbatch = (V + NB - 1) / NB;
   setup_batch_call<G, STAGE != STAGE_NONE>(tvs[0], geom, 0, min(NB, V), ti, pi.nu, pi.nv);
   if (nbatch > 1)
     setup_batch_call<G, STAGE != STAGE_NONE>(tvs[1], geom, NB, min(NB, V - NB), ti, pi.nu, pi.nv);
   __syncthreads();
-  if (STAGE && warp < NS && warp < V) {
+  if (STAGE && !bad && warp < NS && warp < V) {
     const unsigned s = (pos.slot + warp) % NS;
     stage_issue<G>(slots + s * SLOT, map, tvs[0][warp], warp, &pipe.full[s]);
   }
@@ -120,7 +120,7 @@ __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const C
     const int vn = v + NS;
     const TileView& tn = tvs[(vn / NB) & 1][vn % NB];
     if constexpr (CONV) {
-      __syncthreads();  // every warp has seen this phase and is done with F
+      bad = __syncthreads_or(bad);  // every warp has seen this phase and is done with F
       if (t.staged) {
         convert_stage<T, G>(reinterpret_cast<float*>(dyn_smem), reinterpret_cast<const T*>(buf), t);
         __syncthreads();  // F holds view v; the raw slot is free
@@ -145,7 +145,7 @@ __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const C
       }
     }
     if constexpr (STAGE && !CONV) {
-      if (last_warp(&pipe.done[slot]) && vn < V && !bad)
+      if (!bad && last_warp(&pipe.done[slot]) && vn < V)
         stage_issue<G>(buf, map, tn, vn, &pipe.full[slot]);
     }
   }
@@ -174,8 +174,10 @@ __global__ void __launch_bounds__(NT, NS > FWD_NS ? 2 : FWD_MINB)
   extern __shared__ __align__(128) unsigned char dyn_smem[];
   if (STAGE) pipe_init(pipe);
   PipePos<NS> pos;
+  bool bad = false;
   forward_tile<ZB, ZS, NS, T, FDK, STAGE>(proj, &map, pi, geom, vi, vol, blockIdx.x / (ZB / ZS),
-                                      blockIdx.x % (ZB / ZS), tvs, pipe, dyn_smem, pos);
+                                      blockIdx.x % (ZB / ZS), tvs, pipe, dyn_smem, pos, bad);
+  if (STAGE && bad) pipe_drain(pipe);
 }
 
 // z-extent of the forward's tiles
@@ -375,9 +377,10 @@ __global__ void __launch_bounds__(NT, FWD_MINB)
   extern __shared__ __align__(128) unsigned char dyn_smem[];
   pipe_init(pipe);
   PipePos<FWD_NS> pos;
+  bool bad = false;
   const int n = t.njobs, total = t.off_fwd[n];
   for (;;) {
-    __syncthreads();  // every thread is done with the previous tile
+    bad = __syncthreads_or(bad);  // every thread is done with the previous tile
     if (threadIdx.x == 0) item = (int)atomicAdd(counter, 1u);
     __syncthreads();
     const int w = item;
@@ -385,8 +388,9 @@ __global__ void __launch_bounds__(NT, FWD_MINB)
     const int j = batch_find(t.off_fwd, n, w);
     const BatchJob& J = t.job[j];
     forward_tile<ZB, ZB, FWD_NS, T, FDK, STAGE_TILE>((const T*)J.proj, &J.map, J.pi, J.geom, J.vif, J.vol,
-                                       w - t.off_fwd[j], 0, tvs, pipe, dyn_smem, pos);
+                                       w - t.off_fwd[j], 0, tvs, pipe, dyn_smem, pos, bad);
   }
+  if (bad) pipe_drain(pipe);
 }
 
 int forward_zb() { return ZB_FWD; }

@@ -27,9 +27,10 @@ cudaError_t bounds_status(unsigned* flags, long long* first, int op, cudaStream_
   for (auto of : {bounds_status_forward, bounds_status_vjp_motion, bounds_status_vjp_fused,
                   bounds_status_vjp_exact}) {
     unsigned f = 0;
-    long long first_of = -1;
-    if (e == cudaSuccess) e = of(&f, &first_of, op == 1 ? 1 : 0, s);
+    long long first_of = op == 3 ? *first : -1;
+    if (e == cudaSuccess) e = of(&f, &first_of, op == 2 ? 0 : op, s);
     if (e != cudaSuccess) return e;
+    if (op == 3) continue;
     *flags |= f;
     if (*first < 0) *first = first_of;
   }

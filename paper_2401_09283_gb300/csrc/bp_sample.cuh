@@ -150,6 +150,7 @@ enum { BC_STAGED_TAP = 0, BC_GLOBAL_TAP = 1, BC_SCATTER = 2, BC_STAGE_DST = 3, B
 #ifdef BP_BOUNDS_CHECK
 static __device__ unsigned int g_bc_flags;
 static __device__ unsigned long long g_bc_first;
+static __device__ int g_bc_lost_view = -1;  // the view whose footprints never arrive
 static __device__ __noinline__ void bc_fail(unsigned code, int a, int b) {
   atomicOr(&g_bc_flags, 1u << code);
   const unsigned long long rec = (1ull << 63) | ((unsigned long long)code << 56) |
@@ -166,6 +167,10 @@ static inline cudaError_t file_bounds_status(unsigned* flags, long long* first, 
     bc_selftest_kernel<<<1, 1, 0, s>>>();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+  }
+  if (op == 3) {
+    const int v = (int)*first;
+    return cudaMemcpyToSymbol(g_bc_lost_view, &v, sizeof(v));
   }
   cudaError_t e = cudaStreamSynchronize(s);
   unsigned long long f = 0;
@@ -457,6 +462,11 @@ __device__ __forceinline__ f2 bilerp2(f2 tu, f2 tv, f2 d00, f2 d10, f2 d01, f2 d
 // last refills the slot, so no warp waits for another one to free a slot.
 // Every warp waits on full[s] for every view, staged or not: it may then be at
 // most one phase behind, which the parity tells apart.
+//
+// A warp whose wait runs out (a copy that never arrives) is bad: it no longer counts
+// itself as finished, so that no slot is refilled from that step on and the other warps
+// run out of time too, where they need more; what it computes from there on shows as
+// NaN; and it stays for the copies that may still be in flight (pipe_drain).
 template <int NS>
 struct StagePipe {
   unsigned long long full[NS];
@@ -486,6 +496,15 @@ struct PipePos {
   }
 };
 
+// A bad warp, before it ends: give the copies in flight the same time again, so that none
+// lands in shared memory that another CTA has been given.  (Of a slot's two parities one
+// is that of a finished phase, whose wait returns at once.)
+template <int NS>
+__device__ __forceinline__ void pipe_drain(StagePipe<NS>& p) {
+#pragma unroll 1
+  for (int k = 0; k < 2 * NS; ++k) mbar_wait(&p.full[k / 2], k & 1);
+}
+
 // One whole warp: request the footprint of record t (view v) into buf.
 template <typename G>
 __device__ __forceinline__ void stage_issue(unsigned char* buf, const CUtensorMap* map,
@@ -497,6 +516,10 @@ __device__ __forceinline__ void stage_issue(unsigned char* buf, const CUtensorMa
   if ((unsigned)nb > StageGeom<G>::ROWS / BOX_ROWS || (t.sx0 & (StageGeom<G>::CH - 1))) {
     if (lane == 0) bc_fail(BC_STAGE_DST, t.sh, t.sx0);
     nb = 0;
+  }
+  if (nb && v == g_bc_lost_view) {  // announced, never copied
+    if (lane == 0) mbar_arrive_expect(bar, (unsigned)(nb * BOX));
+    return;
   }
 #endif
   if (lane == 0) {

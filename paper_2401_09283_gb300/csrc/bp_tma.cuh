@@ -31,12 +31,18 @@ __device__ __forceinline__ void mbar_arrive_expect(unsigned long long* bar, unsi
 // Wait for the phase of the given parity.  Each try suspends the thread in
 // hardware until the phase completes or the hinted time (10 ms) is over: with
 // the short default time the polling itself took a fifth of the issue slots.
-// Bounded: false after 1024 tries, far beyond any copy.
+// Bounded: false after MBAR_TRIES tries, far beyond any copy (64 in the debug build,
+// where a test lets the wait run out).
+#ifdef BP_BOUNDS_CHECK
+constexpr int MBAR_TRIES = 64;
+#else
+constexpr int MBAR_TRIES = 1024;
+#endif
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity) {
   const unsigned a = smem_addr(bar);
   unsigned ok = 0;
 #pragma unroll 1
-  for (int i = 0; i < 1024; ++i) {
+  for (int i = 0; i < MBAR_TRIES; ++i) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"

@@ -951,7 +951,8 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
     const int in = idx + NS;
     const TileView& tn = tvs[(in / NB) & 1][in % NB];
     if constexpr (CONV) {
-      __syncthreads();  // every warp has seen this phase and is done with F and step idx-1
+      // every warp has seen this phase and is done with F and step idx-1
+      bad = __syncthreads_or(bad);
       if (b > 0 && half == 0 && warp == ((idx + 4) & 7)) record(idx - 1, bad);
       if (t.staged) {
         convert_stage<T, G>(reinterpret_cast<float*>(dyn_smem), reinterpret_cast<const T*>(buf), t);
@@ -978,10 +979,12 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
     if (HALVES == 2 && half == 1) vjp_reduce(ti, S, Z, red[slot][warp]);
     if constexpr (!CONV) {
       if (!STAGE) __syncthreads();  // no pipe to keep the warps within two views
-      if (last_warp(&pipe.done[slot])) {
-        if (half == HALVES - 1) record(idx, bad);
+      if (STAGE && bad) {
+        if (half == HALVES - 1) record(idx, true);
+      } else if (last_warp(&pipe.done[slot])) {
+        if (half == HALVES - 1) record(idx, false);
         __syncwarp();
-        if (STAGE && in < nst && !bad)
+        if (STAGE && in < nst)
           stage_issue<G>(buf, map, tn, vbeg + in / HALVES, &pipe.full[slot]);
       }
     }
@@ -990,6 +993,7 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
     __syncthreads();
     if (warp == 0) record(nst - 1, bad);
   }
+  if (STAGE && bad) pipe_drain(pipe);
 }
 
 template <int ZB, int NS, typename T, bool FDK, bool EXACT, bool PROJ, int STAGE>
