@@ -29,14 +29,16 @@ __device__ __forceinline__ void mbar_arrive_expect(unsigned long long* bar, unsi
 }
 
 // Wait for the phase of the given parity.  Each try suspends the thread in
-// hardware until the phase completes or the hinted time (10 ms) is over: with
+// hardware until the phase completes or the hinted time (20 us) is over: with
 // the short default time the polling itself took a fifth of the issue slots.
-// Bounded: false after MBAR_TRIES tries, far beyond any copy (64 in the debug build,
-// where a test lets the wait run out).
+// Bounded: false after MBAR_TRIES tries.  A try lasts 2 to 3 us whatever the hint
+// (1024 of "10 ms" were over after 3 ms, which memory that has to be paged in could
+// exceed): 2^20 of them are 2 to 3 s, and 20 s at most.  (A limit by the timer in place of the
+// count made the forward spill, 256^3 x 248 3.28 against 3.33 ms.)
 #ifdef BP_BOUNDS_CHECK
-constexpr int MBAR_TRIES = 64;
+constexpr int MBAR_TRIES = 1 << 14;  // a test lets it run out
 #else
-constexpr int MBAR_TRIES = 1024;
+constexpr int MBAR_TRIES = 1 << 20;
 #endif
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity) {
   const unsigned a = smem_addr(bar);
@@ -48,7 +50,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(a), "r"(parity), "r"(10000000u)
+        : "r"(a), "r"(parity), "r"(20000u)
         : "memory");
     if (ok) return true;
   }

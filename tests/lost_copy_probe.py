@@ -73,7 +73,7 @@ def main():
         lose(LOST)
         t = time.time()
         lost = calls(dtype)
-        res["seconds"] = max(res.get("seconds", 0.0), time.time() - t)
+        res["seconds"] = min(res.get("seconds", 1e9), time.time() - t)
         lose(-1)
         again = calls(dtype)
         n = str(dtype)
