@@ -99,14 +99,15 @@ int prepare_views(bp_ctx* ctx, const bp_proj_desc* pd, const double* P, const do
   const double* dvw = (const double*)q;
   CK(stage_in(ctx->s_scale, pd->view_scale, sizeof(float) * V, s, &q), "copy view_scale");
   const float* dsc = (const float*)q;
-  CK(ensure(ctx->geom, sizeof(ViewGeom) * (size_t)V), "alloc view table");
+  // (the view flags behind the table: a call that is being captured may be the first
+  // one that needs them, and cannot allocate)
+  CK(ensure(ctx->geom, (sizeof(ViewGeom) + sizeof(int)) * (size_t)V), "alloc view table");
   // large problems choose the kernel variant per view on the device (two
   // launches, one of which returns at once: ~3 us, so not for small ones)
   *wide = nullptr;
   bpk::FitInfo fit{pd->dtype, nullptr};
   if ((long long)vi.nx * vi.ny * vi.nz * V >= (1LL << 28)) {
-    CK(ensure(ctx->wide, sizeof(int) * (size_t)V), "alloc view flags");
-    fit.wide = (int*)ctx->wide.p;
+    fit.wide = reinterpret_cast<int*>((ViewGeom*)ctx->geom.p + V);
     *wide = fit.wide;
   }
   CK(TL(K_COMPOSE, 1, bpk::launch_compose(*dP, *dmotion, dvw, dsc, V, weight == BP_WEIGHT_FDK,
@@ -185,7 +186,7 @@ void bp_ctx_destroy(bp_ctx* ctx) {
   if (!ctx) return;
   DeviceGuard g(ctx->device);
   cudaDeviceSynchronize();
-  Buf* bufs[] = {&ctx->geom,   &ctx->wide,   &ctx->grad,   &ctx->partials,   &ctx->shblk,      &ctx->fdk_tab,
+  Buf* bufs[] = {&ctx->geom,   &ctx->grad,   &ctx->partials,   &ctx->shblk,      &ctx->fdk_tab,
                  &ctx->s_proj,
                  &ctx->s_P,    &ctx->s_motion, &ctx->s_vw,     &ctx->s_scale,    &ctx->s_vol,
                  &ctx->s_dvol, &ctx->s_out_motion, &ctx->s_out_P, &ctx->s_out_proj,
@@ -202,7 +203,7 @@ const char* bp_last_error(const bp_ctx* ctx) { return ctx ? ctx->err.c_str() : "
 
 long long bp_ctx_workspace_bytes(const bp_ctx* ctx) {
   if (!ctx) return 0;
-  const Buf* bufs[] = {&ctx->geom,   &ctx->wide,   &ctx->grad,   &ctx->partials,   &ctx->shblk,      &ctx->fdk_tab,
+  const Buf* bufs[] = {&ctx->geom,   &ctx->grad,   &ctx->partials,   &ctx->shblk,      &ctx->fdk_tab,
                        &ctx->s_proj,
                        &ctx->s_P,    &ctx->s_motion, &ctx->s_vw,     &ctx->s_scale,    &ctx->s_vol,
                        &ctx->s_dvol, &ctx->s_out_motion, &ctx->s_out_P, &ctx->s_out_proj,
