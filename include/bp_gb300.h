@@ -174,9 +174,14 @@ int bp_forward(bp_ctx* ctx, const void* proj, const bp_proj_desc* pdesc, const d
  *               of 16 bytes per detector pixel of every view for it (4x the
  *               size of dL_dproj; see bp_ctx_workspace_bytes), kept between
  *               calls -- when dL_dproj comes with the motion gradients, only
- *               for projections with 16-byte aligned rows or those that a
- *               large call copies to aligned rows (scratch of the context,
- *               one stack; without memory for either the call does without).
+ *               for projections with 16-byte aligned rows.  It is required
+ *               where rows are whole 16-byte chunks; for other widths the call
+ *               does without where memory is short.  So it does without the
+ *               aligned copy (scratch of the context, one stack) that large
+ *               calls on unaligned rows make: both are taken only after
+ *               everything that the call needs, if they leave three quarters
+ *               of the free memory, and given back when a later call or job
+ *               has no room.
  * Any output may be NULL to skip it (dL_dmotion needs motion or treats it as
  * zero).  With BP_WEIGHT_FDK the derivative of (sid/w)^2 is included. */
 int bp_vjp(bp_ctx* ctx, const float* dL_dvol, const void* proj, const bp_proj_desc* pdesc,

@@ -85,23 +85,35 @@ size_t proj_bytes(const bp_proj_desc* pd) {
 
 constexpr int ZB = bpk::ZB_VJP;
 
-// Stage the per-view inputs and run the FP64 composition into ctx->geom.
-int prepare_views(bp_ctx* ctx, const bp_proj_desc* pd, const double* P, const double* motion,
-                  const double* view_weight, int weight, const VolInfo& vi, cudaStream_t s,
-                  const double** dP, const double** dmotion, const int** wide) {
+// The per-view inputs on the device.
+struct Views {
+  const double *P, *motion, *vw;
+  const float* scale;
+};
+
+// Stage the per-view inputs and make room for the view table.
+int stage_views(bp_ctx* ctx, const bp_proj_desc* pd, const double* P, const double* motion,
+                const double* view_weight, cudaStream_t s, Views* dv) {
   const int V = pd->nviews;
   const void* q = nullptr;
-  CK(stage_in(ctx->s_P, P, sizeof(double) * 12 * V, s, &q), "copy P");
-  *dP = (const double*)q;
-  CK(stage_in(ctx->s_motion, motion, sizeof(double) * 6 * V, s, &q), "copy motion");
-  *dmotion = (const double*)q;
-  CK(stage_in(ctx->s_vw, view_weight, sizeof(double) * V, s, &q), "copy view_weight");
-  const double* dvw = (const double*)q;
-  CK(stage_in(ctx->s_scale, pd->view_scale, sizeof(float) * V, s, &q), "copy view_scale");
-  const float* dsc = (const float*)q;
+  CK(stage_in(ctx, ctx->s_P, P, sizeof(double) * 12 * V, s, &q), "copy P");
+  dv->P = (const double*)q;
+  CK(stage_in(ctx, ctx->s_motion, motion, sizeof(double) * 6 * V, s, &q), "copy motion");
+  dv->motion = (const double*)q;
+  CK(stage_in(ctx, ctx->s_vw, view_weight, sizeof(double) * V, s, &q), "copy view_weight");
+  dv->vw = (const double*)q;
+  CK(stage_in(ctx, ctx->s_scale, pd->view_scale, sizeof(float) * V, s, &q), "copy view_scale");
+  dv->scale = (const float*)q;
   // (the view flags behind the table: a call that is being captured may be the first
   // one that needs them, and cannot allocate)
-  CK(ensure(ctx->geom, (sizeof(ViewGeom) + sizeof(int)) * (size_t)V), "alloc view table");
+  CK(ensure(ctx, ctx->geom, (sizeof(ViewGeom) + sizeof(int)) * (size_t)V), "alloc view table");
+  return BP_OK;
+}
+
+// Run the FP64 composition into ctx->geom.
+int compose_views(bp_ctx* ctx, const bp_proj_desc* pd, const Views& dv, int weight,
+                  const VolInfo& vi, cudaStream_t s, const int** wide) {
+  const int V = pd->nviews;
   // large problems choose the kernel variant per view on the device (two
   // launches, one of which returns at once: ~3 us, so not for small ones)
   *wide = nullptr;
@@ -110,16 +122,30 @@ int prepare_views(bp_ctx* ctx, const bp_proj_desc* pd, const double* P, const do
     fit.wide = reinterpret_cast<int*>((ViewGeom*)ctx->geom.p + V);
     *wide = fit.wide;
   }
-  CK(TL(K_COMPOSE, 1, bpk::launch_compose(*dP, *dmotion, dvw, dsc, V, weight == BP_WEIGHT_FDK,
+  CK(TL(K_COMPOSE, 1, bpk::launch_compose(dv.P, dv.motion, dv.vw, dv.scale, V, weight == BP_WEIGHT_FDK,
                                           pd->sid, vi, (ViewGeom*)ctx->geom.p, nullptr, s,
                                           fit.wide ? &fit : nullptr)),
      "compose");
   return BP_OK;
 }
 
-// Grow a workspace that a call can do without: false where that fails.
-bool ensure_optional(Buf& b, size_t bytes) {
-  if (ensure(b, bytes) == cudaSuccess) return true;
+// Whether a call on s is being captured.
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
+// Grow a workspace that a call can do without: false where that fails, where it would
+// take more than a quarter of the free memory (it is kept, and the program that the
+// memory is left to may not know of it), or in a capture.
+bool ensure_spare(Buf& b, size_t bytes, cudaStream_t s) {
+  if (b.n >= bytes && b.p) return true;
+  size_t fr = 0, tot = 0;
+  if (!capturing(s) && cudaMemGetInfo(&fr, &tot) == cudaSuccess && bytes <= fr / 4 &&
+      ensure(b, bytes) == cudaSuccess)
+    return true;
   cudaGetLastError();
   return false;
 }
@@ -131,29 +157,22 @@ bool ensure_optional(Buf& b, size_t bytes) {
 // pixel, 1-2 ps; staging saves more than 1 ps per voxel-view) and 2^22 of them (~4 us,
 // the launch).  Without memory for it the call runs as before; so does one that is
 // being captured (its graph would hold a workspace that a later, larger call
-// replaces).  Measured: BF16 rows of
-// 401 pixels, 143 x 187 x 161 voxels x 111 views, forward and both gradients 4.35 ->
-// 3.42 ms.
+// replaces).  Measured: BF16 rows of 401 pixels, 143 x 187 x 161 voxels x 111 views,
+// forward and both gradients 4.35 -> 3.42 ms.
 int align_rows(bp_ctx* ctx, const bp_proj_desc* pd, long long nvox, cudaStream_t s,
-               const void** dproj, ProjInfo* pi, bool* copied) {
-  *copied = false;
+               const void** dproj, ProjInfo* pi) {
   const long long rows = (long long)pi->nviews * pi->nv, work = nvox * pi->nviews;
   if (bpk::stage_aligned(*dproj, pd->dtype, *pi) || work < (1LL << 22) || work < rows * pi->nu)
     return BP_OK;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return BP_OK;
-  }
+  if (capturing(s)) return BP_OK;
   const long long es = pd->dtype == BP_F32 ? 4 : 2, rs = (pi->nu * es + 15) / 16 * 16 / es;
-  if (!ensure_optional(ctx->aligned, (size_t)(rows * rs * es))) return BP_OK;
+  if (!ensure_spare(ctx->aligned, (size_t)(rows * rs * es), s)) return BP_OK;
   CK(TL(K_ALIGN, 1, bpk::launch_align_rows(*dproj, pd->dtype, *pi, ctx->aligned.p, rs, s)),
      "align rows");
   *dproj = ctx->aligned.p;
   pi->rs = rs;
   pi->vs = rs * pi->nv;
   pi->seq = 1;  // the sums of the motion gradient keep the order they have without the copy
-  *copied = true;
   return BP_OK;
 }
 
@@ -248,7 +267,7 @@ int bp_probe(bp_ctx* ctx, int kind, double* result, void* stream) {
   int sms = 0;
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device), "bp_probe");
   const long long words = 16LL << 20;  // 64 MiB of scratch for the atomics
-  CK(ensure(ctx->probe, (size_t)words * 4), "bp_probe: scratch");
+  CK(ensure(ctx, ctx->probe, (size_t)words * 4), "bp_probe: scratch");
   cudaStream_t s = (cudaStream_t)stream;
   CK(cudaMemsetAsync(ctx->probe.p, 0, (size_t)words * 4, s), "bp_probe: clear");
   CK(bpk::run_probe(kind, (float*)ctx->probe.p, words, sms, result, s), "bp_probe");
@@ -276,13 +295,13 @@ int bp_compose(bp_ctx* ctx, int nviews, const double* P, const double* motion, d
   DeviceGuard g(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
   const void* q;
-  CK(stage_in(ctx->s_P, P, sizeof(double) * 12 * nviews, s, &q), "copy P");
+  CK(stage_in(ctx, ctx->s_P, P, sizeof(double) * 12 * nviews, s, &q), "copy P");
   const double* dP = (const double*)q;
-  CK(stage_in(ctx->s_motion, motion, sizeof(double) * 6 * nviews, s, &q), "copy motion");
+  CK(stage_in(ctx, ctx->s_motion, motion, sizeof(double) * 6 * nviews, s, &q), "copy motion");
   const double* dm = (const double*)q;
   void* o;
   bool host;
-  CK(stage_out(ctx->s_out_P, Phat, sizeof(double) * 12 * nviews, &o, &host), "alloc Phat");
+  CK(stage_out(ctx, ctx->s_out_P, Phat, sizeof(double) * 12 * nviews, &o, &host), "alloc Phat");
   VolInfo vi{};
   CK(TL(K_COMPOSE, 1, bpk::launch_compose(dP, dm, nullptr, nullptr, nviews, 0, 0.0, vi, nullptr,
                                           (double*)o, s)),
@@ -315,20 +334,20 @@ int bp_forward(bp_ctx* ctx, const void* proj, const bp_proj_desc* pdesc, const d
   cudaStream_t s = (cudaStream_t)stream;
   void* dvol;
   bool host_vol;
-  CK(stage_out(ctx->s_vol, vol, sizeof(float) * nvox, &dvol, &host_vol), "alloc vol");
+  CK(stage_out(ctx, ctx->s_vol, vol, sizeof(float) * nvox, &dvol, &host_vol), "alloc vol");
   if (pdesc->nviews == 0) {
     CK(cudaMemsetAsync(dvol, 0, sizeof(float) * nvox, s), "zero vol");
   } else {
     const VolInfo vi = make_volinfo(vdesc, ZB);
     const void* dproj;
-    CK(stage_in(ctx->s_proj, proj, proj_bytes(pdesc), s, &dproj), "copy proj");
-    const double *dP, *dm;
+    CK(stage_in(ctx, ctx->s_proj, proj, proj_bytes(pdesc), s, &dproj), "copy proj");
+    Views dv;
     const int* wide;
-    st = prepare_views(ctx, pdesc, P, motion, view_weight, weight, vi, s, &dP, &dm, &wide);
+    st = stage_views(ctx, pdesc, P, motion, view_weight, s, &dv);
+    if (!st) st = compose_views(ctx, pdesc, dv, weight, vi, s, &wide);
     if (st) return st;
     ProjInfo pi = make_projinfo(pdesc);
-    bool copied;
-    st = align_rows(ctx, pdesc, nvox, s, &dproj, &pi, &copied);
+    st = align_rows(ctx, pdesc, nvox, s, &dproj, &pi);
     if (st) return st;
     CK(TL(K_FORWARD, wide ? 2 : 1, bpk::launch_forward(dproj, pdesc->dtype, pi,
                                           (const ViewGeom*)ctx->geom.p, vi,
@@ -369,58 +388,62 @@ int bp_vjp(bp_ctx* ctx, const float* dL_dvol, const void* proj, const bp_proj_de
   ProjInfo pi = make_projinfo(pdesc);
   const int ntiles = vi.tiles_x * vi.tiles_y * vi.tiles_z;
   const void* q;
-  CK(stage_in(ctx->s_dvol, dL_dvol, sizeof(float) * nvox, s, &q), "copy dL_dvol");
+  CK(stage_in(ctx, ctx->s_dvol, dL_dvol, sizeof(float) * nvox, s, &q), "copy dL_dvol");
   const float* ddvol = (const float*)q;
   const void* dproj = nullptr;
-  bool copied = false;
-  if (want_geo) {
-    CK(stage_in(ctx->s_proj, proj, proj_bytes(pdesc), s, &dproj), "copy proj");
-    st = align_rows(ctx, pdesc, nvox, s, &dproj, &pi, &copied);
-    if (st) return st;
-  }
-  const double *dP, *dm;
-  const int* wide;
-  st = prepare_views(ctx, pdesc, P, motion, view_weight, weight, vi, s, &dP, &dm, &wide);
+  if (want_geo) CK(stage_in(ctx, ctx->s_proj, proj, proj_bytes(pdesc), s, &dproj), "copy proj");
+  Views dv;
+  st = stage_views(ctx, pdesc, P, motion, view_weight, s, &dv);
   if (st) return st;
   void *om = nullptr, *oP = nullptr, *oD = nullptr;
   bool hm = false, hP = false, hD = false;
-  CK(stage_out(ctx->s_out_motion, dL_dmotion, sizeof(double) * 6 * V, &om, &hm), "alloc out");
-  CK(stage_out(ctx->s_out_P, dL_dPhat, sizeof(double) * 12 * V, &oP, &hP), "alloc out");
+  CK(stage_out(ctx, ctx->s_out_motion, dL_dmotion, sizeof(double) * 6 * V, &om, &hm), "alloc out");
+  CK(stage_out(ctx, ctx->s_out_P, dL_dPhat, sizeof(double) * 12 * V, &oP, &hP), "alloc out");
   const size_t dproj_bytes = sizeof(float) * (size_t)V * pdesc->nv * pdesc->nu;
-  CK(stage_out(ctx->s_out_proj, dL_dproj, dproj_bytes, &oD, &hD), "alloc out");
+  CK(stage_out(ctx, ctx->s_out_proj, dL_dproj, dproj_bytes, &oD, &hD), "alloc out");
   // the data VJP is fused into the motion-VJP kernel when both are wanted
   const bool fuse = want_geo && dL_dproj && nvox > 0;
+  const bool exact = deriv == BP_DERIV_BILINEAR_EXACT;
+  // what the call needs, then what it can do without
+  if (want_geo && !exact)
+    CK(ensure(ctx, ctx->grad, sizeof(float2) * (size_t)V * pdesc->nv * pdesc->nu), "alloc grad");
+  if (want_geo && nvox > 0)
+    CK(ensure(ctx, ctx->partials, sizeof(float) * bpk::PSLOTS * (size_t)V * ntiles),
+       "alloc partials");
+  // the fused data VJP of staged CENTRAL tiles goes through a block image (one vector
+  // reduction per sample), added into dL_dproj by a second kernel of the same launch;
+  // stacks whose rows are not whole 16-byte chunks never needed its memory
+  const size_t blk_bytes = sizeof(float) * (size_t)bpk::block_image_floats(pi);
+  bool blocks = fuse && !pi.seq && bpk::vjp_uses_blocks(dproj, pdesc->dtype, pi, exact);
+  if (blocks) CK(ensure(ctx, ctx->blkimg, blk_bytes), "alloc block image");
+  if (want_geo) {
+    st = align_rows(ctx, pdesc, nvox, s, &dproj, &pi);
+    if (st) return st;
+    if (fuse && !blocks && bpk::vjp_uses_blocks(dproj, pdesc->dtype, pi, exact))
+      blocks = ensure_spare(ctx->blkimg, blk_bytes, s);
+  }
+  const int* wide;
+  st = compose_views(ctx, pdesc, dv, weight, vi, s, &wide);
+  if (st) return st;
   if (dL_dproj) CK(cudaMemsetAsync(oD, 0, dproj_bytes, s), "zero dL_dproj");
   if (want_geo) {
     const float2* grad = nullptr;
-    if (deriv == BP_DERIV_CENTRAL) {
-      CK(ensure(ctx->grad, sizeof(float2) * (size_t)V * pdesc->nv * pdesc->nu), "alloc grad");
+    if (!exact) {
       CK(TL(K_GRAD, 1, bpk::launch_grad_images(dproj, pdesc->dtype, pi, (float2*)ctx->grad.p, s)),
          "grad images");
       grad = (const float2*)ctx->grad.p;
     }
     if (nvox > 0) {
-      CK(ensure(ctx->partials, sizeof(float) * bpk::PSLOTS * (size_t)V * ntiles), "alloc partials");
-      // the fused data VJP of staged CENTRAL tiles goes through a block
-      // image (one vector reduction per sample), added into dL_dproj by a
-      // second kernel of the same launch
-      bool blocks = fuse && bpk::vjp_uses_blocks(dproj, pdesc->dtype, pi,
-                                                 deriv == BP_DERIV_BILINEAR_EXACT);
-      if (blocks && copied)  // (unaligned stacks never needed its memory)
-        blocks = ensure_optional(ctx->blkimg, sizeof(float) * (size_t)bpk::block_image_floats(pi));
-      else if (blocks)
-        CK(ensure(ctx->blkimg, sizeof(float) * (size_t)bpk::block_image_floats(pi)),
-           "alloc block image");
       CK(TL(fuse ? K_VJP_FUSED : K_VJP_MOTION, (wide ? 2 : 1) + (blocks ? 1 : 0),
             bpk::launch_vjp_motion(ddvol, dproj, pdesc->dtype, pi, grad,
                                    (const ViewGeom*)ctx->geom.p, vi, weight == BP_WEIGHT_FDK,
-                                   deriv == BP_DERIV_BILINEAR_EXACT, (float*)ctx->partials.p,
+                                   exact, (float*)ctx->partials.p,
                                    fuse ? (float*)oD : nullptr,
                                    blocks ? (float*)ctx->blkimg.p : nullptr, wide, s)),
          "vjp kernel");
     }
     CK(TL(K_REDUCE, 1, bpk::launch_reduce_chain((const float*)ctx->partials.p, nvox > 0 ? ntiles : 0,
-                                              vi, dP, dm, V, (double*)oP, (double*)om, s)),
+                                              vi, dv.P, dv.motion, V, (double*)oP, (double*)om, s)),
        "reduce kernel");
   }
   if (dL_dproj && !fuse && nvox > 0) {
@@ -428,7 +451,7 @@ int bp_vjp(bp_ctx* ctx, const float* dL_dvol, const void* proj, const bp_proj_de
     po.rs = pdesc->nu;
     po.vs = (long long)pdesc->nu * pdesc->nv;
     const long long bf = bpk::block_image_floats(po);
-    if (bf > 0) CK(ensure(ctx->blkimg, sizeof(float) * (size_t)bf), "alloc block image");
+    if (bf > 0) CK(ensure(ctx, ctx->blkimg, sizeof(float) * (size_t)bf), "alloc block image");
     CK(TL(K_VJP_PROJ, bf > 0 ? 2 : 1,
           bpk::launch_vjp_proj(ddvol, po, (const ViewGeom*)ctx->geom.p, vi,
                                weight == BP_WEIGHT_FDK, (float*)oD,
@@ -462,13 +485,13 @@ int bp_sharpness(bp_ctx* ctx, const float* vol, const bp_vol_desc* vdesc, double
     return BP_OK;
   }
   const void* q;
-  CK(stage_in(ctx->s_vol, vol, sizeof(float) * nvox, s, &q), "copy vol");
+  CK(stage_in(ctx, ctx->s_vol, vol, sizeof(float) * nvox, s, &q), "copy vol");
   void *ol, *og;
   bool hl, hg;
-  CK(stage_out(ctx->s_loss, loss, sizeof(double), &ol, &hl), "alloc loss");
-  CK(stage_out(ctx->s_dvol, dL_dvol, sizeof(float) * nvox, &og, &hg), "alloc grad");
+  CK(stage_out(ctx, ctx->s_loss, loss, sizeof(double), &ol, &hl), "alloc loss");
+  CK(stage_out(ctx, ctx->s_dvol, dL_dvol, sizeof(float) * nvox, &og, &hg), "alloc grad");
   const int nb = bpk::sharpness_blocks(nvox);
-  CK(ensure(ctx->shblk, sizeof(double) * nb), "alloc block sums");
+  CK(ensure(ctx, ctx->shblk, sizeof(double) * nb), "alloc block sums");
   CK(TL(K_SHARPNESS, 2, bpk::launch_sharpness((const float*)q, vdesc->nx, vdesc->ny, vdesc->nz,
                                               (double*)ctx->shblk.p, nb, (double*)ol,
                                               (float*)og, s)),
@@ -500,13 +523,13 @@ int bp_tv(bp_ctx* ctx, const float* vol, const bp_vol_desc* vdesc, double eps, d
     return BP_OK;
   }
   const void* q;
-  CK(stage_in(ctx->s_vol, vol, sizeof(float) * nvox, s, &q), "copy vol");
+  CK(stage_in(ctx, ctx->s_vol, vol, sizeof(float) * nvox, s, &q), "copy vol");
   void *ol, *og;
   bool hl, hg;
-  CK(stage_out(ctx->s_loss, loss, sizeof(double), &ol, &hl), "alloc loss");
-  CK(stage_out(ctx->s_dvol, dL_dvol, sizeof(float) * nvox, &og, &hg), "alloc grad");
+  CK(stage_out(ctx, ctx->s_loss, loss, sizeof(double), &ol, &hl), "alloc loss");
+  CK(stage_out(ctx, ctx->s_dvol, dL_dvol, sizeof(float) * nvox, &og, &hg), "alloc grad");
   const int nb = bpk::sharpness_blocks(nvox);
-  CK(ensure(ctx->shblk, sizeof(double) * nb), "alloc block sums");
+  CK(ensure(ctx, ctx->shblk, sizeof(double) * nb), "alloc block sums");
   CK(TL(K_SHARPNESS, 2, bpk::launch_tv((const float*)q, vdesc->nx, vdesc->ny, vdesc->nz,
                                        (float)eps, (double*)ctx->shblk.p, nb, (double*)ol,
                                        nullptr, 0, (float*)og, s)),
@@ -532,19 +555,19 @@ int opt_step(bp_ctx* ctx, int V, double* theta, const double* grad, double* m1, 
   double* dm2 = m2;
   const bool ht = is_host(theta), h1 = m1 && is_host(m1), h2 = m2 && is_host(m2);
   const void* q;
-  CK(stage_in(ctx->s_grad, grad, b, s, &q), "copy grad");
+  CK(stage_in(ctx, ctx->s_grad, grad, b, s, &q), "copy grad");
   if (ht) {
-    CK(ensure(ctx->s_theta, b), "alloc");
+    CK(ensure(ctx, ctx->s_theta, b), "alloc");
     CK(cudaMemcpyAsync(ctx->s_theta.p, theta, b, cudaMemcpyHostToDevice, s), "copy theta");
     dt = (double*)ctx->s_theta.p;
   }
   if (h1) {
-    CK(ensure(ctx->s_m1, b), "alloc");
+    CK(ensure(ctx, ctx->s_m1, b), "alloc");
     CK(cudaMemcpyAsync(ctx->s_m1.p, m1, b, cudaMemcpyHostToDevice, s), "copy m1");
     dm1 = (double*)ctx->s_m1.p;
   }
   if (h2) {
-    CK(ensure(ctx->s_m2, b), "alloc");
+    CK(ensure(ctx, ctx->s_m2, b), "alloc");
     CK(cudaMemcpyAsync(ctx->s_m2.p, m2, b, cudaMemcpyHostToDevice, s), "copy m2");
     dm2 = (double*)ctx->s_m2.p;
   }
@@ -610,10 +633,10 @@ int bp_akima_motion(bp_ctx* ctx, int n_nodes, int nviews, const double* nodes, d
   DeviceGuard g(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
   const void* q;
-  CK(stage_in(ctx->s_nodes, nodes, sizeof(double) * 6 * n_nodes, s, &q), "copy nodes");
+  CK(stage_in(ctx, ctx->s_nodes, nodes, sizeof(double) * 6 * n_nodes, s, &q), "copy nodes");
   void* o;
   bool host;
-  CK(stage_out(ctx->s_out_motion, theta, sizeof(double) * 6 * nviews, &o, &host), "alloc theta");
+  CK(stage_out(ctx, ctx->s_out_motion, theta, sizeof(double) * 6 * nviews, &o, &host), "alloc theta");
   CK(TL(K_SPLINE, 1, bpk::launch_akima_eval(n_nodes, nviews, (const double*)q, (double*)o, s)),
      "akima");
   if (host) {
@@ -635,12 +658,12 @@ int bp_akima_motion_vjp(bp_ctx* ctx, int n_nodes, int nviews, const double* node
   DeviceGuard g(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
   const void* q;
-  CK(stage_in(ctx->s_nodes, nodes, sizeof(double) * 6 * n_nodes, s, &q), "copy nodes");
+  CK(stage_in(ctx, ctx->s_nodes, nodes, sizeof(double) * 6 * n_nodes, s, &q), "copy nodes");
   const double* dn = (const double*)q;
-  CK(stage_in(ctx->s_grad, dL_dtheta, sizeof(double) * 6 * nviews, s, &q), "copy dL/dtheta");
+  CK(stage_in(ctx, ctx->s_grad, dL_dtheta, sizeof(double) * 6 * nviews, s, &q), "copy dL/dtheta");
   void* o;
   bool host;
-  CK(stage_out(ctx->s_out_nodes, dL_dnodes, sizeof(double) * 6 * n_nodes, &o, &host),
+  CK(stage_out(ctx, ctx->s_out_nodes, dL_dnodes, sizeof(double) * 6 * n_nodes, &o, &host),
      "alloc dL/dnodes");
   CK(TL(K_SPLINE, 1, bpk::launch_akima_vjp(n_nodes, nviews, dn, (const double*)q, (double*)o, s)),
      "akima vjp");
@@ -672,11 +695,11 @@ int bp_fdk_filter(bp_ctx* ctx, const float* raw, int nviews, int nv, int nu, dou
   DeviceGuard g(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
   const void* q;
-  CK(stage_in(ctx->s_proj, raw, sizeof(float) * n, s, &q), "copy raw");
+  CK(stage_in(ctx, ctx->s_proj, raw, sizeof(float) * n, s, &q), "copy raw");
   void* o;
   bool host;
-  CK(stage_out(ctx->s_out_proj, out, sizeof(float) * n, &o, &host), "alloc out");
-  CK(ensure(ctx->fdk_tab, sizeof(float) * bpk::fdk_table_floats(nviews, nu, nv, ext)),
+  CK(stage_out(ctx, ctx->s_out_proj, out, sizeof(float) * n, &o, &host), "alloc out");
+  CK(ensure(ctx, ctx->fdk_tab, sizeof(float) * bpk::fdk_table_floats(nviews, nu, nv, ext)),
      "alloc tables");
   CK(TL(K_FDK, 2, bpk::launch_fdk_filter((const float*)q, nviews, nv, nu, ext, pitch, sid, sdd,
                                          arc, (float*)ctx->fdk_tab.p, (float*)o, s)),

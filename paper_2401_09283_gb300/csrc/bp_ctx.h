@@ -151,6 +151,31 @@ inline cudaError_t ensure(Buf& b, size_t bytes) {
   return cudaSuccess;
 }
 
+// Give back the workspaces that a call can do without (what large calls on unaligned rows
+// keep, and the block image): true where that freed anything but `b`.
+inline bool release_spare(bp_ctx* c, const Buf* b) {
+  bool any = false;
+  for (Buf* q : {&c->aligned, &c->blkimg}) {
+    if (!q->p || q == b) continue;
+    if (!any && cudaDeviceSynchronize() != cudaSuccess) return false;
+    cudaFree(q->p);
+    *q = Buf{};
+    any = true;
+  }
+  return any;
+}
+
+// ensure() for what a call needs: the spare workspaces make room for it.  Within a call
+// these come first, its own spare ones after them.
+inline cudaError_t ensure(bp_ctx* c, Buf& b, size_t bytes) {
+  cudaError_t e = ensure(b, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    if (release_spare(c, &b)) e = ensure(b, bytes);
+  }
+  return e;
+}
+
 inline bool is_host(const void* p) {
   if (!p) return false;
   cudaPointerAttributes a;
@@ -164,12 +189,12 @@ inline bool is_host(const void* p) {
 
 // Returns a device pointer holding `bytes` of the caller's array (copied to
 // `stage` when the caller's pointer is host memory).
-inline cudaError_t stage_in(Buf& stage, const void* p, size_t bytes, cudaStream_t s, const void** out) {
+inline cudaError_t stage_in(bp_ctx* c, Buf& stage, const void* p, size_t bytes, cudaStream_t s, const void** out) {
   if (!p || !is_host(p)) {
     *out = p;
     return cudaSuccess;
   }
-  cudaError_t e = ensure(stage, bytes);
+  cudaError_t e = ensure(c, stage, bytes);
   if (e != cudaSuccess) return e;
   e = cudaMemcpyAsync(stage.p, p, bytes, cudaMemcpyHostToDevice, s);
   *out = stage.p;
@@ -177,13 +202,13 @@ inline cudaError_t stage_in(Buf& stage, const void* p, size_t bytes, cudaStream_
 }
 
 // Device destination for an output (a staging buffer when it is host memory).
-inline cudaError_t stage_out(Buf& stage, void* p, size_t bytes, void** out, bool* host) {
+inline cudaError_t stage_out(bp_ctx* c, Buf& stage, void* p, size_t bytes, void** out, bool* host) {
   *host = p && is_host(p);
   if (!*host) {
     *out = p;
     return cudaSuccess;
   }
-  cudaError_t e = ensure(stage, bytes);
+  cudaError_t e = ensure(c, stage, bytes);
   *out = stage.p;
   return e;
 }
