@@ -110,25 +110,6 @@ int stage_views(bp_ctx* ctx, const bp_proj_desc* pd, const double* P, const doub
   return BP_OK;
 }
 
-// Run the FP64 composition into ctx->geom.
-int compose_views(bp_ctx* ctx, const bp_proj_desc* pd, const Views& dv, int weight,
-                  const VolInfo& vi, cudaStream_t s, const int** wide) {
-  const int V = pd->nviews;
-  // large problems choose the kernel variant per view on the device (two
-  // launches, one of which returns at once: ~3 us, so not for small ones)
-  *wide = nullptr;
-  bpk::FitInfo fit{pd->dtype, nullptr};
-  if ((long long)vi.nx * vi.ny * vi.nz * V >= (1LL << 28)) {
-    fit.wide = reinterpret_cast<int*>((ViewGeom*)ctx->geom.p + V);
-    *wide = fit.wide;
-  }
-  CK(TL(K_COMPOSE, 1, bpk::launch_compose(dv.P, dv.motion, dv.vw, dv.scale, V, weight == BP_WEIGHT_FDK,
-                                          pd->sid, vi, (ViewGeom*)ctx->geom.p, nullptr, s,
-                                          fit.wide ? &fit : nullptr)),
-     "compose");
-  return BP_OK;
-}
-
 // Whether a call on s is being captured.
 bool capturing(cudaStream_t s) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -159,20 +140,48 @@ bool ensure_spare(Buf& b, size_t bytes, cudaStream_t s) {
 // being captured (its graph would hold a workspace that a later, larger call
 // replaces).  Measured: BF16 rows of 401 pixels, 143 x 187 x 161 voxels x 111 views,
 // forward and both gradients 4.35 -> 3.42 ms.
-int align_rows(bp_ctx* ctx, const bp_proj_desc* pd, long long nvox, cudaStream_t s,
+// Returns whether dproj and pi now are the copy's, which compose_views makes.
+bool plan_copy(bp_ctx* ctx, const bp_proj_desc* pd, long long nvox, cudaStream_t s,
                const void** dproj, ProjInfo* pi) {
   const long long rows = (long long)pi->nviews * pi->nv, work = nvox * pi->nviews;
   if (bpk::stage_aligned(*dproj, pd->dtype, *pi) || work < (1LL << 22) || work < rows * pi->nu)
-    return BP_OK;
-  if (capturing(s)) return BP_OK;
+    return false;
   const long long es = pd->dtype == BP_F32 ? 4 : 2, rs = (pi->nu * es + 15) / 16 * 16 / es;
-  if (!ensure_spare(ctx->aligned, (size_t)(rows * rs * es), s)) return BP_OK;
-  CK(TL(K_ALIGN, 1, bpk::launch_align_rows(*dproj, pd->dtype, *pi, ctx->aligned.p, rs, s)),
-     "align rows");
+  if (capturing(s) || !ensure_spare(ctx->aligned, (size_t)(rows * rs * es), s)) return false;
   *dproj = ctx->aligned.p;
   pi->rs = rs;
   pi->vs = rs * pi->nv;
   pi->seq = 1;  // the sums of the motion gradient keep the order they have without the copy
+  return true;
+}
+
+// Run the FP64 composition into ctx->geom, flag the views that are wide where the call
+// chooses its kernel variant by that, and copy the stack `raw` to aligned rows where
+// copied (plan_copy).  proj: the stack that the call samples, NULL for none.
+int compose_views(bp_ctx* ctx, const bp_proj_desc* pd, const Views& dv, int weight,
+                  const VolInfo& vi, cudaStream_t s, const void* proj, const ProjInfo& pi,
+                  const bpk::RawStack& raw, bool copied, const int** wide) {
+  const int V = pd->nviews;
+  // Large problems choose the kernel variant on the device (two launches, one of which
+  // returns at once: 3 to 6 us, so not for small ones), and so do those of 2^22
+  // voxel-views whose detector is more than three times as wide as the volume has
+  // voxels, which mostly are scans of more than 3 px per voxel (64^3 x 200 at 4.8 px, rows
+  // of 351: both copied and staged in vain, exact motion VJP 0.253 -> 0.318 ms).
+  const long long work = (long long)vi.nx * vi.ny * vi.nz * V;
+  const bool choose = proj && bpk::stage_aligned(proj, pd->dtype, pi) &&
+                      (work >= (1LL << 28) ||
+                       (work >= (1LL << 22) && pd->nu > 3LL * (vi.nx > vi.ny ? vi.nx : vi.ny)));
+  bpk::FitInfo fit{pd->dtype, reinterpret_cast<int*>((ViewGeom*)ctx->geom.p + V)};
+  *wide = choose ? fit.wide : nullptr;
+  CK(TL(K_COMPOSE, 1, bpk::launch_compose(dv.P, dv.motion, dv.vw, dv.scale, V,
+                                          weight == BP_WEIGHT_FDK, pd->sid, vi,
+                                          (ViewGeom*)ctx->geom.p, nullptr, s,
+                                          choose ? &fit : nullptr)),
+     "compose");
+  if (copied)
+    CK(TL(K_ALIGN, 1, bpk::launch_align_rows(raw.proj, pd->dtype, raw.pi, ctx->aligned.p, pi.rs,
+                                             *wide, s)),
+       "align rows");
   return BP_OK;
 }
 
@@ -344,14 +353,16 @@ int bp_forward(bp_ctx* ctx, const void* proj, const bp_proj_desc* pdesc, const d
     Views dv;
     const int* wide;
     st = stage_views(ctx, pdesc, P, motion, view_weight, s, &dv);
-    if (!st) st = compose_views(ctx, pdesc, dv, weight, vi, s, &wide);
     if (st) return st;
     ProjInfo pi = make_projinfo(pdesc);
-    st = align_rows(ctx, pdesc, nvox, s, &dproj, &pi);
+    const bpk::RawStack raw{dproj, pi};
+    const bool copied = plan_copy(ctx, pdesc, nvox, s, &dproj, &pi);
+    st = compose_views(ctx, pdesc, dv, weight, vi, s, dproj, pi, raw, copied, &wide);
     if (st) return st;
     CK(TL(K_FORWARD, wide ? 2 : 1, bpk::launch_forward(dproj, pdesc->dtype, pi,
                                           (const ViewGeom*)ctx->geom.p, vi,
-                                          weight == BP_WEIGHT_FDK, (float*)dvol, wide, s)),
+                                          weight == BP_WEIGHT_FDK, (float*)dvol, wide, s,
+                                          copied ? &raw : nullptr)),
        "forward kernel");
   }
   if (host_vol) {
@@ -416,20 +427,19 @@ int bp_vjp(bp_ctx* ctx, const float* dL_dvol, const void* proj, const bp_proj_de
   const size_t blk_bytes = sizeof(float) * (size_t)bpk::block_image_floats(pi);
   bool blocks = fuse && !pi.seq && bpk::vjp_uses_blocks(dproj, pdesc->dtype, pi, exact);
   if (blocks) CK(ensure(ctx, ctx->blkimg, blk_bytes), "alloc block image");
-  if (want_geo) {
-    st = align_rows(ctx, pdesc, nvox, s, &dproj, &pi);
-    if (st) return st;
-    if (fuse && !blocks && bpk::vjp_uses_blocks(dproj, pdesc->dtype, pi, exact))
-      blocks = ensure_spare(ctx->blkimg, blk_bytes, s);
-  }
+  const bpk::RawStack raw{dproj, pi};
+  const bool copied = want_geo && plan_copy(ctx, pdesc, nvox, s, &dproj, &pi);
+  if (fuse && !blocks && bpk::vjp_uses_blocks(dproj, pdesc->dtype, pi, exact))
+    blocks = ensure_spare(ctx->blkimg, blk_bytes, s);
   const int* wide;
-  st = compose_views(ctx, pdesc, dv, weight, vi, s, &wide);
+  st = compose_views(ctx, pdesc, dv, weight, vi, s, dproj, pi, raw, copied, &wide);
   if (st) return st;
   if (dL_dproj) CK(cudaMemsetAsync(oD, 0, dproj_bytes, s), "zero dL_dproj");
   if (want_geo) {
     const float2* grad = nullptr;
     if (!exact) {
-      CK(TL(K_GRAD, 1, bpk::launch_grad_images(dproj, pdesc->dtype, pi, (float2*)ctx->grad.p, s)),
+      CK(TL(K_GRAD, 1, bpk::launch_grad_images(raw.proj, pdesc->dtype, raw.pi, (float2*)ctx->grad.p,
+                                            s)),
          "grad images");
       grad = (const float2*)ctx->grad.p;
     }
@@ -439,7 +449,8 @@ int bp_vjp(bp_ctx* ctx, const float* dL_dvol, const void* proj, const bp_proj_de
                                    (const ViewGeom*)ctx->geom.p, vi, weight == BP_WEIGHT_FDK,
                                    exact, (float*)ctx->partials.p,
                                    fuse ? (float*)oD : nullptr,
-                                   blocks ? (float*)ctx->blkimg.p : nullptr, wide, s)),
+                                   blocks ? (float*)ctx->blkimg.p : nullptr, wide, s,
+                                   copied ? &raw : nullptr)),
          "vjp kernel");
     }
     CK(TL(K_REDUCE, 1, bpk::launch_reduce_chain((const float*)ctx->partials.p, nvox > 0 ? ntiles : 0,

@@ -163,12 +163,19 @@ __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const C
   }
 }
 
+// Whether all n views are wide (all threads of the CTA).
+__device__ __forceinline__ bool all_wide(const int* __restrict__ wide, int n) {
+  bool w = true;
+  for (int j = threadIdx.x; j < n; j += blockDim.x) w = w && wide[j] != 0;
+  return __syncthreads_and(w);
+}
+
 template <int ZB, int ZS, int NS, typename T, bool FDK, int STAGE>
 __global__ void __launch_bounds__(NT, NS > FWD_NS ? 2 : FWD_MINB)
     forward_kernel(const T* __restrict__ proj, const __grid_constant__ CUtensorMap map, ProjInfo pi,
                    const ViewGeom* __restrict__ geom, VolInfo vi, float* __restrict__ vol,
                    const int* __restrict__ wide) {
-  if (wide && (wide[0] != 0) == (STAGE != STAGE_NONE)) return;  // the other variant's launch
+  if (wide && all_wide(wide, pi.nviews) == (STAGE != STAGE_NONE)) return;  // the other's launch
   __shared__ TileView tvs[2][batch_records<STAGE>()];
   __shared__ StagePipe<NS> pipe;
   extern __shared__ __align__(128) unsigned char dyn_smem[];
@@ -184,32 +191,38 @@ __global__ void __launch_bounds__(NT, NS > FWD_NS ? 2 : FWD_MINB)
 constexpr int ZB_FWD = 16;
 
 // Staging needs 16-byte aligned rows; their length does not matter (TMA fills
-// with zeros beyond it).
+// with zeros beyond it).  A tensor map's strides are below 2^40 bytes.
 bool stage_aligned(const void* proj, int dtype, const ProjInfo& pi) {
   const long long es = dtype == 0 ? 4 : 2;
   return ((reinterpret_cast<uintptr_t>(proj) & 15) == 0) && (pi.rs * es) % 16 == 0 &&
-         (pi.vs * es) % 16 == 0;
+         (pi.vs * es) % 16 == 0 && pi.vs * es < (1LL << 40);
 }
 template <typename U>
 __global__ void __launch_bounds__(256)
-    align_rows_kernel(const U* __restrict__ src, ProjInfo pi, U* __restrict__ dst, long long rs) {
-  const long long row = blockIdx.x;  // one CTA per detector row
-  const long long j = row / pi.nv, b = row - j * pi.nv;
-  const U* p = src + j * pi.vs + b * pi.rs;
-  U* q = dst + row * rs;
-  for (int a = threadIdx.x; a < pi.nu; a += blockDim.x) q[a] = p[a];
+    align_rows_kernel(const U* __restrict__ src, ProjInfo pi, U* __restrict__ dst, long long rs,
+                      const int* __restrict__ wide) {
+  if (wide && all_wide(wide, pi.nviews)) return;
+  const long long rows = (long long)pi.nviews * pi.nv;
+  for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
+    const long long j = row / pi.nv, b = row - j * pi.nv;
+    const U* p = src + j * pi.vs + b * pi.rs;
+    U* q = dst + row * rs;
+    for (int a = threadIdx.x; a < pi.nu; a += blockDim.x) q[a] = p[a];
+  }
 }
 
 cudaError_t launch_align_rows(const void* proj, int dtype, const ProjInfo& pi, void* dst,
-                              long long rs, cudaStream_t s) {
+                              long long rs, const int* wide, cudaStream_t s) {
   const long long rows = (long long)pi.nviews * pi.nv;
   if (rows <= 0 || pi.nu <= 0) return cudaSuccess;
-  if (rows > 0x7fffffffLL) return cudaErrorInvalidValue;
+  // CTAs loop over rows where each reads the flags first, else one CTA per row
+  const unsigned ctas =
+      (unsigned)(wide ? (rows < 152 * 16 ? rows : 152 * 16) : (rows < 0x7fffffff ? rows : 0x7fffffff));
   if (dtype == 0)
-    align_rows_kernel<<<(unsigned)rows, 256, 0, s>>>((const unsigned*)proj, pi, (unsigned*)dst, rs);
+    align_rows_kernel<<<ctas, 256, 0, s>>>((const unsigned*)proj, pi, (unsigned*)dst, rs, wide);
   else
-    align_rows_kernel<<<(unsigned)rows, 256, 0, s>>>((const unsigned short*)proj, pi,
-                                                     (unsigned short*)dst, rs);
+    align_rows_kernel<<<ctas, 256, 0, s>>>((const unsigned short*)proj, pi, (unsigned short*)dst, rs,
+                                           wide);
   return cudaGetLastError();
 }
 
@@ -259,7 +272,8 @@ cudaError_t make_stage_map(const void* proj, int dtype, const ProjInfo& pi, CUte
 
 template <int ZS, int NS, typename T, bool FDK>
 static cudaError_t forward_launch(const void* proj, const ProjInfo& pi, const ViewGeom* geom,
-                                  const VolInfo& vi, float* vol, const int* wide, cudaStream_t s) {
+                                  const VolInfo& vi, float* vol, const int* wide, cudaStream_t s,
+                                  const RawStack* raw) {
   const int nblocks = vi.tiles_x * vi.tiles_y * vi.tiles_z * (ZB_FWD / ZS);
   CUtensorMap map{};
   if (wide == WIDE_HALF && stageable<T>(proj, pi) &&
@@ -284,8 +298,8 @@ static cudaError_t forward_launch(const void* proj, const ProjInfo& pi, const Vi
     e = cudaGetLastError();
     if (e != cudaSuccess || !sel) return e;
   }
-  forward_kernel<ZB_FWD, ZS, FWD_NS, T, FDK, STAGE_NONE>
-      <<<nblocks, NT, 0, s>>>((const T*)proj, map, pi, geom, vi, vol, sel);
+  forward_kernel<ZB_FWD, ZS, FWD_NS, T, FDK, STAGE_NONE><<<nblocks, NT, 0, s>>>(
+      (const T*)(raw ? raw->proj : proj), map, raw ? raw->pi : pi, geom, vi, vol, sel);
   return cudaGetLastError();
 }
 
@@ -300,14 +314,14 @@ constexpr int FWD_NS_FEW = 4;
 
 template <typename T, bool FDK>
 static cudaError_t forward_dispatch(const void* proj, const ProjInfo& pi, const ViewGeom* geom,
-                                    const VolInfo& vi, float* vol, const int* wide,
-                                    cudaStream_t s) {
+                                    const VolInfo& vi, float* vol, const int* wide, cudaStream_t s,
+                                    const RawStack* raw) {
   const int n = vi.tiles_x * vi.tiles_y * vi.tiles_z;
   if (n <= FWD_FEW_TILES)
-    return forward_launch<8, FWD_NS_FEW, T, FDK>(proj, pi, geom, vi, vol, wide, s);
+    return forward_launch<8, FWD_NS_FEW, T, FDK>(proj, pi, geom, vi, vol, wide, s, raw);
   if (n <= FWD_SOME_TILES)
-    return forward_launch<8, FWD_NS, T, FDK>(proj, pi, geom, vi, vol, wide, s);
-  return forward_launch<16, FWD_NS, T, FDK>(proj, pi, geom, vi, vol, wide, s);
+    return forward_launch<8, FWD_NS, T, FDK>(proj, pi, geom, vi, vol, wide, s, raw);
+  return forward_launch<16, FWD_NS, T, FDK>(proj, pi, geom, vi, vol, wide, s, raw);
 }
 
 template <typename T, bool FDK>
@@ -334,18 +348,18 @@ cudaError_t prepare_forward(int dtype, int fdk) {
 
 cudaError_t launch_forward(const void* proj, int dtype, const ProjInfo& pi, const ViewGeom* geom,
                            const VolInfo& vi_in, int fdk, float* vol, const int* wide,
-                           cudaStream_t s) {
+                           cudaStream_t s, const RawStack* raw) {
   VolInfo vi = vi_in;  // the forward tiles z by ZB_FWD
   vi.zb = ZB_FWD;
   vi.tiles_z = (vi.nz + ZB_FWD - 1) / ZB_FWD;
   if (dtype == 0)
-    return fdk ? forward_dispatch<float, true>(proj, pi, geom, vi, vol, wide, s)
-               : forward_dispatch<float, false>(proj, pi, geom, vi, vol, wide, s);
+    return fdk ? forward_dispatch<float, true>(proj, pi, geom, vi, vol, wide, s, raw)
+               : forward_dispatch<float, false>(proj, pi, geom, vi, vol, wide, s, raw);
   if (dtype == 1)
-    return fdk ? forward_dispatch<__half, true>(proj, pi, geom, vi, vol, wide, s)
-               : forward_dispatch<__half, false>(proj, pi, geom, vi, vol, wide, s);
-  return fdk ? forward_dispatch<__nv_bfloat16, true>(proj, pi, geom, vi, vol, wide, s)
-             : forward_dispatch<__nv_bfloat16, false>(proj, pi, geom, vi, vol, wide, s);
+    return fdk ? forward_dispatch<__half, true>(proj, pi, geom, vi, vol, wide, s, raw)
+               : forward_dispatch<__half, false>(proj, pi, geom, vi, vol, wide, s, raw);
+  return fdk ? forward_dispatch<__nv_bfloat16, true>(proj, pi, geom, vi, vol, wide, s, raw)
+             : forward_dispatch<__nv_bfloat16, false>(proj, pi, geom, vi, vol, wide, s, raw);
 }
 
 cudaError_t bounds_status_forward(unsigned* flags, long long* first, int op, cudaStream_t s) {

@@ -89,8 +89,10 @@ struct ProjInfo {
 // most half tiles fit the wider half-tile buffers.  `wide` of launch_forward and
 // launch_vjp_motion: NULL, take the staged variant; WIDE_ALL, take the one that
 // reads global memory; WIDE_HALF, stage half tiles (the same job: 59.9 -> 47.0 ms);
-// else one flag per view on the device (launch_compose, fit): the first two are launched and each item runs in
-// the one that suits its first view.
+// else one flag per view on the device (launch_compose, fit): the first two are launched
+// and an item (a forward, a VJP's chunk of views) runs in the one that reads global memory
+// if all its views are wide.  (One that is not takes twice as long there; wide ones among
+// others lose little in the staged variant.)
 struct FitInfo {
   int dtype;
   int* wide;  // [V]
@@ -111,10 +113,16 @@ const int* scan_variant(const double* P, int V, int dtype, const VolInfo& vi);
 
 
 // Whether the staging copies can read a stack (16-byte aligned data and strides),
-// and a copy of one with a row pitch of rs elements.
+// and a copy of one with a row pitch of rs elements (left out if all views are wide).
+// Where such a copy is given to launch_forward or launch_vjp_motion, RawStack is the
+// stack itself, for the variant that reads global memory.
+struct RawStack {
+  const void* proj;
+  ProjInfo pi;
+};
 bool stage_aligned(const void* proj, int dtype, const ProjInfo& pi);
 cudaError_t launch_align_rows(const void* proj, int dtype, const ProjInfo& pi, void* dst,
-                              long long rs, cudaStream_t s);
+                              long long rs, const int* wide, cudaStream_t s);
 // The tensor map that the staging copies read.  half: boxes of the half-tile buffers.
 cudaError_t make_stage_map(const void* proj, int dtype, const ProjInfo& pi, CUtensorMap* map,
                            bool half);
@@ -123,7 +131,7 @@ void stage_extent(int dtype, bool half, int* cols, int* rows);
 
 cudaError_t launch_forward(const void* proj, int dtype, const ProjInfo& pi, const ViewGeom* geom,
                            const VolInfo& vi, int fdk, float* vol, const int* wide,
-                           cudaStream_t s);
+                           cudaStream_t s, const RawStack* raw = nullptr);
 // Set the forward / motion-VJP kernels' shared-memory attributes on the
 // current device (done by the first launch anyway; call before capturing a
 // graph).
@@ -142,7 +150,7 @@ cudaError_t launch_grad_images(const void* proj, int dtype, const ProjInfo& pi, 
 cudaError_t launch_vjp_motion(const float* dvol, const void* proj, int dtype, const ProjInfo& pi,
                               const float2* grad, const ViewGeom* geom, const VolInfo& vi,
                               int fdk, int exact, float* partials, float* dproj, float* blk,
-                              const int* wide, cudaStream_t s);
+                              const int* wide, cudaStream_t s, const RawStack* raw = nullptr);
 long long block_image_floats(const ProjInfo& pi);
 bool vjp_uses_blocks(const void* proj, int dtype, const ProjInfo& pi, int exact);
 

@@ -129,7 +129,7 @@ template <typename T, bool FDK, bool EXACT, bool PROJ>
 cudaError_t vjp_variants(const float* dvol, const void* proj, const ProjInfo& pi,
                          const float2* grad, const ViewGeom* geom, const VolInfo& vi,
                          float* partials, float* dproj, float* blk, int vc, unsigned nblocks,
-                         const int* wide, cudaStream_t s);
+                         const int* wide, cudaStream_t s, const RawStack* raw);
 template <typename T, bool FDK, bool EXACT>
 cudaError_t prepare_vjp_t();
 
@@ -161,7 +161,7 @@ template <typename T, bool FDK, bool EXACT>
 static cudaError_t vjp_dispatch(const float* dvol, const void* proj, const ProjInfo& pi,
                                 const float2* grad, const ViewGeom* geom, const VolInfo& vi,
                                 float* partials, float* dproj, float* blk, const int* wide,
-                                cudaStream_t s) {
+                                cudaStream_t s, const RawStack* raw) {
   const int ntiles = vi.tiles_x * vi.tiles_y * vi.tiles_z;
   // block images only where the staged CENTRAL paths scatter
   const bool useb = dproj && blk && stageable<T>(proj, pi) && !EXACT && BP_VJP_BLOCKS;
@@ -173,12 +173,12 @@ static cudaError_t vjp_dispatch(const float* dvol, const void* proj, const ProjI
   const unsigned nblocks = (unsigned)((long long)ntiles * ((pi.nviews + vc - 1) / vc));
   if (!dproj)
     return vjp_variants<T, FDK, EXACT, false>(dvol, proj, pi, grad, geom, vi, partials, nullptr,
-                                              nullptr, vc, nblocks, wide, s);
+                                              nullptr, vc, nblocks, wide, s, raw);
   cudaError_t e = cudaSuccess;
   if (useb) e = cudaMemsetAsync(blk, 0, sizeof(float) * (size_t)block_image_floats(pi), s);
   if (e == cudaSuccess)
     e = vjp_variants<T, FDK, EXACT, true>(dvol, proj, pi, grad, geom, vi, partials, dproj,
-                                          useb ? blk : nullptr, vc, nblocks, wide, s);
+                                          useb ? blk : nullptr, vc, nblocks, wide, s, raw);
   if (e == cudaSuccess && useb) e = launch_block_combine(blk, pi, dproj, s);
   return e;
 }
@@ -210,31 +210,31 @@ template <typename T>
 static cudaError_t vjp_dispatch_t(int fdk, int exact, const float* dvol, const void* proj,
                                   const ProjInfo& pi, const float2* grad, const ViewGeom* geom,
                                   const VolInfo& vi, float* partials, float* dproj,
-                                  float* blk, const int* wide, cudaStream_t s) {
+                                  float* blk, const int* wide, cudaStream_t s, const RawStack* raw) {
   if (fdk)
     return exact ? vjp_dispatch<T, true, true>(dvol, proj, pi, grad, geom, vi, partials, dproj,
-                                               blk, wide, s)
+                                               blk, wide, s, raw)
                  : vjp_dispatch<T, true, false>(dvol, proj, pi, grad, geom, vi, partials, dproj,
-                                                blk, wide, s);
+                                                blk, wide, s, raw);
   return exact ? vjp_dispatch<T, false, true>(dvol, proj, pi, grad, geom, vi, partials, dproj,
-                                              blk, wide, s)
+                                              blk, wide, s, raw)
                : vjp_dispatch<T, false, false>(dvol, proj, pi, grad, geom, vi, partials, dproj,
-                                               blk, wide, s);
+                                               blk, wide, s, raw);
 }
 
 cudaError_t launch_vjp_motion(const float* dvol, const void* proj, int dtype, const ProjInfo& pi,
                               const float2* grad, const ViewGeom* geom, const VolInfo& vi,
                               int fdk, int exact, float* partials, float* dproj, float* blk,
-                              const int* wide, cudaStream_t s) {
+                              const int* wide, cudaStream_t s, const RawStack* raw) {
   if (vi.zb != ZB_VJP) return cudaErrorInvalidValue;
   if (dtype == 0)
     return vjp_dispatch_t<float>(fdk, exact, dvol, proj, pi, grad, geom, vi, partials, dproj, blk,
-                                 wide, s);
+                                 wide, s, raw);
   if (dtype == 1)
     return vjp_dispatch_t<__half>(fdk, exact, dvol, proj, pi, grad, geom, vi, partials, dproj,
-                                  blk, wide, s);
+                                  blk, wide, s, raw);
   return vjp_dispatch_t<__nv_bfloat16>(fdk, exact, dvol, proj, pi, grad, geom, vi, partials,
-                                       dproj, blk, wide, s);
+                                       dproj, blk, wide, s, raw);
 }
 
 // ------------------------------------------------- VJP w.r.t. the data

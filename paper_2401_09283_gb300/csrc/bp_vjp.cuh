@@ -1003,10 +1003,11 @@ __global__ void __launch_bounds__(NT, NS > VJP_NS ? 2 : VJP_MINB)
                       const float2* __restrict__ grad, const ViewGeom* __restrict__ geom,
                       VolInfo vi, float* __restrict__ partials, float* __restrict__ dproj,
                       float* __restrict__ dblk, int vchunk, const int* __restrict__ wide) {
-  // the other variant's launch takes this item
-  if (wide && (wide[blockIdx.x / (vi.tiles_x * vi.tiles_y * vi.tiles_z) * vchunk] != 0) ==
-                  (STAGE != STAGE_NONE))
-    return;
+  if (wide) {  // are all views of the chunk (at most 32) wide?
+    const int j = blockIdx.x / (vi.tiles_x * vi.tiles_y * vi.tiles_z) * vchunk + (threadIdx.x & 31);
+    const bool w = (int)(threadIdx.x & 31) >= vchunk || j >= pi.nviews || wide[j] != 0;
+    if (__all_sync(0xffffffffu, w) == (STAGE != STAGE_NONE)) return;  // the other's launch
+  }
   __shared__ TileView tvs[2][batch_records<STAGE>()];
   __shared__ float red[NS][NT / 32][12];
   __shared__ StagePipe<NS> pipe;
@@ -1041,7 +1042,8 @@ template <typename T, bool FDK, bool EXACT, bool PROJ>
 cudaError_t vjp_variants(const float* dvol, const void* proj, const ProjInfo& pi,
                                 const float2* grad, const ViewGeom* geom, const VolInfo& vi,
                                 float* partials, float* dproj, float* blk, int vc,
-                                unsigned nblocks, const int* wide, cudaStream_t s) {
+                                unsigned nblocks, const int* wide, cudaStream_t s,
+                                const RawStack* raw) {
   CUtensorMap map{};
   if constexpr (!EXACT && !PROJ) {
     if (wide == WIDE_HALF && stageable<T>(proj, pi) &&
@@ -1061,8 +1063,9 @@ cudaError_t vjp_variants(const float* dvol, const void* proj, const ProjInfo& pi
                   dvol, proj, map, pi, grad, geom, vi, partials, dproj, blk, vc, nblocks, sel, s);
     if (e != cudaSuccess || !sel) return e;
   }
-  return vjp_launch<VJP_NS, T, FDK, EXACT, PROJ, STAGE_NONE>(dvol, proj, map, pi, grad, geom, vi, partials,
-                                                        dproj, nullptr, vc, nblocks, sel, s);
+  return vjp_launch<VJP_NS, T, FDK, EXACT, PROJ, STAGE_NONE>(
+      dvol, raw ? raw->proj : proj, map, raw ? raw->pi : pi, grad, geom, vi, partials, dproj, nullptr,
+      vc, nblocks, sel, s);
 }
 
 template <typename T, bool FDK, bool EXACT>
@@ -1084,7 +1087,7 @@ cudaError_t prepare_vjp_t() {
 #define BP_VJP_VARIANT(T, FDK, EXACT, PROJ)                                                       \
   template cudaError_t vjp_variants<T, FDK, EXACT, PROJ>(                                         \
       const float*, const void*, const ProjInfo&, const float2*, const ViewGeom*, const VolInfo&, \
-      float*, float*, float*, int, unsigned, const int*, cudaStream_t);
+      float*, float*, float*, int, unsigned, const int*, cudaStream_t, const RawStack*);
 #define BP_VJP_VARIANTS(EXACT, PROJ)            \
   BP_VJP_VARIANT(float, false, EXACT, PROJ)     \
   BP_VJP_VARIANT(float, true, EXACT, PROJ)      \
