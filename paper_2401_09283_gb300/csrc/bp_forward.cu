@@ -298,8 +298,12 @@ static cudaError_t forward_launch(const void* proj, const ProjInfo& pi, const Vi
     e = cudaGetLastError();
     if (e != cudaSuccess || !sel) return e;
   }
-  forward_kernel<ZB_FWD, ZS, FWD_NS, T, FDK, STAGE_NONE><<<nblocks, NT, 0, s>>>(
-      (const T*)(raw ? raw->proj : proj), map, raw ? raw->pi : pi, geom, vi, vol, sel);
+  // From global memory half tiles throughout: a warp's taps of one view are then closer
+  // together in the L1 cache (128^3 x 200 at 4.8 px per voxel 1.061 -> 0.957 ms, 256^3 x
+  // 120 at 1.5 px, three iterations with the VJP, 29.3 -> 28.7).
+  forward_kernel<ZB_FWD, 8, FWD_NS, T, FDK, STAGE_NONE>
+      <<<vi.tiles_x * vi.tiles_y * vi.tiles_z * (ZB_FWD / 8), NT, 0, s>>>(
+          (const T*)(raw ? raw->proj : proj), map, raw ? raw->pi : pi, geom, vi, vol, sel);
   return cudaGetLastError();
 }
 
