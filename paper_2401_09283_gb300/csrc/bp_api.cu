@@ -164,13 +164,13 @@ int compose_views(bp_ctx* ctx, const bp_proj_desc* pd, const Views& dv, int weig
   const int V = pd->nviews;
   // Large problems choose the kernel variant on the device (two launches, one of which
   // returns at once: 3 to 6 us, so not for small ones), and so do those of 2^22
-  // voxel-views whose detector is more than three times as wide as the volume has
-  // voxels, which mostly are scans of more than 3 px per voxel (64^3 x 200 at 4.8 px, rows
+  // voxel-views whose detector is more than four times as wide as the volume has
+  // voxels, which mostly are scans of more than 4 px per voxel (64^3 x 200 at 4.8 px, rows
   // of 351: both copied and staged in vain, exact motion VJP 0.253 -> 0.318 ms).
   const long long work = (long long)vi.nx * vi.ny * vi.nz * V;
   const bool choose = proj && bpk::stage_aligned(proj, pd->dtype, pi) &&
                       (work >= (1LL << 28) ||
-                       (work >= (1LL << 22) && pd->nu > 3LL * (vi.nx > vi.ny ? vi.nx : vi.ny)));
+                       (work >= (1LL << 22) && pd->nu > 4LL * (vi.nx > vi.ny ? vi.nx : vi.ny)));
   bpk::FitInfo fit{pd->dtype, reinterpret_cast<int*>((ViewGeom*)ctx->geom.p + V)};
   *wide = choose ? fit.wide : nullptr;
   CK(TL(K_COMPOSE, 1, bpk::launch_compose(dv.P, dv.motion, dv.vw, dv.scale, V,

@@ -48,7 +48,7 @@ def test_chosen_variants_agree_with_the_global_one(kind, deriv, dtype):
     cfg, P, th, proj, delta, origin = scan(kind, 181)
     stored = torch.as_tensor(proj).to(dtype)
     used, shape, vw = stored.double().numpy(), delta.shape, np.full(len(P), 0.02)
-    assert delta.size * len(P) >= 1 << 22 and 181 > 3 * 42
+    assert delta.size * len(P) >= 1 << 22 and 181 > 4 * 42
     p, Pd, thd, vwd, dv = (torch.as_tensor(x, device=DEV) for x in (stored, P, th, vw, delta))
     geo = dict(spacing=(1.0,) * 3, origin=origin, view_weight=vwd, sid=cfg.sid)
 
