@@ -47,20 +47,25 @@ struct FdkTables {
         red(ramp + 2 * ((size_t)nu + 2 * (size_t)ext) - 1) {}
 };
 
-constexpr int RED_VIEWS = 8;  // views per thread of the redundancy table
+// The tables' FP64 functions: a warp's instruction takes 16 cycles of an SM's pipe, and
+// one weight is a chain of some hundred.  Small tables are spread over as many SMs as
+// possible (CTAs of two warps) and take one view per thread; large ones share the fan
+// angle's atan between eight.  13 views of 72 x 105, whole filter: 32.9 us with eight
+// views per thread in CTAs of 256, 24.7 with one, 22.7 with one in CTAs of 64.
+constexpr int RED_VIEWS = 8, TABLE_THREADS = 64;
 
 // [nvh][nuh] (high, low) FP32 parts of the cosine weight, then h[m + ne - 1] for
 // |m| < ne = nu + 2 ext, then the redundancy weight of (view j, column a) at
 // j nu + a.
 __global__ void fdk_tables_kernel(int V, int nu, int nv, int ext, double pitch, double sid,
-                                  double sdd, double arc, float* __restrict__ tab) {
+                                  double sdd, double arc, int rv, float* __restrict__ tab) {
   const double tau = pitch * sid / sdd;
   const bool full = arc >= 2.0 * kPi - 1e-12;
   const double dbeta = full ? arc / V : (V > 1 ? arc / (V - 1) : 0.0);
   const int ne = nu + 2 * ext;
   const FdkTables T(nu, nv, ext);
   const long long nc = (long long)T.nuh * T.nvh, nh = 2LL * ne - 1;
-  const long long nr = (long long)((V + RED_VIEWS - 1) / RED_VIEWS) * nu;
+  const long long nr = (long long)((V + rv - 1) / rv) * nu;  // rv views per thread
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nc + nh + nr;
        e += (long long)gridDim.x * blockDim.x) {
     if (e < nc) {
@@ -74,29 +79,29 @@ __global__ void fdk_tables_kernel(int V, int nu, int nv, int ext, double pitch, 
       tab[T.ramp + (e - nc)] = (float)(-2.0 / (kPi * kPi * tau * tau * (4.0 * m * m - 1.0)));
     } else {
       const long long q = e - nc - nh;
-      const int j0 = (int)(q / nu) * RED_VIEWS, a = (int)(q % nu);
+      const int j0 = (int)(q / nu) * rv, a = (int)(q % nu);
       const double g = full ? 0.0 : atan((a - 0.5 * (nu - 1)) * pitch / sdd);
-      for (int j = j0; j < min(V, j0 + RED_VIEWS); ++j)
+      for (int j = j0; j < min(V, j0 + rv); ++j)
         tab[T.red + (size_t)j * nu + a] = full ? 0.5f : (float)parker_w(j * dbeta, g, arc);
     }
   }
 }
 
 constexpr int ROWS = 4;        // detector rows of a group, interleaved as float4
-constexpr int OUT = 8;         // consecutive outputs per thread
 constexpr int MAX_GROUPS = 8;  // groups per CTA
 constexpr int MAX_THREADS = 512;
 
 // The ramp in shared memory, element m at m + m / 8, shifted by `shift` so that
 // the taps of one block of eight steps lie in one such run: the lanes' loads
 // (eight elements apart) fall in different banks and their offsets are immediates.
+// (With two outputs per thread a block of two steps lies in one.)
 struct RampLayout {
   int c, shift, n;  // index of output 0's first tap; elements
   __host__ __device__ RampLayout(int nu, int ext) {
     const int c0 = ext + (nu + 2 * ext) - 1;
     shift = (7 - c0) & 7;
     c = c0 + shift;
-    n = (nu + OUT - 1) / OUT * OUT + c;
+    n = (nu + 7) / 8 * 8 + c;
   }
   __host__ __device__ static int at(int m) { return m + (m >> 3); }
 };
@@ -123,8 +128,12 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
 // unrolling).  One output of 4 rows per thread loaded 20 bytes for four FMAs.
 // The cosine weight comes from a table as a pair of FP32 values, not from an FP64
 // square root and division per pixel and view (2 FP64 lanes per clock and SM).
-// 248 x 480 rows of 616: 3.76 -> 1.90 ms, the FMAs alone take 1.2 ms (1.93 at 78
-// registers and two CTAs per SM; 2.14 with 8 rows per thread and 126 registers).
+// 248 x 480 rows of 616: 3.74 -> 1.73 ms, the FMAs alone take 1.2 ms (without the
+// compiler's own choice of registers, 78 and two CTAs per SM, 1.5 % more; with 8 rows
+// per thread and 126 registers 13 % more).
+// OUT = 2 for problems of few outputs, whose threads are a serial chain of nu taps each
+// while most of the chip is idle.
+template <int OUT>
 __global__ void __launch_bounds__(MAX_THREADS, 2)
     fdk_conv_kernel(const float* __restrict__ raw, int nu, int nv, int ext, int G, float tau,
                     const float* __restrict__ tab, float* __restrict__ out) {
@@ -179,7 +188,7 @@ __global__ void __launch_bounds__(MAX_THREADS, 2)
 #pragma unroll
     for (int i = 0; i < OUT; ++i) acc[i][0] = acc[i][1] = splat2(0.0f);
 #pragma unroll
-    for (int i = 1; i < OUT; ++i) w[i] = splat2(hb[1 + i]);
+    for (int i = 1; i < OUT; ++i) w[i] = splat2(h[RampLayout::at(a0 + L.c + i)]);
 #pragma unroll 1
     for (int kk = 0; kk + OUT <= ne; kk += OUT) {
 #pragma unroll
@@ -192,7 +201,7 @@ __global__ void __launch_bounds__(MAX_THREADS, 2)
           acc[i][1] = fma2(w[(i - q + OUT) % OUT], x.y, acc[i][1]);
         }
       }
-      hb -= OUT + 1;
+      hb = OUT == 8 ? hb - 9 : h + RampLayout::at(a0 + L.c - kk - OUT);
     }
 #pragma unroll 1
     for (int kk = ne / OUT * OUT; kk < ne; ++kk) {
@@ -215,9 +224,10 @@ __global__ void __launch_bounds__(MAX_THREADS, 2)
         const f2 a = acc[i][r / 2];
         s[i] = tau * __uint_as_float((unsigned)(r % 2 ? a >> 32 : a));
       }
-      if (nu % 4 == 0 && a0 + OUT <= nu && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
-        reinterpret_cast<float4*>(o)[0] = make_float4(s[0], s[1], s[2], s[3]);
-        reinterpret_cast<float4*>(o)[1] = make_float4(s[4], s[5], s[6], s[7]);
+      if (OUT == 8 && nu % 4 == 0 && a0 + OUT <= nu &&
+          (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+        reinterpret_cast<float4*>(o)[0] = make_float4(s[0], s[1], s[2 % OUT], s[3 % OUT]);
+        reinterpret_cast<float4*>(o)[1] = make_float4(s[4 % OUT], s[5 % OUT], s[6 % OUT], s[7 % OUT]);
       } else {
 #pragma unroll
         for (int i = 0; i < OUT; ++i)
@@ -233,28 +243,23 @@ size_t conv_smem(int nu, int ext, int G) {
          sizeof(float) * (size_t)(RampLayout::at(L.n) + 1);
 }
 
-}  // namespace
+// Threads' work (groups of four rows x eight outputs) below which a thread takes two
+// outputs, four warps on each SM, and the row length up to which it does: longer rows
+// take more than one turn of a CTA.  Whole filter, us, one output per thread at first /
+// eight / two: 13 x 72 x 105 (views, rows, columns) 22.7 / 22.7 / 17.7, 4 x 54 x 96 18.6 /
+// 21.6 / 17.7, 1 x 480 x 616 49.3 / 54.4 / 43.0; but 2 x 20 x 1200 113 / 75 / 84.
+constexpr long long FEW_ITEMS = 152 * 32 * 4;
+constexpr int FEW_NU = 768;
 
-size_t fdk_table_floats(int V, int nu, int nv, int ext) {
-  return FdkTables(nu, nv, ext).red + (size_t)V * nu;
-}
-
-cudaError_t launch_fdk_filter(const float* raw, int V, int nv, int nu, int ext, double pitch,
-                              double sid, double sdd, double arc, float* tab, float* out,
-                              cudaStream_t s) {
-  if (V == 0 || nv == 0) return cudaSuccess;
-  const long long n = (long long)fdk_table_floats(V, nu, nv, ext);
-  long long nb = (n + 255) / 256;
-  if (nb > 152 * 16) nb = 152 * 16;
-  fdk_tables_kernel<<<(int)nb, 256, 0, s>>>(V, nu, nv, ext, pitch, sid, sdd, arc, tab);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+template <int OUT>
+cudaError_t conv_launch(const float* raw, int V, int nv, int nu, int ext, double pitch, double sid,
+                        double sdd, const float* tab, float* out, cudaStream_t s) {
   // Groups per CTA: the share of busy threads (whole warps, whole CTAs), best
   // within 56 KiB of shared memory, so that several CTAs are resident.
   const int nt = (nu + OUT - 1) / OUT, groups = (nv + ROWS - 1) / ROWS;
   int G = 1, threads = 0;
   double best = 0.0;
-  for (int g = 1; g <= MAX_GROUPS && g <= groups; ++g) {
+  for (int g = 1; g <= (OUT == 8 ? MAX_GROUPS : 1) && g <= groups; ++g) {
     if (g > 1 && conv_smem(nu, ext, g) > 56 * 1024) break;
     const int t = (g * nt + 31) / 32 * 32 < MAX_THREADS ? (g * nt + 31) / 32 * 32 : MAX_THREADS;
     const int ctas = (groups + g - 1) / g, turns = (g * nt + t - 1) / t;
@@ -267,14 +272,39 @@ cudaError_t launch_fdk_filter(const float* raw, int V, int nv, int nu, int ext, 
   }
   const size_t smem = conv_smem(nu, ext, G);
   if (smem > 48 * 1024) {  // the same limit in every call: calls in other threads agree
-    e = cudaFuncSetAttribute(fdk_conv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             227 * 1024);
+    const cudaError_t e = cudaFuncSetAttribute(
+        fdk_conv_kernel<OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
   }
   dim3 grid((groups + G - 1) / G, V);
-  fdk_conv_kernel<<<grid, threads, smem, s>>>(raw, nu, nv, ext, G, (float)(pitch * sid / sdd), tab,
-                                              out);
+  fdk_conv_kernel<OUT><<<grid, threads, smem, s>>>(raw, nu, nv, ext, G, (float)(pitch * sid / sdd),
+                                                   tab, out);
   return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t fdk_table_floats(int V, int nu, int nv, int ext) {
+  return FdkTables(nu, nv, ext).red + (size_t)V * nu;
+}
+
+cudaError_t launch_fdk_filter(const float* raw, int V, int nv, int nu, int ext, double pitch,
+                              double sid, double sdd, double arc, float* tab, float* out,
+                              cudaStream_t s) {
+  if (V == 0 || nv == 0) return cudaSuccess;
+  const long long n = (long long)fdk_table_floats(V, nu, nv, ext);
+  long long nb = (n + TABLE_THREADS - 1) / TABLE_THREADS, rv = (long long)V * nu / 16384;
+  if (nb > 152 * 64) nb = 152 * 64;
+  rv = rv < 1 ? 1 : rv > RED_VIEWS ? RED_VIEWS : rv;
+  fdk_tables_kernel<<<(int)nb, TABLE_THREADS, 0, s>>>(V, nu, nv, ext, pitch, sid, sdd, arc, (int)rv,
+                                                      tab);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  // few outputs: two per thread, so that four warps per SM have work
+  const long long items = (long long)V * ((nv + ROWS - 1) / ROWS) * ((nu + 7) / 8);
+  return items < FEW_ITEMS && nu <= FEW_NU
+             ? conv_launch<2>(raw, V, nv, nu, ext, pitch, sid, sdd, tab, out, s)
+             : conv_launch<8>(raw, V, nv, nu, ext, pitch, sid, sdd, tab, out, s);
 }
 
 }  // namespace bpk
