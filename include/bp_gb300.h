@@ -180,8 +180,8 @@ int bp_forward(bp_ctx* ctx, const void* proj, const bp_proj_desc* pdesc, const d
  *               aligned copy (scratch of the context, one stack) that large
  *               calls on unaligned rows make: both are taken only after
  *               everything that the call needs, if they leave three quarters
- *               of the free memory, and given back when a later call or job
- *               has no room.
+ *               of the free memory, and the copy is given back when a later
+ *               call or job has no room.
  * Any output may be NULL to skip it (dL_dmotion needs motion or treats it as
  * zero).  With BP_WEIGHT_FDK the derivative of (sid/w)^2 is included. */
 int bp_vjp(bp_ctx* ctx, const float* dL_dvol, const void* proj, const bp_proj_desc* pdesc,

@@ -151,27 +151,22 @@ inline cudaError_t ensure(Buf& b, size_t bytes) {
   return cudaSuccess;
 }
 
-// Give back the workspaces that a call can do without (what large calls on unaligned rows
-// keep, and the block image): true where that freed anything but `b`.
-inline bool release_spare(bp_ctx* c, const Buf* b) {
-  bool any = false;
-  for (Buf* q : {&c->aligned, &c->blkimg}) {
-    if (!q->p || q == b) continue;
-    if (!any && cudaDeviceSynchronize() != cudaSuccess) return false;
-    cudaFree(q->p);
-    *q = Buf{};
-    any = true;
-  }
-  return any;
+// Give back the aligned copy that large calls on unaligned rows keep: true where there was
+// one.  (No captured graph holds it.  The block image stays: a graph may hold that.)
+inline bool release_spare(bp_ctx* c) {
+  if (!c->aligned.p || cudaDeviceSynchronize() != cudaSuccess) return false;
+  cudaFree(c->aligned.p);
+  c->aligned = Buf{};
+  return true;
 }
 
-// ensure() for what a call needs: the spare workspaces make room for it.  Within a call
-// these come first, its own spare ones after them.
+// ensure() for what a call needs: the copy of an earlier call makes room for it.  (A
+// call's own copy comes after everything that it needs.)
 inline cudaError_t ensure(bp_ctx* c, Buf& b, size_t bytes) {
   cudaError_t e = ensure(b, bytes);
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
-    if (release_spare(c, &b)) e = ensure(b, bytes);
+    if (release_spare(c)) e = ensure(b, bytes);
   }
   return e;
 }

@@ -227,7 +227,7 @@ int bp_job_create(bp_ctx* ctx, const void* proj, const bp_proj_desc* pdesc, cons
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return cuda_fail(ctx, cudaGetLastError(), "meminfo");
     avail = (long long)fr - (256LL << 20);
-    if (L.total > avail && release_spare(ctx, nullptr) && cudaMemGetInfo(&fr, &tot) == cudaSuccess)
+    if (L.total > avail && release_spare(ctx) && cudaMemGetInfo(&fr, &tot) == cudaSuccess)
       avail = (long long)fr - (256LL << 20);
   }
   if (L.total > avail)
@@ -247,7 +247,7 @@ int bp_job_create(bp_ctx* ctx, const void* proj, const bp_proj_desc* pdesc, cons
   cudaError_t e = cudaStreamCreateWithFlags(&j->own, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&j->done, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMallocAsync(&j->base, (size_t)L.total, j->own);
-  if (e == cudaErrorMemoryAllocation && release_spare(ctx, nullptr)) {
+  if (e == cudaErrorMemoryAllocation && release_spare(ctx)) {
     cudaGetLastError();
     e = cudaMallocAsync(&j->base, (size_t)L.total, j->own);
   }

@@ -14,6 +14,9 @@
 // 1.5*2^23, bilinear interpolation with FP32 lerps (hardware texture filtering is
 // not used: its weights are 8-bit fixed point).
 //
+// The forward is in bp_forward.cu, the motion VJP in bp_vjp.cuh; here are the gradient
+// images, the choice of the VJP's variant and the stand-alone data VJP.
+//
 // What bounds them (ncu, 256^3 x 128 views): no unit alone.  The L1 data pipe is at
 // 75 % (forward) and 74 % (motion VJP: 12 taps per voxel-view at 1.4 wavefronts),
 // issue at 62 and 59 % (21 and 51 instructions per voxel-view), the FMA pipe at 57 and
@@ -141,9 +144,11 @@ cudaError_t prepare_vjp_t();
 // near BP_VJP_CHUNK_MIB, at most 32 views (c2, fused VJP before the block image:
 // 16 MiB 23.1 ms, 32 MiB 20.3 ms, 64 MiB 18.1 ms, 128 MiB 17.4 ms).  Small ones:
 // one wave of CTAs (a CTA's views are a serial chain) up to ten views each, then
-// at least three waves, so that the last one is not a large part (motion VJP
-// with 32 / 16 / 8 / 4 views per chunk, in a step of 60 views: 96^3 voxels 467 /
-// 438 / 430 / 440 us, 32^3 268 / 231 / 212 / 204 us).
+// at least eight views (from 1.25 waves on) until there are three waves, so that the
+// last one is not a large part (motion VJP with 32 / 16 / 8 / 4 views per chunk, in a
+// step of 60 views: 96^3 voxels 467 / 438 / 430 / 440 us, 32^3 268 / 231 / 212 / 204 us).
+// The stand-alone data VJP takes the same rule (with / without it, us: 32^3 x 60 39 / 113,
+// 64^3 x 248 251 / 290, 96^3 x 120 341 / 364, 128^3 x 248 and larger the same).
 constexpr int VJP_WAVE = 152 * VJP_MINB;
 static int view_chunk(const ProjInfo& pi, long long bytes_per_px, int ntiles) {
   const long long per_view = (long long)pi.nu * pi.nv * bytes_per_px;

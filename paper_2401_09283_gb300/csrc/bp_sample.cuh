@@ -360,9 +360,9 @@ __device__ __forceinline__ void setup_batch(TileView* tvs, const ViewGeom* __res
   if (!EARLY) tvs[b] = t;
 }
 
-// The same as a call, for the forward: inlined three times it took registers from the
-// sample loop (3.43 against 3.46 ms on 256^3 x 248).  The VJP inlines it: as a call,
-// or left to the compiler, its loop spilled (11.1 against 9.6 ms).
+// The same as a call, for the forward: inlined, at three places or at one, it took
+// registers from the sample loop (3.26 against 3.41 to 3.55 ms on 256^3 x 248).  The VJP
+// inlines it at one place (bp_vjp.cuh).
 template <typename G, bool STAGE>
 __device__ __noinline__ void setup_batch_call(TileView* tvs, const ViewGeom* __restrict__ geom,
                                               int j0, int nb, const TileIdx& ti, int nu, int nv) {
