@@ -197,17 +197,24 @@ bool stage_aligned(const void* proj, int dtype, const ProjInfo& pi) {
   return ((reinterpret_cast<uintptr_t>(proj) & 15) == 0) && (pi.rs * es) % 16 == 0 &&
          (pi.vs * es) % 16 == 0 && pi.vs * es < (1LL << 40);
 }
-template <typename U>
+// One CTA per detector row, or, where each reads the view flags first (CHOOSE), CTAs that
+// loop over rows.
+template <typename U, bool CHOOSE>
 __global__ void __launch_bounds__(256)
     align_rows_kernel(const U* __restrict__ src, ProjInfo pi, U* __restrict__ dst, long long rs,
                       const int* __restrict__ wide) {
-  if (wide && all_wide(wide, pi.nviews)) return;
-  const long long rows = (long long)pi.nviews * pi.nv;
-  for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
+  auto copy = [&](long long row) {
     const long long j = row / pi.nv, b = row - j * pi.nv;
     const U* p = src + j * pi.vs + b * pi.rs;
     U* q = dst + row * rs;
     for (int a = threadIdx.x; a < pi.nu; a += blockDim.x) q[a] = p[a];
+  };
+  if constexpr (CHOOSE) {
+    if (all_wide(wide, pi.nviews)) return;
+    const long long rows = (long long)pi.nviews * pi.nv;
+    for (long long row = blockIdx.x; row < rows; row += gridDim.x) copy(row);
+  } else {
+    copy(blockIdx.x);
   }
 }
 
@@ -215,15 +222,17 @@ cudaError_t launch_align_rows(const void* proj, int dtype, const ProjInfo& pi, v
                               long long rs, const int* wide, cudaStream_t s) {
   const long long rows = (long long)pi.nviews * pi.nv;
   if (rows <= 0 || pi.nu <= 0) return cudaSuccess;
-  // CTAs loop over rows where each reads the flags first, else one CTA per row
-  const unsigned ctas =
-      (unsigned)(wide ? (rows < 152 * 16 ? rows : 152 * 16) : (rows < 0x7fffffff ? rows : 0x7fffffff));
+  if (rows > 0x7fffffffLL) return cudaErrorInvalidValue;
+  const unsigned ctas = (unsigned)(wide && rows > 152 * 16 ? 152 * 16 : rows);
+  auto run = [&](auto* kernel, auto* src, auto* to) {
+    kernel<<<ctas, 256, 0, s>>>(src, pi, to, rs, wide);
+    return cudaGetLastError();
+  };
   if (dtype == 0)
-    align_rows_kernel<<<ctas, 256, 0, s>>>((const unsigned*)proj, pi, (unsigned*)dst, rs, wide);
-  else
-    align_rows_kernel<<<ctas, 256, 0, s>>>((const unsigned short*)proj, pi, (unsigned short*)dst, rs,
-                                           wide);
-  return cudaGetLastError();
+    return run(wide ? align_rows_kernel<unsigned, true> : align_rows_kernel<unsigned, false>,
+               (const unsigned*)proj, (unsigned*)dst);
+  return run(wide ? align_rows_kernel<unsigned short, true> : align_rows_kernel<unsigned short, false>,
+             (const unsigned short*)proj, (unsigned short*)dst);
 }
 
 void stage_extent(int dtype, bool half, int* cols, int* rows) {

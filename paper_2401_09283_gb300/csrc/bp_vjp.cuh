@@ -447,6 +447,12 @@ __device__ __forceinline__ Sums6 vjp_view_edge2(unsigned buf, float* pout, float
   return Sums6{{S[0], S[1], S[2]}, {Z[0], Z[1], Z[2]}};
 }
 
+// Whether scatters go to the block image (see vjp_view_central2).
+template <int BLK>
+__device__ __forceinline__ bool to_blocks(const float* qout) {
+  return BP_VJP_BLOCKS && (BLK == 1 || (BLK == 2 && qout));
+}
+
 // The CENTRAL sample loop from a staged central-safe footprint with packed
 // pairs of voxels (k, k+1): the steps of vjp_view in the same order on
 // f32x2 pairs, with the w-component kept negated (na2 = -a2) so that no
@@ -454,9 +460,11 @@ __device__ __forceinline__ Sums6 vjp_view_edge2(unsigned buf, float* pout, float
 // halves of the pair accumulators and added at the end.  ZS slices from dz = zlo on,
 // dcol their upstream gradients.
 // With SEQ the sums are taken sample by sample instead, on top of S and Z.
-// BLK: the fused data VJP goes to the block image qout (a test of qout per sample took
-// three instructions of about 80).
-template <int ZS, typename G, bool FDK, bool PROJ, bool LINES, bool SEQ, bool BLK>
+// BLK: whether the fused data VJP goes to the block image qout: 0 or 1, or 2, a test per
+// sample.  That takes three instructions of about 80, but one copy of the body: with four
+// slots, where there is one CTA per SM or two, two copies spilled (32^3 x 60 views, both
+// gradients, 38.0 against 36.3 us).
+template <int ZS, typename G, bool FDK, bool PROJ, bool LINES, bool SEQ, int BLK>
 __device__ __forceinline__ void vjp_view_central2(unsigned buf, float* pout, float* qout, int nu,
                                                   int nv, const TileView& t, float dx, float dy,
                                                   const float* dcol, float zlo,
@@ -556,7 +564,7 @@ __device__ __forceinline__ void vjp_view_central2(unsigned buf, float* pout, flo
 #endif
         // (iv * nu + iu) from the floor bits, in 32-bit wraparound arithmetic
         const unsigned px = (unsigned)byi * (unsigned)nu + (unsigned)bxi + pofs;
-        if (BLK) {  // one vector reduction into the block image
+        if (to_blocks<BLK>(qout)) {  // one vector reduction into the block image
           red_v4(block_at(qout, px), w[0][h], w[1][h], w[2][h], w[3][h]);
           continue;
         }
@@ -598,7 +606,7 @@ __device__ __forceinline__ void vjp_view_central2(unsigned buf, float* pout, flo
 // consecutive voxels (f32x2), as in the motion loop.  Exact to rounding: the
 // same weights, summed in another order.  dsm holds the tile's dL/dvol as
 // [z][y][x] with a row pitch of TX + 1.
-template <int ZB, bool FDK, bool BLK>
+template <int ZB, bool FDK, int BLK>
 __device__ __forceinline__ void proj_lines(float* __restrict__ pout, float* __restrict__ qout,
                                            int nu, int nv, const TileView& t,
                                            const float* __restrict__ dsm) {
@@ -670,7 +678,7 @@ __device__ __forceinline__ void proj_lines(float* __restrict__ pout, float* __re
       const bool keep = have && bx == cb && by == rb;
       if (have && !keep) {  // the line leaves the open cell: add its four pixels
         const unsigned px = pixel(cb, rb);
-        if (BLK) {
+        if (to_blocks<BLK>(qout)) {
           red_v4(block_at(qout, px), a0, a1, b0, b1);
         } else {
           float* q = pout + px;
@@ -690,7 +698,7 @@ __device__ __forceinline__ void proj_lines(float* __restrict__ pout, float* __re
     }
   }
   const unsigned px = pixel(cb, rb);
-  if (BLK) {
+  if (to_blocks<BLK>(qout)) {
     red_v4(block_at(qout, px), a0, a1, b0, b1);
     return;
   }
@@ -706,7 +714,7 @@ __device__ __forceinline__ void proj_lines(float* __restrict__ pout, float* __re
 // (central-safe) tiles run the packed motion loop and, when the data VJP is fused,
 // the line pass above; the other tiles scatter the data VJP per sample.  ZS slices
 // from dz = zlo on, dcol their upstream gradients.
-template <int ZB, int ZS, typename T, bool FDK, bool EXACT, bool PROJ, int STAGE>
+template <int ZB, int ZS, int NS, typename T, bool FDK, bool EXACT, bool PROJ, int STAGE>
 __device__ __forceinline__ void vjp_tile_view(const T* img, const float2* gimg, unsigned buf,
                                               bool staged, float* pout, float* qout,
                                               const ProjInfo& pi, const TileView& t,
@@ -733,18 +741,22 @@ __device__ __forceinline__ void vjp_tile_view(const T* img, const float2* gimg, 
     // four atomics per sample from the packed loop, with fewer instructions
     if constexpr (PROJ) {
       if (BP_VJP_LINES && fminf(fabsf(t.ru0), fabsf(t.ru1)) <= BP_VJP_LINE_DU * t.W0) {
-        vjp_view_central2<ZB, G, FDK, false, PROJ, false, false>(
+        vjp_view_central2<ZB, G, FDK, false, PROJ, false, 0>(
             buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy, dcol, zlo, S, Z);
-        if (BP_VJP_BLOCKS && qout) proj_lines<ZB, FDK, true>(pout, qout, pi.nu, pi.nv, t, dsm);
-        else proj_lines<ZB, FDK, false>(pout, qout, pi.nu, pi.nv, t, dsm);
+        if (NS > VJP_NS) proj_lines<ZB, FDK, 2>(pout, qout, pi.nu, pi.nv, t, dsm);
+        else if (BP_VJP_BLOCKS && qout) proj_lines<ZB, FDK, 1>(pout, qout, pi.nu, pi.nv, t, dsm);
+        else proj_lines<ZB, FDK, 0>(pout, qout, pi.nu, pi.nv, t, dsm);
         return;
       }
     }
-    if (PROJ && BP_VJP_BLOCKS && qout)
-      vjp_view_central2<ZS, G, FDK, PROJ, PROJ, ZS != ZB, PROJ>(
+    if constexpr (PROJ && NS > VJP_NS)
+      vjp_view_central2<ZS, G, FDK, PROJ, PROJ, ZS != ZB, 2>(
+          buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy, dcol, zlo, S, Z);
+    else if (PROJ && BP_VJP_BLOCKS && qout)
+      vjp_view_central2<ZS, G, FDK, PROJ, PROJ, ZS != ZB, PROJ ? 1 : 0>(
           buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy, dcol, zlo, S, Z);
     else
-      vjp_view_central2<ZS, G, FDK, PROJ, PROJ, ZS != ZB, false>(
+      vjp_view_central2<ZS, G, FDK, PROJ, PROJ, ZS != ZB, 0>(
           buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy, dcol, zlo, S, Z);
   } else if (!EXACT && staged) {
     take(vjp_view_edge2<ZS, G, FDK, PROJ>(buf, pout, qout, pi.nu, pi.nv, t, ti.dx, ti.dy, dcol, zlo,
@@ -932,10 +944,11 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
   for (int idx = 0; idx < nst; ++idx) {
     const int v = vbeg + idx / HALVES, half = idx % HALVES, k = idx / NB, b = idx - k * NB;
     if (b == 0 && (STAGE || k >= 1)) {
-      __syncthreads();  // every warp is done with batch k-1, its records are written
-      if (CONV && warp == 0 && k >= 1)  // (the barrier path writes them one step late)
-        record(idx - 1, bad);
-      if (CONV) __syncthreads();
+      if (k >= 1) {
+        __syncthreads();  // every warp is done with batch k-1, its records are written
+        if (CONV && warp == 0) record(idx - 1, bad);  // (the barrier path writes them one late)
+        if (CONV) __syncthreads();
+      }
 #pragma unroll 1
       for (int q = k ? k + 1 : 0; q <= k + 1 && q < nbatch; ++q) setup(q);
       __syncthreads();
@@ -971,7 +984,7 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
       float* pout = PROJ ? dproj + (long long)v * pi.nv * pi.nu : nullptr;
       float* qout =
           PROJ && dblk ? dblk + (long long)v * 4 * pi.nv * pi.nu : nullptr;
-      vjp_tile_view<ZB, ZS, T, FDK, EXACT, PROJ, STAGE>(
+      vjp_tile_view<ZB, ZS, NS, T, FDK, EXACT, PROJ, STAGE>(
           img, gimg, smem_addr(CONV ? dyn_smem : buf), STAGE && t.staged, pout, qout, pi, t, ti,
           half * ZS - 0.5f * (ZB - 1), delta, dcol + delta_off<PROJ>(half * ZS), finite, dsm, S, Z);
       if (HALVES == 1) vjp_reduce(ti, S, Z, red[slot][warp]);
@@ -1082,7 +1095,6 @@ cudaError_t prepare_vjp_t() {
         vjp_smem_bytes<T, VJP_NS_FEW, EXACT, false>());
   return e;
 }
-
 
 #define BP_VJP_VARIANT(T, FDK, EXACT, PROJ)                                                       \
   template cudaError_t vjp_variants<T, FDK, EXACT, PROJ>(                                         \
