@@ -18,9 +18,9 @@
 // images, the choice of the VJP's variant and the stand-alone data VJP.
 //
 // What bounds them (ncu, 256^3 x 128 views): no unit alone.  The L1 data pipe is at
-// 75 % (forward) and 74 % (motion VJP: 12 taps per voxel-view at 1.4 wavefronts),
-// issue at 62 and 59 % (21 and 51 instructions per voxel-view), the FMA pipe at 57 and
-// 50 %, with the 32 and 24 warps per SM that their registers allow.
+// 72 % (forward) and 73 % (motion VJP: 12 taps per voxel-view at 1.4 wavefronts),
+// issue at 66 and 61 % (21 and 51 instructions per voxel-view), the FMA pipe at 59 and
+// 51 %, with the 32 and 24 warps per SM that their registers allow.
 #include "bp_scatter.cuh"
 
 namespace bpk {
@@ -147,7 +147,7 @@ cudaError_t prepare_vjp_t();
 // at least eight views (from 1.25 waves on) until there are three waves, so that the
 // last one is not a large part (motion VJP with 32 / 16 / 8 / 4 views per chunk, in a
 // step of 60 views: 96^3 voxels 467 / 438 / 430 / 440 us, 32^3 268 / 231 / 212 / 204 us).
-// The stand-alone data VJP takes the same rule (with / without it, us: 32^3 x 60 39 / 113,
+// The stand-alone data VJP takes the same rule (now / before it, us: 32^3 x 60 39 / 113,
 // 64^3 x 248 251 / 290, 96^3 x 120 341 / 364, 128^3 x 248 and larger the same).
 constexpr int VJP_WAVE = 152 * VJP_MINB;
 static int view_chunk(const ProjInfo& pi, long long bytes_per_px, int ntiles) {
