@@ -912,6 +912,12 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
       partials[((long long)(vbeg + e / PSLOTS) * ntiles + tile) * PSLOTS + e % PSLOTS] = 0.0f;
     return;
   }
+  // Where the records are made decides how many registers spill: at one place inside the
+  // loop with two slots (at three places 9.62 against 9.34 ms for the 256^3 x 248 motion
+  // VJP), before it and inside without staging (2.28 against 2.17 ms for 128^3 x 200 at
+  // 4.8 px per voxel) and with four slots, which have registers to spare (32^3 x 60 motion
+  // 47.2 against 45.4 us).
+  constexpr bool BEFORE = STAGE == STAGE_NONE || NS > VJP_NS;
   auto setup = [&](int k) {  // the records of batch k
     auto records = [&](const TileIdx& box) {
       setup_batch<G, STAGE != STAGE_NONE, HALVES, EXACT>(
@@ -920,7 +926,7 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
     };
     // (the box again, not kept over the sample loop: no spills in the motion kernel,
     // 9.34 against 9.19 ms; the fused one has them elsewhere, and more with it)
-    if constexpr (PROJ || EXACT || STAGE == STAGE_NONE) records(ti);
+    if constexpr (PROJ || EXACT || BEFORE) records(ti);
     else records(tile_index<ZB>(vi, tile));
   };
   // the record of step x's view (x is the view's last step)
@@ -930,20 +936,20 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
     if (HALVES == 2) live = live || q[-1].mode != MODE_SKIP;
     vjp_write_record(*q, live, red[x % NS], bad, lane, vbeg + x / HALVES, tile, ntiles, partials);
   };
-  // Where the records are made decides how many registers spill: at one place inside the
-  // loop with staging (at three places 9.62 against 9.34 ms for the 256^3 x 248 motion
-  // VJP), at two without (2.28 against 2.17 ms for 128^3 x 200 at 4.8 px per voxel).
-  if constexpr (STAGE == STAGE_NONE) {
+  if constexpr (BEFORE) {
 #pragma unroll 1
     for (int k = 0; k < min(2, nbatch); ++k) setup(k);
     __syncthreads();
+    if (STAGE && warp < NS && warp < nst)
+      stage_issue<G>(slots + warp * SLOT, map, tvs[0][warp], vbeg + warp / HALVES,
+                     &pipe.full[warp]);
   }
   bool bad = false;
   PipePos<NS> pos;
   float S[3], Z[3];
   for (int idx = 0; idx < nst; ++idx) {
     const int v = vbeg + idx / HALVES, half = idx % HALVES, k = idx / NB, b = idx - k * NB;
-    if (b == 0 && (STAGE || k >= 1)) {
+    if (b == 0 && (!BEFORE || k >= 1)) {
       if (k >= 1) {
         __syncthreads();  // every warp is done with batch k-1, its records are written
         if (CONV && warp == 0) record(idx - 1, bad);  // (the barrier path writes them one late)
@@ -952,7 +958,7 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
 #pragma unroll 1
       for (int q = k ? k + 1 : 0; q <= k + 1 && q < nbatch; ++q) setup(q);
       __syncthreads();
-      if (STAGE && k == 0 && warp < NS && warp < nst)
+      if (STAGE && !BEFORE && k == 0 && warp < NS && warp < nst)
         stage_issue<G>(slots + warp * SLOT, map, tvs[0][warp], vbeg + warp / HALVES,
                        &pipe.full[warp]);
     }
