@@ -463,7 +463,7 @@ __device__ __forceinline__ f2 bilerp2(f2 tu, f2 tv, f2 d00, f2 d10, f2 d01, f2 d
 // Every warp waits on full[s] for every view, staged or not: it may then be at
 // most one phase behind, which the parity tells apart.
 //
-// A warp whose wait runs out (a copy that never arrives) is bad: it no longer counts
+// A warp whose wait runs out (a copy that never arrives; in any lane) is bad: it no longer counts
 // itself as finished, so that no slot is refilled from that step on and the other warps
 // run out of time too, where they need more; what it computes from there on shows as
 // NaN; and it stays for the copies that may still be in flight (pipe_drain).
