@@ -115,7 +115,10 @@ __device__ __forceinline__ void forward_tile(const T* __restrict__ proj, const C
     const TileView& t = tvs[k & 1][b];
     const unsigned slot = pos.slot;
     unsigned char* buf = slots + slot * SLOT;
-    if (STAGE && !bad) bad = !__all_sync(0xffffffffu, mbar_wait(&pipe.full[slot], pos.parity));
+    if (STAGE && !bad) {  // (the lanes poll on their own; with CONV the CTA votes below)
+      const bool ok = mbar_wait(&pipe.full[slot], pos.parity);
+      bad = CONV ? !ok : !__all_sync(0xffffffffu, ok);
+    }
     pos.next();
     const int vn = v + NS;
     const TileView& tn = tvs[(vn / NB) & 1][vn % NB];

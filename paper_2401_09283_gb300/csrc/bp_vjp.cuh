@@ -965,7 +965,10 @@ __device__ __forceinline__ void vjp_item(const float* __restrict__ dvol, const T
     const TileView& t = tvs[k & 1][b];
     const unsigned slot = pos.slot;
     unsigned char* buf = slots + slot * SLOT;
-    if (STAGE && !bad) bad = !__all_sync(0xffffffffu, mbar_wait(&pipe.full[slot], pos.parity));
+    if (STAGE && !bad) {  // (the lanes poll on their own; with CONV the CTA votes below)
+      const bool ok = mbar_wait(&pipe.full[slot], pos.parity);
+      bad = CONV ? !ok : !__all_sync(0xffffffffu, ok);
+    }
     pos.next();
     const int in = idx + NS;
     const TileView& tn = tvs[(in / NB) & 1][in % NB];
